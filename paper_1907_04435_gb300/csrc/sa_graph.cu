@@ -35,24 +35,6 @@ constexpr int kGraphThreads = 256;
 constexpr int kGather = 8;        // summaries a thread loads ahead in the walk
 constexpr int kWalkTile = 2048;   // walk codes staged in shared memory at a time
 
-// Longest run of ones in x, which is not all ones.  With A_k the bits i at which a run of
-// at least k ones starts (A_1 = x, A_{a+b} = A_a & (A_b >> a)), the longest run is the
-// largest n with A_n != 0; it is found bit by bit from 32 down, since it is below 64.
-__device__ __forceinline__ unsigned longest_run(unsigned long long x) {
-    const unsigned long long a1 = x, a2 = a1 & (a1 >> 1), a4 = a2 & (a2 >> 2), a8 = a4 & (a4 >> 4),
-                             a16 = a8 & (a8 >> 8), a32 = a16 & (a16 >> 16);
-    unsigned long long cur = ~0ull;   // A_0
-    unsigned n = 0;
-    unsigned long long c;
-    c = cur & (a32 >> n); if (c) { cur = c; n += 32; }
-    c = cur & (a16 >> n); if (c) { cur = c; n += 16; }
-    c = cur & (a8 >> n);  if (c) { cur = c; n += 8; }
-    c = cur & (a4 >> n);  if (c) { cur = c; n += 4; }
-    c = cur & (a2 >> n);  if (c) { cur = c; n += 2; }
-    c = cur & (a1 >> n);  if (c) { n += 1; }
-    return n;
-}
-
 // grid: x over receivers, y over edges (strided)
 __global__ void k_edge_summary(const unsigned long long* __restrict__ masks, long long R, int n_edges,
                                const int* __restrict__ edge_K, unsigned* __restrict__ summary) {
@@ -63,21 +45,7 @@ __global__ void k_edge_summary(const unsigned long long* __restrict__ masks, lon
         unsigned* __restrict__ se = summary + (long long)e * R;
         for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < R;
              r += (long long)gridDim.x * blockDim.x) {
-            const unsigned long long m = me[r] & low;
-            if (m == 0ull) {            // lit at every step: the most common case
-                se[r] = 0u;
-                continue;
-            }
-            const unsigned pop = (unsigned)__popcll(m);
-            unsigned pre, suf, best;
-            if (pop == (unsigned)K) {
-                pre = suf = best = (unsigned)K;
-            } else {
-                pre = (unsigned)(__ffsll((long long)~m) - 1);            // ones below the first zero
-                suf = (unsigned)__clzll((long long)~(m << (64 - K)));   // ones above the last zero
-                best = longest_run(m);
-            }
-            se[r] = pop | (pre << 8) | (suf << 16) | (best << 24);
+            se[r] = run_summary(me[r] & low, K);
         }
     }
 }

@@ -302,6 +302,40 @@ __device__ __forceinline__ void stitch(RunState& s, uint64_t m, int K, int new_d
     s.run = suffix;
 }
 
+// Longest run of ones in x, which is not all ones.  With A_k the bits i at which a run of
+// at least k ones starts (A_1 = x, A_{a+b} = A_a & (A_b >> a)), the longest run is the
+// largest n with A_n != 0; it is found bit by bit from 32 down, since it is below 64.
+__device__ __forceinline__ unsigned longest_run(unsigned long long x) {
+    const unsigned long long a1 = x, a2 = a1 & (a1 >> 1), a4 = a2 & (a2 >> 2), a8 = a4 & (a4 >> 4),
+                             a16 = a8 & (a8 >> 8), a32 = a16 & (a16 >> 16);
+    unsigned long long cur = ~0ull;   // A_0
+    unsigned n = 0;
+    unsigned long long c;
+    c = cur & (a32 >> n); if (c) { cur = c; n += 32; }
+    c = cur & (a16 >> n); if (c) { cur = c; n += 16; }
+    c = cur & (a8 >> n);  if (c) { cur = c; n += 8; }
+    c = cur & (a4 >> n);  if (c) { cur = c; n += 4; }
+    c = cur & (a2 >> n);  if (c) { cur = c; n += 2; }
+    c = cur & (a1 >> n);  if (c) { n += 1; }
+    return n;
+}
+
+// A block's step mask (K steps, no bit beyond them) in 32 bits: its count, leading run
+// (from bit 0), trailing run (down from bit K - 1) and longest run, 8 bits each.
+__device__ __forceinline__ unsigned run_summary(unsigned long long m, int K) {
+    if (m == 0ull) return 0u;            // lit at every step: the most common case
+    const unsigned pop = (unsigned)__popcll(m);
+    unsigned pre, suf, best;
+    if (pop == (unsigned)K) {
+        pre = suf = best = (unsigned)K;
+    } else {
+        pre = (unsigned)(__ffsll((long long)~m) - 1);            // ones below the first zero
+        suf = (unsigned)__clzll((long long)~(m << (64 - K)));   // ones above the last zero
+        best = longest_run(m);
+    }
+    return pop | (pre << 8) | (suf << 16) | (best << 24);
+}
+
 // ------------------------------------------------------------------ float helpers
 template <int A> __device__ __forceinline__ float comp(const float4& v);
 template <> __device__ __forceinline__ float comp<0>(const float4& v) { return v.x; }
@@ -510,9 +544,14 @@ cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const De
 // traversal mode of the sweep (which = 0) and accrual (which = 1) kernels
 void set_trace_mode(int which, int mode);
 int get_trace_mode(int which);
-// ground raster; `sun` may be the per-step partition (K = 1 blocks) for SA_SWEEP_RASTER
+// ground raster; `sun` may be the per-step partition (K = 1 blocks) for SA_SWEEP_RASTER;
+// out.gross may be null when only the masks are wanted
 cudaError_t launch_raster_ground(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
                                  const DevOut& out, cudaStream_t st);
+
+// the run summary (run_summary) of every block and cell: summaries [n_blocks][R]
+cudaError_t launch_raster_summaries(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
+                                    unsigned* summaries, cudaStream_t st);
 
 // Extruded convex footprints kept on the device (scenes built from footprints).
 struct FootprintSet {

@@ -10,18 +10,23 @@
 // receivers themselves, as one bit per step: no texel resampling, no aliasing, no bias.
 //
 // Per block of <= 64 steps:
-//   k_bin_count / k_bin_fill  one pass over the triangles bins each into the 32 x 32-cell
-//                             tiles its projection can reach during the block (the
-//                             triangle swept along the block's slope box)
-//   k_raster                  one CTA per tile keeps the tile's 1024 x 64-bit slices in
-//                             registers, projects each binned triangle for every step of
-//                             the block and sets bit k of each covered cell; the gross /
-//                             continuous reduction is fused into the epilogue.
+//   k_bin             one pass over the triangles bins each into the 32 x 32-cell tiles its
+//                     projection can reach during the block (the triangle swept along the
+//                     block's slope box)
+//   k_raster_items    one CTA per tile and block keeps the tile's 1024 x 64-bit slices in
+//                     shared memory, projects each binned triangle for every step of the
+//                     block, sets bit k of each covered cell and leaves each cell's run
+//                     summary
+//   k_items_fold      stitches the summaries into the gross / continuous counts
+//   k_raster          one CTA per tile, its blocks in series, the reduction fused (the raster
+//                     in fixed scratch, and the per-step raster of a large grid)
 // With one step per block the same kernels form the per-step shadow raster baseline.
 //
 // Coverage is decided with edge functions evaluated from canonically ordered endpoints,
 // so an edge shared by two projected triangles yields exactly negated values in the two
 // and a cell centre on it is covered by at least one (watertight).
+#include <algorithm>
+
 #include "sa_internal.cuh"
 
 namespace sa {
@@ -84,56 +89,70 @@ __device__ __forceinline__ bool swept_tiles(const float4& a, const float4& b, co
 
 // For a closed scene only triangles facing the sun at some step of the block cast the
 // shadow's coverage (the projection of a closed solid is covered by its sun-facing faces).
-__device__ __forceinline__ bool faces_sun(const float4& a, const float4& b, const float4& c,
-                                          const StepConst* steps, const BlockConst& bc) {
-    const float ux = b.x - a.x, uy = b.y - a.y, uz = b.z - a.z;
-    const float vx = c.x - a.x, vy = c.y - a.y, vz = c.z - a.z;
-    const float nx = uy * vz - uz * vy, ny = uz * vx - ux * vz, nz = ux * vy - uy * vx;
+// n: the triangle's unnormalised normal.  The bounds of n . d over the block's direction
+// box decide most triangles without the loop over its steps; 1e-5 |n|_1 is far more than
+// the rounding of either (3 ulp), so the answer is the loop's.
+__device__ __forceinline__ bool faces_sun(const float3& n, const StepConst* steps, const BlockConst& bc) {
+    const float hi = fmaxf(n.x * bc.dlo[0], n.x * bc.dhi[0]) + fmaxf(n.y * bc.dlo[1], n.y * bc.dhi[1]) +
+                     fmaxf(n.z * bc.dlo[2], n.z * bc.dhi[2]);
+    const float lo = fminf(n.x * bc.dlo[0], n.x * bc.dhi[0]) + fminf(n.y * bc.dlo[1], n.y * bc.dhi[1]) +
+                     fminf(n.z * bc.dlo[2], n.z * bc.dhi[2]);
+    const float tol = 1e-5f * (fabsf(n.x) + fabsf(n.y) + fabsf(n.z));
+    if (hi < -tol) return false;
+    if (lo > tol) return true;
     for (int k = 0; k < bc.K; ++k) {
         const StepConst& s = steps[bc.j0 + k];
-        if (nx * s.dx + ny * s.dy + nz * s.dz > 0.f) return true;
+        if (n.x * s.dx + n.y * s.dy + n.z * s.dz > 0.f) return true;
     }
     return false;
 }
 
-__global__ void k_bin_count(DevScene sc, const StepConst* __restrict__ steps,
-                            const BlockConst* __restrict__ blocks, int b0,
-                            TileGeom g, unsigned* __restrict__ counts) {
+// Bins of blocks [b0, b0 + nbc): a thread loads its triangle once and takes `per` of the
+// blocks (blockIdx.y picks which), so a season's blocks do not read the mesh again each.
+// Counting (FILL false) adds to counts[block][tile]; filling writes the triangle at
+// offsets[block][tile], or at a fixed place of `cap` triangles per bin when offsets is
+// null (a mesh so small that every bin can hold all of it: one pass, nothing to size).
+template <bool FILL>
+__global__ void k_bin(DevScene sc, const StepConst* __restrict__ steps,
+                      const BlockConst* __restrict__ blocks, int b0, int nbc, int per, TileGeom g,
+                      const unsigned* __restrict__ offsets, unsigned cap,
+                      unsigned* __restrict__ counts, int* __restrict__ bins) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int bl = blockIdx.y;
     if (t >= sc.T) return;
     const float4 a = __ldg(&sc.tris[3 * t]), b = __ldg(&sc.tris[3 * t + 1]),
                  c = __ldg(&sc.tris[3 * t + 2]);
     if (!tri_above_ground(a, b, c)) return;
-    // the tile range first: it culls the triangles whose shadow misses the grid before the
-    // per-step facing test (both are conservative, so the order leaves the bins unchanged)
-    int tx0, tx1, ty0, ty1;
-    if (!swept_tiles(a, b, c, blocks[b0 + bl], g, &tx0, &tx1, &ty0, &ty1)) return;
-    if (sc.closed && !faces_sun(a, b, c, steps, blocks[b0 + bl])) return;
-    unsigned* row = counts + (size_t)bl * g.tiles_x * g.tiles_y;
-    for (int ty = ty0; ty <= ty1; ++ty)
-        for (int tx = tx0; tx <= tx1; ++tx) atomicAdd(&row[ty * g.tiles_x + tx], 1u);
+    const float ux = b.x - a.x, uy = b.y - a.y, uz = b.z - a.z;
+    const float vx = c.x - a.x, vy = c.y - a.y, vz = c.z - a.z;
+    const float3 n = make_float3(uy * vz - uz * vy, uz * vx - ux * vz, ux * vy - uy * vx);
+    const int bl0 = blockIdx.y * per, bl1 = min(nbc, bl0 + per);
+    for (int bl = bl0; bl < bl1; ++bl) {
+        const BlockConst& bc = blocks[b0 + bl];
+        // the tile range first: it culls the triangles whose shadow misses the grid before
+        // the facing test (both are conservative, so the order leaves the bins unchanged)
+        int tx0, tx1, ty0, ty1;
+        if (!swept_tiles(a, b, c, bc, g, &tx0, &tx1, &ty0, &ty1)) continue;
+        if (sc.closed && !faces_sun(n, steps, bc)) continue;
+        const size_t row = (size_t)bl * g.tiles_x * g.tiles_y;
+        for (int ty = ty0; ty <= ty1; ++ty)
+            for (int tx = tx0; tx <= tx1; ++tx) {
+                const size_t cell = row + ty * g.tiles_x + tx;
+                const unsigned slot = atomicAdd(&counts[cell], 1u);
+                if (FILL) bins[(offsets ? (size_t)offsets[cell] : cell * cap) + slot] = t;
+            }
+    }
 }
 
-__global__ void k_bin_fill(DevScene sc, const StepConst* __restrict__ steps,
-                           const BlockConst* __restrict__ blocks, int b0,
-                           TileGeom g, const unsigned* __restrict__ offsets,
-                           unsigned* __restrict__ cursor, int* __restrict__ bins) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int bl = blockIdx.y;
-    if (t >= sc.T) return;
-    const float4 a = __ldg(&sc.tris[3 * t]), b = __ldg(&sc.tris[3 * t + 1]),
-                 c = __ldg(&sc.tris[3 * t + 2]);
-    if (!tri_above_ground(a, b, c)) return;
-    int tx0, tx1, ty0, ty1;
-    if (!swept_tiles(a, b, c, blocks[b0 + bl], g, &tx0, &tx1, &ty0, &ty1)) return;
-    if (sc.closed && !faces_sun(a, b, c, steps, blocks[b0 + bl])) return;
-    const size_t row = (size_t)bl * g.tiles_x * g.tiles_y;
-    for (int ty = ty0; ty <= ty1; ++ty)
-        for (int tx = tx0; tx <= tx1; ++tx) {
-            const size_t cell = row + ty * g.tiles_x + tx;
-            bins[offsets[cell] + atomicAdd(&cursor[cell], 1u)] = t;
-        }
+constexpr int kBinThreads = 128;
+
+// Grid of k_bin: enough CTAs for the chip (a few waves) from the triangles alone where the
+// mesh has them, else the blocks are split as well.
+dim3 bin_grid(int T, int nbc, int* per) {
+    const int gx = (T + kBinThreads - 1) / kBinThreads;
+    int gy = std::min(nbc, std::max(1, (152 * 16 + gx - 1) / gx));
+    gy = std::min(gy, 65535);
+    *per = (nbc + gy - 1) / gy;
+    return dim3((unsigned)gx, (unsigned)((nbc + *per - 1) / *per));
 }
 
 struct RasterArgs {
@@ -151,7 +170,10 @@ struct RasterArgs {
     int cull;                        // closed scene: only faces toward the sun
     int run;                         // steps per work unit
     long long R;
-    const int* order;                // tile of each CTA (null: CTA i takes tile i)
+    const int* order;                // tile (item) of each CTA (null: CTA i takes i)
+    unsigned cap;                    // items: triangles per bin when offsets is null
+    int parts;                       // items: parts a block's steps are cut into
+    unsigned* summary;               // items: run summaries [nbc][parts][R] (nullable)
 };
 
 constexpr int kWarpsRaster = kRasterThreads / 32;
@@ -265,6 +287,7 @@ __device__ __forceinline__ void tile_setup(TileSmem& sm, const TileGeom& g, int 
     }
     for (int c = threadIdx.x; c < kTile * kTile; c += kRasterThreads) sm.mask[c] = 0ull;
 }
+
 
 // The steps of one run (kn <= 32 steps from k0) that cover cell (x, y): bit k of the
 // result is step k0 + k.  CULL: closed scene, only front faces count.
@@ -655,8 +678,10 @@ __device__ __forceinline__ void flush_raster_counts(unsigned long long* stats, u
 }
 
 // One CTA per 32 x 32-cell tile, every block of the chunk in order; the gross /
-// continuous state of the thread's four cells stays in registers between blocks.
-template <bool COUNT, bool CULL, int CTAS>
+// continuous state of the tile's cells stays in shared memory between blocks.  It needs no
+// memory per block, so the raster in fixed scratch (launch_raster_ground_in) takes it, and
+// the per-step raster of a large grid; k_raster_items is faster on the rest (below).
+template <bool CULL, int CTAS>
 __global__ void __launch_bounds__(kRasterThreads, CTAS)
 k_raster(RasterArgs ra) {
     __shared__ TileSmem sm;
@@ -687,9 +712,9 @@ k_raster(RasterArgs ra) {
     const float inv_dx = 1.f / g.dx;
     for (int bl = 0; bl < ra.nbc; ++bl) {
         const BlockConst* bcp = &ra.sun.blocks[ra.b0 + bl];
-        const unsigned off = ra.offsets[(size_t)bl * n_tiles + tile];
-        const unsigned cnt = ra.counts[(size_t)bl * n_tiles + tile];
-        const int* bins = ra.bins + off;
+        const size_t bin = (size_t)bl * n_tiles + tile;
+        const unsigned cnt = ra.counts[bin];
+        const int* bins = ra.bins + ra.offsets[bin];
         const float4* tris = ra.sc.tris;
         const int T = ra.sc.T;
         auto fetch = [bins, tris, T](int i, int v, float4* out) {
@@ -697,7 +722,7 @@ k_raster(RasterArgs ra) {
             (void)T;
             return true;
         };
-        raster_block<COUNT, CULL>(sm, fetch, (int)cnt, ra.sun.steps, bcp->j0, bcp->K, tox, toy,
+        raster_block<false, CULL>(sm, fetch, (int)cnt, ra.sun.steps, bcp->j0, bcp->K, tox, toy,
                                   inv_dx, ra.run, n_cell, n_test, n_unit, n_span);
         const int K = bcp->K, new_day = bcp->new_day;
 #pragma unroll
@@ -724,7 +749,115 @@ k_raster(RasterArgs ra) {
         ra.out.run[o] = st.run;
         if (ra.final_chunk && ra.out.minutes) ra.out.minutes[o] = (float)st.gross * ra.out.step_minutes;
     }
+}
+
+// One CTA per item, (block, tile) and one of `parts` consecutive pieces of the block's steps:
+// the items of a small grid's long interval fill the chip where its tiles alone cannot.
+// Each item leaves its cells' run summaries (run_summary, 4 bytes per block and cell), which
+// k_items_fold stitches in time order, and its step masks where they are asked for.
+// Against one CTA per tile with the blocks in series (k_raster), same inputs and bits:
+// 231 x 187 cells, 92 days (56 tiles, 828 blocks) 54.1 -> 4.54 ms; 64^2 cells, one day
+// 216 -> 57 us; 512^2 604 -> 286 us; 2048^2 2.43 -> 2.21 ms (heavy items start first,
+// 23.9 KB of shared memory instead of 35.9); 1024^2 in December 27.5 -> 25.2 ms.
+template <bool COUNT, bool CULL>
+__global__ void __launch_bounds__(kRasterThreads, SA_RASTER_CTAS)
+k_raster_items(RasterArgs ra) {
+    __shared__ TileSmem sm;
+    unsigned long long n_cell = 0, n_test = 0, n_unit = 0, n_span = 0;
+    const TileGeom& g = ra.g;
+    const int n_tiles = g.tiles_x * g.tiles_y;
+    const int item = ra.order ? ra.order[blockIdx.x] : (int)blockIdx.x;
+    const int bl = item / n_tiles, tile = item - bl * n_tiles;
+    const int tx = tile % g.tiles_x, ty = tile / g.tiles_x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int part = blockIdx.y;
+    const BlockConst* bcp = &ra.sun.blocks[ra.b0 + bl];
+    const int k0 = part * bcp->K / ra.parts, K = (part + 1) * bcp->K / ra.parts - k0;
+    const unsigned cnt = ra.counts[item];
+    const int ix = tx * kTile + lane, row0 = warp * 4;
+    if (cnt > 0 && K > 0) {
+        float tox, toy;
+        tile_setup(sm, g, tx, ty, &tox, &toy);
+        const int* bins = ra.bins + (ra.offsets ? (size_t)ra.offsets[item] : (size_t)item * ra.cap);
+        const float4* tris = ra.sc.tris;
+        const int T = ra.sc.T;
+        auto fetch = [bins, tris, T](int i, int v, float4* out) {
+            *out = __ldg(&tris[3 * SA_CHK(bins[i], T, sa::CK_RASTER_BIN) + v]);
+            (void)T;
+            return true;
+        };
+        raster_block<COUNT, CULL>(sm, fetch, (int)cnt, ra.sun.steps, bcp->j0 + k0, K, tox, toy, 1.f / g.dx,
+                                  ra.run, n_cell, n_test, n_unit, n_span);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int iy = ty * kTile + row0 + q;
+        if (ix >= g.nx || iy >= g.ny) continue;
+        const unsigned long long m = (cnt > 0 && K > 0) ? sm.mask[(row0 + q) * kTile + lane] : 0ull;
+        const size_t cell = (size_t)iy * g.nx + ix;
+        if (ra.summary) ra.summary[((size_t)bl * ra.parts + part) * ra.R + cell] = run_summary(m, K);
+        // pieces and one-step blocks share a mask word
+        if (ra.out.masks && m)
+            atomicOr(reinterpret_cast<unsigned long long*>(&ra.out.masks[(size_t)bcp->mask_block * ra.R + cell]),
+                     m << (bcp->mask_bit + k0));
+    }
     if (COUNT) flush_raster_counts(ra.out.stats, n_cell, n_test, n_unit, n_span);
+}
+
+constexpr int kFoldThreads = 128;
+constexpr int kFoldTile = 1024;      // steps-and-day codes staged in shared memory at a time
+constexpr int kFoldAhead = 8;        // summaries a thread loads ahead of their use
+
+// Stitches the chunk's run summaries, in time order, into each cell's gross / continuous
+// state (as stitch does with the masks themselves).
+__global__ void __launch_bounds__(kFoldThreads)
+k_items_fold(const unsigned* __restrict__ summary, long long R, const BlockConst* __restrict__ blocks,
+             int nbc, int parts, DevOut out, int* __restrict__ best, int load_state, int final_chunk) {
+    __shared__ int s_code[kFoldTile];
+    const long long r = (long long)blockIdx.x * kFoldThreads + threadIdx.x;
+    const int n_all = nbc * parts;
+    RunState st{0, 0, 0};
+    if (r < R && load_state) {
+        st.gross = out.gross[r];
+        st.best = best[r];
+        st.run = out.run[r];
+    }
+    for (int p0 = 0; p0 < n_all; p0 += kFoldTile) {
+        const int n = min(kFoldTile, n_all - p0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += kFoldThreads) {
+            const int b = (p0 + i) / parts, q = (p0 + i) - b * parts;
+            const int K = blocks[b].K;
+            s_code[i] = ((q + 1) * K / parts - q * K / parts) | (q == 0 && blocks[b].new_day ? 128 : 0);
+        }
+        __syncthreads();
+        if (r >= R) continue;
+        for (int i = 0; i < n; i += kFoldAhead) {
+            unsigned v[kFoldAhead];
+#pragma unroll
+            for (int q = 0; q < kFoldAhead; ++q) v[q] = i + q < n ? __ldcs(&summary[(size_t)(p0 + i + q) * R + r]) : 0u;
+#pragma unroll
+            for (int q = 0; q < kFoldAhead; ++q) {
+                if (i + q >= n) break;
+                const int code = s_code[i + q], K = code & 127;
+                if (code & 128) st.run = 0;
+                const int pop = (int)(v[q] & 255u);
+                st.gross += pop;
+                if (pop == K) {
+                    st.run += K;
+                    st.best = max(st.best, st.run);
+                } else {
+                    st.best = max(st.best, max(st.run + (int)((v[q] >> 8) & 255u), (int)(v[q] >> 24)));
+                    st.run = (int)((v[q] >> 16) & 255u);
+                }
+            }
+        }
+    }
+    if (r >= R) return;
+    out.gross[r] = st.gross;
+    best[r] = st.best;
+    out.run[r] = st.run;
+    if (final_chunk && out.minutes) out.minutes[r] = (float)st.gross * out.step_minutes;
 }
 
 // --------------------------------------------------------------- batched scenarios
@@ -824,16 +957,15 @@ k_batch(BatchArgs ba) {
     if (COUNT) flush_raster_counts(ba.stats, n_cell, n_test, n_unit, n_span);
 }
 
-// Launch order of the tiles: descending by the triangles binned to them over the chunk's
-// blocks, bucketed at half powers of two.  The CTAs that start last are then the cheap
-// ones, which shortens the launch's tail; the order does not change any result.
-__global__ void k_tile_order(const unsigned* __restrict__ counts, int nbc, int n_tiles,
-                             int* __restrict__ order) {
+// Launch order of the items (of the tiles, over their nbc blocks): descending by the
+// triangles binned to them, bucketed at half powers of two.  The CTAs that start last are then the cheap ones, which shortens the
+// launch's tail; the order does not change any result.
+__global__ void k_item_order(const unsigned* __restrict__ counts, int nbc, int n, int* __restrict__ order) {
     constexpr int kBuckets = 64;
     __shared__ unsigned hist[kBuckets];
     auto bucket = [&](int t) {
         unsigned c = 0;
-        for (int b = 0; b < nbc; ++b) c += counts[(size_t)b * n_tiles + t];
+        for (int b = 0; b < nbc; ++b) c += counts[(size_t)b * n + t];
         if (c <= 1u) return kBuckets - 1;
         const int l = 31 - __clz(c);
         const int key = 2 * l + (int)((c >> (l - 1)) & 1u);     // 2 .. 63
@@ -841,7 +973,7 @@ __global__ void k_tile_order(const unsigned* __restrict__ counts, int nbc, int n
     };
     if (threadIdx.x < kBuckets) hist[threadIdx.x] = 0u;
     __syncthreads();
-    for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) atomicAdd(&hist[bucket(t)], 1u);
+    for (int t = threadIdx.x; t < n; t += blockDim.x) atomicAdd(&hist[bucket(t)], 1u);
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned run = 0;
@@ -852,80 +984,128 @@ __global__ void k_tile_order(const unsigned* __restrict__ counts, int nbc, int n
         }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < n_tiles; t += blockDim.x) order[atomicAdd(&hist[bucket(t)], 1u)] = t;
-}
-
-template <int CTAS>
-void launch_k_raster_as(const RasterArgs& ra, int n_tiles, bool stats, cudaStream_t st) {
-    if (ra.cull) {
-        if (stats) k_raster<true, true, CTAS><<<n_tiles, kRasterThreads, 0, st>>>(ra);
-        else k_raster<false, true, CTAS><<<n_tiles, kRasterThreads, 0, st>>>(ra);
-    } else {
-        if (stats) k_raster<true, false, CTAS><<<n_tiles, kRasterThreads, 0, st>>>(ra);
-        else k_raster<false, false, CTAS><<<n_tiles, kRasterThreads, 0, st>>>(ra);
-    }
+    for (int t = threadIdx.x; t < n; t += blockDim.x) order[atomicAdd(&hist[bucket(t)], 1u)] = t;
 }
 
 // A launch of more tiles than 4 CTAs per SM hold takes the build for SA_RASTER_CTAS
 // resident CTAs per SM (fewer registers, more warps to hide latency); a smaller one, all of
 // whose tiles are resident at once anyway, takes the build for 4 (more registers, no
 // spills).
-void launch_k_raster(const RasterArgs& ra, int n_tiles, bool stats, cudaStream_t st) {
+void launch_k_raster(const RasterArgs& ra, int n_tiles, cudaStream_t st) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 0;
-    if (SA_RASTER_CTAS > 4 && n_tiles > 4 * sms) launch_k_raster_as<SA_RASTER_CTAS>(ra, n_tiles, stats, st);
-    else launch_k_raster_as<4>(ra, n_tiles, stats, st);
+    if (SA_RASTER_CTAS > 4 && n_tiles > 4 * sms) {
+        if (ra.cull) k_raster<true, SA_RASTER_CTAS><<<n_tiles, kRasterThreads, 0, st>>>(ra);
+        else k_raster<false, SA_RASTER_CTAS><<<n_tiles, kRasterThreads, 0, st>>>(ra);
+    } else {
+        if (ra.cull) k_raster<true, 4><<<n_tiles, kRasterThreads, 0, st>>>(ra);
+        else k_raster<false, 4><<<n_tiles, kRasterThreads, 0, st>>>(ra);
+    }
+}
+
+void launch_k_items(const RasterArgs& ra, int n_items, bool stats, cudaStream_t st) {
+    const dim3 grid((unsigned)n_items, (unsigned)ra.parts);
+    if (ra.cull) {
+        if (stats) k_raster_items<true, true><<<grid, kRasterThreads, 0, st>>>(ra);
+        else k_raster_items<false, true><<<grid, kRasterThreads, 0, st>>>(ra);
+    } else {
+        if (stats) k_raster_items<true, false><<<grid, kRasterThreads, 0, st>>>(ra);
+        else k_raster_items<false, false><<<grid, kRasterThreads, 0, st>>>(ra);
+    }
 }
 
 }  // namespace
 
-// Runs every block of `sun` through the accrual raster, in chunks of blocks whose bins
-// fit a bounded scratch budget.  out.run must be scratch [R]; out.continuous may be NULL.
-cudaError_t launch_raster_ground(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
-                                 const DevOut& out, cudaStream_t st) {
+// Pieces each block's steps are cut into: one from 1,824 items (two waves of
+// SA_RASTER_CTAS CTAs on 152 SMs) up, where the items alone fill the chip and a piece only
+// repeats the staging (512^2 cells, 9 blocks, 2,304 items: 0.29 ms in one piece, 0.33 in
+// two), more below it, up to 4 (64^2 cells, 5 blocks, 20 items: 84 us in one, 57 us in four,
+// 54 us in six; 300^2 cells, 900 items: 255 us in one, 232 us in two, 226 us in three).
+static int raster_parts(int n_tiles, int n_blocks) {
+    const long long items = (long long)n_tiles * n_blocks, fill = 152ll * SA_RASTER_CTAS * 2;
+    return (int)std::max(1ll, std::min(4ll, (fill + items - 1) / items));
+}
+
+static TileGeom tile_geom(const DevRecv& rc) {
     TileGeom g;
     g.x0 = rc.x0; g.y0 = rc.y0; g.dx = rc.dx; g.nx = rc.nx; g.ny = rc.ny;
     g.tiles_x = (rc.nx + kTile - 1) / kTile;
     g.tiles_y = (rc.ny + kTile - 1) / kTile;
+    return g;
+}
+
+// Runs every block of `sun` through the accrual raster, in chunks of blocks whose bins
+// fit a bounded scratch budget.  out.run must be scratch [R]; out.continuous may be NULL,
+// and out.gross too when only the masks are wanted.  With `summaries`
+// ([n_blocks][R]) the run summary of every block goes there and out is not touched.
+static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
+                                 const DevOut& out, unsigned* summaries, cudaStream_t st) {
+    const TileGeom g = tile_geom(rc);
     const int n_tiles = g.tiles_x * g.tiles_y;
     const long long R = (long long)rc.nx * rc.ny;
-    if (R == 0) return cudaSuccess;
+    if (R == 0 || sun.n_blocks == 0) return cudaSuccess;
+    // One-step blocks (the per-step raster) of a grid whose tiles fill the chip go by tile: a
+    // summary per step is as much memory as the raster's own work (2048^2 cells, 481 steps:
+    // 30.9 ms by tile, 32.3 by item; 300 x 200 cells, 70 tiles, 241 steps: 4.07 and 0.50 ms).
+    const bool by_tile = !summaries && out.gross && !out.stats && n_tiles >= 4 * 152 &&
+                         sun.S < 8ll * sun.n_blocks;
+    const int parts = summaries || by_tile ? 1 : raster_parts(n_tiles, sun.n_blocks);
+    const bool fold = !summaries && out.gross && !by_tile;
     cudaError_t e = cudaSuccess;
+    // blocks per chunk: 64, and more where a small grid's counters, bins (every triangle in
+    // every tile at the most: the sums stay below 2^31) and run summaries (1 GiB) allow it
+    long long chunk = by_tile ? 64ll : std::max(64ll, std::min((1ll << 20) / n_tiles, (1ll << 31) / ((long long)std::max(sc.T, 1) * n_tiles)));
+    if (fold) chunk = std::min(chunk, std::max(1ll, (1ll << 30) / (4ll * parts * R)));
+    const int max_chunk_blocks = (int)std::min<long long>(sun.n_blocks, chunk);
+    const size_t nc = (size_t)max_chunk_blocks * n_tiles;
+    // a mesh so small that every bin may hold all of it needs no counting pass, no scan and
+    // no read-back of the bins' size
+    const bool direct = !by_tile && sc.T > 0 && (double)nc * sc.T <= (double)(4 << 20);
+    // one block of words: counts | cursor (zeroed together) | offsets | order | total
+    unsigned* words = nullptr;
+    int* bins = nullptr;
     int* best = out.continuous;
     int* best_scratch = nullptr;
-    if (!best) {
+    unsigned* summary = summaries;
+    size_t bins_cap = 0;
+    e = sa::scratch_alloc(&words, sizeof(unsigned) * (4 * nc + 1), st);
+    unsigned *counts = words, *cursor = words + nc, *offsets = words + 2 * nc, *d_total = words + 4 * nc;
+    int* order = reinterpret_cast<int*>(words + 3 * nc);
+    if (e == cudaSuccess && !best && out.gross) {
         e = sa::scratch_alloc(&best_scratch, sizeof(int) * (size_t)R, st);
-        if (e != cudaSuccess) return e;
         best = best_scratch;
     }
-    const int chunk = 64;
-    const int max_chunk_blocks = sun.n_blocks < chunk ? sun.n_blocks : chunk;
-    unsigned *counts = nullptr, *offsets = nullptr, *cursor = nullptr, *d_total = nullptr;
-    int *bins = nullptr, *order = nullptr;
-    size_t bins_cap = 0;
-    const size_t nc = (size_t)max_chunk_blocks * n_tiles;
-    e = sa::scratch_alloc(&counts, sizeof(unsigned) * nc, st);
-    if (e == cudaSuccess) e = sa::scratch_alloc(&offsets, sizeof(unsigned) * nc, st);
-    if (e == cudaSuccess) e = sa::scratch_alloc(&cursor, sizeof(unsigned) * nc, st);
-    if (e == cudaSuccess) e = sa::scratch_alloc(&d_total, sizeof(unsigned), st);
-    if (e == cudaSuccess) e = sa::scratch_alloc(&order, sizeof(int) * (size_t)n_tiles, st);
-    const int tpb = 128;
-    for (int b0 = 0; b0 < sun.n_blocks && e == cudaSuccess; b0 += chunk) {
-        const int nbc = (sun.n_blocks - b0) < chunk ? (sun.n_blocks - b0) : chunk;
+    if (e == cudaSuccess && fold)
+        e = sa::scratch_alloc(&summary, sizeof(unsigned) * (size_t)max_chunk_blocks * parts * (size_t)R, st);
+    if (e == cudaSuccess && direct) {
+        bins_cap = nc * sc.T;
+        e = sa::scratch_alloc(&bins, sizeof(int) * bins_cap, st);
+    }
+    if (e == cudaSuccess && out.gross && out.accumulate_into) {
+        // run lengths never cross calls (calls cover whole days)
+        e = cudaMemsetAsync(out.run, 0, sizeof(int) * (size_t)R, st);
+        if (e == cudaSuccess && !out.continuous) e = cudaMemsetAsync(best, 0, sizeof(int) * (size_t)R, st);
+    }
+    for (int b0 = 0; b0 < sun.n_blocks && e == cudaSuccess; b0 += (int)chunk) {
+        const int nbc = std::min(sun.n_blocks - b0, (int)chunk);
         const size_t ncc = (size_t)nbc * n_tiles;
-        e = cudaMemsetAsync(counts, 0, sizeof(unsigned) * ncc, st);
-        if (e != cudaSuccess) break;
-        e = cudaMemsetAsync(cursor, 0, sizeof(unsigned) * ncc, st);
+        int per = 1;
+        const dim3 grid = bin_grid(std::max(sc.T, 1), nbc, &per);
+        e = cudaMemsetAsync(words, 0, sizeof(unsigned) * (direct ? ncc : nc + ncc), st);
         if (e != cudaSuccess) break;
         unsigned total = 0;
-        if (sc.T > 0) {
-            dim3 grid((sc.T + tpb - 1) / tpb, nbc);
+        if (direct) {
+            KernelTimer kt(KT_RASTER_BIN, st);
+            k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, nullptr,
+                                                      (unsigned)sc.T, counts, bins);
+        } else if (sc.T > 0) {
             {
                 KernelTimer kt(KT_RASTER_BIN, st);
-                k_bin_count<<<grid, tpb, 0, st>>>(sc, sun.steps, sun.blocks, b0, g, counts);
+                k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, nullptr, 0u,
+                                                           counts, nullptr);
             }
-            k_tile_order<<<1, 1024, 0, st>>>(counts, nbc, n_tiles, order);
+            k_item_order<<<1, 1024, 0, st>>>(counts, by_tile ? nbc : 1, by_tile ? n_tiles : (int)ncc, order);
             e = cudaMemcpyAsync(offsets, counts, sizeof(unsigned) * ncc, cudaMemcpyDeviceToDevice, st);
             if (e != cudaSuccess) break;
             e = exclusive_scan_u32(offsets, (long long)ncc, d_total, st);
@@ -942,7 +1122,8 @@ cudaError_t launch_raster_ground(const DevScene& sc, const DevRecv& rc, const De
             }
             if (total > 0) {
                 KernelTimer kt(KT_RASTER_BIN, st);
-                k_bin_fill<<<grid, tpb, 0, st>>>(sc, sun.steps, sun.blocks, b0, g, offsets, cursor, bins);
+                k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, offsets, 0u,
+                                                          cursor, bins);
             }
         } else {
             e = cudaMemsetAsync(offsets, 0, sizeof(unsigned) * ncc, st);
@@ -950,37 +1131,41 @@ cudaError_t launch_raster_ground(const DevScene& sc, const DevRecv& rc, const De
         }
         RasterArgs ra;
         ra.sc = sc; ra.sun = sun; ra.g = g; ra.b0 = b0; ra.nbc = nbc;
-        ra.offsets = offsets; ra.counts = counts; ra.bins = bins;
+        ra.offsets = direct ? nullptr : offsets; ra.counts = counts; ra.bins = bins;
         ra.out = out; ra.best = best;
         ra.load_state = (b0 > 0) || out.accumulate_into;
         ra.final_chunk = (b0 + nbc >= sun.n_blocks);
         ra.R = R;
         ra.cull = sc.closed;
         ra.run = g_raster_run;
-        ra.order = sc.T > 0 ? order : nullptr;
-        if (b0 == 0 && out.accumulate_into) {
-            // run lengths never cross calls (calls cover whole days)
-            e = cudaMemsetAsync(out.run, 0, sizeof(int) * (size_t)R, st);
-            if (e != cudaSuccess) break;
-            if (!out.continuous) {
-                e = cudaMemsetAsync(best, 0, sizeof(int) * (size_t)R, st);
-                if (e != cudaSuccess) break;
-            }
-        }
+        ra.order = sc.T > 0 && !direct ? order : nullptr;
+        ra.cap = direct ? (unsigned)sc.T : 0u;
+        ra.parts = parts;
+        ra.summary = summaries ? summaries + (size_t)b0 * (size_t)R : summary;
         {
             KernelTimer kt(KT_RASTER, st);
-            launch_k_raster(ra, n_tiles, out.stats != nullptr, st);
+            if (by_tile) launch_k_raster(ra, n_tiles, st);
+            else launch_k_items(ra, (int)ncc, out.stats != nullptr, st);
         }
+        if (fold)
+            k_items_fold<<<(unsigned)((R + kFoldThreads - 1) / kFoldThreads), kFoldThreads, 0, st>>>(
+                summary, R, sun.blocks + b0, nbc, parts, out, best, ra.load_state, ra.final_chunk);
         e = cudaGetLastError();
     }
-    if (counts) cudaFreeAsync(counts, st);
-    if (offsets) cudaFreeAsync(offsets, st);
-    if (cursor) cudaFreeAsync(cursor, st);
-    if (d_total) cudaFreeAsync(d_total, st);
-    if (bins) cudaFreeAsync(bins, st);
-    if (order) cudaFreeAsync(order, st);
-    if (best_scratch) cudaFreeAsync(best_scratch, st);
+    for (void* p : {(void*)words, (void*)bins, (void*)best_scratch, fold ? (void*)summary : nullptr})
+        if (p) cudaFreeAsync(p, st);
     return e;
+}
+
+cudaError_t launch_raster_ground(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
+                                 const DevOut& out, cudaStream_t st) {
+    return raster_ground(sc, rc, sun, out, nullptr, st);
+}
+
+cudaError_t launch_raster_summaries(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
+                                    unsigned* summaries, cudaStream_t st) {
+    DevOut out{};
+    return raster_ground(sc, rc, sun, out, summaries, st);
 }
 
 namespace {
@@ -1025,7 +1210,6 @@ cudaError_t launch_raster_ground_in(const DevScene& sc, const DevRecv& rc, const
     const size_t bins_cap = (bytes - off) / sizeof(int);
     DevOut o = out;
     o.run = run;
-    const int tpb = 128;
     // Bins of blocks [b0, b0 + nbc): counts, their exclusive scan into offsets, and the
     // total, read back to the host.
     auto count_chunk = [&](int b0, int nbc, unsigned* total) -> cudaError_t {
@@ -1034,8 +1218,9 @@ cudaError_t launch_raster_ground_in(const DevScene& sc, const DevRecv& rc, const
         cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(unsigned) * ncc, st);
         if (e != cudaSuccess) return e;
         if (sc.T == 0) return cudaMemsetAsync(offsets, 0, sizeof(unsigned) * ncc, st);
-        dim3 grid((sc.T + tpb - 1) / tpb, nbc);
-        k_bin_count<<<grid, tpb, 0, st>>>(sc, sun.steps, sun.blocks, b0, g, counts);
+        int per = 1;
+        const dim3 grid = bin_grid(sc.T, nbc, &per);
+        k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, nullptr, 0u, counts, nullptr);
         e = cudaMemcpyAsync(offsets, counts, sizeof(unsigned) * ncc, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = exclusive_scan_u32_with(offsets, (long long)ncc, partial, d_total, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(total, d_total, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
@@ -1072,8 +1257,9 @@ cudaError_t launch_raster_ground_in(const DevScene& sc, const DevRecv& rc, const
         if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, sizeof(unsigned) * (size_t)c.y * n_tiles, st);
         if (e != cudaSuccess) return e;
         if (total > 0) {
-            dim3 grid((sc.T + tpb - 1) / tpb, c.y);
-            k_bin_fill<<<grid, tpb, 0, st>>>(sc, sun.steps, sun.blocks, c.x, g, offsets, cursor, bins);
+            int per = 1;
+            const dim3 grid = bin_grid(sc.T, c.y, &per);
+            k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, c.x, c.y, per, g, offsets, 0u, cursor, bins);
         }
         RasterArgs ra;
         ra.sc = sc; ra.sun = sun; ra.g = g; ra.b0 = c.x; ra.nbc = c.y;
@@ -1085,7 +1271,10 @@ cudaError_t launch_raster_ground_in(const DevScene& sc, const DevRecv& rc, const
         ra.cull = sc.closed;
         ra.run = g_raster_run;
         ra.order = nullptr;
-        launch_k_raster(ra, n_tiles, out.stats != nullptr, st);
+        ra.cap = 0u;
+        ra.parts = 1;
+        ra.summary = nullptr;
+        launch_k_raster(ra, n_tiles, st);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -1113,10 +1302,11 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     if (e == cudaSuccess) e = cudaMemsetAsync(*counts, 0, sizeof(unsigned) * nc, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, sizeof(unsigned) * nc, st);
     unsigned total = 0;
-    const int tpb = 128;
-    dim3 grid((sc.T + tpb - 1) / tpb > 0 ? (sc.T + tpb - 1) / tpb : 1, sun.n_blocks);
+    int per = 1;
+    const dim3 grid = bin_grid(sc.T > 0 ? sc.T : 1, sun.n_blocks, &per);
     if (e == cudaSuccess && sc.T > 0) {
-        k_bin_count<<<grid, tpb, 0, st>>>(sc, sun.steps, sun.blocks, 0, g, *counts);
+        k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, 0, sun.n_blocks, per, g, nullptr, 0u,
+                                                   *counts, nullptr);
         e = cudaMemcpyAsync(*offsets, *counts, sizeof(unsigned) * nc, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = exclusive_scan_u32(*offsets, (long long)nc, d_total, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&total, d_total, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
@@ -1126,7 +1316,8 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     }
     if (e == cudaSuccess) e = cudaMalloc(bins, sizeof(int) * ((size_t)total + 1));
     if (e == cudaSuccess && total > 0)
-        k_bin_fill<<<grid, tpb, 0, st>>>(sc, sun.steps, sun.blocks, 0, g, *offsets, cursor, *bins);
+        k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, 0, sun.n_blocks, per, g, *offsets, 0u,
+                                                  cursor, *bins);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (cursor) cudaFreeAsync(cursor, st);
