@@ -264,6 +264,7 @@ struct TileSmem {
     float4 d[kMaxBlock];                     // step directions
     float4 ubox[kMaxBlock];                  // per run: (min u.x, max u.x, min u.y, max u.y)
     unsigned long long mask[kTile * kTile];
+    unsigned long long row_full[kTile];      // steps at which every cell of a row is shadowed
     // per warp: cells waiting for their step tests, (unit << 10) | cell, drained 32 at a
     // time so that every lane tests a cell whichever unit it comes from
     unsigned queue[kRasterThreads / 32][64];
@@ -521,9 +522,9 @@ __device__ __forceinline__ void raster_units(TileSmem& sm, int un0, int nu, int 
         if (ridx < total_rows) {
             const UnitRun u = unit_run<CULL>(sm, un, nsub);
             const int row = ((ubox >> 10) & 31) + (ridx - rex);
-            row_span(sm, u, ubox, row, inv_dx, &cs, &w);
-            cs += row * kTile;                      // the row's first cell
             can = (unsigned long long)(u.fr | u.bk) << u.k0;
+            if ((sm.row_full[row] & can) != can) row_span(sm, u, ubox, row, inv_dx, &cs, &w);
+            cs += row * kTile;                      // the row's first cell
         }
         const int cincl = lane_prefix(w);
         const int total = __shfl_sync(0xffffffffu, cincl, 31);
@@ -578,6 +579,7 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
     }
     if (threadIdx.x <= nsub) sm.run_k0[threadIdx.x] = (unsigned char)(threadIdx.x * K / nsub);
     if (threadIdx.x == 0) sm.inv_nsub = 1.f / (float)nsub;
+    if (threadIdx.x < kTile) sm.row_full[threadIdx.x] = 0ull;
     if (threadIdx.x < nsub) {
         const int k0 = threadIdx.x * K / nsub, k1 = (threadIdx.x + 1) * K / nsub;
         float4 b = make_float4(3.4e38f, -3.4e38f, 3.4e38f, -3.4e38f);
@@ -599,7 +601,27 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
             sm.tri[i] = v;
             if (i % 3 == 0) sm.valid[i / 3] = ok ? 1 : 0;
         }
+        // the steps at which a whole row is shadowed already, and (below) the whole tile:
+        // no later triangle can change them there, so its units lose those steps and rows
+        // before their spans are found, and a tile shadowed at every step is done.  A low
+        // sun bins thousands of triangles to a tile that the first few hundred fill
+        // (1024^2 cells, 16 December: 25.0 -> 16.4 ms; the June district is unchanged).
+        if (base > 0) {
+            for (int row = warp; row < kTile; row += kWarpsRaster) {
+                const unsigned long long m = sm.mask[row * kTile + lane];
+                const unsigned lo = __reduce_and_sync(0xffffffffu, (unsigned)m);
+                const unsigned hi = __reduce_and_sync(0xffffffffu, (unsigned)(m >> 32));
+                if (lane == 0) sm.row_full[row] = ((unsigned long long)hi << 32) | lo;
+            }
+        }
         __syncthreads();
+        unsigned long long tile_full = 0ull;
+        if (base > 0) {
+            const unsigned long long m = sm.row_full[lane];
+            tile_full = ((unsigned long long)__reduce_and_sync(0xffffffffu, (unsigned)(m >> 32)) << 32) |
+                        __reduce_and_sync(0xffffffffu, (unsigned)m);
+            if (tile_full == (K >= 64 ? ~0ull : (1ull << K) - 1ull)) break;
+        }
         if (threadIdx.x == 0) sm.next_unit = kWarpsRaster * kUnitClaim;
         // sun-facing steps of each staged triangle: a warp per triangle, a lane per step
         for (int t = warp; t < nt; t += kWarpsRaster) {
@@ -622,6 +644,8 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
                     fr |= (unsigned long long)f << (32 * h);
                     bk |= (unsigned long long)g << (32 * h);
                 }
+                fr &= ~tile_full;
+                bk &= ~tile_full;
                 if (CULL) bk = 0ull;
             }
             if (lane == 0) {

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 import torch
 
-from parity import block_sizes, unpack_masks
+from parity import assert_bits_parity, block_sizes, cached_oracle, unpack_masks, workload
 from synth import city as C
 from synth.sun import sun_table
 
@@ -60,3 +60,20 @@ def test_per_step_raster_equals_the_accrual_raster(cuda_lib, nx, ny):
     a = B.sa_accumulate(scene, grid, sun, 4.0, "accrual_sam")
     b = B.sa_accumulate(scene, grid, sun, 4.0, "sweep_raster")
     assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("closed", [True, False])
+def test_low_sun_tiles_that_fill_up(cuda_lib, closed):
+    """A December afternoon: a tile's bins hold many batches of triangles and its rows fill up
+    before the last, which then are skipped; step masks against the oracle."""
+    B = cuda_lib
+    w = workload("district_small", n_buildings=160, nx=100, ny=90, n_facade=0, doys=(355,), t0=14.0, t1=16.6, step=3.0)
+    scene = B.Scene(w.mesh.verts, w.mesh.tris, w.mesh.tri_building, w.city.B, closed=closed)
+    sun = B.Sun(w.sun.dirs, w.sun.day_start, 64)
+    g = w.ground
+    grid = B.Receivers.ground_grid(g.x0, g.y0, g.dx, g.nx, g.ny)
+    bits, near = cached_oracle("low_sun", w, "ground")
+    tiles = bits.reshape(g.ny, g.nx, -1)
+    assert tiles[32:64, 96:].all(axis=(0, 1)).sum() > 40      # a tile wholly shadowed at most steps
+    got = unpack_masks(B.sa_shadow_masks(scene, grid, sun, "accrual_sam"), block_sizes(w.sun.day_start, 64))
+    assert_bits_parity(got, bits, near)
