@@ -767,9 +767,8 @@ void sa_receivers_destroy(sa_receivers* recv) {
 int64_t sa_receivers_count(const sa_receivers* recv) { return recv ? recv->R : -1; }
 
 // ------------------------------------------------------------------------- accumulate
-static sa_status run_method(const sa_scene* scene, const sa_receivers* recv, const sa_sun* sun,
-                            sa_method method, int32_t iam_levels, sa::DevOut out,
-                            cudaStream_t st, const char* who) {
+static sa_status check_method(const sa_scene* scene, const sa_receivers* recv, const sa_sun* sun,
+                              sa_method method, int32_t iam_levels, const char* who) {
     if (!scene || !recv || !sun) return fail(SA_ERR_INVALID_ARG, "%s: NULL handle", who);
     if (iam_levels < 0 || iam_levels > 8) return fail(SA_ERR_INVALID_ARG, "%s: iam_levels", who);
     const bool raster = method == SA_SWEEP_RASTER || (method == SA_ACCRUAL_SAM && recv->is_grid);
@@ -779,6 +778,15 @@ static sa_status run_method(const sa_scene* scene, const sa_receivers* recv, con
         return fail(SA_ERR_UNSUPPORTED, "%s: raster methods need geometry at z >= 0", who);
     if (method < SA_SWEEP_TRACE || method > SA_IAM)
         return fail(SA_ERR_INVALID_ARG, "%s: unknown method %d", who, (int)method);
+    return SA_OK;
+}
+
+static sa_status run_method(const sa_scene* scene, const sa_receivers* recv, const sa_sun* sun,
+                            sa_method method, int32_t iam_levels, sa::DevOut out,
+                            cudaStream_t st, const char* who) {
+    const sa_status chk = check_method(scene, recv, sun, method, iam_levels, who);
+    if (chk != SA_OK) return chk;
+    const bool raster = method == SA_SWEEP_RASTER || (method == SA_ACCRUAL_SAM && recv->is_grid);
     sa::DevScene dsc = dev_scene(scene);
     sa::DevRecv drc = dev_recv(recv);
     sa::DevSun dsun;
@@ -922,12 +930,15 @@ sa_status sa_accumulate_graph(const sa_scene* scene, const sa_receivers* recv, c
     const long long per_edge = 8ll * R;
     long long fit = std::max(1ll, (4ll << 30) / per_edge);
     if (fit >= 64) fit -= fit % 64;
-    const int chunk = (int)std::min((long long)E, fit);
-    sa_status status = SA_OK;
+    // the ground accrual raster leaves the edges' run summaries itself, without masks
+    const bool direct = method == SA_ACCRUAL_SAM && recv->is_grid;
+    const int chunk = direct ? E : (int)std::min((long long)E, fit);
+    sa_status status = check_method(scene, recv, sun, method, iam_levels, who);
+    if (status != SA_OK) return status;
 #define TRY(x) do { e = (x); if (e != cudaSuccess) goto done; } while (0)
     TRY(sa::scratch_alloc(&summary, sizeof(unsigned) * (size_t)E * (size_t)R, st));
-    TRY(sa::scratch_alloc(&masks, sizeof(unsigned long long) * (size_t)chunk * (size_t)R, st));
-    TRY(sa::scratch_alloc(&scratch, sizeof(int) * (size_t)R, st));
+    if (!direct) TRY(sa::scratch_alloc(&masks, sizeof(unsigned long long) * (size_t)chunk * (size_t)R, st));
+    if (!direct) TRY(sa::scratch_alloc(&scratch, sizeof(int) * (size_t)R, st));
     TRY(sa::scratch_alloc(&d_walk, sizeof(int) * (size_t)nb, st));
     TRY(sa::scratch_alloc(&d_K, sizeof(int) * (size_t)E, st));
     TRY(cudaMemcpyAsync(d_walk, walk.data(), sizeof(int) * (size_t)nb, cudaMemcpyHostToDevice, st));
@@ -939,14 +950,14 @@ sa_status sa_accumulate_graph(const sa_scene* scene, const sa_receivers* recv, c
         sa_sun gs;
         gs.S = sun->S;
         gs.D = e1 - e0;
-        gs.h_steps = sun->h_steps;
+        if (!direct) gs.h_steps = sun->h_steps;
         for (int q = e0; q < e1; ++q) {
             sa::BlockConst bc = sun->h_blocks[(size_t)rep[(size_t)q]];
             bc.mask_block = q - e0;
             bc.mask_bit = 0;
             bc.new_day = 1;
             gs.h_blocks.push_back(bc);
-            for (int i = 0; i < bc.K; ++i) {
+            for (int i = 0; i < bc.K && !direct; ++i) {
                 sa::BlockConst sb = sun->h_step_blocks[(size_t)bc.j0 + i];
                 sb.mask_block = q - e0;
                 sb.mask_bit = i;
@@ -957,8 +968,13 @@ sa_status sa_accumulate_graph(const sa_scene* scene, const sa_receivers* recv, c
         gs.d_steps = sun->d_steps;
         e = upload(gs.h_blocks.data(), gs.h_blocks.size(), 0, &gs.d_blocks, st);
         if (e == cudaSuccess) e = upload(gs.h_step_blocks.data(), gs.h_step_blocks.size(), 0, &gs.d_step_blocks, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)(e1 - e0) * (size_t)R, st);
-        if (e == cudaSuccess) {
+        if (e == cudaSuccess && direct) {
+            const sa::DevSun ds{gs.d_steps, gs.d_blocks, gs.S, E};
+            e = sa::launch_raster_summaries(dev_scene(scene), dev_recv(recv), ds, summary, st);
+        }
+        if (e == cudaSuccess && !direct)
+            e = cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)(e1 - e0) * (size_t)R, st);
+        if (e == cudaSuccess && !direct) {
             sa::DevOut out;
             memset(&out, 0, sizeof(out));
             out.gross = scratch;
@@ -966,7 +982,7 @@ sa_status sa_accumulate_graph(const sa_scene* scene, const sa_receivers* recv, c
             out.write_final = 1;
             status = run_method(scene, recv, &gs, method, iam_levels, out, st, who);
         }
-        if (e == cudaSuccess && status == SA_OK)
+        if (e == cudaSuccess && status == SA_OK && !direct)
             e = sa::launch_edge_summary(masks, R, e1 - e0, d_K + e0, summary + (size_t)e0 * (size_t)R, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (gs.d_blocks) cudaFree(gs.d_blocks);

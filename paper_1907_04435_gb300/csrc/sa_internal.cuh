@@ -689,6 +689,14 @@ long long scan_partials(long long n);
 cudaError_t exclusive_scan_u32_with(unsigned* data, long long n, unsigned* partial,
                                     unsigned* d_total, cudaStream_t st);
 
+// Launch order of n work items (tiles): descending by tc[i] x rc[i] (by tc[i] when rc is
+// null), so that the items that start last are the cheap ones, which shortens a launch's
+// tail; hist is kOrderBuckets words of scratch, *n_work (nullable) the items with work,
+// which come first.  The order within a bucket is arbitrary.
+constexpr int kOrderBuckets = 64;
+cudaError_t launch_work_order(const unsigned* tc, const unsigned* rc, long long n, unsigned* hist,
+                              int* order, unsigned* n_work, cudaStream_t st);
+
 // The ground accrual raster with every scratch buffer carved from `scratch` (bytes long,
 // 256-byte aligned); allocates nothing.  *capacity_error is set to 1 (and cudaSuccess
 // returned) when the receivers' state or a single block's bins do not fit.

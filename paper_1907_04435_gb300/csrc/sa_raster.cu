@@ -145,13 +145,13 @@ __global__ void k_bin(DevScene sc, const StepConst* __restrict__ steps,
 
 constexpr int kBinThreads = 128;
 
-// Grid of k_bin: enough CTAs for the chip (a few waves) from the triangles alone where the
-// mesh has them, else the blocks are split as well.
+// Grid of k_bin: up to 8 blocks a thread.  More would read the mesh less often still, but a
+// triangle inside the grid then makes its atomics for all of them in series (64 blocks a
+// thread, 1.5M triangles, a 1024^2 grid in the middle: 2.76 ms, 8 a thread 1.25); fewer where the triangles alone do not fill the chip.
 dim3 bin_grid(int T, int nbc, int* per) {
     const int gx = (T + kBinThreads - 1) / kBinThreads;
-    int gy = std::min(nbc, std::max(1, (152 * 16 + gx - 1) / gx));
-    gy = std::min(gy, 65535);
-    *per = (nbc + gy - 1) / gy;
+    *per = std::max(1, std::min(8, (int)((long long)gx * nbc / (152 * 16))));
+    if ((nbc + *per - 1) / *per > 65535) *per = (nbc + 65534) / 65535;
     return dim3((unsigned)gx, (unsigned)((nbc + *per - 1) / *per));
 }
 
@@ -833,18 +833,21 @@ constexpr int kFoldTile = 1024;      // steps-and-day codes staged in shared mem
 constexpr int kFoldAhead = 8;        // summaries a thread loads ahead of their use
 
 // Stitches the chunk's run summaries, in time order, into each cell's gross / continuous
-// state (as stitch does with the masks themselves).
+// state (as stitch does with the masks themselves), VEC cells per thread.  Bound by memory
+// on a large grid (4 bytes in per block, 12 out; four cells per thread: 16-byte loads, 2048^2
+// cells x 9 blocks 79 -> 37 us); a small one keeps a cell per thread for the parallelism.
+template <int VEC>
 __global__ void __launch_bounds__(kFoldThreads)
 k_items_fold(const unsigned* __restrict__ summary, long long R, const BlockConst* __restrict__ blocks,
              int nbc, int parts, DevOut out, int* __restrict__ best, int load_state, int final_chunk) {
     __shared__ int s_code[kFoldTile];
-    const long long r = (long long)blockIdx.x * kFoldThreads + threadIdx.x;
+    const long long r = ((long long)blockIdx.x * kFoldThreads + threadIdx.x) * VEC;
     const int n_all = nbc * parts;
-    RunState st{0, 0, 0};
-    if (r < R && load_state) {
-        st.gross = out.gross[r];
-        st.best = best[r];
-        st.run = out.run[r];
+    RunState st[VEC];
+#pragma unroll
+    for (int c = 0; c < VEC; ++c) {
+        st[c] = RunState{0, 0, 0};
+        if (r < R && load_state) st[c] = RunState{out.gross[r + c], out.run[r + c], best[r + c]};
     }
     for (int p0 = 0; p0 < n_all; p0 += kFoldTile) {
         const int n = min(kFoldTile, n_all - p0);
@@ -857,31 +860,74 @@ k_items_fold(const unsigned* __restrict__ summary, long long R, const BlockConst
         __syncthreads();
         if (r >= R) continue;
         for (int i = 0; i < n; i += kFoldAhead) {
-            unsigned v[kFoldAhead];
+            unsigned v[kFoldAhead][VEC];
 #pragma unroll
-            for (int q = 0; q < kFoldAhead; ++q) v[q] = i + q < n ? __ldcs(&summary[(size_t)(p0 + i + q) * R + r]) : 0u;
+            for (int q = 0; q < kFoldAhead; ++q) {
+                const unsigned* at = summary + (size_t)(p0 + i + q) * R + r;
+                if (i + q >= n) {
+#pragma unroll
+                    for (int c = 0; c < VEC; ++c) v[q][c] = 0u;
+                } else if (VEC == 4) {
+                    const uint4 x = __ldcs(reinterpret_cast<const uint4*>(at));
+                    v[q][0] = x.x; v[q][VEC > 1 ? 1 : 0] = x.y; v[q][VEC > 2 ? 2 : 0] = x.z; v[q][VEC > 3 ? 3 : 0] = x.w;
+                } else {
+                    v[q][0] = __ldcs(at);
+                }
+            }
 #pragma unroll
             for (int q = 0; q < kFoldAhead; ++q) {
                 if (i + q >= n) break;
                 const int code = s_code[i + q], K = code & 127;
-                if (code & 128) st.run = 0;
-                const int pop = (int)(v[q] & 255u);
-                st.gross += pop;
-                if (pop == K) {
-                    st.run += K;
-                    st.best = max(st.best, st.run);
-                } else {
-                    st.best = max(st.best, max(st.run + (int)((v[q] >> 8) & 255u), (int)(v[q] >> 24)));
-                    st.run = (int)((v[q] >> 16) & 255u);
+#pragma unroll
+                for (int c = 0; c < VEC; ++c) {
+                    RunState& s = st[c];
+                    const unsigned x = v[q][c];
+                    if (code & 128) s.run = 0;
+                    const int pop = (int)(x & 255u);
+                    s.gross += pop;
+                    if (pop == K) {
+                        s.run += K;
+                        s.best = max(s.best, s.run);
+                    } else {
+                        s.best = max(s.best, max(s.run + (int)((x >> 8) & 255u), (int)(x >> 24)));
+                        s.run = (int)((x >> 16) & 255u);
+                    }
                 }
             }
         }
     }
     if (r >= R) return;
-    out.gross[r] = st.gross;
-    best[r] = st.best;
-    out.run[r] = st.run;
-    if (final_chunk && out.minutes) out.minutes[r] = (float)st.gross * out.step_minutes;
+    const float dt = out.step_minutes;
+    if (VEC == 4) {
+        const RunState &a = st[0], &b = st[VEC > 1 ? 1 : 0], &c = st[VEC > 2 ? 2 : 0], &d = st[VEC > 3 ? 3 : 0];
+        *reinterpret_cast<int4*>(out.gross + r) = make_int4(a.gross, b.gross, c.gross, d.gross);
+        *reinterpret_cast<int4*>(best + r) = make_int4(a.best, b.best, c.best, d.best);
+        if (!final_chunk) *reinterpret_cast<int4*>(out.run + r) = make_int4(a.run, b.run, c.run, d.run);
+        else if (out.minutes)
+            *reinterpret_cast<float4*>(out.minutes + r) =
+                make_float4((float)a.gross * dt, (float)b.gross * dt, (float)c.gross * dt, (float)d.gross * dt);
+    } else {
+        out.gross[r] = st[0].gross;
+        best[r] = st[0].best;
+        if (!final_chunk) out.run[r] = st[0].run;
+        else if (out.minutes) out.minutes[r] = (float)st[0].gross * dt;
+    }
+}
+
+// Four cells per thread from a million cells up, where every row of summaries and every
+// output starts on 16 bytes.
+void launch_k_fold(const unsigned* summary, long long R, const BlockConst* blocks, int nbc, int parts,
+                   const DevOut& out, int* best, int load_state, int final_chunk, cudaStream_t st) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(out.gross) | reinterpret_cast<uintptr_t>(best) |
+                         reinterpret_cast<uintptr_t>(out.run) | reinterpret_cast<uintptr_t>(out.minutes) |
+                         reinterpret_cast<uintptr_t>(summary);
+    if (R >= (1 << 20) && R % 4 == 0 && (at & 15) == 0) {
+        const unsigned g = (unsigned)((R / 4 + kFoldThreads - 1) / kFoldThreads);
+        k_items_fold<4><<<g, kFoldThreads, 0, st>>>(summary, R, blocks, nbc, parts, out, best, load_state, final_chunk);
+    } else {
+        const unsigned g = (unsigned)((R + kFoldThreads - 1) / kFoldThreads);
+        k_items_fold<1><<<g, kFoldThreads, 0, st>>>(summary, R, blocks, nbc, parts, out, best, load_state, final_chunk);
+    }
 }
 
 // --------------------------------------------------------------- batched scenarios
@@ -981,34 +1027,14 @@ k_batch(BatchArgs ba) {
     if (COUNT) flush_raster_counts(ba.stats, n_cell, n_test, n_unit, n_span);
 }
 
-// Launch order of the items (of the tiles, over their nbc blocks): descending by the
-// triangles binned to them, bucketed at half powers of two.  The CTAs that start last are then the cheap ones, which shortens the
-// launch's tail; the order does not change any result.
-__global__ void k_item_order(const unsigned* __restrict__ counts, int nbc, int n, int* __restrict__ order) {
-    constexpr int kBuckets = 64;
-    __shared__ unsigned hist[kBuckets];
-    auto bucket = [&](int t) {
-        unsigned c = 0;
-        for (int b = 0; b < nbc; ++b) c += counts[(size_t)b * n + t];
-        if (c <= 1u) return kBuckets - 1;
-        const int l = 31 - __clz(c);
-        const int key = 2 * l + (int)((c >> (l - 1)) & 1u);     // 2 .. 63
-        return kBuckets - 1 - key;
-    };
-    if (threadIdx.x < kBuckets) hist[threadIdx.x] = 0u;
-    __syncthreads();
-    for (int t = threadIdx.x; t < n; t += blockDim.x) atomicAdd(&hist[bucket(t)], 1u);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned run = 0;
-        for (int k = 0; k < kBuckets; ++k) {
-            const unsigned h = hist[k];
-            hist[k] = run;
-            run += h;
-        }
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < n; t += blockDim.x) order[atomicAdd(&hist[bucket(t)], 1u)] = t;
+// Launch order of the tiles when a CTA takes all blocks of a tile: as launch_work_order, by
+// the triangles binned to the tile over the chunk's blocks.
+__global__ void k_tile_sums(const unsigned* __restrict__ counts, int nbc, int n_tiles, unsigned* __restrict__ sums) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n_tiles) return;
+    unsigned c = 0;
+    for (int b = 0; b < nbc; ++b) c += counts[(size_t)b * n_tiles + t];
+    sums[t] = c;
 }
 
 // A launch of more tiles than 4 CTAs per SM hold takes the build for SA_RASTER_CTAS
@@ -1086,15 +1112,16 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
     // a mesh so small that every bin may hold all of it needs no counting pass, no scan and
     // no read-back of the bins' size
     const bool direct = !by_tile && sc.T > 0 && (double)nc * sc.T <= (double)(4 << 20);
-    // one block of words: counts | cursor (zeroed together) | offsets | order | total
+    // one block of words: counts | cursor (zeroed together) | offsets | order | total | buckets
     unsigned* words = nullptr;
     int* bins = nullptr;
     int* best = out.continuous;
     int* best_scratch = nullptr;
     unsigned* summary = summaries;
     size_t bins_cap = 0;
-    e = sa::scratch_alloc(&words, sizeof(unsigned) * (4 * nc + 1), st);
-    unsigned *counts = words, *cursor = words + nc, *offsets = words + 2 * nc, *d_total = words + 4 * nc;
+    e = sa::scratch_alloc(&words, sizeof(unsigned) * (4 * nc + 1 + kOrderBuckets), st);
+    unsigned *counts = words, *cursor = words + nc, *offsets = words + 2 * nc, *d_total = words + 4 * nc,
+             *hist = d_total + 1;
     int* order = reinterpret_cast<int*>(words + 3 * nc);
     if (e == cudaSuccess && !best && out.gross) {
         e = sa::scratch_alloc(&best_scratch, sizeof(int) * (size_t)R, st);
@@ -1129,7 +1156,13 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
                 k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, nullptr, 0u,
                                                            counts, nullptr);
             }
-            k_item_order<<<1, 1024, 0, st>>>(counts, by_tile ? nbc : 1, by_tile ? n_tiles : (int)ncc, order);
+            if (by_tile) {       // the sums borrow the offsets, which are written below
+                k_tile_sums<<<(n_tiles + 255) / 256, 256, 0, st>>>(counts, nbc, n_tiles, offsets);
+                e = launch_work_order(offsets, nullptr, n_tiles, hist, order, nullptr, st);
+            } else {
+                e = launch_work_order(counts, nullptr, (long long)ncc, hist, order, nullptr, st);
+            }
+            if (e != cudaSuccess) break;
             e = cudaMemcpyAsync(offsets, counts, sizeof(unsigned) * ncc, cudaMemcpyDeviceToDevice, st);
             if (e != cudaSuccess) break;
             e = exclusive_scan_u32(offsets, (long long)ncc, d_total, st);
@@ -1172,8 +1205,7 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
             else launch_k_items(ra, (int)ncc, out.stats != nullptr, st);
         }
         if (fold)
-            k_items_fold<<<(unsigned)((R + kFoldThreads - 1) / kFoldThreads), kFoldThreads, 0, st>>>(
-                summary, R, sun.blocks + b0, nbc, parts, out, best, ra.load_state, ra.final_chunk);
+            launch_k_fold(summary, R, sun.blocks + b0, nbc, parts, out, best, ra.load_state, ra.final_chunk, st);
         e = cudaGetLastError();
     }
     for (void* p : {(void*)words, (void*)bins, (void*)best_scratch, fold ? (void*)summary : nullptr})

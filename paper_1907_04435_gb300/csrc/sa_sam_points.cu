@@ -480,59 +480,6 @@ k_sam_tile(TileArgs ta) {
     }
 }
 
-// Launch order of the light-space tiles: descending by (triangles x receivers), bucketed at
-// half powers of two; tiles with no pair go last and are not launched.  The order changes
-// no result, only which CTAs start last (the cheap ones, which shortens the tail).
-constexpr int kOrderBuckets = 64;
-
-__device__ __forceinline__ int pair_bucket(unsigned tcount, unsigned rcount) {
-    const unsigned long long c = (unsigned long long)tcount * rcount;
-    if (c == 0ull) return kOrderBuckets - 1;
-    if (c == 1ull) return kOrderBuckets - 2;
-    const int l = 63 - __clzll(c);
-    const int key = min(kOrderBuckets - 2, 2 * l + (int)((c >> (l - 1)) & 1ull));
-    return kOrderBuckets - 2 - key;
-}
-
-__global__ void k_order_hist(const unsigned* __restrict__ tc, const unsigned* __restrict__ rc,
-                             long long n, unsigned* __restrict__ hist) {
-    __shared__ unsigned h[kOrderBuckets];
-    if (threadIdx.x < kOrderBuckets) h[threadIdx.x] = 0u;
-    __syncthreads();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) atomicAdd(&h[pair_bucket(tc[i], rc[i])], 1u);
-    __syncthreads();
-    if (threadIdx.x < kOrderBuckets && h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], h[threadIdx.x]);
-}
-
-// exclusive scan of the histogram into the bucket cursors; n_work = tiles with a pair
-__global__ void k_order_scan(unsigned* __restrict__ hist, unsigned* __restrict__ n_work) {
-    if (threadIdx.x != 0) return;
-    unsigned run = 0;
-    for (int k = 0; k < kOrderBuckets; ++k) {
-        const unsigned h = hist[k];
-        hist[k] = run;
-        run += h;
-        if (k == kOrderBuckets - 2) *n_work = run;
-    }
-}
-
-__global__ void k_order_fill(const unsigned* __restrict__ tc, const unsigned* __restrict__ rc,
-                             long long n, unsigned* __restrict__ cursor, int* __restrict__ order) {
-    __shared__ unsigned h[kOrderBuckets], base[kOrderBuckets];
-    if (threadIdx.x < kOrderBuckets) h[threadIdx.x] = 0u;
-    __syncthreads();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int b = i < n ? pair_bucket(tc[i], rc[i]) : -1;
-    unsigned rank = 0;
-    if (b >= 0) rank = atomicAdd(&h[b], 1u);
-    __syncthreads();
-    if (threadIdx.x < kOrderBuckets && h[threadIdx.x])
-        base[threadIdx.x] = atomicAdd(&cursor[threadIdx.x], h[threadIdx.x]);
-    __syncthreads();
-    if (b >= 0) order[base[b] + rank] = (int)i;
-}
-
 // Stitch the chunk's blocks, in order, into each receiver's gross / continuous state.
 __global__ void k_points_fold(long long R, const int* __restrict__ perm,
                               const BlockConst* __restrict__ blocks, int nbc,
@@ -743,7 +690,7 @@ cudaError_t launch_sam_points(const DevScene& sc, const float* scene_box, const 
         TRYB(sa::scratch_alloc(&roff, sizeof(unsigned) * nt, st));
         TRYB(sa::scratch_alloc(&rcur, sizeof(unsigned) * nt, st));
         TRYB(sa::scratch_alloc(&d_total, 2 * sizeof(unsigned), st));   // bin total, tiles with work
-        TRYB(sa::scratch_alloc(&hist, sizeof(unsigned) * kOrderBuckets, st));
+        TRYB(sa::scratch_alloc(&hist, sizeof(unsigned) * kOrderBuckets, st));   // zeroed by the launch
         TRYB(sa::scratch_alloc(&order, sizeof(int) * nt, st));
         TRYB(sa::scratch_alloc(&rbins, sizeof(int) * (size_t)R * n_runs, st));
         TRYB(cudaMemcpyAsync(d_runs, hr.data(), sizeof(RunLight) * hr.size(), cudaMemcpyHostToDevice, st));
@@ -752,18 +699,13 @@ cudaError_t launch_sam_points(const DevScene& sc, const float* scene_box, const 
         TRYB(cudaMemsetAsync(tcur, 0, sizeof(unsigned) * nt, st));
         TRYB(cudaMemsetAsync(rcn, 0, sizeof(unsigned) * nt, st));
         TRYB(cudaMemsetAsync(rcur, 0, sizeof(unsigned) * nt, st));
-        TRYB(cudaMemsetAsync(hist, 0, sizeof(unsigned) * kOrderBuckets, st));
         const dim3 gt((unsigned)std::max(1, (sc.T + 127) / 128), n_runs);
         const dim3 gr((unsigned)((R + 255) / 256), n_runs);
         unsigned totals[2] = {0u, 0u};
-        const unsigned go = (unsigned)((nt + 255) / 256);
         if (e == cudaSuccess) {
             if (sc.T > 0) k_lt_bin<<<gt, 128, 0, st>>>(sc, sun.steps, d_runs, n_runs, false, tc, nullptr, nullptr, nullptr);
             k_lr_bin<<<gr, 256, 0, st>>>(rc.orig, R, d_runs, n_runs, false, rcn, nullptr, nullptr, nullptr);
-            k_order_hist<<<go, 256, 0, st>>>(tc, rcn, (long long)nt, hist);
-            k_order_scan<<<1, 32, 0, st>>>(hist, d_total + 1);
-            k_order_fill<<<go, 256, 0, st>>>(tc, rcn, (long long)nt, hist, order);
-            e = cudaGetLastError();
+            e = launch_work_order(tc, rcn, (long long)nt, hist, order, d_total + 1, st);
         }
         TRYB(cudaMemcpyAsync(toff, tc, sizeof(unsigned) * nt, cudaMemcpyDeviceToDevice, st));
         TRYB(cudaMemcpyAsync(roff, rcn, sizeof(unsigned) * nt, cudaMemcpyDeviceToDevice, st));

@@ -95,6 +95,56 @@ __global__ void k_scan_apply(unsigned* __restrict__ data, long long n,
     }
 }
 
+// ------------------------------------------------------------------------- work order
+// Buckets of the work counts tc[i] x rc[i] (tc[i] alone when rc is null) at half powers of
+// two, the heaviest first; items without work come last.
+__device__ __forceinline__ int work_bucket(const unsigned* tc, const unsigned* rc, long long i) {
+    const unsigned long long c = (unsigned long long)tc[i] * (rc ? rc[i] : 1u);
+    if (c == 0ull) return kOrderBuckets - 1;
+    if (c == 1ull) return kOrderBuckets - 2;
+    const int l = 63 - __clzll(c);
+    const int key = min(kOrderBuckets - 2, 2 * l + (int)((c >> (l - 1)) & 1ull));
+    return kOrderBuckets - 2 - key;
+}
+
+__global__ void k_order_hist(const unsigned* __restrict__ tc, const unsigned* __restrict__ rc,
+                             long long n, unsigned* __restrict__ hist) {
+    __shared__ unsigned h[kOrderBuckets];
+    if (threadIdx.x < kOrderBuckets) h[threadIdx.x] = 0u;
+    __syncthreads();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) atomicAdd(&h[work_bucket(tc, rc, i)], 1u);
+    __syncthreads();
+    if (threadIdx.x < kOrderBuckets && h[threadIdx.x]) atomicAdd(&hist[threadIdx.x], h[threadIdx.x]);
+}
+
+// exclusive scan of the histogram into the bucket cursors; *n_work (nullable) = items with work
+__global__ void k_order_scan(unsigned* __restrict__ hist, unsigned* __restrict__ n_work) {
+    static_assert(kOrderBuckets == 64, "two buckets per lane");
+    const int lane = threadIdx.x;
+    const unsigned a = hist[2 * lane], b = hist[2 * lane + 1];
+    const unsigned ex = warp_incl_scan(a + b) - (a + b);
+    hist[2 * lane] = ex;
+    hist[2 * lane + 1] = ex + a;
+    if (lane == 31 && n_work) *n_work = ex + a;      // all but the last bucket
+}
+
+__global__ void k_order_fill(const unsigned* __restrict__ tc, const unsigned* __restrict__ rc,
+                             long long n, unsigned* __restrict__ cursor, int* __restrict__ order) {
+    __shared__ unsigned h[kOrderBuckets], base[kOrderBuckets];
+    if (threadIdx.x < kOrderBuckets) h[threadIdx.x] = 0u;
+    __syncthreads();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = i < n ? work_bucket(tc, rc, i) : -1;
+    unsigned rank = 0;
+    if (b >= 0) rank = atomicAdd(&h[b], 1u);
+    __syncthreads();
+    if (threadIdx.x < kOrderBuckets && h[threadIdx.x])
+        base[threadIdx.x] = atomicAdd(&cursor[threadIdx.x], h[threadIdx.x]);
+    __syncthreads();
+    if (b >= 0) order[base[b] + rank] = (int)i;
+}
+
 // ------------------------------------------------------------------------ radix sort
 constexpr int kSortThreads = 256;
 constexpr int kSortRounds = 8;                              // keys per thread per tile
@@ -191,6 +241,17 @@ cudaError_t exclusive_scan_u32_with(unsigned* data, long long n, unsigned* parti
     k_scan_reduce<<<np, kScanThreads, 0, st>>>(data, n, partial);
     k_scan_partials<<<1, kScanThreads, 0, st>>>(partial, np, d_total);
     k_scan_apply<<<np, kScanThreads, 0, st>>>(data, n, partial);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_work_order(const unsigned* tc, const unsigned* rc, long long n, unsigned* hist,
+                              int* order, unsigned* n_work, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(unsigned) * kOrderBuckets, st);
+    if (e != cudaSuccess || n <= 0) return e;
+    const unsigned g = (unsigned)((n + 255) / 256);
+    k_order_hist<<<g, 256, 0, st>>>(tc, rc, n, hist);
+    k_order_scan<<<1, 32, 0, st>>>(hist, n_work);
+    k_order_fill<<<g, 256, 0, st>>>(tc, rc, n, hist, order);
     return cudaGetLastError();
 }
 
