@@ -12,22 +12,25 @@
 //   k_flip_count / k_flip_fill  walk each receiver's forward step masks (from the accrual
 //                               raster) and list the intervals whose end statuses differ;
 //                               intervals without a flip add dt * chi to S directly.
-//   k_flip_solve                per flip, in FP64: find the buildings that shadow the
-//                               receiver at the shadowed end (FP32 BVH traversal), locate
-//                               each one's flip a*_b on the exact prism test, in a
-//                               projective parameter of the same arc in which every prism
-//                               constraint is linear: an FP32 bisection brackets the flip,
-//                               the pair of constraints that close the entry interval there
-//                               gives it in closed form, and FP64 statuses on both sides
-//                               confirm it (otherwise an FP64 bisection finds it); then
-//                               take the first (lit -> shadow) or last (shadow -> lit), and
-//                               if the flip is the shadow of a roof edge e of building b
-//                               crossing the receiver, differentiate the grazing condition
+//   k_arcs                      the FP64 constants of every interval's arc.
+//   k_flip_solve                per flip: find the buildings that shadow the receiver at the
+//                               shadowed end (FP32 BVH traversal), locate each one's flip
+//                               a*_b on the exact prism test, in a projective parameter of
+//                               the same arc in which every prism constraint is linear: the
+//                               pair of constraints that close the entry interval at the
+//                               flip is found in FP32, with margins that certify it, and
+//                               gives the flip in closed form in FP64 (without the margins,
+//                               an FP64 search finds it); then take the first (lit ->
+//                               shadow) or last (shadow -> lit), and if the flip is the
+//                               shadow of a roof edge e of building b crossing the
+//                               receiver, differentiate the grazing condition
 //                                  G(a, h) = A_e + h B_e(a) = 0,  B_e(a) = c_e x u(a),
 //                               u = d_xy / d_z:  da*/dh = -B_e / (h dB_e/da).  A flip caused
 //                               by a vertical edge does not depend on h.
 #include <float.h>
 #include <string.h>
+
+#include <algorithm>
 
 #include "sa_internal.cuh"
 
@@ -40,55 +43,123 @@ constexpr int kMaxCand = 8;
 constexpr int kBisect = 40;   // halvings of [0, 1]: the flip to 1e-12 of a step
 constexpr int kLinEdges = 8;  // footprints up to this many edges take the linear form
 constexpr int kBisectF = 22;  // FP32 halvings that bracket a flip before its closed form
+constexpr int kSolveThreads = 128;
+constexpr int kSumCtas = 512;
 constexpr double kSide = 1e-10;   // FP64 status checks this far on both sides of a root
 
-// Visits every interval (j, j+1) inside a day of receiver r: f(j, chi0, chi1).
-template <class F>
-__device__ void for_intervals(const unsigned long long* masks, long long R, const BlockConst* blocks,
-                              int n_blocks, long long r, F f) {
-    int prev = -1;
-    int prev_j = -1;
-    for (int b = 0; b < n_blocks; ++b) {
-        const BlockConst& bc = blocks[b];
-        if (bc.new_day) prev = -1;
-        const unsigned long long m = masks[(long long)bc.mask_block * R + r] >> bc.mask_bit;
-        for (int k = 0; k < bc.K; ++k) {
-            const int c = (int)((m >> k) & 1ull);
-            if (prev >= 0) f(prev_j, prev, c);
-            prev = c;
-            prev_j = bc.j0 + k;
-        }
-    }
+// Step mask of a block for receiver r, and the status of the step before it in the same day
+// (none: the block's own first step, which makes no interval and no flip).
+struct BlockBits {
+    unsigned long long m;       // bit k: shadowed at step j0 + k
+    unsigned long long before;  // bit k: shadowed at the step before it
+    unsigned long long pairs;   // bit k: step k ends an interval (the first of a day ends none)
+};
+
+__device__ __forceinline__ BlockBits block_bits(const unsigned long long* masks, long long R,
+                                                const BlockConst& bc, long long r, bool& carry) {
+    BlockBits b;
+    const unsigned long long full = bc.K >= 64 ? ~0ull : ((1ull << bc.K) - 1ull);
+    b.m = (masks[(long long)bc.mask_block * R + r] >> bc.mask_bit) & full;
+    b.before = ((b.m << 1) | (carry ? 1ull : 0ull)) & full;
+    b.pairs = bc.new_day ? full & ~1ull : full;
+    carry = (b.m >> (bc.K - 1)) & 1ull;
+    return b;
 }
 
-__global__ void k_flip_count(const unsigned long long* __restrict__ masks, long long R,
+// Sum of s over the CTA's threads in a fixed order (at thread 0; at most 1,024 threads).
+__device__ __forceinline__ double cta_sum(double s) {
+    __shared__ double s_part[32];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(kFull, s, o);
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (unsigned w = 1; w < blockDim.x / 32; ++w) s += s_part[w];
+    return s;
+}
+
+// Sums whose order depends on n alone, so that S repeats to the last bit.
+__global__ void k_sum(const double* __restrict__ x, long long n, double* __restrict__ part) {
+    double s = 0.0;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        s += x[i];
+    s = cta_sum(s);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+
+__global__ void k_sum_pair(const double* __restrict__ x, const double* __restrict__ y, double* __restrict__ S) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < kSumCtas; i += blockDim.x) s += x[i] + y[i];
+    s = cta_sum(s);
+    if (threadIdx.x == 0) *S = s;
+}
+
+// The list's order: groups of consecutive blocks, in each the grid's 8 x 4-cell patches, one
+// warp each.  Flips that neighbours see at nearly the same time, mostly of one edge, then
+// share a warp in k_flip_solve: their rays visit the same nodes and their derivatives go to
+// the same building (k_flip_solve 8.9 -> 6.9 ms before the
+// certified search).
+struct FlipOrder {
+    int nx, ny, tiles_x;
+    long long n;          // threads: 32 per patch
+    int per;              // blocks per group
+};
+
+__device__ __forceinline__ long long patch_cell(const FlipOrder& g, long long t) {
+    const long long p = t >> 5;
+    const int lane = (int)(t & 31), tx = (int)(p % g.tiles_x);
+    const long long ix = tx * 8 + (lane & 7), iy = (p / g.tiles_x) * 4 + (lane >> 3);
+    return ix < g.nx && iy < g.ny ? iy * g.nx + ix : -1;
+}
+
+// Flips per group and receiver (counts [groups][n]), and the minutes of the intervals
+// without one: both are counts of bits (481 steps one by one took 1.10 ms on 600k cells,
+// whose masks are 43 MB).
+__global__ void k_flip_count(const unsigned long long* __restrict__ masks, long long R, FlipOrder g,
                              const BlockConst* __restrict__ blocks, int n_blocks,
                              const float* __restrict__ weights, double dt,
-                             unsigned* __restrict__ counts, double* __restrict__ S) {
-    const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+                             unsigned* __restrict__ counts, double* __restrict__ part) {
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long r = t < g.n ? patch_cell(g, t) : -1;
     double s = 0.0;
-    if (r < R) {
-        unsigned n = 0;
-        double steady = 0.0;
-        for_intervals(masks, R, blocks, n_blocks, r, [&](int, int c0, int c1) {
-            if (c0 != c1) ++n; else steady += c0;
-        });
-        counts[r] = n;
-        s = steady * dt * (weights ? (double)weights[r] : 1.0);
+    if (t < g.n) {
+        unsigned n = 0, steady = 0;
+        bool carry = false;
+        for (int b = 0; b < n_blocks; ++b) {
+            if (r >= 0) {
+                const BlockBits w = block_bits(masks, R, blocks[b], r, carry);
+                n += __popcll((w.m ^ w.before) & w.pairs);
+                steady += __popcll(w.m & w.before & w.pairs);
+            }
+            if ((b + 1) % g.per == 0 || b + 1 == n_blocks) {
+                counts[(long long)(b / g.per) * g.n + t] = n;
+                n = 0;
+            }
+        }
+        if (r >= 0) s = (double)steady * dt * (weights ? (double)weights[r] : 1.0);
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(kFull, s, o);
-    if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(S, s);
+    s = cta_sum(s);
+    if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-__global__ void k_flip_fill(const unsigned long long* __restrict__ masks, long long R,
+__global__ void k_flip_fill(const unsigned long long* __restrict__ masks, long long R, FlipOrder g,
                             const BlockConst* __restrict__ blocks, int n_blocks,
                             const unsigned* __restrict__ offsets, int4* __restrict__ flips) {
-    const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    unsigned w = offsets[r];
-    for_intervals(masks, R, blocks, n_blocks, r, [&](int j, int c0, int c1) {
-        if (c0 != c1) flips[w++] = make_int4((int)(r & 0x7fffffff), (int)(r >> 31), j, c0);
-    });
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long r = t < g.n ? patch_cell(g, t) : -1;
+    if (r < 0) return;
+    unsigned w = 0;
+    bool carry = false;
+    for (int b = 0; b < n_blocks; ++b) {
+        if (b % g.per == 0) w = offsets[(long long)(b / g.per) * g.n + t];
+        const BlockBits q = block_bits(masks, R, blocks[b], r, carry);
+        unsigned long long f = (q.m ^ q.before) & q.pairs;
+        while (f) {
+            const int k = __ffsll((long long)f) - 1;
+            f &= f - 1ull;
+            flips[w++] = make_int4((int)(r & 0x7fffffff), (int)(r >> 31), blocks[b].j0 + k - 1,
+                                   (int)((q.before >> k) & 1ull));
+        }
+    }
 }
 
 struct Vec3 { double x, y, z; };
@@ -103,6 +174,32 @@ struct Arc {
     Vec3 a, b;
     double theta, sin_theta;
 };
+
+// The arc from step j to step j + 1, one per interval: unit end a, chord e = b - a, angle.
+struct ArcConst {
+    double ax, ay, az, ex, ey, ez;
+    double theta, sin_theta, omc;     // omc = 1 - cos theta = |e|^2 / 2
+    double inv_theta;                 // 1 / theta (0 for a degenerate arc)
+};
+
+__global__ void k_arcs(const StepConst* __restrict__ steps, int n, ArcConst* __restrict__ arcs) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const Vec3 a = unit(steps[j]), b = unit(steps[j + 1]);
+    ArcConst c;
+    c.ax = a.x; c.ay = a.y; c.az = a.z;
+    c.ex = b.x - a.x; c.ey = b.y - a.y; c.ez = b.z - a.z;
+    const double nx = a.y * b.z - a.z * b.y, ny = a.z * b.x - a.x * b.z, nz = a.x * b.y - a.y * b.x;
+    c.sin_theta = sqrt(nx * nx + ny * ny + nz * nz);
+    c.omc = 0.5 * (c.ex * c.ex + c.ey * c.ey + c.ez * c.ez);
+    c.theta = atan2(c.sin_theta, 1.0 - c.omc);
+    c.inv_theta = c.theta < 1e-12 ? 0.0 : 1.0 / c.theta;
+    arcs[j] = c;
+}
+
+__device__ __forceinline__ Arc arc_of(const ArcConst& c) {
+    return Arc{Vec3{c.ax, c.ay, c.az}, Vec3{c.ax + c.ex, c.ay + c.ey, c.az + c.ez}, c.theta, c.sin_theta};
+}
 
 __device__ __forceinline__ Vec3 arc_dir(const Arc& c, double al) {
     if (c.theta < 1e-12) {
@@ -299,16 +396,209 @@ __device__ bool pair_root(const PrismLin& P, int il, int iu, double* be) {
     return true;
 }
 
-// slerp parameter of the projective parameter be (see prism_along)
-__device__ __forceinline__ double slerp_param(const Arc& arc, double be) {
-    if (arc.theta < 1e-12) return be;
-    const double dx = fma(be, arc.b.x - arc.a.x, arc.a.x);
-    const double dy = fma(be, arc.b.y - arc.a.y, arc.a.y);
-    const double dz = fma(be, arc.b.z - arc.a.z, arc.a.z);
-    const double cx = arc.a.y * dz - arc.a.z * dy, cy = arc.a.z * dx - arc.a.x * dz,
-                 cz = arc.a.x * dy - arc.a.y * dx;
-    const double ang = atan2(sqrt(cx * cx + cy * cy + cz * cz), arc.a.x * dx + arc.a.y * dy + arc.a.z * dz);
-    return fmin(1.0, fmax(0.0, ang / arc.theta));
+// slerp parameter of the projective parameter be (see prism_along): the angle from a to
+// d = a + be e has |a x d| = be sin theta and a . d = 1 - be (1 - cos theta).
+__device__ __forceinline__ double slerp_param(const ArcConst& c, double be) {
+    if (c.inv_theta == 0.0) return be;
+    double ang;
+    if (c.theta < 0.1) {
+        // steps up to about 20 minutes: the arctangent's power series (the next term is below
+        // 1e-18 of the first at t = 0.1)
+        const double t = be * c.sin_theta / (1.0 - be * c.omc), q = t * t;
+        double p = -1.0 / 15.0;
+        p = fma(p, q, 1.0 / 13.0);
+        p = fma(p, q, -1.0 / 11.0);
+        p = fma(p, q, 1.0 / 9.0);
+        p = fma(p, q, -1.0 / 7.0);
+        p = fma(p, q, 0.2);
+        p = fma(p, q, -1.0 / 3.0);
+        ang = fma(t * q, p, t);
+    } else {
+        ang = atan2(be * c.sin_theta, 1.0 - be * c.omc);
+    }
+    return fmin(1.0, fmax(0.0, ang * c.inv_theta));
+}
+
+// Flip of one building along the arc, searched in FP64: s0 is its status at be = 0.  False
+// when the statuses at the ends are not those of a flip.
+__device__ __noinline__ bool solve_fp64(const FootprintSet& fs, const float* heights, int b, double px,
+                                        double py, const Arc& arc, bool s0, double* be_star) {
+    const int fa = fs.fp_off[b], v = fs.fp_off[b + 1] - fa;
+    if (v <= kLinEdges) {
+        PrismLin P;
+        prism_lin_setup(P, fs.xy, fa, v, (double)heights[b], px, py, arc);
+        if (prism_lin_inside(P, 0.0) != s0 || prism_lin_inside(P, 1.0) == s0) return false;
+        // bracket in FP32, then the closed form of the pair of constraints that close the
+        // interval, confirmed by FP64 statuses on both sides of it
+        PrismLinF F;
+        prism_lin_to_f(P, F);
+        float flo = 0.f, fhi = 1.f;
+        for (int it = 0; it < kBisectF; ++it) {
+            const float mid = 0.5f * (flo + fhi);
+            if (prism_lin_inside_f(F, mid) == s0) flo = mid; else fhi = mid;
+        }
+        int il, iu;
+        prism_lin_active(P, s0 ? (double)flo : (double)fhi, &il, &iu);
+        double r;
+        if (pair_root(P, il, iu, &r) && r > kSide && r < 1.0 - kSide &&
+            fabs(r - 0.5 * ((double)flo + (double)fhi)) < 1e-4 &&
+            prism_lin_inside(P, r - kSide) == s0 && prism_lin_inside(P, r + kSide) != s0) {
+            *be_star = r;
+            return true;
+        }
+        double lo = 0.0, hi = 1.0;   // invariant: status(lo) == status at the start
+        for (int it = 0; it < kBisect; ++it) {
+            const double mid = 0.5 * (lo + hi);
+            if (prism_lin_inside(P, mid) == s0) lo = mid; else hi = mid;
+        }
+        *be_star = 0.5 * (lo + hi);
+        return true;
+    }
+    if (prism_along(fs, heights, b, px, py, arc, 0.0) != s0) return false;
+    if (prism_along(fs, heights, b, px, py, arc, 1.0) == s0) return false;
+    double lo = 0.0, hi = 1.0;
+    for (int it = 0; it < kBisect; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        if (prism_along(fs, heights, b, px, py, arc, mid) == s0) lo = mid; else hi = mid;
+    }
+    *be_star = 0.5 * (lo + hi);
+    return true;
+}
+
+// The same flip with FP64 only where it counts.  The statuses inside(be) form an interval of
+// the arc (the prism is convex), so the flip is where one pair of bounds -- lower edge il,
+// upper edge or roof iu -- closes the entry interval.  The pair is found in FP32 from the
+// lit end: the pair that is closed there has its root nearer to the flip, and the pair closed
+// at that root replaces it until none is.  It is accepted only with margins far above the
+// FP32 errors (1e-4 of the point's own distance, against 2e-5): every other constraint is
+// slack at the root and at the shadowed end.  The root itself, and its derivative with respect to h, are FP64 from the two
+// constraints' exact coefficients.  FP64 runs at 1/64 of the FP32 rate here, and the search
+// in it kept that pipe 83 % busy (park of 600k cells, 200 buildings: 12.2 ms for all flips,
+// now 1.06, and 0.67 for the 6 % that are left to it).
+// Returns 1 with the root, 0 when undecided.  *dbe_dh: derivative of a roof-edge flip.
+__device__ __forceinline__ int solve_fast(const FootprintSet& fs, int fa, int v, float h, float px, float py,
+                                          const ArcConst& arc, bool c0, double* be_star, double* dbe_dh) {
+    const float ax = (float)arc.ax, ay = (float)arc.ay, az = (float)arc.az;
+    const float ex = (float)arc.ex, ey = (float)arc.ey, ez = (float)arc.ez;
+    // constraint i: A_i d_z(be) + z (E0_i + be E1_i) >= 0 for the heights z inside; its margin is
+    // T_i (reach + z), T_i = 1e-4 |c_i| (padding: i >= v is never read)
+    float A[kLinEdges], E0[kLinEdges], E1[kLinEdges], T[kLinEdges];
+    const float2* xy = fs.xy + fa;
+    float reach = 1.f;
+    float2 p0 = xy[0];
+    const float2 first = p0;
+#pragma unroll
+    for (int i = 0; i < kLinEdges; ++i) {
+        if (i < v) {
+            const float2 p1 = i + 1 < v ? xy[i + 1] : first;
+            const float cx = p1.x - p0.x, cy = p1.y - p0.y, dx = px - p0.x, dy = py - p0.y;
+            A[i] = cx * dy - cy * dx;
+            E0[i] = cx * ay - cy * ax;
+            E1[i] = cx * ey - cy * ex;
+            T[i] = (fabsf(cx) + fabsf(cy)) * 1e-4f;
+            reach = fmaxf(reach, fabsf(dx) + fabsf(dy));
+            p0 = p1;
+        } else {
+            A[i] = E0[i] = E1[i] = T[i] = 0.f;
+        }
+    }
+    auto bounds = [&](float be, float& L, float& U, int& il, int& iu) {
+        const float dz = fmaf(be, ez, az);
+        L = 0.f; U = h; il = -1; iu = -1;
+#pragma unroll
+        for (int i = 0; i < kLinEdges; ++i) {
+            const float den = fmaf(be, E1[i], E0[i]);
+            const float z = __fdividef(-A[i] * dz, den);
+            if (i < v && den > 0.f && z > L) { L = z; il = i; }
+            if (i < v && den < 0.f && z < U) { U = z; iu = i; }
+        }
+    };
+    // every constraint but il and iu holds with its margin at height z
+    auto slack = [&](float be, float z, int il, int iu) {
+        const float dz = fmaf(be, ez, az);
+        bool ok = true;
+#pragma unroll
+        for (int i = 0; i < kLinEdges; ++i)
+            ok &= i >= v || i == il || i == iu ||
+                  fmaf(z, fmaf(be, E1[i], E0[i]), A[i] * dz) > T[i] * (reach + z);
+        return ok;
+    };
+    const float sh = c0 ? 0.f : 1.f, lit = 1.f - sh;
+    const float zm = 1e-4f * (h + reach);          // margin of heights
+    float L, U;
+    int il, iu;
+    int pl = -2, pu = -2;
+    float be = lit;
+    bool done = false;
+    for (int it = 0; it < 6 && !done; ++it) {
+        bounds(be, L, U, il, iu);
+        if ((il == pl && iu == pu) || (it > 0 && L <= U)) { done = true; break; }
+        if (il < 0 || L <= U) return 0;
+        pl = il; pu = iu;
+        float Ai = 0.f, E0i = 0.f, E1i = 0.f, Aj = 0.f, E0j = 0.f, E1j = 0.f;
+#pragma unroll
+        for (int i = 0; i < kLinEdges; ++i) {
+            if (i == il) { Ai = A[i]; E0i = E0[i]; E1i = E1[i]; }
+            if (i == iu) { Aj = A[i]; E0j = E0[i]; E1j = E1[i]; }
+        }
+        be = iu < 0 ? __fdividef(-fmaf(Ai, az, h * E0i), fmaf(Ai, ez, h * E1i))
+                    : __fdividef(Aj * E0i - Ai * E0j, Ai * E1j - Aj * E1i);
+        if (!(be > 0.f && be < 1.f)) return 0;
+    }
+    if (!done) return 0;
+    // FP64: the pair's exact coefficients, and its root
+    auto coef = [&](int i, double* a, double* e0, double* e1) {
+        const float2 p = xy[i], q = i + 1 == v ? first : xy[i + 1];
+        const double cx = (double)q.x - (double)p.x, cy = (double)q.y - (double)p.y;
+        *a = cx * ((double)py - (double)p.y) - cy * ((double)px - (double)p.x);
+        *e0 = cx * arc.ay - cy * arc.ax;
+        *e1 = cx * arc.ey - cy * arc.ex;
+    };
+    double ai, e0i, e1i, r;
+    coef(pl, &ai, &e0i, &e1i);
+    *dbe_dh = 0.0;
+    double num, den;
+    if (pu < 0) {
+        den = fma(ai, arc.ez, (double)h * e1i);
+        num = -fma(ai, arc.az, (double)h * e0i);
+    } else {
+        double aj, e0j, e1j;
+        coef(pu, &aj, &e0j, &e1j);
+        den = ai * e1j - aj * e1i;
+        num = aj * e0i - ai * e0j;
+    }
+    if (den == 0.0) return 0;
+    const double inv = 1.0 / den;
+    r = num * inv;
+    if (!(r > 1e-6 && r < 1.0 - 1e-6)) return 0;
+    // closed toward the lit end
+    const double side = fma((double)lit, den, -num);
+    if (!(pu < 0 ? side < 0.0 : side > 0.0)) return 0;
+    const double dl = fma(r, e1i, e0i);
+    if (pu < 0) *dbe_dh = -dl * inv;
+    // certificates at the root and at the lit end
+    const float rf = (float)r;
+    float Al = 0.f, E0l = 0.f, E1l = 0.f, Au = 0.f, E0u = -1.f, E1u = 0.f, Tl = 0.f, Tu = 0.f;
+#pragma unroll
+    for (int i = 0; i < kLinEdges; ++i) {
+        if (i == pl) { Al = A[i]; E0l = E0[i]; E1l = E1[i]; Tl = T[i]; }
+        if (i == pu) { Au = A[i]; E0u = E0[i]; E1u = E1[i]; Tu = T[i]; }
+    }
+    // at be: the pair's denominators above a hundredth of their edge (z then errs by 2e-5 of
+    // reach + z at the most), its mean height within the prism, every other constraint slack
+    // there.  At the root the two bounds meet, so the others hold around it; at the shadowed
+    // end the pair is open (the root lies between it and the lit end), so some height between
+    // its bounds is inside.
+    auto holds = [&](float at) {
+        const float dz = fmaf(at, ez, az), denl = fmaf(at, E1l, E0l), denu = fmaf(at, E1u, E0u);
+        const float zl = __fdividef(-Al * dz, denl);
+        const float z = 0.5f * (zl + (pu < 0 ? h : __fdividef(-Au * dz, denu)));
+        return denl > 100.f * Tl && denu < -100.f * Tu && z > zm && (pu < 0 || z < h - zm) && slack(at, z, pl, pu);
+    };
+    const bool ok = fmaf(lit, E1l, E0l) > 100.f * Tl && fmaf(lit, E1u, E0u) < -100.f * Tu && holds(rf) && holds(sh);
+    if (!ok) return 0;
+    *be_star = r;
+    return 1;
 }
 
 // Buildings hit by the FP32 ray from o toward step s (all hits, not only the first).
@@ -346,20 +636,24 @@ struct SolveArgs {
     FootprintSet fs;
     const float* heights;
     const StepConst* steps;
+    const ArcConst* arcs;
     float x0, y0, dx;
     int nx;
     const float* weights;
     double dt;
     const int4* flips;
     long long n_flips;
-    double* S;
+    unsigned* later;         // flips left to the FP64 search, and how many
+    unsigned* n_later;
+    double* minutes;         // each flip's part of S
     double* dSdh;
 };
 
-__global__ void k_flip_solve(SolveArgs a) {
-    const long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= a.n_flips) return;
-    const int4 fl = a.flips[f];
+// The flip of one list entry: adds its minutes to s; returns the building whose roof edge
+// casts it and the contribution to that building's derivative, or -1; -2 (FAST) when a
+// building's flip is not certified and the whole entry is left to the FP64 search.
+template <bool FAST>
+__device__ __forceinline__ int solve_flip(const SolveArgs& a, const int4& fl, double& s, double& grad) {
     const long long r = (long long)(unsigned)fl.x | ((long long)fl.y << 31);
     const int j = fl.z, c0 = fl.w;
     const int ix = (int)(r % a.nx), iy = (int)(r / a.nx);
@@ -367,95 +661,105 @@ __global__ void k_flip_solve(SolveArgs a) {
     o.x = __fadd_rn(a.x0, __fmul_rn(__fadd_rn((float)ix, 0.5f), a.dx));
     o.y = __fadd_rn(a.y0, __fmul_rn(__fadd_rn((float)iy, 0.5f), a.dx));
     o.z = 0.f;
-    const double px = o.x, py = o.y;
     const double w = a.weights ? (double)a.weights[r] : 1.0;
-    Arc arc;
-    arc.a = unit(a.steps[j]);
-    arc.b = unit(a.steps[j + 1]);
-    double cd = arc.a.x * arc.b.x + arc.a.y * arc.b.y + arc.a.z * arc.b.z;
-    cd = fmin(cd, 1.0);
-    arc.theta = acos(cd);
-    arc.sin_theta = sin(arc.theta);
     // candidates: buildings hit at the shadowed end
     int ids[kMaxCand];
-    const StepConst& ss = a.steps[c0 ? j : j + 1];
-    const int n = hit_buildings(a.sc, o, ss, ids);
-    const double al_sh = c0 ? 0.0 : 1.0, al_lit = c0 ? 1.0 : 0.0;
-    double best = c0 ? -1.0 : 2.0;
+    const int n = hit_buildings(a.sc, o, a.steps[c0 ? j : j + 1], ids);
+    const ArcConst arc = a.arcs[j];
+    double best = c0 ? -1.0 : 2.0, best_dh = 0.0;
     int bbest = -1;
     for (int q = 0; q < n; ++q) {
         const int b = ids[q];
-        const bool s0 = c0 != 0;
         const int fa = a.fs.fp_off[b], v = a.fs.fp_off[b + 1] - fa;
-        double be_star = -1.0;
-        if (v <= kLinEdges) {
-            PrismLin P;
-            prism_lin_setup(P, a.fs.xy, fa, v, (double)a.heights[b], px, py, arc);
-            if (!prism_lin_inside(P, al_sh) || prism_lin_inside(P, al_lit)) continue;
-            // bracket in FP32, then the closed form of the pair of constraints that close
-            // the interval, confirmed by FP64 statuses on both sides of it
-            PrismLinF F;
-            prism_lin_to_f(P, F);
-            float flo = 0.f, fhi = 1.f;
-            for (int it = 0; it < kBisectF; ++it) {
-                const float mid = 0.5f * (flo + fhi);
-                if (prism_lin_inside_f(F, mid) == s0) flo = mid; else fhi = mid;
-            }
-            int il, iu;
-            prism_lin_active(P, s0 ? (double)flo : (double)fhi, &il, &iu);
-            double r;
-            if (pair_root(P, il, iu, &r) && r > kSide && r < 1.0 - kSide &&
-                fabs(r - 0.5 * ((double)flo + (double)fhi)) < 1e-4 &&
-                prism_lin_inside(P, r - kSide) == s0 && prism_lin_inside(P, r + kSide) != s0) {
-                be_star = r;
-            } else {
-                double lo = 0.0, hi = 1.0;   // invariant: status(lo) == status at the start
-                for (int it = 0; it < kBisect; ++it) {
-                    const double mid = 0.5 * (lo + hi);
-                    if (prism_lin_inside(P, mid) == s0) lo = mid; else hi = mid;
-                }
-                be_star = 0.5 * (lo + hi);
-            }
-        } else {
-            if (!prism_along(a.fs, a.heights, b, px, py, arc, al_sh)) continue;
-            if (prism_along(a.fs, a.heights, b, px, py, arc, al_lit)) continue;
-            double lo = 0.0, hi = 1.0;
-            for (int it = 0; it < kBisect; ++it) {
-                const double mid = 0.5 * (lo + hi);
-                if (prism_along(a.fs, a.heights, b, px, py, arc, mid) == s0) lo = mid; else hi = mid;
-            }
-            be_star = 0.5 * (lo + hi);
+        double be = -1.0, dh = 0.0;
+        if (FAST) {
+            if (v > kLinEdges || !solve_fast(a.fs, fa, v, a.heights[b], o.x, o.y, arc, c0 != 0, &be, &dh)) return -2;
+        } else if (!solve_fp64(a.fs, a.heights, b, (double)o.x, (double)o.y, arc_of(arc), c0 != 0, &be)) {
+            continue;
         }
-        const double as = slerp_param(arc, be_star);
-        if (c0 ? (as > best) : (as < best)) { best = as; bbest = b; }
+        // the slerp parameter grows with be
+        if (c0 ? (be > best) : (be < best)) { best = be; best_dh = dh; bbest = b; }
     }
     if (bbest < 0) {
         // No single building explains the flip in FP64 (a step status decided within FP32
         // rounding of a boundary): the flip time is unknown, count half the interval and
         // no derivative.
-        atomicAdd(a.S, 0.5 * a.dt * w);
-        return;
+        s += 0.5 * a.dt * w;
+        return -1;
     }
-    atomicAdd(a.S, a.dt * w * (c0 ? best : 1.0 - best));
+    const double al = slerp_param(arc, best);
+    s += a.dt * w * (c0 ? al : 1.0 - al);
+    const double sf = c0 ? 1.0 : -1.0;
+    if (FAST) {
+        if (best_dh == 0.0) return -1;                            // vertical-edge event
+        // d alpha / d be = |d x d'| / (|d|^2 theta) on the arc d = a + be e
+        const double dal = arc.inv_theta == 0.0
+                               ? 1.0
+                               : arc.sin_theta * arc.inv_theta / (1.0 - 2.0 * arc.omc * best * (1.0 - best));
+        grad = w * a.dt * sf * best_dh * dal;
+        return bbest;
+    }
     // is the flip the shadow of a roof edge?  (entry through edge e exactly at height h)
     const int fa = a.fs.fp_off[bbest], v = a.fs.fp_off[bbest + 1] - fa;
-    const double h = (double)a.heights[bbest];
-    const Vec3 d = arc_dir(arc, best);
-    const Vec3 dd = arc_ddir(arc, best);
+    const double h = (double)a.heights[bbest], px = o.x, py = o.y;
+    const Arc ac = arc_of(arc);
+    const Vec3 d = arc_dir(ac, al);
+    const Vec3 dd = arc_ddir(ac, al);
     const double ux = d.x / d.z, uy = d.y / d.z;
     const double dux = (dd.x * d.z - d.x * dd.z) / (d.z * d.z);
     const double duy = (dd.y * d.z - d.y * dd.z) / (d.z * d.z);
     const Entry e = prism(a.fs.xy, fa, v, h, px, py, ux, uy);
     const double tol = 1e-6 * (h + 1.0);
-    if (e.elo < 0 || fabs(e.zlo - h) > tol || e.zhi < h - tol) return;   // vertical-edge event
+    if (e.elo < 0 || fabs(e.zlo - h) > tol || e.zhi < h - tol) return -1;   // vertical-edge event
     const float2 p0 = a.fs.xy[fa + e.elo], p1 = a.fs.xy[fa + (e.elo + 1 == v ? 0 : e.elo + 1)];
     const double cx = (double)p1.x - (double)p0.x, cy = (double)p1.y - (double)p0.y;
     const double Bc = cx * uy - cy * ux;
     const double dB = cx * duy - cy * dux;
-    if (dB == 0.0) return;
-    const double dadh = -Bc / (h * dB);
-    const double sf = c0 ? 1.0 : -1.0;
-    atomicAdd(&a.dSdh[bbest], w * a.dt * sf * dadh);
+    if (dB == 0.0) return -1;
+    grad = w * a.dt * sf * (-Bc / (h * dB));
+    return bbest;
+}
+
+// One flip per thread: first every flip by the certified search (FAST), then the ones it left
+// over, packed so that no warp runs the FP64 search for one lane.  The minutes go to a list
+// that is summed in a fixed order (an atomic per flip on S alone serialised at the L2), the
+// derivatives are summed per warp and building before their atomics.
+template <bool FAST>
+__global__ void __launch_bounds__(kSolveThreads) k_flip_solve(SolveArgs a) {
+    const int lane = threadIdx.x & 31;
+    const long long n = FAST ? a.n_flips : (long long)*a.n_later;
+    for (long long f0 = (long long)blockIdx.x * kSolveThreads; f0 < n; f0 += (long long)gridDim.x * kSolveThreads) {
+        const long long f = f0 + threadIdx.x;
+        double s = 0.0, grad = 0.0;
+        int b = -1;
+        if (f < n) {
+            const long long i = FAST ? f : (long long)a.later[f];
+            b = solve_flip<FAST>(a, a.flips[i], s, grad);
+            a.minutes[i] = s;
+        }
+        __syncwarp();
+        if (FAST) {
+            const unsigned left = __ballot_sync(kFull, b == -2);
+            unsigned at = 0;
+            if (lane == 0 && left) at = atomicAdd(a.n_later, (unsigned)__popc(left));
+            at = __shfl_sync(kFull, at, 0);
+            if (b == -2) a.later[at + __popc(left & ((1u << lane) - 1u))] = (unsigned)f;
+        }
+        // sum over the lanes of the same building (pairs of peers first, then pairs of pairs), and
+        // one atomic by its first lane
+        const unsigned same = __match_any_sync(kFull, b);
+        const int leader = __ffs(same) - 1;
+        unsigned above = same & (0xfffffffeu << lane);
+        unsigned rank = __popc(same & ((1u << lane) - 1u));
+        while (__any_sync(kFull, above != 0u)) {
+            const int next = __ffs(above) - 1;
+            const double t = __shfl_sync(kFull, grad, next < 0 ? lane : next);
+            if (next >= 0) grad += t;
+            above &= ~__ballot_sync(kFull, rank & 1u);
+            rank >>= 1;
+        }
+        if (b >= 0 && lane == leader) atomicAdd(&a.dSdh[b], grad);
+    }
 }
 
 __global__ void k_to_float(const double* __restrict__ in, float* __restrict__ out, int n) {
@@ -476,50 +780,68 @@ cudaError_t launch_height_grad(const DevScene& sc, const FootprintSet& fs, const
     unsigned* counts = nullptr;
     unsigned* d_total = nullptr;
     int4* flips = nullptr;
-    int* gross = nullptr;
+    ArcConst* arcs = nullptr;
+    double *steady = nullptr, *minutes = nullptr;
+    unsigned* later = nullptr;
     const int B = fs.B;
 #define TRY(x) do { e = (x); if (e != cudaSuccess) goto done; } while (0)
     TRY(sa::scratch_alloc(&dsdh, sizeof(double) * (B > 0 ? B : 1), st));
-    TRY(sa::scratch_alloc(&S, sizeof(double), st));
+    TRY(sa::scratch_alloc(&S, sizeof(double) * (1 + kSumCtas), st));      // S and its flips' partial sums
     TRY(cudaMemsetAsync(dsdh, 0, sizeof(double) * (B > 0 ? B : 1), st));
-    TRY(cudaMemsetAsync(S, 0, sizeof(double), st));
+    TRY(cudaMemsetAsync(S, 0, sizeof(double) * (1 + kSumCtas), st));
     if (R > 0 && sun.n_blocks > 0) {
         TRY(sa::scratch_alloc(&masks, sizeof(unsigned long long) * (size_t)R * sun.n_blocks, st));
         TRY(cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)R * sun.n_blocks, st));
-        TRY(sa::scratch_alloc(&gross, sizeof(int) * (size_t)R, st));
         {
             DevOut out;
-            memset(&out, 0, sizeof(out));
-            out.gross = gross;
+            memset(&out, 0, sizeof(out));                  // only the masks are wanted
             out.masks = reinterpret_cast<uint64_t*>(masks);
-            int* run = nullptr;
-            TRY(sa::scratch_alloc(&run, sizeof(int) * (size_t)R, st));
-            out.run = run;
-            e = launch_raster_ground(sc, rc, sun, out, st);
-            cudaFreeAsync(run, st);
-            if (e != cudaSuccess) goto done;
+            TRY(launch_raster_ground(sc, rc, sun, out, st));
         }
-        TRY(sa::scratch_alloc(&counts, sizeof(unsigned) * (size_t)R, st));
+        constexpr int kGroups = 32;         // of blocks, at the most
+        FlipOrder go;
+        go.nx = rc.nx; go.ny = rc.ny; go.tiles_x = (rc.nx + 7) / 8;
+        go.n = 32ll * go.tiles_x * ((rc.ny + 3) / 4);
+        go.per = (sun.n_blocks + kGroups - 1) / kGroups;
+        const long long slots = go.n * ((sun.n_blocks + go.per - 1) / go.per);
+        TRY(sa::scratch_alloc(&counts, sizeof(unsigned) * (size_t)slots, st));
         TRY(sa::scratch_alloc(&d_total, sizeof(unsigned), st));
         const double dt = step_minutes;
-        const unsigned grid = (unsigned)((R + 255) / 256);
-        k_flip_count<<<grid, 256, 0, st>>>(masks, R, sun.blocks, sun.n_blocks, weights, dt, counts, S);
+        const unsigned grid = (unsigned)((go.n + 255) / 256);
+        TRY(sa::scratch_alloc(&steady, sizeof(double) * (kSumCtas + (size_t)grid), st));
+        k_flip_count<<<grid, 256, 0, st>>>(masks, R, go, sun.blocks, sun.n_blocks, weights, dt, counts,
+                                           steady + kSumCtas);
         TRY(cudaGetLastError());
-        TRY(exclusive_scan_u32(counts, R, d_total, st));
+        TRY(exclusive_scan_u32(counts, slots, d_total, st));
         unsigned total = 0;
         TRY(cudaMemcpyAsync(&total, d_total, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
         TRY(cudaStreamSynchronize(st));
         if (total > 0) {
             TRY(sa::scratch_alloc(&flips, sizeof(int4) * (size_t)total, st));
-            k_flip_fill<<<grid, 256, 0, st>>>(masks, R, sun.blocks, sun.n_blocks, counts, flips);
+            k_flip_fill<<<grid, 256, 0, st>>>(masks, R, go, sun.blocks, sun.n_blocks, counts, flips);
+            TRY(sa::scratch_alloc(&arcs, sizeof(ArcConst) * (size_t)sun.S, st));
+            k_arcs<<<(sun.S + 127) / 128, 128, 0, st>>>(sun.steps, sun.S - 1, arcs);
             SolveArgs sa;
+            sa.arcs = arcs;
             sa.sc = sc; sa.fs = fs; sa.heights = d_heights; sa.steps = sun.steps;
             sa.x0 = rc.x0; sa.y0 = rc.y0; sa.dx = rc.dx; sa.nx = rc.nx;
             sa.weights = weights; sa.dt = dt; sa.flips = flips; sa.n_flips = total;
-            sa.S = S; sa.dSdh = dsdh;
-            k_flip_solve<<<(unsigned)((total + 127) / 128), 128, 0, st>>>(sa);
+            TRY(sa::scratch_alloc(&minutes, sizeof(double) * (size_t)total, st));
+            sa.minutes = minutes; sa.dSdh = dsdh;
+            TRY(sa::scratch_alloc(&later, sizeof(unsigned) * ((size_t)total + 1), st));
+            TRY(cudaMemsetAsync(later, 0, sizeof(unsigned), st));
+            sa.n_later = later;
+            sa.later = later + 1;
+            const unsigned ctas = (unsigned)(((long long)total + kSolveThreads - 1) / kSolveThreads);
+            k_flip_solve<true><<<ctas, kSolveThreads, 0, st>>>(sa);
+            k_flip_solve<false><<<std::min(ctas, 152u * 16u), kSolveThreads, 0, st>>>(sa);
+            k_sum<<<kSumCtas, 256, 0, st>>>(minutes, total, S + 1);
             TRY(cudaGetLastError());
         }
+        // S: the steady intervals, then the flips
+        k_sum<<<kSumCtas, 256, 0, st>>>(steady + kSumCtas, grid, steady);
+        k_sum_pair<<<1, 256, 0, st>>>(steady, S + 1, S);
+        TRY(cudaGetLastError());
     }
     if (B > 0) k_to_float<<<(B + 255) / 256, 256, 0, st>>>(dsdh, dS_dh, B);
     TRY(cudaGetLastError());
@@ -531,7 +853,10 @@ done:
     if (counts) cudaFreeAsync(counts, st);
     if (d_total) cudaFreeAsync(d_total, st);
     if (flips) cudaFreeAsync(flips, st);
-    if (gross) cudaFreeAsync(gross, st);
+    if (arcs) cudaFreeAsync(arcs, st);
+    if (later) cudaFreeAsync(later, st);
+    if (steady) cudaFreeAsync(steady, st);
+    if (minutes) cudaFreeAsync(minutes, st);
     return e;
 #undef TRY
 }
