@@ -57,9 +57,10 @@ typedef enum {
  *   SA_SWEEP_RASTER   per-step shadow raster of ground receivers: each step projects
  *                     the triangles onto the ground separately (the per-minute
  *                     shadow-map baseline, Sec. 8.1).  Ground grids only.
- *   SA_ACCRUAL_TRACE  ray-traced accrual: one BVH traversal per receiver and block of
- *                     <= 64 steps, whose query is the whole fan of the block's rays
- *                     (the moving-shadow observation of Sec. 3.2 applied to rays).
+ *   SA_ACCRUAL_TRACE  ray-traced accrual: one BVH traversal per group of 128 neighbouring
+ *                     receivers and run of <= 27 steps (per warp and block for thin point
+ *                     sets), whose query is the whole fan of the run's rays (the
+ *                     moving-shadow observation of Sec. 3.2 applied to rays).
  *   SA_ACCRUAL_SAM    shadow accrual map (Sec. 4): one pass over the geometry serves all
  *                     the steps of a block (ground grids: the receiver-space accrual
  *                     raster) or of a run of <= 32 steps (points: a light-space map

@@ -336,6 +336,24 @@ __device__ __forceinline__ unsigned run_summary(unsigned long long m, int K) {
     return pop | (pre << 8) | (suf << 16) | (best << 24);
 }
 
+// ------------------------------------------------------------------ Morton codes
+__device__ __forceinline__ unsigned expand_bits10(unsigned v) {
+    v &= 0x3ffu;
+    v = (v | (v << 16)) & 0x030000FFu;
+    v = (v | (v << 8)) & 0x0300F00Fu;
+    v = (v | (v << 4)) & 0x030C30C3u;
+    v = (v | (v << 2)) & 0x09249249u;
+    return v;
+}
+
+// 30-bit code of a point of the unit cube
+__device__ __forceinline__ unsigned morton30(float x, float y, float z) {
+    unsigned ix = (unsigned)fminf(fmaxf(x * 1024.f, 0.f), 1023.f);
+    unsigned iy = (unsigned)fminf(fmaxf(y * 1024.f, 0.f), 1023.f);
+    unsigned iz = (unsigned)fminf(fmaxf(z * 1024.f, 0.f), 1023.f);
+    return (expand_bits10(ix) << 2) | (expand_bits10(iy) << 1) | expand_bits10(iz);
+}
+
 // ------------------------------------------------------------------ float helpers
 template <int A> __device__ __forceinline__ float comp(const float4& v);
 template <> __device__ __forceinline__ float comp<0>(const float4& v) { return v.x; }
@@ -516,12 +534,15 @@ struct DevRecv {
     const float4* nrm;      // facade normals in the same order, or null
     const int* perm;
     long long R;
+    const unsigned* order = nullptr;   // regrouping of the points (sorted indices), or null
 };
 
 struct DevSun {
     const StepConst* steps;
     const BlockConst* blocks;
     int S, n_blocks;
+    int max_K = kMaxBlock;      // steps of the longest block, or a bound
+    float max_slope = 0.f;      // largest |d_xy| / d_z of a block's slope box, if known
 };
 
 // outputs / state (state buffers hold gross, run, best per receiver in output order)
@@ -539,7 +560,8 @@ struct DevOut {
 
 cudaError_t launch_sweep_trace(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
                                const DevOut& out, cudaStream_t st);
-cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
+// (recv_box: bounds of point receivers, lo.xyz hi.xyz)
+cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const float* recv_box, const DevSun& sun,
                                  const DevOut& out, cudaStream_t st);
 // traversal mode of the sweep (which = 0) and accrual (which = 1) kernels
 void set_trace_mode(int which, int mode);
@@ -549,6 +571,11 @@ int get_trace_mode(int which);
 cudaError_t launch_raster_ground(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
                                  const DevOut& out, cudaStream_t st);
 
+// Stitches run summaries [nbc blocks][parts][R] of consecutive blocks, in time order, into the
+// receivers' gross / run / best state (loaded if load_state; the run is not written by the
+// final chunk, the minutes only by it).
+void launch_fold(const unsigned* summary, long long R, const BlockConst* blocks, int nbc, int parts,
+                 const DevOut& out, int* best, int load_state, int final_chunk, cudaStream_t st);
 // the run summary (run_summary) of every block and cell: summaries [n_blocks][R]
 cudaError_t launch_raster_summaries(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
                                     unsigned* summaries, cudaStream_t st);
@@ -679,8 +706,9 @@ cudaError_t sort_points(const float* d_pos, const float* d_nrm, long long n, flo
                         float4* d_nrm_sorted, int* d_perm, cudaStream_t st, long long* bad_out,
                         float* box_out);
 
-// radix sort of (key, value) pairs by key (stable, 32-bit keys), in place via scratch
-cudaError_t radix_sort_pairs(unsigned* keys, unsigned* vals, long long n, cudaStream_t st);
+// radix sort of (key, value) pairs by the low `bits` (16 or 32) of their keys (stable, the
+// rest zero), in place via scratch
+cudaError_t radix_sort_pairs(unsigned* keys, unsigned* vals, long long n, cudaStream_t st, int bits = 32);
 
 // exclusive scan of n uint32 (in place); writes the total to *d_total if non-null
 cudaError_t exclusive_scan_u32(unsigned* data, long long n, unsigned* d_total, cudaStream_t st);

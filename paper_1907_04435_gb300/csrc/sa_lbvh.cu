@@ -18,22 +18,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ unsigned expand_bits10(unsigned v) {
-    v &= 0x3ffu;
-    v = (v | (v << 16)) & 0x030000FFu;
-    v = (v | (v << 8)) & 0x0300F00Fu;
-    v = (v | (v << 4)) & 0x030C30C3u;
-    v = (v | (v << 2)) & 0x09249249u;
-    return v;
-}
-
-__device__ __forceinline__ unsigned morton3(float x, float y, float z) {
-    unsigned ix = (unsigned)fminf(fmaxf(x * 1024.f, 0.f), 1023.f);
-    unsigned iy = (unsigned)fminf(fmaxf(y * 1024.f, 0.f), 1023.f);
-    unsigned iz = (unsigned)fminf(fmaxf(z * 1024.f, 0.f), 1023.f);
-    return (expand_bits10(ix) << 2) | (expand_bits10(iy) << 1) | expand_bits10(iz);
-}
-
 // order-preserving float <-> uint map for atomic min / max
 __device__ __forceinline__ unsigned f2o(float f) {
     unsigned u = __float_as_uint(f);
@@ -125,7 +109,7 @@ __global__ void k_morton(const float4* __restrict__ raw, long long nt,
     float4 a = raw[3 * t], b = raw[3 * t + 1], c = raw[3 * t + 2];
     float cx = (a.x + b.x + c.x) * (1.f / 3.f), cy = (a.y + b.y + c.y) * (1.f / 3.f),
           cz = (a.z + b.z + c.z) * (1.f / 3.f);
-    keys[t] = morton3((cx - lo[0]) * inv[0], (cy - lo[1]) * inv[1], (cz - lo[2]) * inv[2]);
+    keys[t] = morton30((cx - lo[0]) * inv[0], (cy - lo[1]) * inv[1], (cz - lo[2]) * inv[2]);
     vals[t] = (unsigned)t;
 }
 
@@ -412,7 +396,7 @@ __global__ void k_points_morton(const float4* __restrict__ o, const float* __res
         inv[k] = ext > 0.f ? 1.f / ext : 0.f;
     }
     float4 p = o[i];
-    unsigned key = morton3((p.x - lo[0]) * inv[0], (p.y - lo[1]) * inv[1], (p.z - lo[2]) * inv[2]);
+    unsigned key = morton30((p.x - lo[0]) * inv[0], (p.y - lo[1]) * inv[1], (p.z - lo[2]) * inv[2]);
     if (nrm) {
         const float az = atan2f(nrm[3 * i + 1], nrm[3 * i]);          // (-pi, pi]
         unsigned sector = (unsigned)((az + 3.14159265f) * (16.f / 6.2831853f));

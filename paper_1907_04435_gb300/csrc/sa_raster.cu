@@ -914,22 +914,6 @@ k_items_fold(const unsigned* __restrict__ summary, long long R, const BlockConst
     }
 }
 
-// Four cells per thread from a million cells up, where every row of summaries and every
-// output starts on 16 bytes.
-void launch_k_fold(const unsigned* summary, long long R, const BlockConst* blocks, int nbc, int parts,
-                   const DevOut& out, int* best, int load_state, int final_chunk, cudaStream_t st) {
-    const uintptr_t at = reinterpret_cast<uintptr_t>(out.gross) | reinterpret_cast<uintptr_t>(best) |
-                         reinterpret_cast<uintptr_t>(out.run) | reinterpret_cast<uintptr_t>(out.minutes) |
-                         reinterpret_cast<uintptr_t>(summary);
-    if (R >= (1 << 20) && R % 4 == 0 && (at & 15) == 0) {
-        const unsigned g = (unsigned)((R / 4 + kFoldThreads - 1) / kFoldThreads);
-        k_items_fold<4><<<g, kFoldThreads, 0, st>>>(summary, R, blocks, nbc, parts, out, best, load_state, final_chunk);
-    } else {
-        const unsigned g = (unsigned)((R + kFoldThreads - 1) / kFoldThreads);
-        k_items_fold<1><<<g, kFoldThreads, 0, st>>>(summary, R, blocks, nbc, parts, out, best, load_state, final_chunk);
-    }
-}
-
 // --------------------------------------------------------------- batched scenarios
 // A persistent launch over work items (interval, variant, tile of the variant's region).
 // Each item rasters every block of its interval for one tile: the base city's binned
@@ -1066,6 +1050,22 @@ void launch_k_items(const RasterArgs& ra, int n_items, bool stats, cudaStream_t 
 }
 
 }  // namespace
+
+// Four cells per thread from a million cells up, where every row of summaries and every
+// output starts on 16 bytes.
+void launch_fold(const unsigned* summary, long long R, const BlockConst* blocks, int nbc, int parts,
+                 const DevOut& out, int* best, int load_state, int final_chunk, cudaStream_t st) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(out.gross) | reinterpret_cast<uintptr_t>(best) |
+                         reinterpret_cast<uintptr_t>(out.run) | reinterpret_cast<uintptr_t>(out.minutes) |
+                         reinterpret_cast<uintptr_t>(summary);
+    if (R >= (1 << 20) && R % 4 == 0 && (at & 15) == 0) {
+        const unsigned g = (unsigned)((R / 4 + kFoldThreads - 1) / kFoldThreads);
+        k_items_fold<4><<<g, kFoldThreads, 0, st>>>(summary, R, blocks, nbc, parts, out, best, load_state, final_chunk);
+    } else {
+        const unsigned g = (unsigned)((R + kFoldThreads - 1) / kFoldThreads);
+        k_items_fold<1><<<g, kFoldThreads, 0, st>>>(summary, R, blocks, nbc, parts, out, best, load_state, final_chunk);
+    }
+}
 
 // Pieces each block's steps are cut into: one from 1,824 items (two waves of
 // SA_RASTER_CTAS CTAs on 152 SMs) up, where the items alone fill the chip and a piece only
@@ -1205,7 +1205,7 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
             else launch_k_items(ra, (int)ncc, out.stats != nullptr, st);
         }
         if (fold)
-            launch_k_fold(summary, R, sun.blocks + b0, nbc, parts, out, best, ra.load_state, ra.final_chunk, st);
+            launch_fold(summary, R, sun.blocks + b0, nbc, parts, out, best, ra.load_state, ra.final_chunk, st);
         e = cudaGetLastError();
     }
     for (void* p : {(void*)words, (void*)bins, (void*)best_scratch, fold ? (void*)summary : nullptr})

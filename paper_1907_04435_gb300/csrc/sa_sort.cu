@@ -255,7 +255,7 @@ cudaError_t launch_work_order(const unsigned* tc, const unsigned* rc, long long 
     return cudaGetLastError();
 }
 
-cudaError_t radix_sort_pairs(unsigned* keys, unsigned* vals, long long n, cudaStream_t st) {
+cudaError_t radix_sort_pairs(unsigned* keys, unsigned* vals, long long n, cudaStream_t st, int bits) {
     if (n <= 1) return cudaSuccess;
     const int n_tiles = (int)((n + kSortTile - 1) / kSortTile);
     unsigned *k2 = nullptr, *v2 = nullptr, *hist = nullptr;
@@ -268,7 +268,7 @@ cudaError_t radix_sort_pairs(unsigned* keys, unsigned* vals, long long n, cudaSt
         return e;
     }
     unsigned *ka = keys, *va = vals, *kb = k2, *vb = v2;
-    for (int shift = 0; shift < 32 && e == cudaSuccess; shift += 8) {
+    for (int shift = 0; shift < bits && e == cudaSuccess; shift += 8) {
         k_radix_hist<<<n_tiles, kSortThreads, 0, st>>>(ka, n, shift, hist, n_tiles);
         e = exclusive_scan_u32(hist, (long long)kRadix * n_tiles, nullptr, st);
         if (e != cudaSuccess) break;
@@ -277,7 +277,7 @@ cudaError_t radix_sort_pairs(unsigned* keys, unsigned* vals, long long n, cudaSt
         unsigned* t = ka; ka = kb; kb = t;
         t = va; va = vb; vb = t;
     }
-    // four passes: the result is back in the caller's buffers
+    // two or four passes: the result is back in the caller's buffers
     cudaFreeAsync(k2, st);
     cudaFreeAsync(v2, st);
     cudaFreeAsync(hist, st);
