@@ -40,6 +40,12 @@ struct sa_batch {
     cudaGraphExec_t exec = nullptr;
     int* g_counts = nullptr;
     int* g_impact = nullptr;
+    // runs from the base masks (k_batch_delta), where they fit and tiles are skipped
+    bool by_delta = false;
+    sa::BatchDelta delta{};
+    int4* d_work = nullptr;                         // its items
+    int n_work = 0;
+    long long max_cells = 0;
 };
 
 namespace sa {
@@ -61,9 +67,10 @@ inline int __float_as_int_host(float f) {
     return i;
 }
 
-sa::BatchLaunch launch_of(const sa_batch* b, int* counts, int* impact, int n_items, int ctas,
+// share: the first 1 / share of the work items
+sa::BatchLaunch launch_of(const sa_batch* b, int* counts, int* impact, int share, int ctas,
                           int run, unsigned long long* stats) {
-    sa::BatchLaunch bl;
+    sa::BatchLaunch bl{};
     bl.base.nodes = b->base->bvh.nodes;
     bl.base.tris = b->base->bvh.tris;
     bl.base.n_nodes = b->base->bvh.n_nodes;
@@ -72,8 +79,13 @@ sa::BatchLaunch launch_of(const sa_batch* b, int* counts, int* impact, int n_ite
     bl.grid = b->grid;
     bl.intervals = b->d_iv;
     bl.variants = b->d_var;
-    bl.items = b->d_items;
-    bl.n_items = n_items;
+    bl.items = b->by_delta ? b->d_work : b->d_items;
+    const int n = b->by_delta ? b->n_work : b->n_items;
+    bl.n_items = share > 1 ? std::max(std::min(n, 1), n / share) : n;
+    bl.delta = b->by_delta ? &b->delta : nullptr;
+    bl.V = b->V;
+    bl.I = b->I;
+    bl.max_cells = b->max_cells;
     bl.counter = b->d_counter;
     bl.removed = b->d_removed;
     bl.tower_tris = b->d_towers;
@@ -175,14 +187,36 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
-    b->ctas = 4 * b->sms;
+    b->ctas = sa::raster_ctas_per_sm() * b->sms;     // 16 variants: 6.2 ms at 4 CTAs per SM, 4.9 at 6
     b->run = sa::get_raster_run();
-    if (e == cudaSuccess) e = dev_copy(b, hv.data(), hv.size(), &b->d_var);
     if (e == cudaSuccess) e = dev_copy(b, towers.data(), towers.size(), &b->d_towers);
     if (e == cudaSuccess) e = dev_copy(b, v->removed_ids, (size_t)n_rem, &b->d_removed);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(unsigned));
     if (e == cudaSuccess) b->owned.push_back(b->d_counter);
-    // per interval: base bins and base counts
+    // The base masks of every interval, where they take at most a quarter of the device's free
+    // memory (8 bytes per cell and block: 453 MB for 1024^2 cells, two intervals of 3 days);
+    // without them, or with the tile skipping off, every run rasters its tiles whole.
+    size_t mask_words = 0;
+    for (int i = 0; i < n_intervals; ++i) mask_words += intervals[i]->h_blocks.size() * (size_t)grid->R;
+    unsigned long long* masks = nullptr;
+    if (e == cudaSuccess && mask_words > 0 && V > 0 && sa::get_batch_tile_skip()) {
+        size_t free_b = 0, total_b = 0;
+        e = cudaMemGetInfo(&free_b, &total_b);
+        if (e == cudaSuccess && mask_words * 8 <= free_b / 4) {
+            if (sa::scratch_alloc(&masks, mask_words * 8, st) == cudaSuccess) {
+                b->owned.push_back(masks);
+                e = cudaMemsetAsync(masks, 0, mask_words * 8, st);
+                b->by_delta = true;
+            } else {
+                cudaGetLastError();
+                masks = nullptr;
+            }
+        }
+    }
+    b->delta.masks = masks;
+    b->delta.R = grid->R;
+    size_t mask_off = 0;
+    // per interval: base bins, base counts and base masks
     sa::DevScene dsc;
     dsc.nodes = base->bvh.nodes; dsc.tris = base->bvh.tris; dsc.n_nodes = base->bvh.n_nodes;
     dsc.T = (int)base->T; dsc.closed = base->closed;
@@ -208,22 +242,28 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
             int *bc = nullptr, *run = nullptr;
             e = cudaMalloc(&bc, sizeof(int) * (size_t)grid->R);
             if (e == cudaSuccess) b->owned.push_back(bc);
+            if (e == cudaSuccess) e = cudaMemsetAsync(bc, 0, sizeof(int) * (size_t)grid->R, st);
             if (e == cudaSuccess) e = sa::scratch_alloc(&run, sizeof(int) * (size_t)grid->R, st);
             if (e == cudaSuccess) {
                 sa::DevOut o;
                 memset(&o, 0, sizeof(o));
                 o.gross = bc;
                 o.run = run;
+                if (masks) o.masks = reinterpret_cast<uint64_t*>(masks + mask_off);
                 e = sa::launch_raster_ground(dsc, b->grid, ds, o, st);
                 cudaFreeAsync(run, st);
             }
             bi.base_counts = bc;
         }
+        bi.mask_off = mask_off;
+        mask_off += (size_t)ds.n_blocks * (size_t)grid->R;
         b->h_iv.push_back(bi);
     }
     if (e == cudaSuccess) e = dev_copy(b, b->h_iv.data(), b->h_iv.size(), &b->d_iv);
     // Boxes of what each variant changes: its removed base buildings and its towers.
     std::vector<std::vector<float>> changed(V);     // per variant: lo.xyz hi.xyz ...
+    std::vector<float4> boxes;                      // the same for the device, and the removed
+    std::vector<int> rem_tri;                       // buildings' triangles
     if (e == cudaSuccess && V > 0) {
         std::vector<float4> bt((size_t)base->T * 3);
         if (base->T > 0)
@@ -243,12 +283,26 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
                 bb[3] = std::max(bb[3], p.x); bb[4] = std::max(bb[4], p.y); bb[5] = std::max(bb[5], p.z);
             }
         }
+        // the triangles of every building, in order
+        std::vector<int> first((size_t)std::max(base->n_buildings, 0) + 1, 0), of((size_t)base->T);
+        if (b->by_delta) {
+            auto id = [&](long long t) { const int i = __float_as_int_host(bt[3 * t].w); return i >= 0 && i < base->n_buildings ? i : -1; };
+            for (long long t = 0; t < base->T; ++t) if (id(t) >= 0) ++first[(size_t)id(t) + 1];
+            for (size_t q = 1; q < first.size(); ++q) first[q] += first[q - 1];
+            std::vector<int> at(first);
+            for (long long t = 0; t < base->T; ++t) if (id(t) >= 0) of[(size_t)at[(size_t)id(t)]++] = (int)t;
+        }
         for (int k = 0; k < V; ++k) {
+            hv[k].remtri_off = (int)rem_tri.size();
             for (int q = v->removed_off[k]; q < v->removed_off[k + 1]; ++q) {
                 const int bid = v->removed_ids[q];
                 if (bid < 0 || bid >= base->n_buildings) continue;
                 changed[k].insert(changed[k].end(), &bbox[6 * (size_t)bid], &bbox[6 * (size_t)bid] + 6);
+                if (b->by_delta)
+                    rem_tri.insert(rem_tri.end(), of.begin() + first[(size_t)bid], of.begin() + first[(size_t)bid + 1]);
             }
+            const size_t n_removed = changed[k].size() / 6;
+            hv[k].n_remtri = (int)rem_tri.size() - hv[k].remtri_off;
             for (int t = v->tower_off[k]; t < v->tower_off[k + 1]; ++t) {
                 float b6[6] = {3.4e38f, 3.4e38f, 3.4e38f, -3.4e38f, -3.4e38f, -3.4e38f};
                 for (int q = 0; q < 3; ++q)
@@ -259,8 +313,24 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
                     }
                 changed[k].insert(changed[k].end(), b6, b6 + 6);
             }
+            hv[k].box_off = (int)boxes.size() / 2;
+            for (size_t q = 0; q < changed[k].size(); q += 6) {
+                const float* c = &changed[k][q];
+                if (c[0] > c[3]) continue;                     // a building without triangles
+                boxes.push_back(make_float4(c[0], c[1], c[2], q / 6 < n_removed ? 1.f : 0.f));
+                boxes.push_back(make_float4(c[3], c[4], c[5], 0.f));
+            }
+            hv[k].n_box = (int)boxes.size() / 2 - hv[k].box_off;
+            b->max_cells = std::max(b->max_cells, (long long)hv[k].nx * hv[k].ny);
         }
     }
+    float4* d_boxes = nullptr;
+    int* d_rem_tri = nullptr;
+    if (e == cudaSuccess) e = dev_copy(b, hv.data(), hv.size(), &b->d_var);
+    if (e == cudaSuccess && b->by_delta) e = dev_copy(b, boxes.data(), boxes.size(), &d_boxes);
+    if (e == cudaSuccess && b->by_delta) e = dev_copy(b, rem_tri.data(), rem_tri.size(), &d_rem_tri);
+    b->delta.boxes = d_boxes;
+    b->delta.rem_tri = d_rem_tri;
     // Work items: every tile of every variant's region, for every interval.  A tile is
     // marked affected if the shadow of a changed box, swept over the interval's slope
     // range, can reach it (one cell of margin); other tiles keep the base counts.
@@ -302,7 +372,27 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
     b->n_affected = 0;
     for (const int4& it : items) b->n_affected += it.w;
     b->n_items = (int)items.size();
-    if (e == cudaSuccess) e = dev_copy(b, items.data(), items.size(), &b->d_items);
+    if (e == cudaSuccess && b->by_delta) {
+        // the blocks of the affected tiles that a change reaches, one item each; a batch with
+        // more than 64M of them rasters its tiles whole
+        int4* d_tiles = nullptr;
+        int max_blocks = 0;
+        for (const sa::BatchInterval& iv : b->h_iv) max_blocks = std::max(max_blocks, iv.n_blocks);
+        unsigned n_work = 0;
+        int* order = nullptr;
+        e = dev_copy(b, items.data(), (size_t)b->n_affected, &d_tiles);
+        if (e == cudaSuccess)
+            e = sa::pick_batch_items(launch_of(b, nullptr, nullptr, 1, 0, 0, nullptr), d_tiles, b->n_affected, max_blocks,
+                                     1u << 26, &n_work, &b->d_work, &order, st);
+        if (b->d_work) b->owned.push_back(b->d_work);
+        if (order) b->owned.push_back(order);
+        b->delta.order = order;
+        b->n_work = (int)std::min(n_work, 1u << 26);
+        if (n_work > (1u << 26)) b->by_delta = false;
+    }
+    if (!b->by_delta && e == cudaSuccess) {
+        e = dev_copy(b, items.data(), items.size(), &b->d_items);
+    }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
@@ -334,7 +424,7 @@ sa_status sa_batch_run(sa_batch* b, int32_t* counts, int32_t* impact, void* stre
         drop_graph(b);
         e = cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            cudaError_t le = sa::launch_batch(launch_of(b, counts, impact, b->n_items, b->ctas, b->run, nullptr),
+            cudaError_t le = sa::launch_batch(launch_of(b, counts, impact, 1, b->ctas, b->run, nullptr),
                                               b->capture);
             e = cudaStreamEndCapture(b->capture, &b->graph);
             if (le != cudaSuccess) e = le;
@@ -357,7 +447,6 @@ sa_status sa_batch_run(sa_batch* b, int32_t* counts, int32_t* impact, void* stre
 sa_status sa_batch_tune(sa_batch* b, int32_t* best_ctas, int32_t* best_run, void* stream) {
     if (!b) return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_tune: NULL batch");
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    const int n = std::max(1, b->n_items / 8);
     int* scratch = nullptr;
     cudaError_t e = sa::scratch_alloc(&scratch, sizeof(int) * (size_t)std::max<long long>(1, b->I * b->cells_per_interval), st);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -368,7 +457,7 @@ sa_status sa_batch_tune(sa_batch* b, int32_t* best_ctas, int32_t* best_run, void
     const int runs[3] = {8, 16, 24};
     for (int c = 2; c <= sa::raster_ctas_per_sm() && e == cudaSuccess; ++c)
         for (int r : runs) {
-            const sa::BatchLaunch bl = launch_of(b, scratch, nullptr, n, c * b->sms, r, nullptr);
+            const sa::BatchLaunch bl = launch_of(b, scratch, nullptr, 8, c * b->sms, r, nullptr);
             e = sa::launch_batch(bl, st);                                   // warm-up
             if (e == cudaSuccess) e = cudaEventRecord(e0, st);
             if (e == cudaSuccess) e = sa::launch_batch(bl, st);
@@ -400,7 +489,7 @@ sa_status sa_batch_work_counters(sa_batch* b, uint64_t* counters, void* stream) 
     if (e == cudaSuccess)
         e = sa::scratch_alloc(&scratch, sizeof(int) * (size_t)std::max<long long>(1, b->I * b->cells_per_interval), st);
     if (e == cudaSuccess)
-        e = sa::launch_batch(launch_of(b, scratch, nullptr, b->n_items, b->ctas, b->run,
+        e = sa::launch_batch(launch_of(b, scratch, nullptr, 1, b->ctas, b->run,
                                        reinterpret_cast<unsigned long long*>(counters)), st);
     if (scratch) cudaFreeAsync(scratch, st);
     if (e != cudaSuccess) return sa::report_error(SA_ERR_CUDA, cudaGetErrorString(e));

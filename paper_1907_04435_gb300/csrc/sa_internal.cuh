@@ -630,12 +630,24 @@ struct BatchInterval {
     const int* bins;
     const int* base_counts;       // [R] gross of the base city (nullable)
     long long out_base;           // offset of this interval's outputs
+    size_t mask_off;              // first word of this interval's base masks (BatchDelta)
 };
 struct BatchVariant {
     int tower_off, n_tower;       // triangles in the tower list
     int rem_off, n_rem;           // ids in the removed list
     int ix0, iy0, nx, ny;         // region in cells of the base grid
     long long out_off;            // offset within an interval's outputs
+    int box_off, n_box;           // changed boxes: removed buildings and tower triangles
+    int remtri_off, n_remtri;     // base triangles of the removed buildings
+};
+// What a batch keeps of the base city beyond its bins and counts, so that a run rasters only
+// what the variants change.
+struct BatchDelta {
+    const unsigned long long* masks;   // base step masks: per interval [n_blocks][R] at mask_off
+    long long R;
+    const float4* boxes;               // (lo.xyz, 1 = removed building), (hi.xyz, 0)
+    const int* rem_tri;                // base triangles of removed buildings, per variant
+    const int* order;                  // launch order of the items, heaviest first
 };
 // Base bins of every block of one interval over all tiles (device, caller frees with
 // cudaFree): offsets / counts [n_blocks][tiles], bins [total].
@@ -656,6 +668,9 @@ struct BatchLaunch {
     unsigned long long* stats;
     int ctas;                     // persistent CTAs
     int run;                      // raster steps per work unit
+    const BatchDelta* delta;      // non-null: items are those of pick_batch_items, for k_batch_delta
+    int V, I;
+    long long max_cells;          // cells of the largest region
 };
 void set_raster_run(int run);
 int get_raster_run();
@@ -665,6 +680,11 @@ int get_point_run();
 void set_batch_tile_skip(int on);
 int get_batch_tile_skip();
 cudaError_t launch_batch(const BatchLaunch& bl, cudaStream_t st);
+// Items of k_batch_delta for n affected tiles (interval, variant, tile) of bl's batch, and their
+// launch order (device, freed by the caller with cudaFree); *n_items above max_items: none
+// are made.  Synchronises st.
+cudaError_t pick_batch_items(const BatchLaunch& bl, const int4* d_tiles, long long n, int max_blocks,
+                             unsigned max_items, unsigned* n_items, int4** items, int** order, cudaStream_t st);
 
 // shadow accrual map of point receivers in light space (scene_box, recv_box: lo.xyz hi.xyz)
 cudaError_t launch_sam_points(const DevScene& sc, const float* scene_box, const DevRecv& rc,

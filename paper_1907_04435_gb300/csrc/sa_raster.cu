@@ -570,11 +570,13 @@ __device__ __forceinline__ void raster_units(TileSmem& sm, int un0, int nu, int 
 // <= 32 steps), bounds the run's swept projection, spreads its lanes over the covered
 // cells (row-major, 32 at a time) and per cell tests the run's steps with the expanded
 // edge functions; step bits are ORed into sm.mask.  Leaves sm.mask complete for the block.
+// prefilled: sm.mask holds bits from the start, whose full rows are skipped at once.
 template <bool COUNT, bool CULL, class Fetch>
 __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const StepConst* steps,
                              int j0, int K, float tox, float toy, float inv_dx, int kSub,
                              unsigned long long& n_cell, unsigned long long& n_test,
-                             unsigned long long& n_unit, unsigned long long& n_span) {
+                             unsigned long long& n_unit, unsigned long long& n_span,
+                             bool prefilled = false) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nsub = (K + kSub - 1) / kSub;
     __syncthreads();
@@ -633,7 +635,7 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
         // before their spans are found, and a tile shadowed at every step is done.  A low
         // sun bins thousands of triangles to a tile that the first few hundred fill
         // (1024^2 cells, 16 December: 25.0 -> 16.4 ms; the June district is unchanged).
-        if (base > 0) {
+        if (base > 0 || prefilled) {
             for (int row = warp; row < kTile; row += kWarpsRaster) {
                 const unsigned long long m = sm.mask[row * kTile + lane];
                 const unsigned lo = __reduce_and_sync(0xffffffffu, (unsigned)m);
@@ -643,11 +645,12 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
         }
         __syncthreads();
         unsigned long long tile_full = 0ull;
-        if (base > 0) {
+        if (base > 0 || prefilled) {
             const unsigned long long m = sm.row_full[lane];
             tile_full = ((unsigned long long)__reduce_and_sync(0xffffffffu, (unsigned)(m >> 32)) << 32) |
                         __reduce_and_sync(0xffffffffu, (unsigned)m);
-            if (tile_full == (K >= 64 ? ~0ull : (1ull << K) - 1ull)) break;
+            const unsigned long long all = K >= 64 ? ~0ull : (1ull << K) - 1ull;
+            if ((tile_full & all) == all) break;
         }
         if (threadIdx.x == 0) sm.next_unit = kWarpsRaster * kUnitClaim;
         // sun-facing steps of each staged triangle: a warp per triangle, a lane per step
@@ -1038,6 +1041,223 @@ k_batch(BatchArgs ba) {
     if (COUNT) flush_raster_counts(ba.stats, n_cell, n_test, n_unit, n_span);
 }
 
+// Batched scenarios from the base city's step masks.  A variant's mask of a tile and block
+// differs from the base mask only where its removed buildings or its towers cast shadow, and
+// every decision is the OR of the same exact tests, so it is put together from them:
+//   - a block no changed box's swept shadow reaches keeps the base counts;
+//   - bits no removed triangle covers stay as they are; the others are decided again by the
+//     base bins without the removed buildings, everything else counting as filled so that
+//     the raster passes over it;
+//   - the towers' triangles are ORed in on top.
+// An item is one (interval, variant, tile, block) that k_batch_pick found changed; its change
+// of the gross counts is added to the outputs, which k_batch_base has set to the base
+// counts.  Against k_batch (every block of an affected tile rastered whole): 16 variants x 2
+// intervals x 3 days over 1024^2 cells 18.2 -> 4.97 ms (bound by the towers' rasters, half of
+// their cells lit, and by the barriers of small launches of work).
+constexpr int kChangeList = 256;          // changed triangles picked per round
+
+// Triangles of k_batch_delta's rasters: item i is tris[map[list[i]]] (either index may be
+// absent); one of the removed buildings' triangles is skipped.
+struct DeltaFetch {
+    const float4* tris;
+    const int* map;
+    const int* list;
+    const int* rem;
+    int n_rem;
+    __device__ __forceinline__ bool operator()(int i, int v, float4* out) const {
+        int t = list ? list[i] : i;
+        if (map) t = map[t];
+        const float4 x = __ldg(&tris[3ll * t + v]);
+        *out = x;
+        if (v != 0 || n_rem == 0) return true;
+        const int bid = __float_as_int(x.w);
+        for (int q = 0; q < n_rem; ++q)
+            if (rem[q] == bid) return false;
+        return true;
+    }
+};
+
+// One copy of the unrolled step tests for the three rasters of a block.
+template <bool COUNT, bool CULL>
+__device__ __noinline__ void raster_block_call(TileSmem& sm, const DeltaFetch& fetch, int n, const StepConst* steps,
+                                               const BlockConst& bc, float tox, float toy, float inv_dx, int kSub,
+                                               bool prefilled, unsigned long long* cnt) {
+    raster_block<COUNT, CULL>(sm, fetch, n, steps, bc.j0, bc.K, tox, toy, inv_dx, kSub, cnt[0], cnt[1], cnt[2], cnt[3],
+                              prefilled);
+}
+
+// Can the shadow of a box (corners lo, hi; z >= 0), swept over the block, reach tile (tx, ty)?
+__device__ __forceinline__ bool box_reaches(const float4& lo, const float4& hi, const BlockConst& bc,
+                                            const TileGeom& g, int tx, int ty) {
+    const float h = fmaxf(hi.z, 0.f), inv = 1.f / (kTile * g.dx);
+    const float x0 = lo.x - fmaxf(h * bc.uxhi, 0.f), x1 = hi.x - fminf(h * bc.uxlo, 0.f);
+    const float y0 = lo.y - fmaxf(h * bc.uyhi, 0.f), y1 = hi.y - fminf(h * bc.uylo, 0.f);
+    // one cell of margin on every side absorbs rounding, as in swept_tiles
+    return floorf((x0 - g.x0 - g.dx) * inv) <= (float)tx && floorf((x1 - g.x0 + g.dx) * inv) >= (float)tx &&
+           floorf((y0 - g.y0 - g.dx) * inv) <= (float)ty && floorf((y1 - g.y0 + g.dx) * inv) >= (float)ty;
+}
+
+template <bool COUNT, bool CULL>
+__global__ void __launch_bounds__(kRasterThreads, SA_RASTER_CTAS)
+k_batch_delta(BatchArgs ba, BatchDelta bd) {
+    __shared__ TileSmem sm;
+    __shared__ int s_list[kChangeList];
+    __shared__ int s_item, s_n;
+    unsigned long long cnt[4] = {0ull, 0ull, 0ull, 0ull};       // cell set-ups, step tests, units, spans
+    const TileGeom& g = ba.g;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row0 = warp * 4;
+    const float inv_dx = 1.f / g.dx;
+    const int n_tiles = g.tiles_x * g.tiles_y;
+    while (true) {
+        __syncthreads();
+        if (tid == 0) s_item = (int)atomicAdd(ba.counter, 1u);
+        __syncthreads();
+        const int item = s_item;
+        if (item >= ba.n_items) break;
+        // interval, variant, tile, block * 4 + (removed buildings reach it) * 2 + (towers do)
+        const int4 it = ba.items[bd.order[item]];
+        const BatchInterval& iv = ba.intervals[it.x];
+        const BatchVariant& var = ba.variants[it.y];
+        const int tile = it.z, bl = it.w >> 2;
+        const bool remv = it.w & 2, tow = it.w & 1;
+        const int tx = tile % g.tiles_x, ty = tile / g.tiles_x;
+        const int ix = tx * kTile + lane;
+        const float4* towers = ba.tower_tris + 3ll * var.tower_off;
+        const int* rem = ba.removed + var.rem_off;
+        const int n_rem = var.n_rem;
+        const int* rem_tri = bd.rem_tri + var.remtri_off;
+        const float4* tris = ba.base_tris;
+        const BlockConst& bc = iv.blocks[bl];
+        float tox, toy;
+        tile_setup(sm, g, tx, ty, &tox, &toy);
+        unsigned long long base[4], now[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int iy = ty * kTile + row0 + q;
+            base[q] = (ix < g.nx && iy < g.ny)
+                          ? __ldg(&bd.masks[(size_t)bl * bd.R + iv.mask_off + (size_t)iy * g.nx + ix]) : 0ull;
+            now[q] = base[q];
+            if (remv) sm.mask[(row0 + q) * kTile + lane] = 0ull;
+        }
+        // rasters the changed triangles pick(i) < n that reach the tile, kChangeList at a time
+        auto raster_changed = [&](DeltaFetch f, int n, bool prefilled) {
+            for (int i0 = 0; i0 < n; i0 += kChangeList) {
+                __syncthreads();
+                if (tid == 0) s_n = 0;
+                __syncthreads();
+                const int i = i0 + tid;
+                bool pick = false;
+                if (i < n) {
+                    const float4* t = f.tris + 3ll * (f.map ? f.map[i] : i);
+                    const float4 a = __ldg(t), b = __ldg(t + 1), c = __ldg(t + 2);
+                    int x0, x1, y0, y1;
+                    pick = tri_above_ground(a, b, c) && swept_tiles(a, b, c, bc, g, &x0, &x1, &y0, &y1) &&
+                           tx >= x0 && tx <= x1 && ty >= y0 && ty <= y1;
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, pick);
+                int at = 0;
+                if (lane == 0 && bal) at = atomicAdd(&s_n, __popc(bal));
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (pick) s_list[at + __popc(bal & ((1u << lane) - 1u))] = i;
+                __syncthreads();
+                const int m = s_n;
+                f.list = s_list;
+                if (m > 0)
+                    raster_block_call<COUNT, CULL>(sm, f, m, iv.steps, bc, tox, toy, inv_dx, ba.run, prefilled, cnt);
+            }
+        };
+        if (remv) {
+            raster_changed(DeltaFetch{tris, rem_tri, nullptr, nullptr, 0}, var.n_remtri, false);
+            __syncthreads();
+            bool any = false;
+            unsigned long long open[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int cell = (row0 + q) * kTile + lane;
+                open[q] = base[q] & sm.mask[cell];         // bits to decide again
+                now[q] = base[q] & ~open[q];
+                any |= open[q] != 0ull;
+                sm.mask[cell] = ~open[q];
+            }
+            if (__syncthreads_or(any)) {
+                const size_t bin = (size_t)bl * n_tiles + tile;
+                raster_block_call<COUNT, CULL>(sm, DeltaFetch{tris, iv.bins + iv.offsets[bin], nullptr, rem, n_rem},
+                                               (int)iv.counts[bin], iv.steps, bc, tox, toy, inv_dx, ba.run, true, cnt);
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < 4; ++q) now[q] |= sm.mask[(row0 + q) * kTile + lane] & open[q];
+            }
+        }
+        if (tow) {
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sm.mask[(row0 + q) * kTile + lane] = now[q];
+            raster_changed(DeltaFetch{towers, nullptr, nullptr, nullptr, 0}, var.n_tower, true);
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) now[q] = sm.mask[(row0 + q) * kTile + lane];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int iy = ty * kTile + row0 + q;
+            const int lx = ix - var.ix0, ly = iy - var.iy0;
+            const int delta = __popcll(now[q]) - __popcll(base[q]);
+            if (delta == 0 || ix >= g.nx || iy >= g.ny || lx < 0 || ly < 0 || lx >= var.nx || ly >= var.ny) continue;
+            const long long o = iv.out_base + var.out_off + (long long)ly * var.nx + lx;
+            atomicAdd(&ba.counts_out[o], delta);
+            if (ba.impact_out) atomicAdd(&ba.impact_out[o], delta);
+        }
+    }
+    if (COUNT) flush_raster_counts(ba.stats, cnt[0], cnt[1], cnt[2], cnt[3]);
+}
+
+// The work items of k_batch_delta: for every affected (interval, variant, tile) and block,
+// whether a changed box's shadow, swept over the block, can reach the tile.  Counts them
+// (items null), or appends them with their weights: the base triangles to raster again, and
+// the boxes.
+__global__ void k_batch_pick(TileGeom g, const BatchInterval* __restrict__ intervals,
+                             const BatchVariant* __restrict__ variants, const float4* __restrict__ boxes,
+                             const int4* __restrict__ tiles, long long n, int max_blocks,
+                             unsigned* __restrict__ total, int4* __restrict__ items, unsigned* __restrict__ weights) {
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n * max_blocks;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int4 t = tiles[i / max_blocks];
+        const int bl = (int)(i % max_blocks);
+        const BatchInterval& iv = intervals[t.x];
+        if (bl >= iv.n_blocks) continue;
+        const BatchVariant& var = variants[t.y];
+        const int tx = t.z % g.tiles_x, ty = t.z / g.tiles_x;
+        bool remv = false;
+        unsigned n_rem = 0, n_tow = 0;
+        for (int q = 0; q < var.n_box; ++q) {
+            const float4 lo = __ldg(&boxes[2 * (var.box_off + q)]), hi = __ldg(&boxes[2 * (var.box_off + q) + 1]);
+            if (!box_reaches(lo, hi, iv.blocks[bl], g, tx, ty)) continue;
+            if (lo.w != 0.f) { remv = true; ++n_rem; }
+            else ++n_tow;
+        }
+        if (!n_rem && !n_tow) continue;
+        const unsigned at = atomicAdd(total, 1u);
+        if (!items) continue;
+        items[at] = make_int4(t.x, t.y, t.z, bl * 4 + (remv ? 2 : 0) + (n_tow ? 1 : 0));
+        weights[at] = 1u + 4u * n_tow + (remv ? 16u * n_rem + iv.counts[(size_t)bl * g.tiles_x * g.tiles_y + t.z] : 0u);
+    }
+}
+
+// The base counts, and no impact, for every cell of every region.
+__global__ void k_batch_base(BatchArgs ba, int V, int I) {
+    for (int iv = blockIdx.y; iv < V * I; iv += gridDim.y) {
+        const BatchInterval& bi = ba.intervals[iv / V];
+        const BatchVariant& var = ba.variants[iv % V];
+        const long long n = (long long)var.nx * var.ny, o0 = bi.out_base + var.out_off;
+        for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
+            const long long ly = c / var.nx, lx = c - ly * var.nx;
+            ba.counts_out[o0 + c] = bi.base_counts[(var.iy0 + ly) * ba.g.nx + var.ix0 + lx];
+            if (ba.impact_out) ba.impact_out[o0 + c] = 0;
+        }
+    }
+}
+
 // Launch order of the tiles when a CTA takes all blocks of a tile: as launch_work_order, by
 // the triangles binned to the tile over the chunk's blocks.
 __global__ void k_tile_sums(const unsigned* __restrict__ counts, int nbc, int n_tiles, unsigned* __restrict__ sums) {
@@ -1417,6 +1637,40 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
 
 int raster_ctas_per_sm() { return SA_RASTER_CTAS; }
 
+cudaError_t pick_batch_items(const BatchLaunch& bl, const int4* d_tiles, long long n, int max_blocks,
+                             unsigned max_items, unsigned* n_items, int4** items, int** order, cudaStream_t st) {
+    *n_items = 0;
+    *items = nullptr;
+    *order = nullptr;
+    if (n == 0 || max_blocks == 0) return cudaSuccess;
+    const TileGeom g = tile_geom(bl.grid);
+    unsigned *words = nullptr, *weights = nullptr;
+    cudaError_t e = sa::scratch_alloc(&words, sizeof(unsigned) * (2 + kOrderBuckets), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(words, 0, sizeof(unsigned) * 2, st);
+    const unsigned ctas = (unsigned)std::min(152ll * 32, (n * max_blocks + 127) / 128);
+    unsigned total = 0;
+    if (e == cudaSuccess) {
+        k_batch_pick<<<ctas, 128, 0, st>>>(g, bl.intervals, bl.variants, bl.delta->boxes, d_tiles, n, max_blocks,
+                                           words, nullptr, nullptr);
+        e = cudaMemcpyAsync(&total, words, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess && total > 0 && total <= max_items) {
+        e = cudaMalloc(items, sizeof(int4) * (size_t)total);
+        if (e == cudaSuccess) e = cudaMalloc(order, sizeof(int) * (size_t)total);
+        if (e == cudaSuccess) e = sa::scratch_alloc(&weights, sizeof(unsigned) * (size_t)total, st);
+        if (e == cudaSuccess) {
+            k_batch_pick<<<ctas, 128, 0, st>>>(g, bl.intervals, bl.variants, bl.delta->boxes, d_tiles, n, max_blocks,
+                                               words + 1, *items, weights);
+            e = launch_work_order(weights, nullptr, total, words + 2, *order, nullptr, st);
+        }
+    }
+    if (words) cudaFreeAsync(words, st);
+    if (weights) cudaFreeAsync(weights, st);
+    *n_items = total;
+    return e;
+}
+
 cudaError_t launch_batch(const BatchLaunch& bl, cudaStream_t st) {
     BatchArgs ba;
     ba.g.x0 = bl.grid.x0; ba.g.y0 = bl.grid.y0; ba.g.dx = bl.grid.dx;
@@ -1438,6 +1692,22 @@ cudaError_t launch_batch(const BatchLaunch& bl, cudaStream_t st) {
     ba.stats = bl.stats;
     cudaError_t e = cudaMemsetAsync(bl.counter, 0, sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
+    if (bl.delta) {
+        const int VI = bl.V * bl.I;
+        if (VI > 0 && bl.max_cells > 0) {
+            const dim3 grid((unsigned)std::min(1024ll, (bl.max_cells + 255) / 256), (unsigned)std::min(VI, 65535));
+            k_batch_base<<<grid, 256, 0, st>>>(ba, bl.V, bl.I);
+        }
+        if (bl.n_items == 0) return cudaGetLastError();
+        if (ba.cull) {
+            if (bl.stats) k_batch_delta<true, true><<<bl.ctas, kRasterThreads, 0, st>>>(ba, *bl.delta);
+            else k_batch_delta<false, true><<<bl.ctas, kRasterThreads, 0, st>>>(ba, *bl.delta);
+        } else {
+            if (bl.stats) k_batch_delta<true, false><<<bl.ctas, kRasterThreads, 0, st>>>(ba, *bl.delta);
+            else k_batch_delta<false, false><<<bl.ctas, kRasterThreads, 0, st>>>(ba, *bl.delta);
+        }
+        return cudaGetLastError();
+    }
     if (bl.n_items == 0) return cudaSuccess;
     if (ba.cull) {
         if (bl.stats) k_batch<true, true><<<bl.ctas, kRasterThreads, 0, st>>>(ba);
