@@ -35,19 +35,16 @@ namespace {
 
 constexpr int kTile = 32;               // cells per tile side
 constexpr int kRasterThreads = 256;     // 8 warps x 4 rows each
-// triangles staged per batch (<= 128: a unit index t x runs + run stays below 2^13, which
-// the float quotient that decodes it and the queue's 13 bits for it both need)
+// triangles staged per batch (<= 64: a unit packs its triangle in 6 bits)
 #ifndef SA_RASTER_BATCH
 #define SA_RASTER_BATCH 64
 #endif
 constexpr int kTriBatch = SA_RASTER_BATCH;
-// work units a warp claims at a time (<= 32: one lane each while their boxes are bounded)
-#ifndef SA_RASTER_CLAIM
-#define SA_RASTER_CLAIM 4
-#endif
-constexpr int kUnitClaim = SA_RASTER_CLAIM;
+static_assert(kTriBatch <= 64, "a unit packs its triangle in 6 bits");
+// work units (triangle, run of steps) of a batch: one per thread
+constexpr int kMaxUnits = kRasterThreads;
 // resident CTAs per SM the raster kernels are compiled for (registers: 65536 / (256 x this));
-// 6 is also what their 35.9 KB of shared memory allows
+// 6 is also what the item kernels' 32 KB of shared memory allow
 #ifndef SA_RASTER_CTAS
 #define SA_RASTER_CTAS 6
 #endif
@@ -246,34 +243,50 @@ __device__ __forceinline__ EdgeLin edge_lin(const EdgeRef& e) {
     return l;
 }
 
-// Shared memory of one tile: staged triangles (xy tile-local), their sun-facing step
-// masks, the block's directions, ground slopes and per-run slope boxes, the tile's 64-bit
-// step masks and its cell centres.
+// Shared memory of one tile: staged triangles (xy tile-local), the block's directions, ground
+// slopes and per-run slope boxes, the batch's work units, the tile's step masks and its
+// cell centres.
 struct TileSmem {
     float4 tri[kTriBatch * 3];
-    unsigned long long front[kTriBatch];     // steps with n . d > 0
-    unsigned long long back[kTriBatch];      // steps with n . d < 0 (open scenes only)
-    int valid[kTriBatch];
     // the staged triangles' edge functions (EdgeLin, 6 floats each), 20 floats apart so
     // that a cell's test reads them as five float4
     float edges[kTriBatch * 20];
-    float2 u[kMaxBlock];
-    // slopes of steps (k, k + 1) packed for the paired step tests: [0][i] starts at step
-    // 2i, [1][i] at step 2i + 1 (the last pair of a block repeats its last step)
-    unsigned long long upx[2][kMaxBlock / 2], upy[2][kMaxBlock / 2];
     float4 d[kMaxBlock];                     // step directions
+    // slopes (u.x of two steps, u.y of the same two) for the paired step tests: [0][i] starts
+    // at step 2i, [1][i] at step 2i + 1 (the last pair of a block repeats its last step)
+    float4 up[2][kMaxBlock / 2];
+    float2 u[kMaxBlock];
     float4 ubox[kMaxBlock];                  // per run: (min u.x, max u.x, min u.y, max u.y)
     float4 uend[kMaxBlock];                  // per run: slopes of its first and last step
     float2 udev[kMaxBlock];                  // per run: largest |u - chord| over its steps
-    unsigned long long mask[kTile * kTile];
+    // step masks of the cells, steps 0..31 and 32..63 apart: 32-bit shared atomics are one
+    // instruction, 64-bit ones a compare-and-swap loop
+    unsigned lo[kTile * kTile], hi[kTile * kTile];
     unsigned long long row_full[kTile];      // steps at which every cell of a row is shadowed
-    // per warp: cells waiting for their step tests, (unit << 10) | cell, drained 32 at a
+    // the batch's units that reach the tile: columns and rows (unit_box) | triangle << 20 |
+    // run << 26, the run's facing steps (front; back, open scenes only), and the unit's
+    // first row in the list of all units' rows; first[g] is the unit of row 32 g
+    unsigned unit[kMaxUnits], fr[kMaxUnits], bk[kMaxUnits];
+    unsigned short start[kMaxUnits];
+    unsigned char first[kMaxUnits + 1];
+    unsigned made;                           // rows << 9 | units
+    int next_row;                            // next rows to hand out
+    // per warp: the covered rows of a claim, (first cell - first position, unit, steps it can
+    // set), and cells waiting for their step tests, (unit << 10) | cell, drained 32 at a
     // time so that every lane tests a cell whichever unit it comes from
+    int4 row[kRasterThreads / 32][32];
     unsigned queue[kRasterThreads / 32][64];
     float xl[kTile], yl[kTile];
-    int next_unit;                           // next work unit of the batch to hand out
-    float inv_nsub;                          // 1 / runs of the block
+    unsigned char valid[kTriBatch];
     unsigned char run_k0[kMaxBlock + 1];     // first step of each run, and K
+
+    __device__ __forceinline__ unsigned long long mask(int cell) const {
+        return ((unsigned long long)hi[cell] << 32) | lo[cell];
+    }
+    __device__ __forceinline__ void set_mask(int cell, unsigned long long m) {
+        lo[cell] = (unsigned)m;
+        hi[cell] = (unsigned)(m >> 32);
+    }
 };
 
 // Tile origin and cell centres in tile-local coordinates; the centres are rounded exactly
@@ -288,16 +301,17 @@ __device__ __forceinline__ void tile_setup(TileSmem& sm, const TileGeom& g, int 
         const int q = threadIdx.x - kTile;
         sm.yl[q] = __fadd_rn(g.y0, __fmul_rn(__fadd_rn((float)(ty * kTile + q), 0.5f), g.dx)) - *toy;
     }
-    for (int c = threadIdx.x; c < kTile * kTile; c += kRasterThreads) sm.mask[c] = 0ull;
+    for (int c = threadIdx.x; c < kTile * kTile; c += kRasterThreads) sm.set_mask(c, 0ull);
 }
 
 
-// The steps of one run (kn <= 32 steps from k0) that cover cell (x, y): bit k of the
-// result is step k0 + k.  CULL: closed scene, only front faces count.
+// The steps of one run (from k0) that cover cell (x, y): bit k of the result is step k0 + k.
+// kmax: steps of the block's longest run, the same for every lane; fr and bk drop the steps
+// beyond a shorter run.  CULL: closed scene, only front faces count.
 template <bool CULL>
 __device__ __forceinline__ unsigned cell_steps(const TileSmem& sm, const EdgeLin& E0,
                                                const EdgeLin& E1, const EdgeLin& E2, float x,
-                                               float y, int k0, int kn, unsigned fr, unsigned bk) {
+                                               float y, int k0, int kmax, unsigned fr, unsigned bk) {
     float P[3], QX[3], QY[3];
     const EdgeLin* ee[3] = {&E0, &E1, &E2};
 #pragma unroll
@@ -315,8 +329,7 @@ __device__ __forceinline__ unsigned cell_steps(const TileSmem& sm, const EdgeLin
         QX2[q] = f2_pack(QX[q], QX[q]);
         QY2[q] = f2_pack(QY[q], QY[q]);
     }
-    const unsigned long long* upx = sm.upx[k0 & 1] + (k0 >> 1);
-    const unsigned long long* upy = sm.upy[k0 & 1] + (k0 >> 1);
+    const ulonglong2* up = reinterpret_cast<const ulonglong2*>(sm.up[k0 & 1]) + (k0 >> 1);
     // Fully unrolled over the longest run.  A step covers the cell from the front when no
     // edge value has its sign bit set (+0 counts as inside, -0 as outside): that bit is
     // shifted in from the sign word, so the front mask comes out in reverse step order.
@@ -325,11 +338,11 @@ __device__ __forceinline__ unsigned cell_steps(const TileSmem& sm, const EdgeLin
     unsigned hf = 0, hb = 0;
 #pragma unroll
     for (int k = 0; k < 32; k += 2) {
-        if (k >= kn) break;
-        const unsigned long long ux = upx[k >> 1], uy = upy[k >> 1];
+        if (k >= kmax) break;
+        const ulonglong2 u = up[k >> 1];
         float f[3][2];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) f2_unpack(f2_fma(QY2[q], uy, f2_fma(QX2[q], ux, P2[q])), f[q][0], f[q][1]);
+        for (int q = 0; q < 3; ++q) f2_unpack(f2_fma(QY2[q], u.y, f2_fma(QX2[q], u.x, P2[q])), f[q][0], f[q][1]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const unsigned a = __float_as_uint(f[0][h]), b = __float_as_uint(f[1][h]), c = __float_as_uint(f[2][h]);
@@ -338,67 +351,47 @@ __device__ __forceinline__ unsigned cell_steps(const TileSmem& sm, const EdgeLin
         }
     }
     // steps 0 .. K2 - 1 (an odd run's last pair repeats a step beyond it, which the masks
-    // below drop) back in order: step k at bit k
-    const int K2 = (kn + 1) & ~1;
+    // drop) back in order: step k at bit k
+    const int K2 = (kmax + 1) & ~1;
     hf = __brev(hf) >> (32 - K2);
     return CULL ? (hf & fr) : ((hf & fr) | (hb & bk));
 }
 
-// Step tests of up to 32 queued cells, one per lane: each item names its work unit
-// (triangle of the staged batch and run of the block) and its cell; the unit's run, its
-// facing steps and the triangle's canonical edges are read back from shared memory.
+// Step tests of up to 32 queued cells (n >= 1), one per lane: each item names its work unit
+// and its cell; the unit's run, its facing steps and the triangle's canonical edges are
+// read back from shared memory.
 template <bool COUNT, bool CULL>
-__device__ __forceinline__ void drain_cells(TileSmem& sm, const unsigned* q, int n, int nsub,
+__device__ __forceinline__ void drain_cells(TileSmem& sm, const unsigned* q, int n, int kmax,
                                             unsigned long long& n_cell,
                                             unsigned long long& n_test) {
     const int lane = threadIdx.x & 31;
-    if (lane >= n) return;
-    const unsigned item = q[lane];
-    const int un = (int)(item >> 10), cell = (int)(item & 1023u);
-    const int t = (int)(((float)un + 0.5f) * sm.inv_nsub), sub = un - t * nsub;
-    const int k0 = sm.run_k0[sub], kn = sm.run_k0[sub + 1] - k0;
-    const unsigned run_bits = (kn >= 32) ? 0xffffffffu : ((1u << kn) - 1u);
-    const unsigned fr = (unsigned)(sm.front[t] >> k0) & run_bits;
-    const unsigned bk = CULL ? 0u : ((unsigned)(sm.back[t] >> k0) & run_bits);
+    const unsigned item = q[lane < n ? lane : 0];
+    const int j = (int)(item >> 10), cell = (int)SA_CHK(item & 1023u, kTile * kTile, sa::CK_RASTER_CELL);
+    const unsigned un = sm.unit[j];
+    const int t = (int)((un >> 20) & 63u), sub = (int)(un >> 26), k0 = sm.run_k0[sub];
+    const unsigned fr = sm.fr[j], bk = CULL ? 0u : sm.bk[j];
     const float4* ef = reinterpret_cast<const float4*>(&sm.edges[20 * t]);
     const float4 f0 = ef[0], f1 = ef[1], f2 = ef[2], f3 = ef[3], f4 = ef[4];
     const EdgeLin E0{f0.x, f0.y, f0.z, f0.w, f1.x, f1.y};
     const EdgeLin E1{f1.z, f1.w, f2.x, f2.y, f2.z, f2.w};
     const EdgeLin E2{f3.x, f3.y, f3.z, f3.w, f4.x, f4.y};
-    if (COUNT) { ++n_cell; n_test += kn; }
+    if (COUNT && lane < n) { ++n_cell; n_test += sm.run_k0[sub + 1] - k0; }
     const unsigned hit = cell_steps<CULL>(sm, E0, E1, E2, sm.xl[cell & (kTile - 1)],
-                                          sm.yl[cell >> 5], k0, kn, fr, bk);
-    if (hit) atomicOr(&sm.mask[SA_CHK(cell, kTile * kTile, sa::CK_RASTER_CELL)], (unsigned long long)hit << k0);
-}
-
-// A work unit is triangle t of the staged batch and run `sub` of the block, un = t nsub +
-// sub; (un + 1/2) / nsub is at least 1 / (2 nsub) from an integer, far beyond the float
-// quotient's rounding (relative 2^-23) for un < 2^13.
-struct UnitRun {
-    int t, sub, k0;
-    unsigned fr, bk;     // the run's steps the triangle faces (front; back, open scenes only)
-};
-
-template <bool CULL>
-__device__ __forceinline__ UnitRun unit_run(const TileSmem& sm, int un, int nsub) {
-    UnitRun u;
-    u.t = (int)(((float)un + 0.5f) * sm.inv_nsub);
-    u.sub = un - u.t * nsub;
-    u.k0 = sm.run_k0[u.sub];
-    const int kn = sm.run_k0[u.sub + 1] - u.k0;       // balanced runs
-    const unsigned run_bits = (kn >= 32) ? 0xffffffffu : ((1u << kn) - 1u);
-    u.fr = (unsigned)(sm.front[u.t] >> u.k0) & run_bits;
-    u.bk = CULL ? 0u : ((unsigned)(sm.back[u.t] >> u.k0) & run_bits);
-    return u;
+                                          sm.yl[cell >> 5], k0, kmax, fr, bk);
+    const unsigned long long m = (unsigned long long)hit << k0;
+    if (lane < n) {
+        if ((unsigned)m) atomicOr(&sm.lo[cell], (unsigned)m);
+        if ((unsigned)(m >> 32)) atomicOr(&sm.hi[cell], (unsigned)(m >> 32));
+    }
 }
 
 // The cells of the tile whose centres (k + 0.5) dx fall in the swept bounding box of the
-// run's projections, with 0.01 cell of slack, as columns c0..c1 and rows r0..r1 packed
-// 5 bits each (c0 | c1 << 5 | r0 << 10 | r1 << 15); -1 when the unit reaches no cell.
-__device__ __forceinline__ int unit_box(const TileSmem& sm, const UnitRun& u, float inv_dx) {
-    if ((u.fr | u.bk) == 0u) return -1;
-    const float4 a = sm.tri[3 * u.t], b = sm.tri[3 * u.t + 1], c = sm.tri[3 * u.t + 2];
-    const float4 ub = sm.ubox[u.sub];
+// projections of triangle t over run `sub`, with 0.01 cell of slack, as columns c0..c1 and
+// rows r0..r1 packed 5 bits each (c0 | c1 << 5 | r0 << 10 | r1 << 15); -1 when it reaches no
+// cell.
+__device__ __forceinline__ int unit_box(const TileSmem& sm, int t, int sub, float inv_dx) {
+    const float4 a = sm.tri[3 * t], b = sm.tri[3 * t + 1], c = sm.tri[3 * t + 2];
+    const float4 ub = sm.ubox[sub];
     const float uxlo = ub.x, uxhi = ub.y, uylo = ub.z, uyhi = ub.w;
     const float az = fmaxf(a.z, 0.f), bz = fmaxf(b.z, 0.f), cz = fmaxf(c.z, 0.f);
     const float xmin = fminf(a.x - az * uxhi, fminf(b.x - bz * uxhi, c.x - cz * uxhi));
@@ -425,14 +418,14 @@ __device__ __forceinline__ int unit_box(const TileSmem& sm, const UnitRun& u, fl
 // times the run's slope box, which a tall triangle or a low sun made far too wide (24 % of
 // the district's cell set-ups met no step, 88 % in December): district ground 2.16 -> 2.10
 // ms, 1024^2 cells on 16 December 15.6 -> 5.03 ms, 231 x 187 cells, 92 days 4.21 -> 4.09 ms.
-__device__ __forceinline__ void row_span(const TileSmem& sm, const UnitRun& u, int box, int row,
+__device__ __forceinline__ void row_span(const TileSmem& sm, int t, int sub, int box, int row,
                                          float inv_dx, int* cs, int* w) {
     *cs = 0;
     *w = 0;
     const int c0 = box & 31, c1 = (box >> 5) & 31;
-    const float4 a = sm.tri[3 * u.t], b = sm.tri[3 * u.t + 1], c = sm.tri[3 * u.t + 2];
-    const float4 ue = sm.uend[u.sub];
-    const float2 dv = sm.udev[u.sub];
+    const float4 a = sm.tri[3 * t], b = sm.tri[3 * t + 1], c = sm.tri[3 * t + 2];
+    const float4 ue = sm.uend[sub];
+    const float2 dv = sm.udev[sub];
     const float az = fmaxf(a.z, 0.f), bz = fmaxf(b.z, 0.f), cz = fmaxf(c.z, 0.f);
     const float zm = fmaxf(az, fmaxf(bz, cz));
     const float slack = 0.15f + 2e-3f * inv_dx;                 // in cells
@@ -478,18 +471,6 @@ __device__ __forceinline__ void row_span(const TileSmem& sm, const UnitRun& u, i
     }
 }
 
-// Index of the lane whose inclusive prefix sum first exceeds idx (incl non-decreasing over
-// the lanes, idx < its value in lane 31).
-__device__ __forceinline__ int prefix_lane(int incl, int idx) {
-    int j = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-        const int v = __shfl_sync(0xffffffffu, incl, j + step - 1);
-        if (v <= idx) j += step;
-    }
-    return j;
-}
-
 __device__ __forceinline__ int lane_prefix(int x) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -500,77 +481,76 @@ __device__ __forceinline__ int lane_prefix(int x) {
     return x;
 }
 
-// Up to 32 work units un0 .. un0 + nu - 1, expanded level by level so that every lane
-// has work: one lane per unit bounds its swept box; one lane per covered row finds the
-// row's span; one lane per covered cell checks whether the cell is already shadowed at
-// every step its unit could set (a stale read only skips less) and queues the others,
-// (unit << 10) | cell, for the step tests, 32 at a time whichever unit they come from.
+// Rows rb .. rb + 31 of the batch's units: one lane per row finds its unit and its span; one
+// lane per covered cell checks whether the cell is already shadowed at every step its unit
+// could set (a stale read only skips less) and queues the others, (unit << 10) | cell, for
+// the step tests, 32 at a time whichever unit they come from.
 template <bool COUNT, bool CULL>
-__device__ __forceinline__ void raster_units(TileSmem& sm, int un0, int nu, int nsub, float inv_dx,
-                                             int& qn, unsigned long long& n_cell,
-                                             unsigned long long& n_test,
-                                             unsigned long long& n_unit,
-                                             unsigned long long& n_span) {
-    const int lane = threadIdx.x & 31;
-    int box = -1;
-    if (lane < nu) box = unit_box(sm, unit_run<CULL>(sm, un0 + lane, nsub), inv_dx);
-    const int rows = box < 0 ? 0 : ((box >> 15) & 31) - ((box >> 10) & 31) + 1;
-    if (COUNT) {
-        const unsigned reach = __ballot_sync(0xffffffffu, rows > 0);
-        if (lane == 0) n_unit += (unsigned long long)__popc(reach);
+__device__ __forceinline__ void raster_rows(TileSmem& sm, int rb, int rows, int n_units, int kmax, float inv_dx,
+                                            int& qn, unsigned long long& n_cell,
+                                            unsigned long long& n_test, unsigned long long& n_span) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned upto = 0xffffffffu >> (31 - lane);           // this lane and the ones below
+    unsigned* q = sm.queue[warp];
+    // the units that start within these rows follow the one that holds row rb: their starts
+    // are distinct, so a lane's unit is the count of starts up to it
+    const int j0 = sm.first[rb >> 5];
+    const int jn = j0 + 1 + lane, at = jn < n_units ? (int)sm.start[jn] - rb : 32;
+    const unsigned starts = __reduce_or_sync(0xffffffffu, at < 32 ? 1u << at : 0u);
+    const int j = j0 + __popc(starts & upto), ridx = rb + lane;
+    int cs = 0, w = 0;
+    unsigned long long can = 0ull;
+    if (ridx < rows) {
+        const unsigned un = sm.unit[j];
+        const int row = (int)((un >> 10) & 31u) + (ridx - sm.start[j]), sub = (int)(un >> 26);
+        can = (unsigned long long)(CULL ? sm.fr[j] : (sm.fr[j] | sm.bk[j])) << sm.run_k0[sub];
+        if ((sm.row_full[row] & can) != can)
+            row_span(sm, (int)((un >> 20) & 63u), sub, (int)(un & 0xfffffu), row, inv_dx, &cs, &w);
+        cs += row * kTile;                                      // the row's first cell
     }
-    const int rincl = lane_prefix(rows);
-    const int total_rows = __shfl_sync(0xffffffffu, rincl, 31);
-    unsigned* q = sm.queue[threadIdx.x >> 5];
-    for (int rb = 0; rb < total_rows; rb += 32) {
-        // this lane's (unit, row)
-        const int ridx = rb + lane;
-        const int i = prefix_lane(rincl, ridx) & 31;
-        const int rex = __shfl_sync(0xffffffffu, rincl - rows, i);
-        const int ubox = __shfl_sync(0xffffffffu, box, i);
-        const int un = un0 + i;
-        int cs = 0, w = 0;
-        unsigned long long can = 0ull;
-        if (ridx < total_rows) {
-            const UnitRun u = unit_run<CULL>(sm, un, nsub);
-            const int row = ((ubox >> 10) & 31) + (ridx - rex);
-            can = (unsigned long long)(u.fr | u.bk) << u.k0;
-            if ((sm.row_full[row] & can) != can) row_span(sm, u, ubox, row, inv_dx, &cs, &w);
-            cs += row * kTile;                      // the row's first cell
-        }
-        const int cincl = lane_prefix(w);
-        const int total = __shfl_sync(0xffffffffu, cincl, 31);
-        if (COUNT && lane == 0) n_span += (unsigned long long)total;
-        const int cex = cincl - w;
-        for (int base = 0; base < total; base += 32) {
-            const int idx = base + lane;
-            const int j = prefix_lane(cincl, idx) & 31;
-            const int ex = __shfl_sync(0xffffffffu, cex, j);
-            const int cj = __shfl_sync(0xffffffffu, cs, j);
-            const int uj = __shfl_sync(0xffffffffu, un, j);
-            const unsigned long long cn = __shfl_sync(0xffffffffu, can, j);
-            const int cell = cj + (idx - ex);
-            const bool need = idx < total &&
-                              (sm.mask[SA_CHK(cell, kTile * kTile, sa::CK_RASTER_CELL)] & cn) != cn;
-            const unsigned bal = __ballot_sync(0xffffffffu, need);
-            if (need) q[qn + __popc(bal & ((1u << lane) - 1u))] = ((unsigned)uj << 10) | (unsigned)cell;
-            qn += __popc(bal);
-            if (qn >= 32) {
-                __syncwarp();
-                drain_cells<COUNT, CULL>(sm, q + (qn - 32), 32, nsub, n_cell, n_test);
-                qn -= 32;
-                __syncwarp();
-            }
+    const int cincl = lane_prefix(w);
+    const int total = __shfl_sync(0xffffffffu, cincl, 31);
+    if (COUNT && lane == 0) n_span += (unsigned long long)total;
+    const int cex = cincl - w;
+    const unsigned some = __ballot_sync(0xffffffffu, w > 0);
+    // the rows with cells, in order
+    if (w > 0)
+        sm.row[warp][__popc(some & (upto >> 1))] = make_int4(cs - cex, j, (int)(unsigned)can, (int)(unsigned)(can >> 32));
+    __syncwarp();
+    int before = -1;                                            // rows that started before this window, less one
+    for (int base = 0; base < total; base += 32) {
+        const int from = cex - base;
+        const unsigned begun = __reduce_or_sync(0xffffffffu, w > 0 && (unsigned)from < 32u ? 1u << from : 0u);
+        const int idx = base + lane;
+        const bool in = idx < total;
+        const int4 info = sm.row[warp][in ? before + __popc(begun & upto) : 0];
+        before += __popc(begun);
+        const int cell = in ? (int)SA_CHK(info.x + idx, kTile * kTile, sa::CK_RASTER_CELL) : 0;
+        const bool need = in && (((unsigned)info.z & ~sm.lo[cell]) | ((unsigned)info.w & ~sm.hi[cell])) != 0u;
+        const unsigned bal = __ballot_sync(0xffffffffu, need);
+        if (need) q[qn + __popc(bal & (upto >> 1))] = ((unsigned)info.y << 10) | (unsigned)cell;
+        qn += __popc(bal);
+        if (qn >= 32) {
+            __syncwarp();
+            drain_cells<COUNT, CULL>(sm, q + (qn - 32), 32, kmax, n_cell, n_test);
+            qn -= 32;
+            __syncwarp();
         }
     }
+    __syncwarp();
 }
 
 // One block of steps of one tile: the n triangles given by fetch(i, vertex, &v) (false =
-// skip the triangle) are staged in batches; each warp takes work units (triangle, run of
-// <= 32 steps), bounds the run's swept projection, spreads its lanes over the covered
-// cells (row-major, 32 at a time) and per cell tests the run's steps with the expanded
-// edge functions; step bits are ORed into sm.mask.  Leaves sm.mask complete for the block.
-// prefilled: sm.mask holds bits from the start, whose full rows are skipped at once.
+// skip the triangle) are staged in batches.  A work unit is a triangle and a run of <= 32
+// steps; one thread per unit finds its facing steps and swept box, the units that reach
+// the tile list their rows, and warps take 32 rows at a time (raster_rows); step bits are
+// ORed into the masks.  Leaves the masks complete for the block.
+// prefilled: the masks hold bits from the start, whose full rows are skipped at once.
+// Bound by issue slots (77 % busy, 26 of 32 lanes active).  Against warps that claimed four
+// units at a time and expanded them lane by lane (a binary search in shuffles for every row
+// and cell, 64-bit shared atomics, step loops of differing lengths): district ground 2.10 ->
+// 1.65 ms, 231 x 187 cells x 92 days 4.09 -> 3.38 ms, 16 scenarios 4.43 -> 3.38 ms.  48
+// triangles a batch measure the same, 32 2 % more, 5 and 4 CTAs per SM 3 and 9 % more.
 template <bool COUNT, bool CULL, class Fetch>
 __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const StepConst* steps,
                              int j0, int K, float tox, float toy, float inv_dx, int kSub,
@@ -578,7 +558,8 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
                              unsigned long long& n_unit, unsigned long long& n_span,
                              bool prefilled = false) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nsub = (K + kSub - 1) / kSub;
+    const int nsub = (K + kSub - 1) / kSub, kmax = (K + nsub - 1) / nsub;
+    const int batch = min(kTriBatch, kMaxUnits / nsub);
     __syncthreads();
     if (threadIdx.x < K) {
         const StepConst& s = steps[j0 + threadIdx.x];
@@ -588,11 +569,9 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
     __syncthreads();
     if (threadIdx.x < K) {
         const int k = threadIdx.x, k1 = min(k + 1, K - 1);
-        sm.upx[k & 1][k >> 1] = f2_pack(sm.u[k].x, sm.u[k1].x);
-        sm.upy[k & 1][k >> 1] = f2_pack(sm.u[k].y, sm.u[k1].y);
+        sm.up[k & 1][k >> 1] = make_float4(sm.u[k].x, sm.u[k1].x, sm.u[k].y, sm.u[k1].y);
     }
     if (threadIdx.x <= nsub) sm.run_k0[threadIdx.x] = (unsigned char)(threadIdx.x * K / nsub);
-    if (threadIdx.x == 0) sm.inv_nsub = 1.f / (float)nsub;
     if (threadIdx.x < kTile) sm.row_full[threadIdx.x] = 0ull;
     // per run, a warp with a step per lane: the slope box, the end steps, and the largest
     // deviation from the chord between them
@@ -619,8 +598,8 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
             sm.udev[run] = make_float2(dx + ulp, dy + ulp);
         }
     }
-    for (int base = 0; base < n; base += kTriBatch) {
-        const int nt = min(kTriBatch, n - base);
+    for (int base = 0; base < n; base += batch) {
+        const int nt = min(batch, n - base);
         __syncthreads();
         for (int i = threadIdx.x; i < nt * 3; i += kRasterThreads) {
             float4 v;
@@ -637,11 +616,14 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
         // (1024^2 cells, 16 December: 25.0 -> 16.4 ms; the June district is unchanged).
         if (base > 0 || prefilled) {
             for (int row = warp; row < kTile; row += kWarpsRaster) {
-                const unsigned long long m = sm.mask[row * kTile + lane];
-                const unsigned lo = __reduce_and_sync(0xffffffffu, (unsigned)m);
-                const unsigned hi = __reduce_and_sync(0xffffffffu, (unsigned)(m >> 32));
+                const unsigned lo = __reduce_and_sync(0xffffffffu, sm.lo[row * kTile + lane]);
+                const unsigned hi = __reduce_and_sync(0xffffffffu, sm.hi[row * kTile + lane]);
                 if (lane == 0) sm.row_full[row] = ((unsigned long long)hi << 32) | lo;
             }
+        }
+        if (threadIdx.x == 0) {
+            sm.next_row = kWarpsRaster * 32;
+            sm.made = 0u;
         }
         __syncthreads();
         unsigned long long tile_full = 0ull;
@@ -652,62 +634,66 @@ __device__ void raster_block(TileSmem& sm, const Fetch& fetch, int n, const Step
             const unsigned long long all = K >= 64 ? ~0ull : (1ull << K) - 1ull;
             if ((tile_full & all) == all) break;
         }
-        if (threadIdx.x == 0) sm.next_unit = kWarpsRaster * kUnitClaim;
-        // sun-facing steps of each staged triangle: a warp per triangle, a lane per step
-        for (int t = warp; t < nt; t += kWarpsRaster) {
-            unsigned long long fr = 0, bk = 0;
+        if (threadIdx.x < nt * 3) {
+            const int t = threadIdx.x / 3, e = threadIdx.x - 3 * t;
+            const EdgeLin l = edge_lin(edge_ref(sm.tri[threadIdx.x], sm.tri[e == 2 ? 3 * t : threadIdx.x + 1]));
+            float* o = &sm.edges[20 * t + 6 * e];
+            o[0] = l.pa; o[1] = l.pb; o[2] = l.pc; o[3] = l.ra; o[4] = l.qc; o[5] = l.rc;
+        }
+        // this thread's unit: triangle t, run sub (neighbouring lanes share the run)
+        int box = -1, t = 0, sub = 0;
+        unsigned fr = 0u, bk = 0u;
+        if (threadIdx.x < nt * nsub) {
+            sub = threadIdx.x / nt;
+            t = threadIdx.x - sub * nt;
             if (sm.valid[t]) {
                 const float4 a = sm.tri[3 * t], b = sm.tri[3 * t + 1], c = sm.tri[3 * t + 2];
                 const float ux = b.x - a.x, uy = b.y - a.y, uz = b.z - a.z;
                 const float vx = c.x - a.x, vy = c.y - a.y, vz = c.z - a.z;
                 const float nx = uy * vz - uz * vy, ny = uz * vx - ux * vz, nz = ux * vy - uy * vx;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int k = lane + 32 * h;
-                    float nd = 0.f;
-                    if (k < K) {
-                        const float4 d = sm.d[k];
-                        nd = nx * d.x + ny * d.y + nz * d.z;
-                    }
-                    const unsigned f = __ballot_sync(0xffffffffu, nd > 0.f);
-                    const unsigned g = __ballot_sync(0xffffffffu, nd < 0.f);
-                    fr |= (unsigned long long)f << (32 * h);
-                    bk |= (unsigned long long)g << (32 * h);
+                const int k0 = sm.run_k0[sub], kn = sm.run_k0[sub + 1] - k0;
+                for (int k = 0; k < kn; ++k) {
+                    const float4 d = sm.d[k0 + k];
+                    const float nd = nx * d.x + ny * d.y + nz * d.z;
+                    if (nd > 0.f) fr |= 1u << k;
+                    if (!CULL && nd < 0.f) bk |= 1u << k;
                 }
-                fr &= ~tile_full;
-                bk &= ~tile_full;
-                if (CULL) bk = 0ull;
-            }
-            if (lane == 0) {
-                sm.front[t] = fr;
-                sm.back[t] = bk;
-            }
-            if (lane < 3) {
-                const float4& p = sm.tri[3 * t + lane];
-                const float4& q = sm.tri[3 * t + (lane == 2 ? 0 : lane + 1)];
-                const EdgeLin e = edge_lin(edge_ref(p, q));
-                float* o = &sm.edges[20 * t + 6 * lane];
-                o[0] = e.pa; o[1] = e.pb; o[2] = e.pc; o[3] = e.ra; o[4] = e.qc; o[5] = e.rc;
+                const unsigned open = ~(unsigned)(tile_full >> k0);
+                fr &= open;
+                bk &= open;
+                if (fr | bk) box = unit_box(sm, t, sub, inv_dx);
             }
         }
+        const int rows = box < 0 ? 0 : ((box >> 15) & 31) - ((box >> 10) & 31) + 1;
+        const unsigned live = __ballot_sync(0xffffffffu, rows > 0);
+        const int rincl = lane_prefix(rows);
+        unsigned slot = 0u;
+        if (lane == 31 && live) slot = atomicAdd(&sm.made, ((unsigned)rincl << 9) | (unsigned)__popc(live));
+        slot = __shfl_sync(0xffffffffu, slot, 31);
+        if (rows > 0) {
+            const int j = (int)(slot & 511u) + __popc(live & ((1u << lane) - 1u)), start = (int)(slot >> 9) + rincl - rows;
+            sm.unit[j] = (unsigned)box | ((unsigned)t << 20) | ((unsigned)sub << 26);
+            sm.fr[j] = fr;
+            if (!CULL) sm.bk[j] = bk;
+            sm.start[j] = (unsigned short)start;
+            const int g = (start + 31) >> 5;                    // at most one multiple of 32 in its rows
+            if (32 * g < start + rows) sm.first[g] = (unsigned char)j;
+        }
+        if (COUNT && lane == 0) n_unit += (unsigned long long)__popc(live);
         __syncthreads();
-        const int units = nt * nsub;
-        // warps take kUnitClaim units at a time from a shared counter, so an expensive
-        // group does not hold the warps that would otherwise wait for its warp at the next
-        // barrier (the next group is claimed before this one is worked, hiding the
-        // atomic's latency)
-        int un = warp * kUnitClaim;
-        int qn = 0;
-        while (un < units) {
+        const int n_units = (int)(sm.made & 511u), n_rows = (int)(sm.made >> 9);
+        // warps take 32 rows at a time from a shared counter, so an expensive group does not
+        // hold the warps that would otherwise wait for its warp at the next barrier (the
+        // next group is claimed before this one is worked, hiding the atomic's latency)
+        int rb = warp * 32, qn = 0;
+        while (rb < n_rows) {
             int nx = 0;
-            if (lane == 0) nx = atomicAdd(&sm.next_unit, kUnitClaim);
-            raster_units<COUNT, CULL>(sm, un, min(kUnitClaim, units - un), nsub, inv_dx, qn, n_cell, n_test,
-                                      n_unit, n_span);
-            un = __shfl_sync(0xffffffffu, nx, 0);
+            if (lane == 0) nx = atomicAdd(&sm.next_row, 32);
+            raster_rows<COUNT, CULL>(sm, rb, n_rows, n_units, kmax, inv_dx, qn, n_cell, n_test, n_span);
+            rb = __shfl_sync(0xffffffffu, nx, 0);
         }
         // the queue's last cells, before the batch's triangles are replaced
-        __syncwarp();
-        drain_cells<COUNT, CULL>(sm, sm.queue[warp], qn, nsub, n_cell, n_test);
+        if (qn > 0) drain_cells<COUNT, CULL>(sm, sm.queue[warp], qn, kmax, n_cell, n_test);
         __syncwarp();
     }
     __syncthreads();
@@ -782,8 +768,8 @@ k_raster(RasterArgs ra) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int cell = (row0 + q) * kTile + lane;
-            const unsigned long long m = sm.mask[cell];
-            sm.mask[cell] = 0ull;
+            const unsigned long long m = sm.mask(cell);
+            sm.set_mask(cell, 0ull);
             RunState st = s_st[cell];
             stitch(st, m, K, new_day);
             s_st[cell] = st;
@@ -847,7 +833,7 @@ k_raster_items(RasterArgs ra) {
     for (int q = 0; q < 4; ++q) {
         const int iy = ty * kTile + row0 + q;
         if (ix >= g.nx || iy >= g.ny) continue;
-        const unsigned long long m = (cnt > 0 && K > 0) ? sm.mask[(row0 + q) * kTile + lane] : 0ull;
+        const unsigned long long m = (cnt > 0 && K > 0) ? sm.mask((row0 + q) * kTile + lane) : 0ull;
         const size_t cell = (size_t)iy * g.nx + ix;
         if (ra.summary) ra.summary[((size_t)bl * ra.parts + part) * ra.R + cell] = run_summary(m, K);
         // pieces and one-step blocks share a mask word
@@ -1018,8 +1004,8 @@ k_batch(BatchArgs ba) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int cell = (row0 + q) * kTile + lane;
-                const unsigned long long m = sm.mask[cell];
-                sm.mask[cell] = 0ull;
+                const unsigned long long m = sm.mask(cell);
+                sm.set_mask(cell, 0ull);
                 RunState st = s_st[cell];
                 stitch(st, m, bc.K, bc.new_day);
                 s_st[cell] = st;
@@ -1138,7 +1124,7 @@ k_batch_delta(BatchArgs ba, BatchDelta bd) {
             base[q] = (ix < g.nx && iy < g.ny)
                           ? __ldg(&bd.masks[(size_t)bl * bd.R + iv.mask_off + (size_t)iy * g.nx + ix]) : 0ull;
             now[q] = base[q];
-            if (remv) sm.mask[(row0 + q) * kTile + lane] = 0ull;
+            if (remv) sm.set_mask((row0 + q) * kTile + lane, 0ull);
         }
         // rasters the changed triangles pick(i) < n that reach the tile, kChangeList at a time
         auto raster_changed = [&](DeltaFetch f, int n, bool prefilled) {
@@ -1175,10 +1161,10 @@ k_batch_delta(BatchArgs ba, BatchDelta bd) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int cell = (row0 + q) * kTile + lane;
-                open[q] = base[q] & sm.mask[cell];         // bits to decide again
+                open[q] = base[q] & sm.mask(cell);         // bits to decide again
                 now[q] = base[q] & ~open[q];
                 any |= open[q] != 0ull;
-                sm.mask[cell] = ~open[q];
+                sm.set_mask(cell, ~open[q]);
             }
             if (__syncthreads_or(any)) {
                 const size_t bin = (size_t)bl * n_tiles + tile;
@@ -1186,17 +1172,17 @@ k_batch_delta(BatchArgs ba, BatchDelta bd) {
                                                (int)iv.counts[bin], iv.steps, bc, tox, toy, inv_dx, ba.run, true, cnt);
                 __syncthreads();
 #pragma unroll
-                for (int q = 0; q < 4; ++q) now[q] |= sm.mask[(row0 + q) * kTile + lane] & open[q];
+                for (int q = 0; q < 4; ++q) now[q] |= sm.mask((row0 + q) * kTile + lane) & open[q];
             }
         }
         if (tow) {
             __syncthreads();
 #pragma unroll
-            for (int q = 0; q < 4; ++q) sm.mask[(row0 + q) * kTile + lane] = now[q];
+            for (int q = 0; q < 4; ++q) sm.set_mask((row0 + q) * kTile + lane, now[q]);
             raster_changed(DeltaFetch{towers, nullptr, nullptr, nullptr, 0}, var.n_tower, true);
             __syncthreads();
 #pragma unroll
-            for (int q = 0; q < 4; ++q) now[q] = sm.mask[(row0 + q) * kTile + lane];
+            for (int q = 0; q < 4; ++q) now[q] = sm.mask((row0 + q) * kTile + lane);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
