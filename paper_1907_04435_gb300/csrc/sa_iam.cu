@@ -10,11 +10,15 @@
 //               q_{K-1}.  The same is done from the block's last step with the pieces
 //               running backwards (the paper's t_n -> t_1 map), which catches stretching
 //               shadows and sources missed by the first map.
-//   k_iam_fold  folds each cell's 64-bit vector into its gross / continuous state and
-//               clears it for the next block.
-// The bit vectors live in one uint64 per cell; drawing uses atomicOr, skipped when the
-// bit is already set.  This is the paper's approximate method: it is compared with its
+//   k_iam_fold  folds the blocks' 64-bit vectors of each cell into its gross / continuous
+//               state.
+// The bit vectors live in one uint64 per cell and block; drawing gathers a line's bits in a
+// cell and uses one atomicOr.  All blocks go in one launch: one launch per block left
+// the chip waiting for the longest warps of each (4.81 -> 3.20 ms; 64^2 cells 2.95 ms ->
+// 0.29 with the gathered marks).  This is the paper's approximate method: it is compared with its
 // own FP64 restatement and with the exact result (the paper's area-error bar).
+#include <algorithm>
+
 #include "sa_internal.cuh"
 
 namespace sa {
@@ -103,13 +107,30 @@ struct Grid {
     int nx, ny;
 };
 
-__device__ __forceinline__ void mark(unsigned long long* masks, long long cell, unsigned long long bit) {
-    if (!(__ldcg(&masks[cell]) & bit)) atomicOr(&masks[cell], bit);
-}
+// Marks of a thread's shadow line: consecutive pieces mostly stay in one cell, so its bits are
+// gathered and ORed into memory once, when the line leaves it.  (Reading the word first to
+// skip bits that are set made every lane of the warp wait: 3.20 ms against 2.76 for 613 x 457
+// cells x 481 steps.)
+struct Marker {
+    unsigned long long* masks;
+    long long cell;
+    unsigned long long bits;
+    __device__ __forceinline__ void flush() {
+        if (bits) atomicOr(&masks[cell], bits);
+    }
+    __device__ __forceinline__ void mark(long long c, unsigned long long bit) {
+        if (c != cell) {
+            flush();
+            cell = c;
+            bits = 0ull;
+        }
+        bits |= bit;
+    }
+};
 
 // Every closed grid cell touched by the segment P -> Q gets `bit`.
 __device__ void draw_segment(const Grid& g, float px, float py, float qx, float qy,
-                             unsigned long long* masks, unsigned long long bit) {
+                             Marker& mk, unsigned long long bit) {
     const float inv = 1.f / g.dx;
     const float ymin = fminf(py, qy), ymax = fmaxf(py, qy);
     int iy0 = (int)ceilf((ymin - g.y0) * inv) - 1;
@@ -134,14 +155,16 @@ __device__ void draw_segment(const Grid& g, float px, float py, float qx, float 
         int ix1 = (int)floorf((xb - g.x0) * inv);
         ix0 = max(ix0, 0);
         ix1 = min(ix1, g.nx - 1);
-        for (int ix = ix0; ix <= ix1; ++ix) mark(masks, (long long)iy * g.nx + ix, bit);
+        for (int ix = ix0; ix <= ix1; ++ix) mk.mark((long long)iy * g.nx + ix, bit);
     }
 }
 
 __global__ void __launch_bounds__(32 * kWarps)
-k_iam_draw(DevScene sc, Grid g, const StepConst* __restrict__ steps, int j0, int K, int L,
-           unsigned long long* __restrict__ masks) {
+k_iam_draw(DevScene sc, Grid g, const StepConst* __restrict__ steps, const BlockConst* __restrict__ blocks,
+           int L, unsigned long long* __restrict__ all_masks) {
     const int lane = threadIdx.x & 31;
+    const int j0 = blocks[blockIdx.y].j0, K = blocks[blockIdx.y].K;
+    Marker mk{all_masks + (long long)blockIdx.y * g.nx * g.ny, -1, 0ull};
     const long long warp_id = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5);
     const int tiles_x = (g.nx + 7) >> 3;
     const long long n_warps = (long long)tiles_x * ((g.ny + 3) >> 2);
@@ -171,26 +194,27 @@ k_iam_draw(DevScene sc, Grid g, const StepConst* __restrict__ steps, int j0, int
                 for (int k = 0; k + 1 < K; ++k) {
                     const float qx = fmaf(-sz, steps[j0 + k + 1].ux, sx);
                     const float qy = fmaf(-sz, steps[j0 + k + 1].uy, sy);
-                    draw_segment(g, px, py, qx, qy, masks, 1ull << k);
+                    draw_segment(g, px, py, qx, qy, mk, 1ull << k);
                     px = qx; py = qy;
                 }
-                draw_segment(g, px, py, px, py, masks, 1ull << (K - 1));
+                draw_segment(g, px, py, px, py, mk, 1ull << (K - 1));
             } else {
                 float px = fmaf(-sz, steps[j0 + K - 1].ux, sx), py = fmaf(-sz, steps[j0 + K - 1].uy, sy);
                 for (int k = K - 1; k >= 1; --k) {
                     const float qx = fmaf(-sz, steps[j0 + k - 1].ux, sx);
                     const float qy = fmaf(-sz, steps[j0 + k - 1].uy, sy);
-                    draw_segment(g, px, py, qx, qy, masks, 1ull << k);
+                    draw_segment(g, px, py, qx, qy, mk, 1ull << k);
                     px = qx; py = qy;
                 }
-                draw_segment(g, px, py, px, py, masks, 1ull);
+                draw_segment(g, px, py, px, py, mk, 1ull);
             }
         }
     }
+    mk.flush();
 }
 
-__global__ void k_iam_fold(long long R, int K, int new_day, int mask_block,
-                           unsigned long long* __restrict__ masks, DevOut out, int first,
+__global__ void k_iam_fold(long long R, const BlockConst* __restrict__ blocks, int nbc,
+                           const unsigned long long* __restrict__ masks, DevOut out, int first,
                            int last) {
     const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= R) return;
@@ -200,39 +224,43 @@ __global__ void k_iam_fold(long long R, int K, int new_day, int mask_block,
         st.best = out.continuous ? out.continuous[r] : 0;
         st.run = (first) ? 0 : out.run[r];
     }
-    const unsigned long long m = masks[r];
-    masks[r] = 0ull;
-    stitch(st, m, K, new_day);
+    for (int b = 0; b < nbc; ++b) {
+        const unsigned long long m = masks[(long long)b * R + r];
+        stitch(st, m, blocks[b].K, blocks[b].new_day);
+        if (out.masks && m) out.masks[(long long)blocks[b].mask_block * R + r] |= m;
+    }
     out.gross[r] = st.gross;
     if (out.continuous) out.continuous[r] = st.best;
     out.run[r] = st.run;
-    if (out.masks) out.masks[(long long)mask_block * R + r] |= m;
     if (last && out.minutes) out.minutes[r] = (float)st.gross * out.step_minutes;
 }
 
 }  // namespace
 
 cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
-                       const BlockConst* h_blocks, int L, const DevOut& out, cudaStream_t st) {
+                       int L, const DevOut& out, cudaStream_t st) {
     const long long R = (long long)rc.nx * rc.ny;
     if (R == 0) return cudaSuccess;
     if (L < 1 || L > kMaxLevels) return cudaErrorInvalidValue;
+    // the blocks go in one launch, as many as 1 GiB of masks holds
+    const int chunk = (int)std::max(1ll, std::min({(long long)sun.n_blocks, 65535ll, (1ll << 30) / (8ll * R)}));
+    const size_t words = (size_t)R * chunk;
     unsigned long long* masks = nullptr;
-    cudaError_t e = sa::scratch_alloc(&masks, sizeof(unsigned long long) * (size_t)R, st);
+    cudaError_t e = sa::scratch_alloc(&masks, sizeof(unsigned long long) * words, st);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)R, st);
     Grid g{rc.x0, rc.y0, rc.dx, rc.nx, rc.ny};
     const long long warps = (long long)((rc.nx + 7) / 8) * ((rc.ny + 3) / 4);
     const unsigned ctas = (unsigned)((warps + kWarps - 1) / kWarps);
-    for (int b = 0; b < sun.n_blocks && e == cudaSuccess; ++b) {
-        const BlockConst& bc = h_blocks[b];
+    for (int b0 = 0; b0 < sun.n_blocks && e == cudaSuccess; b0 += chunk) {
+        const int nbc = std::min(chunk, sun.n_blocks - b0);
+        e = cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)R * nbc, st);
+        if (e != cudaSuccess) break;
         {
             KernelTimer kt(KT_IAM, st);
-            k_iam_draw<<<ctas, 32 * kWarps, 0, st>>>(sc, g, sun.steps, bc.j0, bc.K, L, masks);
+            k_iam_draw<<<dim3(ctas, (unsigned)nbc), 32 * kWarps, 0, st>>>(sc, g, sun.steps, sun.blocks + b0, L, masks);
         }
-        k_iam_fold<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(R, bc.K, bc.new_day, bc.mask_block,
-                                                               masks, out, b == 0,
-                                                               b == sun.n_blocks - 1);
+        k_iam_fold<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(R, sun.blocks + b0, nbc, masks, out, b0 == 0,
+                                                               b0 + nbc == sun.n_blocks);
         e = cudaGetLastError();
     }
     cudaError_t e2 = cudaFreeAsync(masks, st);

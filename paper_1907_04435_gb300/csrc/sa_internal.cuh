@@ -693,9 +693,9 @@ cudaError_t launch_sam_points(const DevScene& sc, const float* scene_box, const 
                               const std::vector<StepConst>& h_steps, const DevOut& out,
                               cudaStream_t st);
 
-// inverse accrual map of a ground grid (h_blocks: host copy of the block constants)
+// inverse accrual map of a ground grid
 cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
-                       const BlockConst* h_blocks, int L, const DevOut& out, cudaStream_t st);
+                       int L, const DevOut& out, cudaStream_t st);
 
 // LBVH build (device), returns node / triangle arrays owned by the caller
 struct LbvhBuild {
