@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "sa_handles.cuh"
+#include "sa_light.cuh"
 
 namespace sa {
 
@@ -106,25 +107,31 @@ __global__ void k_shadow_score(const int* __restrict__ steps, long long R, int n
 // these partition the region's shadowed cell-steps -- except the ones the raster marks
 // shadowed whose FP32 ray grazes past every triangle (shadow edges), counted apart.
 //
-// A first pass lists, per run of <= 32 consecutive steps of a block, the region's cells
-// with a shadowed step in it.  One warp then takes 32 listed cells of one run and walks
-// the depth-first node list once with the fan of the run's rays as its query (as the
-// ray-traced accrual does): every triangle in the fan is tested exactly (Plucker form,
-// with its distance) against the lane's shadowed steps it can reach.  Per lane and step
-// the nearest hit (distance, building) is kept in shared memory, and per lane and run a
-// short list of kCastList (building, steps met) pairs; a lane whose
-// run meets more buildings than the list holds counts its casting again ray by ray, with
-// a list of kRayList buildings per ray.  Counts are integers, credited by atomics on
-// per-building totals (runs of equal nearest buildings are credited at once).
-constexpr int kContribWarps = 2;
-constexpr int kContribRun = 32;             // steps per fan traversal
-constexpr int kCastList = 8;                // buildings per lane and run in the fan pass
-constexpr int kRayList = 2 * kContribRun;   // buildings per ray in the per-ray recount
+// A first pass lists, per run of <= 16 consecutive steps of a block, the region's cells
+// with a shadowed step in it.  A CTA then takes 128 listed cells of one run and walks the
+// BVH once for all of them (walk_group, as the ray-traced accrual does): the pairs of a
+// cell and a triangle that the run's rays may reach are tested exactly at each of the
+// cell's shadowed steps (Plucker form, with the distance).  Per cell and step the nearest
+// hit is kept in shared memory -- distance and triangle in one 64-bit key, so the minimum
+// does not depend on the order; equal distances go to the lower triangle index, as a walk
+// of the node list in its order gives -- and per cell and run a short list of kCastList
+// (building, steps met) pairs.  Where a cell's run meets more buildings than the list holds,
+// the CTA walks again for those cells, once per class of building ids modulo kCastSplit,
+// and where a class does not fit either, modulo the next power of it.  Counts are integers,
+// credited by atomics on per-building totals (runs of equal nearest buildings are credited
+// at once).
+constexpr int kCastList = 12;               // buildings per cell and run: what five CTAs per SM leave
+constexpr unsigned kCastSplit = 4;          // classes per level when the list runs out
+constexpr int kCastLevels = 16;             // 4^15 classes of 2^31 ids: none holds more than the list
+constexpr unsigned kRayMost = 64;           // buildings a ray may meet: more are reported
+constexpr int kContribChunk = 64;           // triangles staged per pass
+constexpr int kContribCtas = 5;             // resident CTAs per SM
 
 struct ContribArgs {
     DevScene sc;
     const StepConst* steps;
-    const BlockConst* runs;           // runs of <= 32 steps; mask_block / mask_bit locate them
+    const BlockConst* runs;           // runs of <= kContribRun steps; mask_block / mask_bit locate them
+    const RunLight* lights;           // their light-space constants
     int n_runs;
     const unsigned long long* masks;  // the raster's step masks [blocks][R]
     long long R;
@@ -141,47 +148,40 @@ struct ContribArgs {
     const int* items;                 // run r's cells at item0[r] .. item0[r] + n_items[r]
     const unsigned* item0;            // [n_runs]
     const unsigned* n_items;          // [n_runs]
-    const int* warp_base;             // [n_runs + 1] first warp of each run
+    const int* cta_base;              // [n_runs + 1] first CTA of each run
 };
 
-// Per warp, in shared memory; Id is a 16-bit building id when the scene has fewer than
-// 65,536 buildings (the smaller footprint keeps more warps resident), else 32-bit.
-template <class Id>
-struct ContribWarpSmem {
-    float t[kContribRun][32];         // nearest hit distance per step and lane
-    Id b[kContribRun][32];            // its building
-    Id cb[kCastList][32];             // casting list: building
-    unsigned cm[kCastList][32];       //               steps whose ray meets it
+// A CTA's shared memory.
+struct ContribSmem {
+    unsigned long long key[kContribRun][kTileThreads];   // nearest hit: distance bits, triangle + 1
+    int cb[kCastList][kTileThreads];          // casting list: building, -1 when free
+    unsigned cm[kCastList][kTileThreads];     //               steps whose ray meets it
+    LightSmem<kContribChunk> l;               // l.m: the cells' shadowed steps
+    GroupSmem<kContribChunk, 512> g;
+    unsigned over[kCastLevels][kTileThreads / 32];   // per level, the cells whose list ran out
 };
+static_assert(sizeof(ContribSmem) <= 227 * 1024 / kContribCtas - 1024, "resident CTAs per SM");
 
-// what the kernel reads of a step: its direction and the direction's reciprocals
-struct ContribStep {
-    float dx, dy, dz, ix, iy, iz;
-};
-
-// Plucker test with the hit distance (t = ((a - o) . n) / (d . n)), the same decision as
-// plucker_hit.
-__device__ __forceinline__ bool plucker_hit_t(const PluckerTri& p, const ContribStep& s, float tmin,
-                                              float* t) {
-    if (!plucker_hit(p, s.dx, s.dy, s.dz, tmin)) return false;
-    const float nd = fmaf(s.dz, p.nz, fmaf(s.dy, p.ny, __fmul_rn(s.dx, p.nx)));
-    *t = p.aon / nd;
-    return true;
-}
-
-// Work list of the fan traversal: per run, the region's cells with at least one shadowed
-// step in it, in patch order (8 x 4 cells per patch, patches row by row), so that the 32
-// cells a traversal warp takes stay close together.  Cells shadowed at no step of a run
+// Work list of the traversal: per run, the region's cells with at least one shadowed
+// step in it, in patch order (8 x 4 cells per patch; strips of kStrip patch rows, column by column), so
+// that the 128 cells a CTA takes stay close together.  Cells shadowed at no step of a run
 // cost nothing there.  Two passes over the patches: counts per (run, patch), then -- after
 // an exclusive scan of the counts into offsets -- the cells themselves.
+constexpr int kStrip = 8;
+
+__host__ __device__ inline long long contrib_patches(int bnx, int bny) {
+    return (long long)((bnx + 7) / 8) * (((bny + 3) / 4 + kStrip - 1) / kStrip * kStrip);
+}
+
 __global__ void k_contrib_items(ContribArgs a, bool fill, unsigned* __restrict__ counts,
                                 const unsigned* __restrict__ offsets, int* __restrict__ items) {
     const int lane = threadIdx.x & 31;
     const int tiles_x = (a.bnx + 7) >> 3;
-    const long long n_patches = (long long)tiles_x * ((a.bny + 3) >> 2);
+    const long long n_patches = contrib_patches(a.bnx, a.bny);
     const long long warp_id = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (warp_id >= n_patches) return;                                  // whole warps
-    const int ty = (int)(warp_id / tiles_x), tx = (int)(warp_id - (long long)ty * tiles_x);
+    const int strip = (int)(warp_id / (tiles_x * kStrip)), at = (int)(warp_id - (long long)strip * tiles_x * kStrip);
+    const int tx = at / kStrip, ty = strip * kStrip + at % kStrip;
     const int lx = tx * 8 + (lane & 7), ly = ty * 4 + (lane >> 3);
     const int ix = a.bx0 + lx, iy = a.by0 + ly;
     const float x = __fadd_rn(a.x0, __fmul_rn(__fadd_rn((float)ix, 0.5f), a.dx));
@@ -203,18 +203,90 @@ __global__ void k_contrib_items(ContribArgs a, bool fill, unsigned* __restrict__
     }
 }
 
-template <class Id>
-__global__ void __launch_bounds__(32 * kContribWarps)
+// Tests n <= 32 queued pairs of a warp, one per lane: the hits of a pair's wanted steps go
+// into its cell's keys (nearest) and casting list.
+__device__ __forceinline__ void drain_contrib(ContribSmem& s, const unsigned short* q, int n, int kn, int n_b,
+                                              bool nearest, unsigned* over) {
+    const int lane = threadIdx.x & 31;
+    if (lane >= n) return;
+    const unsigned e = q[lane];
+    const int who = (int)(e >> 8), t = (int)(e & 0xffu);
+    LightSmem<kContribChunk>& l = s.l;
+    const float4 p = l.o[who];
+    const float4 a = l.tri[3 * t], b = l.tri[3 * t + 1], c = l.tri[3 * t + 2], nv = l.n[t];
+    const PluckerTri pt = plucker_setup_n(make_float3(p.x, p.y, p.z), a, b, c, make_float3(nv.x, nv.y, nv.z));
+    unsigned long long M[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) M[i][j] = f2_pack(pt.m[i][j], pt.m[i][j]);
+    unsigned m = 0;
+#pragma unroll
+    for (int k = 0; k < kContribRun; k += 2) {
+        if (k >= kn) break;
+        const unsigned long long dx = l.d2[k >> 1][0], dy = l.d2[k >> 1][1], dz = l.d2[k >> 1][2];
+        float sv[3][2];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            f2_unpack(f2_fma(dz, M[i][2], f2_fma(dy, M[i][1], f2_mul(dx, M[i][0]))), sv[i][0], sv[i][1]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (min3f(sv[0][h], sv[1][h], sv[2][h]) >= 0.f || max3f(sv[0][h], sv[1][h], sv[2][h]) <= 0.f)
+                m |= 1u << (k + h);
+    }
+    m &= l.m[who];
+    // inside the edges at a wanted step: the distance decides (plucker_hit's roundings)
+    unsigned hits = 0;
+    const unsigned tri = l.front[t];                  // its index + 1
+    while (m) {
+        const int k = __ffs(m) - 1;
+        m &= m - 1u;
+        float dx[2], dy[2], dz[2];
+        f2_unpack(l.d2[k >> 1][0], dx[0], dx[1]);
+        f2_unpack(l.d2[k >> 1][1], dy[0], dy[1]);
+        f2_unpack(l.d2[k >> 1][2], dz[0], dz[1]);
+        const bool odd = k & 1;
+        const float nd = fmaf(odd ? dz[1] : dz[0], pt.nz,
+                              fmaf(odd ? dy[1] : dy[0], pt.ny, __fmul_rn(odd ? dx[1] : dx[0], pt.nx)));
+        const float lim = __fmul_rn(p.w, nd);
+        if ((nd > 0.f && pt.aon > lim) || (nd < 0.f && pt.aon < lim)) {
+            hits |= 1u << k;
+            const unsigned long long key =
+                ((unsigned long long)__float_as_uint(pt.aon / nd) << 32) | tri;   // distance > 0
+            if (nearest && key < *(volatile unsigned long long*)&s.key[k][who]) atomicMin(&s.key[k][who], key);
+        }
+    }
+    if (hits) {
+        const int bid = (int)SA_CHK(__float_as_int(a.w), n_b, sa::CK_CONTRIB_BUILDING);
+        int i = 0;
+        for (; i < kCastList; ++i) {
+            int cur = *(volatile int*)&s.cb[i][who];
+            if (cur < 0) {
+                cur = atomicCAS(&s.cb[i][who], -1, bid);
+                if (cur < 0) cur = bid;
+            }
+            if (cur == bid) break;
+        }
+        if (i < kCastList) atomicOr(&s.cm[i][who], hits);
+        else atomicOr(&over[who >> 5], 1u << (who & 31));
+    }
+}
+
+// Bound by the latency of the pairs' culls and tests at 20 warps per SM (the keys and lists
+// fill its shared memory).  512 x 512 cells, 2000 buildings, 481 steps in June, the whole
+// call: 3.49 ms with a warp walking the node list with 32 cells' fans, 1.86 ms grouped (2.21
+// in runs of 32 steps with eight list entries, which leave 16 warps per SM, and patches row
+// by row; patches in strips of 8 rows 1.86, of 4 1.95, row by row 2.41).  A December day,
+// where a run meets more buildings than a list holds: 1000 buildings, 300 x 200 cells 24.9
+// -> 6.4 ms (a recount ray by ray for those cells: 16.6; classes of 8 and lists of 8: 7.0).
+__global__ void __launch_bounds__(kTileThreads, kContribCtas)
 k_building_contribution(ContribArgs a) {
-    __shared__ ContribWarpSmem<Id> s_w[kContribWarps];
-    __shared__ BlockConst s_bc[kContribWarps];
-    __shared__ ContribStep s_st[kContribWarps][kContribRun];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int warp_id = (int)(blockIdx.x * kContribWarps + wib);
-    if (warp_id >= a.warp_base[a.n_runs]) return;                       // whole warps
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    ContribSmem& s = *reinterpret_cast<ContribSmem*>(s_raw);
+    const int tid = threadIdx.x, lane = tid & 31;
     int r = 0;
-    while (a.warp_base[r + 1] <= warp_id) ++r;
-    const unsigned slot = (unsigned)(warp_id - a.warp_base[r]) * 32u + (unsigned)lane;
+    while (a.cta_base[r + 1] <= (int)blockIdx.x) ++r;
+    const unsigned slot = (unsigned)((int)blockIdx.x - a.cta_base[r]) * (unsigned)kTileThreads + (unsigned)tid;
     const bool live = slot < a.n_items[r];
     const long long cell = live ? (long long)SA_CHK(a.items[(long long)a.item0[r] + slot], a.R, sa::CK_CONTRIB_CELL) : 0;
     const int ix = (int)(cell % a.nx), iy = (int)(cell / a.nx);
@@ -222,152 +294,92 @@ k_building_contribution(ContribArgs a) {
     o.x = __fadd_rn(a.x0, __fmul_rn(__fadd_rn((float)ix, 0.5f), a.dx));
     o.y = __fadd_rn(a.y0, __fmul_rn(__fadd_rn((float)iy, 0.5f), a.dx));
     o.z = 0.f;
-    ContribWarpSmem<Id>& w = s_w[wib];
-    BlockConst& bc = s_bc[wib];
-    ContribStep* ss = s_st[wib];
-    unsigned long long n_graze = 0, n_over = 0;
-    {
-        for (int q = lane; q < (int)(sizeof(BlockConst) / 4); q += 32)
-            reinterpret_cast<int*>(&bc)[q] = reinterpret_cast<const int*>(&a.runs[r])[q];
-        __syncwarp();
-        const int K = bc.K;
-        if (lane < K) {
-            const StepConst& sk = a.steps[bc.j0 + lane];
-            ss[lane] = ContribStep{sk.dx, sk.dy, sk.dz, sk.ix, sk.iy, sk.iz};
+    const BlockConst& bc = a.runs[r];
+    const RunLight& rl = a.lights[r];
+    const int K = bc.K;
+    const unsigned run_bits = K >= 32 ? 0xffffffffu : ((1u << K) - 1u);
+    const unsigned m = live ? (unsigned)(a.masks[(long long)bc.mask_block * a.R + cell] >> bc.mask_bit) & run_bits : 0u;
+    for (int k = 0; k < K; ++k) s.key[k][tid] = ~0ull;
+    const float4 p = make_float4(o.x, o.y, o.z, kGroundTmin);
+    s.l.o[tid] = p;
+    stage_directions(s.l, a.steps, rl);
+    unsigned long long n_graze = 0, n_over = 0, n_box = 0;
+    unsigned found = 0u;
+    // pass (level, rem): buildings with id = rem modulo mod = kCastSplit^level, for the cells
+    // whose list ran out a level above
+    int level = 0;
+    unsigned mod = 1, rem = 0;
+    while (true) {
+        const bool mine = level == 0 ? live : ((s.over[level - 1][tid >> 5] >> lane) & 1u) != 0u;
+#pragma unroll
+        for (int e = 0; e < kCastList; ++e) {
+            s.cb[e][tid] = -1;
+            s.cm[e][tid] = 0u;
         }
-        const unsigned run_bits = K >= 32 ? 0xffffffffu : ((1u << K) - 1u);
-        unsigned m = 0u;
-        if (live) m = (unsigned)(a.masks[(long long)bc.mask_block * a.R + cell] >> bc.mask_bit) & run_bits;
-        __syncwarp();
-        for (int k = 0; k < K; ++k) w.t[k][lane] = 3.4e38f;
-        int n_list = 0;
-        bool ovf = false;
-        unsigned found = 0u;
-        const bool wedge = bc.wedge_ok != 0.f;
-        const bool want = m != 0u;
-        for (int i = 0; i < a.sc.n_nodes;) {
-            const float4 lo = __ldg(&a.sc.nodes[2 * i]);
-            const float4 hi = __ldg(&a.sc.nodes[2 * i + 1]);
-            const int esc = SA_ESC(__float_as_int(lo.w), i, a.sc.n_nodes, sa::CK_CONTRIB_ESCAPE);
-            const int tri = SA_LEAF(__float_as_int(hi.w), a.sc.T, sa::CK_CONTRIB_LEAF);
-            const bool in = want && (wedge ? fan_box(o, bc, lo, hi) : slope_box(o, bc, lo, hi));
-            if (tri >= 0) {
-                unsigned cand = 0u;
-                float4 ta, tb, tc;
-                if (in) {
-                    ta = __ldg(&a.sc.tris[3 * tri]);
-                    tb = __ldg(&a.sc.tris[3 * tri + 1]);
-                    tc = __ldg(&a.sc.tris[3 * tri + 2]);
-                    if (plane_reachable(o, ta, tb, tc, bc)) {
-                        int ka, kb;
-                        candidate_steps(o, bc, bc.psi, ta, tb, tc, &ka, &kb);
-                        if (ka <= kb) {
-                            const unsigned hi_bits = kb >= 31 ? 0xffffffffu : ((2u << kb) - 1u);
-                            cand = m & hi_bits & ~((1u << ka) - 1u);
-                        }
+        if (lane == 0) s.over[level][tid >> 5] = 0u;
+        s.l.m[tid] = mine ? m : 0u;
+        walk_group<false>(
+            s.l, s.g, a.sc, rl, mine, p,
+            [&](int tri) {
+                const bool in = mod == 1u || (unsigned)__float_as_int(__ldg(&a.sc.tris[3 * tri]).w) % mod == rem;
+                return in ? (unsigned)tri + 1u : 0u;
+            },
+            n_box, [&](int nt, float la, float lb) {
+                light_pass(s.l, rl, nt, mine, p, la, lb, [&](const unsigned short* q, int n) {
+                    drain_contrib(s, q, n, K, a.n_b, level == 0, s.over[level]);
+                });
+                return false;
+            });
+        const bool ovf = (s.over[level][tid >> 5] >> lane) & 1u;
+        if (level == 0) {
+            // nearest: runs of steps with the same nearest building are credited at once
+            int cur = -1, last = -1;
+            unsigned long long cnt = 0;
+            for (unsigned rest = m; rest;) {
+                const int k = __ffs(rest) - 1;
+                rest &= rest - 1u;
+                const unsigned long long key = s.key[k][tid];
+                s.key[k][tid] = 0ull;                 // from here on: buildings met at the step
+                if (key == ~0ull) continue;
+                found |= 1u << k;
+                const int tri = (int)((unsigned)key - 1u);
+                if (tri != last) {
+                    last = tri;
+                    const int bid = (int)SA_CHK(__float_as_int(__ldg(&a.sc.tris[3 * tri]).w), a.n_b, sa::CK_CONTRIB_BUILDING);
+                    if (bid != cur) {
+                        if (cnt) atomicAdd(&a.near_cnt[cur], cnt);
+                        cur = bid;
+                        cnt = 0;
                     }
                 }
-                const int wa = __reduce_min_sync(0xffffffffu, cand ? __ffs(cand) - 1 : 32);
-                const int wb = __reduce_max_sync(0xffffffffu, cand ? 31 - __clz(cand) : -1);
-                if (wa <= wb) {
-                    unsigned hits = 0u;
-                    PluckerTri pt;
-                    if (cand) pt = plucker_setup(o, ta, tb, tc);
-                    const int bid = cand ? (int)SA_CHK(__float_as_int(ta.w), a.n_b, sa::CK_CONTRIB_BUILDING) : 0;
-                    for (int k = wa; k <= wb; ++k) {
-                        float t;
-                        if (((cand >> k) & 1u) && plucker_hit_t(pt, ss[k], kGroundTmin, &t)) {
-                            hits |= 1u << k;
-                            if (t < w.t[k][lane]) {
-                                w.t[k][lane] = t;
-                                w.b[k][lane] = (Id)bid;
-                            }
-                        }
-                    }
-                    if (hits) {
-                        found |= hits;
-                        int e = 0;
-                        while (e < n_list && (int)w.cb[e][lane] != bid) ++e;
-                        if (e < n_list) {
-                            w.cm[e][lane] |= hits;
-                        } else if (n_list < kCastList) {
-                            w.cb[n_list][lane] = (Id)bid;
-                            w.cm[n_list][lane] = hits;
-                            ++n_list;
-                        } else {
-                            ovf = true;
-                        }
-                    }
-                }
-                i = esc;
-            } else {
-                i = __any_sync(0xffffffffu, in) ? i + 1 : esc;
+                ++cnt;
+            }
+            if (cnt) atomicAdd(&a.near_cnt[cur], cnt);
+            n_graze += (unsigned long long)__popc(m & ~found);
+        }
+        if (mine && !ovf) {
+            for (int e = 0; e < kCastList && s.cb[e][tid] >= 0; ++e) {
+                const unsigned met = s.cm[e][tid];
+                atomicAdd(&a.cast_cnt[s.cb[e][tid]], (unsigned long long)__popc(met));
+                if (level > 0)
+                    for (unsigned w = met; w; w &= w - 1u) ++s.key[__ffs(w) - 1][tid];
             }
         }
-        // nearest: runs of steps with the same nearest building are credited at once
-        n_graze += (unsigned long long)__popc(m & ~found);
-        unsigned rest = m & found;
-        int cur = -1;
-        unsigned long long cnt = 0;
-        while (rest) {
-            const int k = __ffs(rest) - 1;
-            rest &= rest - 1u;
-            const int bid = (int)w.b[k][lane];
-            if (bid != cur) {
-                if (cnt) atomicAdd(&a.near_cnt[cur], cnt);
-                cur = bid;
-                cnt = 0;
+        if (__syncthreads_or(ovf)) {          // split the pass
+            ++level;
+            mod *= kCastSplit;
+        } else {                              // the next class, or the next one a level above
+            while (level > 0 && rem >= mod - mod / kCastSplit) {
+                rem -= mod - mod / kCastSplit;
+                mod /= kCastSplit;
+                --level;
             }
-            ++cnt;
-        }
-        if (cnt) atomicAdd(&a.near_cnt[cur], cnt);
-        if (!ovf) {
-            for (int e = 0; e < n_list; ++e)
-                atomicAdd(&a.cast_cnt[(int)w.cb[e][lane]], (unsigned long long)__popc(w.cm[e][lane]));
-        }
-        // more buildings than the list holds: casting again, ray by ray (each lane alone;
-        // the nearest arrays, no longer needed, hold the ray's list -- with 16-bit ids a
-        // lane's list spans other lanes' columns of t, hence the warp barrier)
-        __syncwarp();
-        Id* ids = reinterpret_cast<Id*>(&w.t[0][0]);       // kRayList x 32 ids over t (and b)
-        unsigned todo = ovf ? (m & found) : 0u;
-        while (todo) {
-            const int k = __ffs(todo) - 1;
-            todo &= todo - 1u;
-            const ContribStep& s = ss[k];
-            int n_ids = 0;
-            bool lost = false;
-            for (int i = 0; i < a.sc.n_nodes;) {
-                const float4 lo = __ldg(&a.sc.nodes[2 * i]);
-                const float4 hi = __ldg(&a.sc.nodes[2 * i + 1]);
-                const int esc = SA_ESC(__float_as_int(lo.w), i, a.sc.n_nodes, sa::CK_CONTRIB_ESCAPE);
-                const int tri = SA_LEAF(__float_as_int(hi.w), a.sc.T, sa::CK_CONTRIB_LEAF);
-                const bool in = hit_box(o, s.ix, s.iy, s.iz, lo, hi);
-                if (tri >= 0) {
-                    if (in) {
-                        const float4 ta = __ldg(&a.sc.tris[3 * tri]);
-                        const float4 tb = __ldg(&a.sc.tris[3 * tri + 1]);
-                        const float4 tc = __ldg(&a.sc.tris[3 * tri + 2]);
-                        const PluckerTri pt = plucker_setup(o, ta, tb, tc);
-                        if (plucker_hit(pt, s.dx, s.dy, s.dz, kGroundTmin)) {
-                            const int bid = (int)SA_CHK(__float_as_int(ta.w), a.n_b, sa::CK_CONTRIB_BUILDING);
-                            int e = 0;
-                            while (e < n_ids && (int)ids[e * 32 + lane] != bid) ++e;
-                            if (e == n_ids) {
-                                if (n_ids < kRayList) ids[(n_ids++) * 32 + lane] = (Id)bid;
-                                else lost = true;
-                            }
-                        }
-                    }
-                    i = esc;
-                } else {
-                    i = in ? i + 1 : esc;
-                }
-            }
-            for (int e = 0; e < n_ids; ++e) atomicAdd(&a.cast_cnt[(int)ids[e * 32 + lane]], 1ull);
-            if (lost) ++n_over;
+            if (level == 0) break;
+            rem += mod / kCastSplit;
         }
     }
+    for (unsigned rest = found; rest; rest &= rest - 1u)
+        if (s.key[__ffs(rest) - 1][tid] > kRayMost) ++n_over;
     for (int q = 16; q > 0; q >>= 1) {
         n_graze += __shfl_down_sync(0xffffffffu, n_graze, q);
         n_over += __shfl_down_sync(0xffffffffu, n_over, q);
@@ -390,7 +402,8 @@ cudaError_t launch_building_contribution(const DevScene& sc, const DevRecv& rc, 
     const size_t n_cnt = 2 * (size_t)B + 2;
     cudaError_t e = cudaSuccess;
     unsigned long long *masks = nullptr, *cnt = nullptr;
-    int *gross = nullptr, *run = nullptr, *items = nullptr, *wbase = nullptr;
+    int *items = nullptr, *cbase = nullptr;
+    RunLight* lights = nullptr;
     unsigned *pcnt = nullptr, *poff = nullptr, *runinfo = nullptr;
     double2* dp = nullptr;
     BlockConst* druns = nullptr;
@@ -419,18 +432,16 @@ cudaError_t launch_building_contribution(const DevScene& sc, const DevRecv& rc, 
         // the accrual raster's per-block step masks mark the shadowed steps
         TRY(sa::scratch_alloc(&masks, sizeof(unsigned long long) * (size_t)R * sun.n_blocks, st));
         TRY(cudaMemsetAsync(masks, 0, sizeof(unsigned long long) * (size_t)R * sun.n_blocks, st));
-        TRY(sa::scratch_alloc(&gross, sizeof(int) * (size_t)R, st));
-        TRY(sa::scratch_alloc(&run, sizeof(int) * (size_t)R, st));
         {
             DevOut out;
             memset(&out, 0, sizeof(out));
-            out.gross = gross;
-            out.run = run;
             out.masks = reinterpret_cast<uint64_t*>(masks);
             TRY(launch_raster_ground(sc, rc, sun, out, st));
         }
+        TRY(sa::scratch_alloc(&lights, sizeof(RunLight) * runs.size(), st));
+        TRY(launch_run_lights(sun.steps, druns, (int)runs.size(), 1, lights, st));
         ContribArgs ca;
-        ca.sc = sc; ca.steps = sun.steps; ca.runs = druns; ca.n_runs = (int)runs.size();
+        ca.sc = sc; ca.steps = sun.steps; ca.runs = druns; ca.lights = lights; ca.n_runs = (int)runs.size();
         ca.masks = masks; ca.R = R;
         ca.x0 = rc.x0; ca.y0 = rc.y0; ca.dx = rc.dx; ca.nx = rc.nx;
         ca.bx0 = (int)fx0; ca.by0 = (int)fy0;
@@ -439,11 +450,11 @@ cudaError_t launch_building_contribution(const DevScene& sc, const DevRecv& rc, 
         ca.cast_cnt = cnt; ca.near_cnt = cnt + B; ca.stats = cnt + 2 * B; ca.n_b = B;
         // the work lists: per run, the cells with a shadowed step in it, in patch order
         const int nr = (int)runs.size();
-        const long long patches = (long long)((ca.bnx + 7) / 8) * ((ca.bny + 3) / 4);
+        const long long patches = contrib_patches(ca.bnx, ca.bny);
         const long long nslots = patches * nr;
         TRY(sa::scratch_alloc(&pcnt, sizeof(unsigned) * (size_t)(nslots + 1), st));
         TRY(sa::scratch_alloc(&poff, sizeof(unsigned) * (size_t)(nslots + 1), st));
-        TRY(sa::scratch_alloc(&wbase, sizeof(int) * (size_t)(nr + 1), st));
+        TRY(sa::scratch_alloc(&cbase, sizeof(int) * (size_t)(nr + 1), st));
         TRY(sa::scratch_alloc(&runinfo, sizeof(unsigned) * 2 * (size_t)nr, st));
         const unsigned pblocks = (unsigned)((patches + 3) / 4);
         k_contrib_items<<<pblocks, 128, 0, st>>>(ca, false, pcnt, nullptr, nullptr);
@@ -453,9 +464,8 @@ cudaError_t launch_building_contribution(const DevScene& sc, const DevRecv& rc, 
         TRY(exclusive_scan_u32(poff, nslots + 1, nullptr, st));
         // per run: its first item and its count (run r's offsets start at slot r x patches)
         std::vector<unsigned> h_off((size_t)nr + 1);
-        for (int r = 0; r <= nr; ++r)
-            TRY(cudaMemcpyAsync(&h_off[(size_t)r], poff + (size_t)r * patches, sizeof(unsigned),
-                                cudaMemcpyDeviceToHost, st));
+        TRY(cudaMemcpy2DAsync(h_off.data(), sizeof(unsigned), poff, sizeof(unsigned) * (size_t)patches,
+                              sizeof(unsigned), (size_t)nr + 1, cudaMemcpyDeviceToHost, st));
         TRY(cudaStreamSynchronize(st));
         const unsigned total = h_off[(size_t)nr];
         TRY(sa::scratch_alloc(&items, sizeof(int) * ((size_t)total + 1), st));
@@ -466,17 +476,17 @@ cudaError_t launch_building_contribution(const DevScene& sc, const DevRecv& rc, 
         for (int r = 0; r < nr; ++r) {
             h_run[(size_t)r] = h_off[(size_t)r];
             h_run[(size_t)nr + r] = h_off[(size_t)r + 1] - h_off[(size_t)r];
-            h_base[(size_t)r + 1] = h_base[(size_t)r] + (int)((h_run[(size_t)nr + r] + 31u) / 32u);
+            h_base[(size_t)r + 1] = h_base[(size_t)r] + (int)((h_run[(size_t)nr + r] + kTileThreads - 1u) / kTileThreads);
         }
         TRY(cudaMemcpyAsync(runinfo, h_run.data(), sizeof(unsigned) * 2 * (size_t)nr, cudaMemcpyHostToDevice, st));
-        TRY(cudaMemcpyAsync(wbase, h_base.data(), sizeof(int) * (size_t)(nr + 1), cudaMemcpyHostToDevice, st));
-        ca.items = items; ca.item0 = runinfo; ca.n_items = runinfo + nr; ca.warp_base = wbase;
-        const long long warps = h_base[(size_t)nr];
-        if (warps > 0) {
+        TRY(cudaMemcpyAsync(cbase, h_base.data(), sizeof(int) * (size_t)(nr + 1), cudaMemcpyHostToDevice, st));
+        ca.items = items; ca.item0 = runinfo; ca.n_items = runinfo + nr; ca.cta_base = cbase;
+        const int ctas = h_base[(size_t)nr];
+        if (ctas > 0) {
             KernelTimer kt(KT_CONTRIB, st);
-            const unsigned ctas = (unsigned)((warps + kContribWarps - 1) / kContribWarps);
-            if (B <= 65535) k_building_contribution<unsigned short><<<ctas, 32 * kContribWarps, 0, st>>>(ca);
-            else k_building_contribution<int><<<ctas, 32 * kContribWarps, 0, st>>>(ca);
+            TRY(cudaFuncSetAttribute(k_building_contribution, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(ContribSmem)));
+            k_building_contribution<<<(unsigned)ctas, kTileThreads, sizeof(ContribSmem), st>>>(ca);
         }
         TRY(cudaGetLastError());
     }
@@ -492,8 +502,8 @@ cudaError_t launch_building_contribution(const DevScene& sc, const DevRecv& rc, 
         stats_out[1] = h_cnt[2 * (size_t)B + 1];
     }
 done:
-    for (void* p : {(void*)masks, (void*)cnt, (void*)gross, (void*)run, (void*)dp, (void*)druns,
-                    (void*)items, (void*)pcnt, (void*)poff, (void*)runinfo, (void*)wbase})
+    for (void* p : {(void*)masks, (void*)cnt, (void*)lights, (void*)dp, (void*)druns,
+                    (void*)items, (void*)pcnt, (void*)poff, (void*)runinfo, (void*)cbase})
         if (p) cudaFreeAsync(p, st);
     return e;
 #undef TRY

@@ -44,7 +44,6 @@ const char* check_site_name(int site) {
         "ground raster: binned triangle", "ground raster: tile cell", "binning: bin slot",
         "light-space map: binned triangle", "light-space map: binned receiver",
         "light-space map: receiver permutation", "light-space map: receiver mask",
-        "building contribution: leaf triangle", "building contribution: escape link",
         "building contribution: building id", "building contribution: listed cell",
         "inverse map: leaf triangle",
         "inverse map: escape link", "height adjoint: leaf triangle", "height adjoint: escape link"};

@@ -24,8 +24,8 @@ namespace sa {
 // the flag the checks compile to nothing.
 enum CheckSite {
     CK_NONE = 0, CK_TRACE_LEAF, CK_TRACE_ESCAPE, CK_RASTER_BIN, CK_RASTER_CELL, CK_BIN_SLOT,
-    CK_POINTS_TRI, CK_POINTS_RECV, CK_POINTS_PERM, CK_POINTS_MASK, CK_CONTRIB_LEAF,
-    CK_CONTRIB_ESCAPE, CK_CONTRIB_BUILDING, CK_CONTRIB_CELL, CK_IAM_LEAF, CK_IAM_ESCAPE, CK_ADJ_LEAF,
+    CK_POINTS_TRI, CK_POINTS_RECV, CK_POINTS_PERM, CK_POINTS_MASK,
+    CK_CONTRIB_BUILDING, CK_CONTRIB_CELL, CK_IAM_LEAF, CK_IAM_ESCAPE, CK_ADJ_LEAF,
     CK_ADJ_ESCAPE, CK_SITES
 };
 const char* check_site_name(int site);
@@ -599,7 +599,8 @@ cudaError_t launch_height_grad(const DevScene& sc, const FootprintSet& fs, const
 
 // building contribution over a polygonal region (sa_analysis.cu); casting_out and
 // nearest_out are host arrays of n_buildings, stats_out two host counters (cell-steps past
-// 32 buildings, shadowed cell-steps whose ray met no building)
+// 64 buildings, shadowed cell-steps whose ray met no building)
+constexpr int kContribRun = 16;   // steps of a run, at the most
 cudaError_t launch_building_contribution(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
                                          const std::vector<BlockConst>& runs, int n_buildings,
                                          const float* poly_xy, int n, double* casting_out,

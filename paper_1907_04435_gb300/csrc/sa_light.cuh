@@ -147,23 +147,25 @@ __host__ __device__ inline void light_finish(const LightBasis& L, const LightSte
     rl->bn = (float)(s.mx[2] * (1.0 + 1e-6) + 1e-12);
 }
 
-// Shared memory of a CTA.
+// Shared memory of a CTA that stages CHUNK triangles at a time.
+template <int CHUNK>
 struct LightSmem {
     // staged triangles: vertices in .xyz; .w of the second and third vertex hold the
     // bounds of d . n over the run's steps (run_dot_bounds)
-    float4 tri[kTriChunk * 3];
-    float4 n[kTriChunk];              // normals (origin-independent set-up), highest vertex z in .w
-    float4 box[kTriChunk];            // light box (amin, amax, bmin, bmax), widened by the slack
-    float4 edge[3][kTriChunk];        // light-space edge lines (nx, ny, c + slack, drift)
-    unsigned front[kTriChunk];        // steps to test
+    float4 tri[CHUNK * 3];
+    float4 n[CHUNK];              // normals (origin-independent set-up), highest vertex z in .w
+    float4 box[CHUNK];            // light box (amin, amax, bmin, bmax), widened by the slack
+    float4 edge[3][CHUNK];        // light-space edge lines (nx, ny, c + slack, drift)
+    unsigned front[CHUNK];        // steps to test
     unsigned long long d2[kRunMax / 2][3];   // directions of steps (k, k + 1), k even
     float4 o[kTileThreads];           // receiver origins (and t_min) of the pass
     unsigned m[kTileThreads];         // their step bits
     unsigned short q[kTileThreads / 32][kQueue];         // pair queues: receiver slot << 8 | triangle
-    unsigned char list[kTileThreads / 32][kTriChunk];    // triangles near the warp's receivers
+    unsigned char list[kTileThreads / 32][CHUNK];    // triangles near the warp's receivers
 };
 
-__device__ __forceinline__ void stage_directions(LightSmem& sm, const StepConst* steps, const RunLight& rl) {
+template <class Smem>
+__device__ __forceinline__ void stage_directions(Smem& sm, const StepConst* steps, const RunLight& rl) {
     if (2 * threadIdx.x < rl.kn) {
         const int k = 2 * threadIdx.x, k1 = min(k + 1, rl.kn - 1);
         const StepConst& s = steps[rl.j0 + rl.k0 + k];
@@ -220,7 +222,8 @@ __device__ __forceinline__ void light_edges(const float* pa, const float* pb, co
 }
 
 // Stages triangle (a, b, c) of the scene in slot i; the caller sets sm.front[i].
-__device__ __forceinline__ void stage_triangle(LightSmem& sm, int i, const float4* tris, int t,
+template <class Smem>
+__device__ __forceinline__ void stage_triangle(Smem& sm, int i, const float4* tris, int t,
                                                const RunLight& rl, const float* ref) {
                 const float4 a = __ldg(&tris[3 * t]), b = __ldg(&tris[3 * t + 1]),
                              c = __ldg(&tris[3 * t + 2]);
@@ -244,8 +247,8 @@ __device__ __forceinline__ void stage_triangle(LightSmem& sm, int i, const float
                 sm.tri[3 * i + 2].w = ndb.y;
 }
 
-template <bool COUNT>
-__device__ __forceinline__ void drain_pairs(LightSmem& sm, const unsigned short* q, int n, int lane,
+template <bool COUNT, class Smem>
+__device__ __forceinline__ void drain_pairs(Smem& sm, const unsigned short* q, int n, int lane,
                                             int kn, unsigned long long& n_pair,
                                             unsigned long long& n_test) {
     const bool live = lane < n;
@@ -321,11 +324,11 @@ __device__ __forceinline__ void drain_pairs(LightSmem& sm, const unsigned short*
 // One pass of a warp's 32 receivers (sm.o, sm.m; light coordinates la, lb) over the nt staged
 // triangles: the triangles no ray of any of them can reach are dropped for the whole warp
 // at once, the other pairs are culled per lane, queued, and tested 32 at a time.
-template <bool COUNT>
-__device__ __forceinline__ void light_pass(LightSmem& sm, const RunLight& rl, int nt, bool live, const float4& p,
-                                           float la, float lb, unsigned long long& n_pair,
-                                           unsigned long long& n_test) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kn = rl.kn;
+// drain(queue, n) tests n <= 32 pairs, receiver slot << 8 | triangle each, one per lane.
+template <class Smem, class Drain>
+__device__ __forceinline__ void light_pass(Smem& sm, const RunLight& rl, int nt, bool live, const float4& p,
+                                           float la, float lb, Drain drain) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned short* q = sm.q[warp];
     // the warp's receivers' light-space box and lowest height
     float wa0 = live ? la : 3.4e38f, wa1 = live ? la : -3.4e38f;
@@ -340,7 +343,7 @@ __device__ __forceinline__ void light_pass(LightSmem& sm, const RunLight& rl, in
     }
     int nl = 0;
     for (int t0 = 0; t0 < nt; t0 += 32) {
-        const int t = t0 + lane;           // < kTriChunk: the arrays are read in bounds
+        const int t = t0 + lane;           // < the chunk: the arrays are read in bounds
         const float rise = sm.n[t].w - wz;
         const float h = fmaxf(rise, 0.f);
         const float4 bx = sm.box[t];
@@ -393,11 +396,138 @@ __device__ __forceinline__ void light_pass(LightSmem& sm, const RunLight& rl, in
         if (n >= 32 || (j == nl && n > 0)) {
             const int cnt = min(n, 32);
             __syncwarp();
-            drain_pairs<COUNT>(sm, q + (n - cnt), cnt, lane, kn, n_pair, n_test);
+            drain(q + (n - cnt), cnt);
             n -= cnt;
             __syncwarp();
         }
     }
 }
+
+// ------------------------------------------------------------------- grouped traversal
+// CHUNK triangles staged at a time, a node stack of STACK entries
+template <int CHUNK, int STACK>
+struct GroupSmem {
+    int stack[STACK];
+    int leaf[CHUNK + kTileThreads];
+    int nst, nleaf;
+    float box[kTileThreads / 32][6];
+};
+
+// Walks the BVH once for a CTA's group of receivers (one per thread: origin and t_min p) with
+// all of their fans of a run as the query, kTileThreads nodes at a time from a shared
+// stack: in the run's light space a ray at height h above its receiver lies within the
+// receiver's coordinates widened by h times the run's drift box, so a node is entered when
+// its projected box reaches the group's, widened by the rise to the node's top.  The
+// leaves' triangles are staged CHUNK at a time (sm.front: front(tri), not 0), and
+// pass(nt, la, lb) takes them; it returns whether the thread's receiver needs no more, and the walk ends when
+// none does.  sm.o must be set, sm.m too if pass uses it.
+template <bool COUNT, int CHUNK, int STACK, class Front, class Pass>
+__device__ __forceinline__ void walk_group(LightSmem<CHUNK>& sm, GroupSmem<CHUNK, STACK>& gs, const DevScene& sc,
+                                           const RunLight& rl, bool active, const float4& p, Front front,
+                                           unsigned long long& n_box, Pass pass) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the group's box, and its centre as the reference point
+    float lo[3] = {p.x, p.y, p.z}, hi[3] = {p.x, p.y, p.z};
+    for (int q = 0; q < 3; ++q) {
+        if (!active) { lo[q] = 3.4e38f; hi[q] = -3.4e38f; }
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[q] = fminf(lo[q], __shfl_xor_sync(kAll, lo[q], o));
+            hi[q] = fmaxf(hi[q], __shfl_xor_sync(kAll, hi[q], o));
+        }
+        if (lane == 0) { gs.box[warp][q] = lo[q]; gs.box[warp][3 + q] = hi[q]; }
+    }
+    if (tid == 0) {
+        gs.stack[0] = 0;
+        gs.nst = sc.n_nodes > 0 ? 1 : 0;
+        gs.nleaf = 0;
+    }
+    __syncthreads();
+    float ref[3], half[3];
+    for (int q = 0; q < 3; ++q) {
+        float a = gs.box[0][q], b = gs.box[0][3 + q];
+        for (int w = 1; w < kTileThreads / 32; ++w) {
+            a = fminf(a, gs.box[w][q]);
+            b = fmaxf(b, gs.box[w][3 + q]);
+        }
+        ref[q] = 0.5f * (a + b);
+        half[q] = 0.5f * (b - a);
+    }
+    const float zlow = ref[2] - half[2] - 0.01f;
+    // half extents of the group in light space, with the culls' slack
+    const float ga = fabsf(rl.e1[0]) * half[0] + fabsf(rl.e1[1]) * half[1] + fabsf(rl.e1[2]) * half[2] + kLightSlack;
+    const float gb = fabsf(rl.e2[0]) * half[0] + fabsf(rl.e2[1]) * half[1] + fabsf(rl.e2[2]) * half[2] + kLightSlack;
+    float la, lb;
+    light_ab(rl, ref, p.x, p.y, p.z, &la, &lb);
+    while (true) {
+        __syncthreads();
+        int nst = gs.nst, nleaf = gs.nleaf;
+        while (nst > 0 && nleaf < CHUNK) {
+            // a wave pops up to kTileThreads nodes and pushes at most twice as many; near the
+            // stack's end it goes node by node, and the tree's depth (<= 62) fits what is left
+            const int take = min(kTileThreads, min(nst, max(1, STACK - 96 - nst)));
+            const int i = tid < take ? gs.stack[nst - 1 - tid] : -1;
+            __syncthreads();
+            if (tid == 0) gs.nst = nst - take;
+            __syncthreads();
+            bool in = false;
+            int tri = -1;
+            if (i >= 0) {
+                const float4 nlo = __ldg(&sc.nodes[2 * i]);
+                const float4 nhi = __ldg(&sc.nodes[2 * i + 1]);
+                tri = SA_LEAF(__float_as_int(nhi.w), sc.T, sa::CK_TRACE_LEAF);
+                if (COUNT) ++n_box;
+                const float hx = 0.5f * (nhi.x - nlo.x), hy = 0.5f * (nhi.y - nlo.y), hz = 0.5f * (nhi.z - nlo.z);
+                float a, b;
+                light_ab(rl, ref, nlo.x + hx, nlo.y + hy, nlo.z + hz, &a, &b);
+                const float ra = fmaf(fabsf(rl.e1[2]), hz, fmaf(fabsf(rl.e1[1]), hy, fabsf(rl.e1[0]) * hx));
+                const float rb = fmaf(fabsf(rl.e2[2]), hz, fmaf(fabsf(rl.e2[1]), hy, fabsf(rl.e2[0]) * hx));
+                const float rise = nhi.z - zlow;
+                in = (rise >= 0.f) & (fmaf(rise, rl.da_hi, ga) >= a - ra) & (fmaf(-rise, rl.da_lo, -ga) <= a + ra) &
+                     (fmaf(rise, rl.db_hi, gb) >= b - rb) & (fmaf(-rise, rl.db_lo, -gb) <= b + rb);
+            }
+            const bool leaf = in && tri >= 0, node = in && tri < 0;
+            const unsigned bn = __ballot_sync(kAll, node), bl = __ballot_sync(kAll, leaf);
+            int pn = 0, pl = 0;
+            if (lane == 0) {
+                if (bn) pn = atomicAdd(&gs.nst, 2 * __popc(bn));
+                if (bl) pl = atomicAdd(&gs.nleaf, __popc(bl));
+            }
+            pn = __shfl_sync(kAll, pn, 0);
+            pl = __shfl_sync(kAll, pl, 0);
+            const unsigned below = (1u << lane) - 1u;
+            if (node) {
+                // in depth-first order the left child follows, and the right one follows it
+                const int left = i + 1;
+                const int right = SA_ESC(__float_as_int(__ldg(&sc.nodes[2 * left]).w), left, sc.n_nodes, sa::CK_TRACE_ESCAPE);
+                gs.stack[pn + 2 * __popc(bn & below)] = right;
+                gs.stack[pn + 2 * __popc(bn & below) + 1] = left;
+            }
+            if (leaf) gs.leaf[pl + __popc(bl & below)] = tri;
+            __syncthreads();
+            nst = gs.nst;
+            nleaf = gs.nleaf;
+        }
+        const int nt = min(nleaf, CHUNK), left = nleaf - nt;
+        if (nt == 0) break;
+        if (tid < nt) {
+            const int tri = gs.leaf[tid];
+            stage_triangle(sm, tid, sc.tris, tri, rl, ref);
+            sm.front[tid] = front(tri);
+        }
+        const int carry = tid < left ? gs.leaf[nt + tid] : 0;
+        __syncthreads();
+        if (tid < left) gs.leaf[tid] = carry;
+        if (tid == 0) gs.nleaf = left;
+        const bool done = pass(nt, la, lb);
+        __syncwarp();
+        if (__syncthreads_and(done)) break;
+    }
+}
+
+// Light-space constants of the runs that n blocks are cut into (piece q of K steps runs from
+// q K / parts): one warp per run, a lane per step.
+cudaError_t launch_run_lights(const StepConst* steps, const BlockConst* blocks, int n_blocks, int parts,
+                              RunLight* runs, cudaStream_t st);
 
 }  // namespace sa

@@ -160,7 +160,7 @@ struct TileArgs {
 template <bool COUNT>
 __global__ void __launch_bounds__(kTileThreads, SA_TILE_CTAS)
 k_sam_tile(TileArgs ta) {
-    __shared__ LightSmem sm;
+    __shared__ LightSmem<kTriChunk> sm;
     unsigned long long n_pair = 0, n_test = 0;
     const int tile = ta.order[blockIdx.x];
     const unsigned tcnt = ta.t_cnt[tile], rcnt = ta.r_cnt[tile];
@@ -188,7 +188,9 @@ k_sam_tile(TileArgs ta) {
             sm.m[threadIdx.x] = 0u;
             float la = 0.f, lb = 0.f;
             light_ab(rl, rl.c, p.x, p.y, p.z, &la, &lb);
-            light_pass<COUNT>(sm, rl, nt, live, p, la, lb, n_pair, n_test);
+            light_pass(sm, rl, nt, live, p, la, lb, [&](const unsigned short* q, int n) {
+                drain_pairs<COUNT>(sm, q, n, lane, rl.kn, n_pair, n_test);
+            });
             __syncwarp();
             const unsigned m = sm.m[threadIdx.x];
             if (live && m) atomicOr(&ta.masks[(long long)rl.blk * ta.R + s], (unsigned long long)m << rl.k0);

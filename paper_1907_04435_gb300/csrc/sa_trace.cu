@@ -194,11 +194,8 @@ k_sweep(DevScene sc, DevRecv rc, DevSun sun, DevOut out) {
 }
 
 // ------------------------------------------------------------------- accrual trace
-constexpr int kStack = 1024;      // node stack of a CTA's traversal
 constexpr int kAccrualRun = 27;   // steps per run, at the most (<= kRunMax)
 
-// Light-space constants of the runs a chunk's blocks are cut into (piece q of K steps runs from
-// q K / parts): one warp per run, a lane per step.
 __global__ void k_run_lights(const StepConst* __restrict__ steps, const BlockConst* __restrict__ blocks, int n,
                              int parts, RunLight* __restrict__ runs) {
     const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
@@ -246,27 +243,21 @@ __device__ __forceinline__ Receiver load_group_receiver(const DevRecv& rc, long 
     return r;
 }
 
-// Ray-traced accrual of one run of steps for 128 neighbouring receivers.  The CTA walks the
-// BVH once with all of their fans as its query, 128 nodes at a time from a shared stack: in
-// the run's light space (sa_light.cuh) a ray at height h above its receiver lies within
-// the receiver's coordinates widened by h times the run's drift box, so a node is entered
-// when its projected box reaches the group's, widened by the rise to the node's top.  The
-// leaves' triangles are staged 128 at a time, and each warp culls and tests the pairs of
-// its receivers with them, exactly and per step, as the light-space map does; a group
-// shadowed at every step stops.  Bound by issue in the pair culls and tests.  The traversal
-// by one warp's 32 fans (k_accrual_fan, 80 instructions a node for every warp of receivers
-// and block in series) took 3.43 ms on 517 x 389 cells x 481 steps, 2.35 ms as items; the
-// grouped one 0.83 ms.  1024^2 cells: 13.8 -> 4.03 ms; 1M facade points: 16.5 -> 6.7 ms.
+// Ray-traced accrual of one run of steps for 128 neighbouring receivers: the CTA walks the
+// BVH once for all of them (walk_group), and each warp culls and tests the pairs of its
+// receivers with the leaves' triangles, exactly and per step, as the light-space map does;
+// a group shadowed at every step stops.  Bound by issue in the pair culls and tests.  The
+// traversal by one warp's 32 fans (k_accrual_fan, 80 instructions a node for every warp of
+// receivers and block in series) took 3.43 ms on 517 x 389 cells x 481 steps, 2.35 ms as
+// items; the grouped one 0.83 ms.  1024^2 cells: 13.8 -> 4.03 ms; 1M facade points: 16.5 ->
+// 6.7 ms.
 template <bool COUNT>
 __global__ void __launch_bounds__(kTileThreads, 8)
 k_accrual(DevScene sc, DevRecv rc, DevSun sun, DevOut out, TraceItems it, const RunLight* __restrict__ runs) {
-    __shared__ LightSmem sm;
-    __shared__ int s_stack[kStack];
-    __shared__ int s_leaf[2 * kTriChunk];
-    __shared__ int s_nst, s_nleaf;
-    __shared__ float s_group[kTileThreads / 32][6];
+    __shared__ LightSmem<kTriChunk> sm;
+    __shared__ GroupSmem<kTriChunk, 1024> gs;
     unsigned long long n_box = 0, n_pair = 0, n_test = 0;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     const RunLight& rl = runs[blockIdx.y];
     const BlockConst& bc = sun.blocks[it.b0 + (int)blockIdx.y / it.parts];
     const Receiver r = load_group_receiver(rc, blockIdx.x);
@@ -274,104 +265,16 @@ k_accrual(DevScene sc, DevRecv rc, DevSun sun, DevOut out, TraceItems it, const 
     const unsigned full = kn >= 32 ? 0xffffffffu : ((1u << kn) - 1u);
     sm.m[tid] = 0u;
     if (kn > 0) {
-        // the group's box, and its centre as the reference point
-        float lo[3] = {r.o.x, r.o.y, r.o.z}, hi[3] = {r.o.x, r.o.y, r.o.z};
-        for (int q = 0; q < 3; ++q) {
-            if (!r.active) { lo[q] = 3.4e38f; hi[q] = -3.4e38f; }
-            for (int o = 16; o > 0; o >>= 1) {
-                lo[q] = fminf(lo[q], __shfl_xor_sync(kFull, lo[q], o));
-                hi[q] = fmaxf(hi[q], __shfl_xor_sync(kFull, hi[q], o));
-            }
-            if (lane == 0) { s_group[warp][q] = lo[q]; s_group[warp][3 + q] = hi[q]; }
-        }
         const float4 p = make_float4(r.o.x, r.o.y, r.o.z, r.tmin);
         sm.o[tid] = p;
         stage_directions(sm, sun.steps, rl);
-        if (tid == 0) {
-            s_stack[0] = 0;
-            s_nst = sc.n_nodes > 0 ? 1 : 0;
-            s_nleaf = 0;
-        }
-        __syncthreads();
-        float ref[3], half[3];
-        for (int q = 0; q < 3; ++q) {
-            float a = s_group[0][q], b = s_group[0][3 + q];
-            for (int w = 1; w < kTileThreads / 32; ++w) {
-                a = fminf(a, s_group[w][q]);
-                b = fmaxf(b, s_group[w][3 + q]);
-            }
-            ref[q] = 0.5f * (a + b);
-            half[q] = 0.5f * (b - a);
-        }
-        const float zlow = ref[2] - half[2] - 0.01f;
-        // half extents of the group in light space, with the culls' slack
-        const float ga = fabsf(rl.e1[0]) * half[0] + fabsf(rl.e1[1]) * half[1] + fabsf(rl.e1[2]) * half[2] + kLightSlack;
-        const float gb = fabsf(rl.e2[0]) * half[0] + fabsf(rl.e2[1]) * half[1] + fabsf(rl.e2[2]) * half[2] + kLightSlack;
-        float la, lb;
-        light_ab(rl, ref, p.x, p.y, p.z, &la, &lb);
-        while (true) {
-            __syncthreads();
-            int nst = s_nst, nleaf = s_nleaf;
-            while (nst > 0 && nleaf < kTriChunk) {
-                // a wave pops up to 128 nodes and pushes at most twice as many; near the stack's
-                // end it goes node by node, and the tree's depth (<= 62) fits what is left
-                const int take = min(kTileThreads, min(nst, max(1, kStack - 96 - nst)));
-                const int i = tid < take ? s_stack[nst - 1 - tid] : -1;
-                __syncthreads();
-                if (tid == 0) s_nst = nst - take;
-                __syncthreads();
-                bool in = false;
-                int tri = -1;
-                if (i >= 0) {
-                    const float4 nlo = __ldg(&sc.nodes[2 * i]);
-                    const float4 nhi = __ldg(&sc.nodes[2 * i + 1]);
-                    tri = SA_LEAF(__float_as_int(nhi.w), sc.T, sa::CK_TRACE_LEAF);
-                    if (COUNT) ++n_box;
-                    const float hx = 0.5f * (nhi.x - nlo.x), hy = 0.5f * (nhi.y - nlo.y), hz = 0.5f * (nhi.z - nlo.z);
-                    float a, b;
-                    light_ab(rl, ref, nlo.x + hx, nlo.y + hy, nlo.z + hz, &a, &b);
-                    const float ra = fmaf(fabsf(rl.e1[2]), hz, fmaf(fabsf(rl.e1[1]), hy, fabsf(rl.e1[0]) * hx));
-                    const float rb = fmaf(fabsf(rl.e2[2]), hz, fmaf(fabsf(rl.e2[1]), hy, fabsf(rl.e2[0]) * hx));
-                    const float rise = nhi.z - zlow;
-                    in = (rise >= 0.f) & (fmaf(rise, rl.da_hi, ga) >= a - ra) & (fmaf(-rise, rl.da_lo, -ga) <= a + ra) &
-                         (fmaf(rise, rl.db_hi, gb) >= b - rb) & (fmaf(-rise, rl.db_lo, -gb) <= b + rb);
-                }
-                const bool leaf = in && tri >= 0, node = in && tri < 0;
-                const unsigned bn = __ballot_sync(kFull, node), bl = __ballot_sync(kFull, leaf);
-                int pn = 0, pl = 0;
-                if (lane == 0) {
-                    if (bn) pn = atomicAdd(&s_nst, 2 * __popc(bn));
-                    if (bl) pl = atomicAdd(&s_nleaf, __popc(bl));
-                }
-                pn = __shfl_sync(kFull, pn, 0);
-                pl = __shfl_sync(kFull, pl, 0);
-                const unsigned below = (1u << lane) - 1u;
-                if (node) {
-                    // in depth-first order the left child follows, and the right one follows it
-                    const int left = i + 1;
-                    const int right = SA_ESC(__float_as_int(__ldg(&sc.nodes[2 * left]).w), left, sc.n_nodes, sa::CK_TRACE_ESCAPE);
-                    s_stack[pn + 2 * __popc(bn & below)] = right;
-                    s_stack[pn + 2 * __popc(bn & below) + 1] = left;
-                }
-                if (leaf) s_leaf[pl + __popc(bl & below)] = tri;
-                __syncthreads();
-                nst = s_nst;
-                nleaf = s_nleaf;
-            }
-            const int nt = min(nleaf, kTriChunk), left = nleaf - nt;
-            if (nt == 0) break;
-            if (tid < nt) {
-                stage_triangle(sm, tid, sc.tris, s_leaf[tid], rl, ref);
-                sm.front[tid] = full;
-            }
-            const int carry = tid < left ? s_leaf[nt + tid] : 0;
-            __syncthreads();
-            if (tid < left) s_leaf[tid] = carry;
-            if (tid == 0) s_nleaf = left;
-            light_pass<COUNT>(sm, rl, nt, r.active && sm.m[tid] != full, p, la, lb, n_pair, n_test);
+        walk_group<COUNT>(sm, gs, sc, rl, r.active, p, [full](int) { return full; }, n_box, [&](int nt, float la, float lb) {
+            light_pass(sm, rl, nt, r.active && sm.m[tid] != full, p, la, lb, [&](const unsigned short* q, int n) {
+                drain_pairs<COUNT>(sm, q, n, lane, kn, n_pair, n_test);
+            });
             __syncwarp();
-            if (__syncthreads_and(!r.active || sm.m[tid] == full)) break;
-        }
+            return !r.active || sm.m[tid] == full;
+        });
     }
     store_item(out, rc, r, it, sm.m[tid], kn, bc.mask_block, bc.mask_bit + rl.k0);
     if (COUNT) flush_counts(out, n_box, n_test);
@@ -654,6 +557,13 @@ cudaError_t launch_sweep_trace(const DevScene& sc, const DevRecv& rc, const DevS
     return cudaGetLastError();
 }
 
+cudaError_t launch_run_lights(const StepConst* steps, const BlockConst* blocks, int n_blocks, int parts,
+                              RunLight* runs, cudaStream_t st) {
+    const int n = n_blocks * parts;
+    if (n > 0) k_run_lights<<<(n + 3) / 4, 128, 0, st>>>(steps, blocks, n, parts, runs);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const float* recv_box, const DevSun& sun,
                                  const DevOut& out, cudaStream_t st) {
     const long long warps = host_warps(rc);
@@ -698,7 +608,8 @@ cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const fl
             e = sa::scratch_alloc(&runs, sizeof(RunLight) * (size_t)sun.n_blocks * parts, st);
             if (e == cudaSuccess)
                 e = by_items(rg, sun, out, parts, st, [&](const TraceItems& it, unsigned ny) {
-                    k_run_lights<<<(ny * 32 + 127) / 128, 128, 0, st>>>(sun.steps, sun.blocks + it.b0, (int)ny, parts, runs);
+                    const cudaError_t el = launch_run_lights(sun.steps, sun.blocks + it.b0, (int)ny / parts, parts, runs, st);
+                    if (el != cudaSuccess) return el;
                     if (out.stats) k_accrual<true><<<dim3(groups, ny), kTileThreads, 0, st>>>(sc, rg, sun, out, it, runs);
                     else k_accrual<false><<<dim3(groups, ny), kTileThreads, 0, st>>>(sc, rg, sun, out, it, runs);
                     return cudaGetLastError();
