@@ -325,7 +325,7 @@ k_building_contribution(ContribArgs a) {
                 return in ? (unsigned)tri + 1u : 0u;
             },
             n_box, [&](int nt, float la, float lb) {
-                light_pass(s.l, rl, nt, mine, p, la, lb, [&](const unsigned short* q, int n) {
+                light_pass(s.l, rl, nt, mine, p, la, lb, 0u, [&](const unsigned short* q, int n) {
                     drain_contrib(s, q, n, K, a.n_b, level == 0, s.over[level]);
                 });
                 return false;

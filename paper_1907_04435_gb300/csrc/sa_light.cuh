@@ -324,10 +324,11 @@ __device__ __forceinline__ void drain_pairs(Smem& sm, const unsigned short* q, i
 // One pass of a warp's 32 receivers (sm.o, sm.m; light coordinates la, lb) over the nt staged
 // triangles: the triangles no ray of any of them can reach are dropped for the whole warp
 // at once, the other pairs are culled per lane, queued, and tested 32 at a time.
-// drain(queue, n) tests n <= 32 pairs, receiver slot << 8 | triangle each, one per lane.
+// drain(queue, n) tests n <= 32 pairs, receiver slot << 8 | triangle each, one per lane.  A
+// receiver whose sm.m has come to `full` needs no more, and the pass ends when none does.
 template <class Smem, class Drain>
 __device__ __forceinline__ void light_pass(Smem& sm, const RunLight& rl, int nt, bool live, const float4& p,
-                                           float la, float lb, Drain drain) {
+                                           float la, float lb, unsigned full, Drain drain) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned short* q = sm.q[warp];
     // the warp's receivers' light-space box and lowest height
@@ -361,8 +362,9 @@ __device__ __forceinline__ void light_pass(Smem& sm, const RunLight& rl, int nt,
     }
     int n = 0;
     __syncwarp();
-    // a lane without a receiver rises below every triangle
-    const float pz = live ? p.z : 3.4e38f;
+    // a lane without a receiver, or done, rises below every triangle
+    float pz = live ? p.z : 3.4e38f;
+    const float da_hi = rl.da_hi, da_lo = rl.da_lo, db_hi = rl.db_hi, db_lo = rl.db_lo;
     // j == nl drains the queue's last pairs: one call site keeps the unrolled step
     // tests in the instruction cache once
     for (int j = 0; j <= nl; ++j) {
@@ -370,8 +372,8 @@ __device__ __forceinline__ void light_pass(Smem& sm, const RunLight& rl, int nt,
         const float rise = j < nl ? sm.n[t].w - pz : -3.4e38f;
         const float h = fmaxf(rise, 0.f);
         const float4 bx = sm.box[t];
-        bool pass = (rise >= -0.01f) & (fmaf(h, rl.da_hi, la) >= bx.x) & (fmaf(-h, rl.da_lo, la) <= bx.y) &
-                    (fmaf(h, rl.db_hi, lb) >= bx.z) & (fmaf(-h, rl.db_lo, lb) <= bx.w);
+        bool pass = (rise >= -0.01f) & (fmaf(h, da_hi, la) >= bx.x) & (fmaf(-h, da_lo, la) <= bx.y) &
+                    (fmaf(h, db_hi, lb) >= bx.z) & (fmaf(-h, db_lo, lb) <= bx.w);
         if (pass) {
 #pragma unroll
             for (int q3 = 0; q3 < 3; ++q3) {
@@ -399,6 +401,8 @@ __device__ __forceinline__ void light_pass(Smem& sm, const RunLight& rl, int nt,
             drain(q + (n - cnt), cnt);
             n -= cnt;
             __syncwarp();
+            if (sm.m[threadIdx.x] == full) pz = 3.4e38f;
+            if (__all_sync(0xffffffffu, pz == 3.4e38f)) break;   // and the queued pairs are theirs
         }
     }
 }

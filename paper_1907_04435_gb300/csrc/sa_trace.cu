@@ -269,7 +269,7 @@ k_accrual(DevScene sc, DevRecv rc, DevSun sun, DevOut out, TraceItems it, const 
         sm.o[tid] = p;
         stage_directions(sm, sun.steps, rl);
         walk_group<COUNT>(sm, gs, sc, rl, r.active, p, [full](int) { return full; }, n_box, [&](int nt, float la, float lb) {
-            light_pass(sm, rl, nt, r.active && sm.m[tid] != full, p, la, lb, [&](const unsigned short* q, int n) {
+            light_pass(sm, rl, nt, r.active && sm.m[tid] != full, p, la, lb, full, [&](const unsigned short* q, int n) {
                 drain_pairs<COUNT>(sm, q, n, lane, kn, n_pair, n_test);
             });
             __syncwarp();
