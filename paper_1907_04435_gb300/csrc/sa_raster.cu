@@ -60,17 +60,17 @@ __device__ __forceinline__ bool tri_above_ground(const float4& a, const float4& 
 
 // Conservative tile range of a triangle swept over a slope box.
 __device__ __forceinline__ bool swept_tiles(const float4& a, const float4& b, const float4& c,
-                                            const BlockConst& bc, const TileGeom& g, int* tx0,
-                                            int* tx1, int* ty0, int* ty1) {
+                                            float uxlo, float uxhi, float uylo, float uyhi,
+                                            const TileGeom& g, int* tx0, int* tx1, int* ty0, int* ty1) {
     float xmin = 3.4e38f, xmax = -3.4e38f, ymin = 3.4e38f, ymax = -3.4e38f;
     const float4* v[3] = {&a, &b, &c};
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         const float z = fmaxf(v[q]->z, 0.f);
-        xmin = fminf(xmin, v[q]->x - z * bc.uxhi);
-        xmax = fmaxf(xmax, v[q]->x - z * bc.uxlo);
-        ymin = fminf(ymin, v[q]->y - z * bc.uyhi);
-        ymax = fmaxf(ymax, v[q]->y - z * bc.uylo);
+        xmin = fminf(xmin, v[q]->x - z * uxhi);
+        xmax = fmaxf(xmax, v[q]->x - z * uxlo);
+        ymin = fminf(ymin, v[q]->y - z * uyhi);
+        ymax = fmaxf(ymax, v[q]->y - z * uylo);
     }
     const float inv = 1.f / (kTile * g.dx);
     // one cell of margin on every side absorbs rounding of the projections
@@ -104,18 +104,68 @@ __device__ __forceinline__ bool faces_sun(const float3& n, const StepConst* step
     return false;
 }
 
-// Bins of blocks [b0, b0 + nbc): a thread loads its triangle once and takes `per` of the
+// The triangles whose shadow may reach the grid at some step of blocks [0, n_blocks): the
+// tile range swept over the union of the blocks' slope boxes, with swept_tiles's own margin
+// (so a triangle it drops has no tile in any block).  A grid in the middle of a city is
+// reached by few: 1024^2 cells among 1.3M triangles, 132 blocks, 3 chunks of k_bin 1.25 ms
+// -> 0.27 in 2 and 16 us here; 231 x 187 cells, 92 days 3.38 -> 3.06 ms.
+constexpr int kReachThreads = 256;
+__global__ void __launch_bounds__(kReachThreads)
+k_reach(DevScene sc, const BlockConst* __restrict__ blocks, int n_blocks, TileGeom g, unsigned* __restrict__ n,
+        int* __restrict__ list) {
+    __shared__ float s_box[kReachThreads / 32][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float x0 = 3.4e38f, x1 = -3.4e38f, y0 = 3.4e38f, y1 = -3.4e38f;
+    for (int b = threadIdx.x; b < n_blocks; b += kReachThreads) {
+        x0 = fminf(x0, blocks[b].uxlo);
+        x1 = fmaxf(x1, blocks[b].uxhi);
+        y0 = fminf(y0, blocks[b].uylo);
+        y1 = fmaxf(y1, blocks[b].uyhi);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        x0 = fminf(x0, __shfl_xor_sync(0xffffffffu, x0, o));
+        x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, o));
+        y0 = fminf(y0, __shfl_xor_sync(0xffffffffu, y0, o));
+        y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
+    }
+    if (lane == 0) { s_box[warp][0] = x0; s_box[warp][1] = x1; s_box[warp][2] = y0; s_box[warp][3] = y1; }
+    __syncthreads();
+    for (int w = 0; w < kReachThreads / 32; ++w) {
+        x0 = fminf(x0, s_box[w][0]);
+        x1 = fmaxf(x1, s_box[w][1]);
+        y0 = fminf(y0, s_box[w][2]);
+        y1 = fmaxf(y1, s_box[w][3]);
+    }
+    for (long long base = (long long)blockIdx.x * kReachThreads; base < sc.T; base += (long long)gridDim.x * kReachThreads) {
+        const long long t = base + threadIdx.x;
+        bool in = false;
+        if (t < sc.T) {
+            const float4 a = __ldg(&sc.tris[3 * t]), b = __ldg(&sc.tris[3 * t + 1]), c = __ldg(&sc.tris[3 * t + 2]);
+            int tx0, tx1, ty0, ty1;
+            in = tri_above_ground(a, b, c) && swept_tiles(a, b, c, x0, x1, y0, y1, g, &tx0, &tx1, &ty0, &ty1);
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        unsigned at = 0u;
+        if (lane == 0 && bal) at = atomicAdd(n, (unsigned)__popc(bal));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (in) list[at + __popc(bal & ((1u << lane) - 1u))] = (int)t;
+    }
+}
+
+// Bins of blocks [b0, b0 + nbc), of the n triangles of `list` (null: of all): a thread loads
+// its triangle once and takes `per` of the
 // blocks (blockIdx.y picks which), so a season's blocks do not read the mesh again each.
 // Counting (FILL false) adds to counts[block][tile]; filling writes the triangle at
 // offsets[block][tile], or at a fixed place of `cap` triangles per bin when offsets is
 // null (a mesh so small that every bin can hold all of it: one pass, nothing to size).
 template <bool FILL>
-__global__ void k_bin(DevScene sc, const StepConst* __restrict__ steps,
+__global__ void k_bin(DevScene sc, const int* __restrict__ list, int n_list, const StepConst* __restrict__ steps,
                       const BlockConst* __restrict__ blocks, int b0, int nbc, int per, TileGeom g,
                       const unsigned* __restrict__ offsets, unsigned cap,
                       unsigned* __restrict__ counts, int* __restrict__ bins) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= sc.T) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_list) return;
+    const int t = list ? __ldg(&list[i]) : i;
     const float4 a = __ldg(&sc.tris[3 * t]), b = __ldg(&sc.tris[3 * t + 1]),
                  c = __ldg(&sc.tris[3 * t + 2]);
     if (!tri_above_ground(a, b, c)) return;
@@ -128,7 +178,7 @@ __global__ void k_bin(DevScene sc, const StepConst* __restrict__ steps,
         // the tile range first: it culls the triangles whose shadow misses the grid before
         // the facing test (both are conservative, so the order leaves the bins unchanged)
         int tx0, tx1, ty0, ty1;
-        if (!swept_tiles(a, b, c, bc, g, &tx0, &tx1, &ty0, &ty1)) continue;
+        if (!swept_tiles(a, b, c, bc.uxlo, bc.uxhi, bc.uylo, bc.uyhi, g, &tx0, &tx1, &ty0, &ty1)) continue;
         if (sc.closed && !faces_sun(n, steps, bc)) continue;
         const size_t row = (size_t)bl * g.tiles_x * g.tiles_y;
         for (int ty = ty0; ty <= ty1; ++ty)
@@ -1138,7 +1188,8 @@ k_batch_delta(BatchArgs ba, BatchDelta bd) {
                     const float4* t = f.tris + 3ll * (f.map ? f.map[i] : i);
                     const float4 a = __ldg(t), b = __ldg(t + 1), c = __ldg(t + 2);
                     int x0, x1, y0, y1;
-                    pick = tri_above_ground(a, b, c) && swept_tiles(a, b, c, bc, g, &x0, &x1, &y0, &y1) &&
+                    pick = tri_above_ground(a, b, c) &&
+                           swept_tiles(a, b, c, bc.uxlo, bc.uxhi, bc.uylo, bc.uyhi, g, &x0, &x1, &y0, &y1) &&
                            tx >= x0 && tx <= x1 && ty >= y0 && ty <= y1;
                 }
                 const unsigned bal = __ballot_sync(0xffffffffu, pick);
@@ -1338,13 +1389,45 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
     cudaError_t e = cudaSuccess;
     // blocks per chunk: 64, and more where a small grid's counters, bins (every triangle in
     // every tile at the most: the sums stay below 2^31) and run summaries (1 GiB) allow it
-    long long chunk = by_tile ? 64ll : std::max(64ll, std::min((1ll << 20) / n_tiles, (1ll << 31) / ((long long)std::max(sc.T, 1) * n_tiles)));
-    if (fold) chunk = std::min(chunk, std::max(1ll, (1ll << 30) / (4ll * parts * R)));
-    const int max_chunk_blocks = (int)std::min<long long>(sun.n_blocks, chunk);
-    const size_t nc = (size_t)max_chunk_blocks * n_tiles;
+    auto chunk_blocks = [&](int T) {
+        long long chunk = by_tile ? 64ll : std::max(64ll, std::min((1ll << 20) / n_tiles, (1ll << 31) / ((long long)std::max(T, 1) * n_tiles)));
+        if (fold) chunk = std::min(chunk, std::max(1ll, (1ll << 30) / (4ll * parts * R)));
+        return (int)std::min<long long>(sun.n_blocks, chunk);
+    };
     // a mesh so small that every bin may hold all of it needs no counting pass, no scan and
     // no read-back of the bins' size
-    const bool direct = !by_tile && sc.T > 0 && (double)nc * sc.T <= (double)(4 << 20);
+    auto is_direct = [&](int chunk, int T) {
+        return !by_tile && T > 0 && (double)chunk * n_tiles * T <= (double)(4 << 20);
+    };
+    // Many blocks or a large mesh: the triangles that reach the grid at all are listed first
+    // (k_reach and a read-back, 20 us), and where they are the lesser part, only they go
+    // on.  4M (triangle, block) pairs are about as much in the two passes of k_bin.
+    int T = sc.T, chunk = chunk_blocks(T);
+    int* list = nullptr;
+    unsigned* d_reach = nullptr;
+    if (!is_direct(chunk, T) && (long long)T * sun.n_blocks >= (4ll << 20)) {
+        unsigned n = 0;
+        e = sa::scratch_alloc(&d_reach, sizeof(unsigned), st);
+        if (e == cudaSuccess) e = sa::scratch_alloc(&list, sizeof(int) * (size_t)T, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(d_reach, 0, sizeof(unsigned), st);
+        if (e == cudaSuccess) {
+            KernelTimer kt(KT_RASTER_BIN, st);
+            k_reach<<<(unsigned)std::min(152 * 8, (T + kReachThreads - 1) / kReachThreads), kReachThreads, 0, st>>>(
+                sc, sun.blocks, sun.n_blocks, g, d_reach, list);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&n, d_reach, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e == cudaSuccess && n <= (unsigned)T / 2) {
+            T = (int)n;
+            chunk = chunk_blocks(T);
+        } else if (list) {
+            cudaFreeAsync(list, st);
+            list = nullptr;
+        }
+    }
+    const size_t nc = (size_t)chunk * n_tiles;
+    const bool direct = is_direct(chunk, T);
     // one block of words: counts | cursor (zeroed together) | offsets | order | total | buckets
     unsigned* words = nullptr;
     int* bins = nullptr;
@@ -1352,7 +1435,7 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
     int* best_scratch = nullptr;
     unsigned* summary = summaries;
     size_t bins_cap = 0;
-    e = sa::scratch_alloc(&words, sizeof(unsigned) * (4 * nc + 1 + kOrderBuckets), st);
+    if (e == cudaSuccess) e = sa::scratch_alloc(&words, sizeof(unsigned) * (4 * nc + 1 + kOrderBuckets), st);
     unsigned *counts = words, *cursor = words + nc, *offsets = words + 2 * nc, *d_total = words + 4 * nc,
              *hist = d_total + 1;
     int* order = reinterpret_cast<int*>(words + 3 * nc);
@@ -1361,9 +1444,9 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
         best = best_scratch;
     }
     if (e == cudaSuccess && fold)
-        e = sa::scratch_alloc(&summary, sizeof(unsigned) * (size_t)max_chunk_blocks * parts * (size_t)R, st);
+        e = sa::scratch_alloc(&summary, sizeof(unsigned) * (size_t)chunk * parts * (size_t)R, st);
     if (e == cudaSuccess && direct) {
-        bins_cap = nc * sc.T;
+        bins_cap = nc * (size_t)T;
         e = sa::scratch_alloc(&bins, sizeof(int) * bins_cap, st);
     }
     if (e == cudaSuccess && out.gross && out.accumulate_into) {
@@ -1371,22 +1454,22 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
         e = cudaMemsetAsync(out.run, 0, sizeof(int) * (size_t)R, st);
         if (e == cudaSuccess && !out.continuous) e = cudaMemsetAsync(best, 0, sizeof(int) * (size_t)R, st);
     }
-    for (int b0 = 0; b0 < sun.n_blocks && e == cudaSuccess; b0 += (int)chunk) {
-        const int nbc = std::min(sun.n_blocks - b0, (int)chunk);
+    for (int b0 = 0; b0 < sun.n_blocks && e == cudaSuccess; b0 += chunk) {
+        const int nbc = std::min(sun.n_blocks - b0, chunk);
         const size_t ncc = (size_t)nbc * n_tiles;
         int per = 1;
-        const dim3 grid = bin_grid(std::max(sc.T, 1), nbc, &per);
+        const dim3 grid = bin_grid(std::max(T, 1), nbc, &per);
         e = cudaMemsetAsync(words, 0, sizeof(unsigned) * (direct ? ncc : nc + ncc), st);
         if (e != cudaSuccess) break;
         unsigned total = 0;
         if (direct) {
             KernelTimer kt(KT_RASTER_BIN, st);
-            k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, nullptr,
-                                                      (unsigned)sc.T, counts, bins);
-        } else if (sc.T > 0) {
+            k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, list, T, sun.steps, sun.blocks, b0, nbc, per, g, nullptr,
+                                                      (unsigned)T, counts, bins);
+        } else if (T > 0) {
             {
                 KernelTimer kt(KT_RASTER_BIN, st);
-                k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, nullptr, 0u,
+                k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, list, T, sun.steps, sun.blocks, b0, nbc, per, g, nullptr, 0u,
                                                            counts, nullptr);
             }
             if (by_tile) {       // the sums borrow the offsets, which are written below
@@ -1412,7 +1495,7 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
             }
             if (total > 0) {
                 KernelTimer kt(KT_RASTER_BIN, st);
-                k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, offsets, 0u,
+                k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, list, T, sun.steps, sun.blocks, b0, nbc, per, g, offsets, 0u,
                                                           cursor, bins);
             }
         } else {
@@ -1428,8 +1511,8 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
         ra.R = R;
         ra.cull = sc.closed;
         ra.run = g_raster_run;
-        ra.order = sc.T > 0 && !direct ? order : nullptr;
-        ra.cap = direct ? (unsigned)sc.T : 0u;
+        ra.order = T > 0 && !direct ? order : nullptr;
+        ra.cap = direct ? (unsigned)T : 0u;
         ra.parts = parts;
         ra.summary = summaries ? summaries + (size_t)b0 * (size_t)R : summary;
         {
@@ -1441,7 +1524,7 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
             launch_fold(summary, R, sun.blocks + b0, nbc, parts, out, best, ra.load_state, ra.final_chunk, st);
         e = cudaGetLastError();
     }
-    for (void* p : {(void*)words, (void*)bins, (void*)best_scratch, fold ? (void*)summary : nullptr})
+    for (void* p : {(void*)words, (void*)bins, (void*)best_scratch, (void*)list, (void*)d_reach, fold ? (void*)summary : nullptr})
         if (p) cudaFreeAsync(p, st);
     return e;
 }
@@ -1509,7 +1592,7 @@ cudaError_t launch_raster_ground_in(const DevScene& sc, const DevRecv& rc, const
         if (sc.T == 0) return cudaMemsetAsync(offsets, 0, sizeof(unsigned) * ncc, st);
         int per = 1;
         const dim3 grid = bin_grid(sc.T, nbc, &per);
-        k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, b0, nbc, per, g, nullptr, 0u, counts, nullptr);
+        k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, nullptr, sc.T, sun.steps, sun.blocks, b0, nbc, per, g, nullptr, 0u, counts, nullptr);
         e = cudaMemcpyAsync(offsets, counts, sizeof(unsigned) * ncc, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = exclusive_scan_u32_with(offsets, (long long)ncc, partial, d_total, st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(total, d_total, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
@@ -1548,7 +1631,7 @@ cudaError_t launch_raster_ground_in(const DevScene& sc, const DevRecv& rc, const
         if (total > 0) {
             int per = 1;
             const dim3 grid = bin_grid(sc.T, c.y, &per);
-            k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, c.x, c.y, per, g, offsets, 0u, cursor, bins);
+            k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, nullptr, sc.T, sun.steps, sun.blocks, c.x, c.y, per, g, offsets, 0u, cursor, bins);
         }
         RasterArgs ra;
         ra.sc = sc; ra.sun = sun; ra.g = g; ra.b0 = c.x; ra.nbc = c.y;
@@ -1594,7 +1677,7 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     int per = 1;
     const dim3 grid = bin_grid(sc.T > 0 ? sc.T : 1, sun.n_blocks, &per);
     if (e == cudaSuccess && sc.T > 0) {
-        k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, 0, sun.n_blocks, per, g, nullptr, 0u,
+        k_bin<false><<<grid, kBinThreads, 0, st>>>(sc, nullptr, sc.T, sun.steps, sun.blocks, 0, sun.n_blocks, per, g, nullptr, 0u,
                                                    *counts, nullptr);
         e = cudaMemcpyAsync(*offsets, *counts, sizeof(unsigned) * nc, cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = exclusive_scan_u32(*offsets, (long long)nc, d_total, st);
@@ -1605,7 +1688,7 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     }
     if (e == cudaSuccess) e = cudaMalloc(bins, sizeof(int) * ((size_t)total + 1));
     if (e == cudaSuccess && total > 0)
-        k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, sun.steps, sun.blocks, 0, sun.n_blocks, per, g, *offsets, 0u,
+        k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, nullptr, sc.T, sun.steps, sun.blocks, 0, sun.n_blocks, per, g, *offsets, 0u,
                                                   cursor, *bins);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
