@@ -925,10 +925,15 @@ sa_status sa_accumulate_graph(const sa_scene* scene, const sa_receivers* recv, c
         return e == cudaSuccess ? SA_OK : cuda_fail(e, who);
     }
     std::vector<int> edge_K((size_t)E);
-    for (int q = 0; q < E; ++q) edge_K[(size_t)q] = K[(size_t)rep[(size_t)q]];
+    std::vector<int2> edges((size_t)E);
+    for (int q = 0; q < E; ++q) {
+        edge_K[(size_t)q] = K[(size_t)rep[(size_t)q]];
+        edges[(size_t)q] = make_int2(edge_K[(size_t)q], wt[(size_t)q]);
+    }
     unsigned* summary = nullptr;
     unsigned long long* masks = nullptr;
     int *d_walk = nullptr, *d_K = nullptr, *scratch = nullptr;
+    int2* d_edges = nullptr;
     // one chunk of edges' masks at a time, at most 4 GiB (the scratch pool keeps 4 GiB
     // across synchronisations; larger chunks are mapped again on every call), in multiples
     // of the raster's own 64-block chunks where it holds that many
@@ -946,6 +951,8 @@ sa_status sa_accumulate_graph(const sa_scene* scene, const sa_receivers* recv, c
     if (!direct) TRY(sa::scratch_alloc(&scratch, sizeof(int) * (size_t)R, st));
     TRY(sa::scratch_alloc(&d_walk, sizeof(int) * (size_t)nb, st));
     TRY(sa::scratch_alloc(&d_K, sizeof(int) * (size_t)E, st));
+    TRY(sa::scratch_alloc(&d_edges, sizeof(int2) * (size_t)E, st));
+    TRY(cudaMemcpyAsync(d_edges, edges.data(), sizeof(int2) * (size_t)E, cudaMemcpyHostToDevice, st));
     TRY(cudaMemcpyAsync(d_walk, walk.data(), sizeof(int) * (size_t)nb, cudaMemcpyHostToDevice, st));
     TRY(cudaMemcpyAsync(d_K, edge_K.data(), sizeof(int) * (size_t)E, cudaMemcpyHostToDevice, st));
     for (int e0 = 0; e0 < E; e0 += chunk) {
@@ -995,10 +1002,10 @@ sa_status sa_accumulate_graph(const sa_scene* scene, const sa_receivers* recv, c
         gs.d_steps = nullptr;
         if (e != cudaSuccess || status != SA_OK) goto done;
     }
-    TRY(sa::launch_graph_reduce(summary, R, d_walk, nb, step_minutes, gross_steps, gross_minutes,
+    TRY(sa::launch_graph_reduce(summary, R, d_walk, nb, d_edges, E, step_minutes, gross_steps, gross_minutes,
                                 continuous_steps, st));
 done:
-    for (void* p : {(void*)summary, (void*)masks, (void*)scratch, (void*)d_walk, (void*)d_K})
+    for (void* p : {(void*)summary, (void*)masks, (void*)scratch, (void*)d_walk, (void*)d_K, (void*)d_edges})
         if (p) cudaFreeAsync(p, st);
 #undef TRY
     if (status != SA_OK) return status;

@@ -17,7 +17,8 @@
 //                     popcount (Eq. 1: each edge's count times its weight), and the longest
 //                     continuous run, stitched along each day's path of edges in time order
 //                     from the prefix / longest / suffix runs (Sec. 6, continuous shadows).
-//                     The days' paths are one walk of packed codes staged in shared memory.
+//                     The days' paths are one walk of packed codes staged in shared memory,
+//                     with the receivers' summaries beside it while the edges are few.
 #include <math.h>
 
 #include <algorithm>
@@ -103,6 +104,92 @@ __global__ void __launch_bounds__(kGraphThreads) k_graph_reduce(
     }
 }
 
+// The same from summaries staged in shared memory, each read once instead of once per
+// block of its edge.  The order-free parts are taken while staging: the count of an edge
+// times its weight, and its longest run (every edge is on the walk).  What the walk then
+// follows is the run across blocks, from each edge's prefix and suffix (a byte each; a
+// prefix of K steps is a full block): the longest run takes in run + prefix, and the run
+// becomes the suffix, plus the run so far where the block is full.  A thread takes two
+// receivers, 32 bits an edge.  Bound by issue and the read of the summaries: 1024^2 cells,
+// 132 edges, 828 blocks 1161 us from global memory (3.5 GB out of L2) -> 454.
+constexpr int kStagedThreads = 128;
+constexpr int kStagedRecv = 2 * kStagedThreads;
+constexpr int kStagedWalk = 512;  // walk codes staged at a time
+constexpr size_t kStagedBytes = 216 * 1024, kStagedTwo = 104 * 1024;
+
+__device__ __forceinline__ unsigned staged_edge(unsigned s, int w, int& g, int& best) {
+    g += (int)(s & 255u) * w;
+    best = max(best, (int)(s >> 24));
+    return (s >> 8) & 0xffffu;
+}
+
+__device__ __forceinline__ void staged_step(unsigned pre, unsigned suf, int K, int keep, int& run, int& best) {
+    run &= keep;                                                  // 0 at a new day
+    best = max(best, run + (int)pre);
+    run = ((int)pre == K ? run : 0) + (int)suf;
+}
+
+// edges: (K, weight) of each edge
+__global__ void __launch_bounds__(kStagedThreads)
+k_graph_reduce_staged(const unsigned* __restrict__ summary, long long R, const int2* __restrict__ edges, int n_edges,
+                      const int* __restrict__ walk, int n_walk, float step_minutes, int* __restrict__ gross,
+                      float* __restrict__ minutes, int* __restrict__ continuous) {
+    extern __shared__ unsigned s_word[];                          // [n_edges][kStagedThreads]
+    __shared__ int4 s_walk[kStagedWalk];                          // the edge's row, keep, K
+    const int tid = threadIdx.x;
+    const long long r0 = (long long)blockIdx.x * kStagedRecv + tid, r1 = r0 + kStagedThreads;
+    int g0 = 0, g1 = 0, best0 = 0, best1 = 0, run0 = 0, run1 = 0;
+    for (int e = 0; e < n_edges; e += kGather) {
+        unsigned u[kGather], v[kGather];
+#pragma unroll
+        for (int q = 0; q < kGather; ++q) {
+            const unsigned* row = summary + (long long)(e + q) * R;
+            u[q] = e + q < n_edges && r0 < R ? __ldcs(&row[r0]) : 0u;
+            v[q] = e + q < n_edges && r1 < R ? __ldcs(&row[r1]) : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q < kGather; ++q) {
+            if (e + q >= n_edges) break;
+            const int w = __ldg(&edges[e + q]).y;
+            const unsigned a = staged_edge(u[q], w, g0, best0), b = staged_edge(v[q], w, g1, best1);
+            s_word[(e + q) * kStagedThreads + tid] = a | (b << 16);
+        }
+    }
+    for (int p0 = 0; p0 < n_walk; p0 += kStagedWalk) {
+        const int n = min(kStagedWalk, n_walk - p0);
+        __syncthreads();
+        for (int i = tid; i < n; i += kStagedThreads) {
+            const int code = __ldg(&walk[p0 + i]);
+            s_walk[i] = make_int4((code & 0xFFFFF) * kStagedThreads, code & (1 << 27) ? 0 : -1, (code >> 20) & 127, 0);
+        }
+        __syncthreads();
+        auto step = [&](const int4& c, unsigned w) {
+            staged_step(w & 255u, (w >> 8) & 255u, c.z, c.y, run0, best0);
+            staged_step((w >> 16) & 255u, w >> 24, c.z, c.y, run1, best1);
+        };
+        int i = 0;
+        for (; i + kGather <= n; i += kGather) {
+            int4 c[kGather];
+            unsigned w[kGather];
+#pragma unroll
+            for (int q = 0; q < kGather; ++q) c[q] = s_walk[i + q];
+#pragma unroll
+            for (int q = 0; q < kGather; ++q) w[q] = s_word[c[q].x + tid];
+#pragma unroll
+            for (int q = 0; q < kGather; ++q) step(c[q], w[q]);
+        }
+        for (; i < n; ++i) step(s_walk[i], s_word[s_walk[i].x + tid]);
+    }
+    auto put = [&](long long r, int g, int best) {
+        if (r >= R) return;
+        gross[r] = g;
+        if (minutes) minutes[r] = (float)g * step_minutes;
+        if (continuous) continuous[r] = best;
+    };
+    put(r0, g0, best0);
+    put(r1, g1, best1);
+}
+
 int grid_for(long long items) {
     const long long b = (items + kGraphThreads - 1) / kGraphThreads;
     return (int)(b < 152ll * 16 ? (b > 0 ? b : 1) : 152ll * 16);
@@ -158,10 +245,23 @@ cudaError_t launch_edge_summary(const unsigned long long* masks, long long R, in
 }
 
 cudaError_t launch_graph_reduce(const unsigned* summary, long long R, const int* d_walk, int n_walk,
-                                float step_minutes, int* gross, float* minutes, int* continuous,
-                                cudaStream_t st) {
+                                const int2* d_edges, int n_edges, float step_minutes, int* gross,
+                                float* minutes, int* continuous, cudaStream_t st) {
     if (R <= 0) return cudaSuccess;
     KernelTimer kt(KT_GRAPH, st);
+    const size_t bytes = sizeof(unsigned) * kStagedThreads * (size_t)n_edges;
+    const long long ctas = (R + kStagedRecv - 1) / kStagedRecv;
+    // Staged while two CTAs fit an SM; with one (600 x 600 cells: 285 edges), where the walk is
+    // long against the staging: 3194 blocks 1690 -> 958 us, 828 blocks 462 and 481.
+    const bool staged = bytes <= kStagedTwo || (bytes <= kStagedBytes && n_walk >= 6 * n_edges);
+    if (staged && ctas <= 0x7fffffffll) {
+        const cudaError_t e = cudaFuncSetAttribute(k_graph_reduce_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)kStagedBytes);
+        if (e != cudaSuccess) return e;
+        k_graph_reduce_staged<<<(unsigned)ctas, kStagedThreads, bytes, st>>>(
+            summary, R, d_edges, n_edges, d_walk, n_walk, step_minutes, gross, minutes, continuous);
+        return cudaGetLastError();
+    }
     k_graph_reduce<<<grid_for(R), kGraphThreads, 0, st>>>(summary, R, d_walk, n_walk, step_minutes, gross,
                                                           minutes, continuous);
     return cudaGetLastError();

@@ -616,10 +616,11 @@ void direction_graph(const float* dirs, int n_blocks, const int* j0, const int* 
 cudaError_t launch_edge_summary(const unsigned long long* masks, long long R, int n_edges,
                                 const int* d_edge_K, unsigned* summary, cudaStream_t st);
 // gross / minutes / continuous per receiver from the summaries along each day's path; the
-// walk holds every block in time order as edge | K << 20 | (first block of a day) << 27
+// walk holds every block in time order as edge | K << 20 | (first block of a day) << 27, and
+// the edges are (K, blocks on the walk)
 cudaError_t launch_graph_reduce(const unsigned* summary, long long R, const int* d_walk, int n_walk,
-                                float step_minutes, int* gross, float* minutes, int* continuous,
-                                cudaStream_t st);
+                                const int2* d_edges, int n_edges, float step_minutes, int* gross,
+                                float* minutes, int* continuous, cudaStream_t st);
 
 // batched scenarios (device-side descriptors; see sa_raster.cu)
 struct BatchInterval {
