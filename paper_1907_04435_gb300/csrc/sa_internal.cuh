@@ -331,7 +331,9 @@ __device__ __forceinline__ unsigned run_summary(unsigned long long m, int K) {
     } else {
         pre = (unsigned)(__ffsll((long long)~m) - 1);            // ones below the first zero
         suf = (unsigned)__clzll((long long)~(m << (64 - K)));   // ones above the last zero
-        best = longest_run(m);
+        // one run of ones (adding its lowest bit clears it) is its own longest
+        const unsigned long long low = m & (0ull - m);
+        best = ((m + low) & m) == 0ull ? pop : (unsigned)longest_run(m);
     }
     return pop | (pre << 8) | (suf << 16) | (best << 24);
 }

@@ -322,8 +322,9 @@ struct TileSmem {
     unsigned made;                           // rows << 9 | units
     int next_row;                            // next rows to hand out
     // per warp: the covered rows of a claim, (first cell - first position, unit, steps it can
-    // set), and cells waiting for their step tests, (unit << 10) | cell, drained 32 at a
-    // time so that every lane tests a cell whichever unit it comes from
+    // set), and cells waiting for their step tests, unit << 22 | triangle << 16 | first step of
+    // its run << 10 | cell, drained 32 at a time so that every lane tests a cell whichever
+    // unit it comes from
     int4 row[kRasterThreads / 32][32];
     unsigned queue[kRasterThreads / 32][64];
     float xl[kTile], yl[kTile];
@@ -416,16 +417,19 @@ __device__ __forceinline__ void drain_cells(TileSmem& sm, const unsigned* q, int
                                             unsigned long long& n_test) {
     const int lane = threadIdx.x & 31;
     const unsigned item = q[lane < n ? lane : 0];
-    const int j = (int)(item >> 10), cell = (int)SA_CHK(item & 1023u, kTile * kTile, sa::CK_RASTER_CELL);
-    const unsigned un = sm.unit[j];
-    const int t = (int)((un >> 20) & 63u), sub = (int)(un >> 26), k0 = sm.run_k0[sub];
+    const int j = (int)(item >> 22), cell = (int)SA_CHK(item & 1023u, kTile * kTile, sa::CK_RASTER_CELL);
+    const int t = (int)((item >> 16) & 63u), k0 = (int)((item >> 10) & 63u);
     const unsigned fr = sm.fr[j], bk = CULL ? 0u : sm.bk[j];
     const float4* ef = reinterpret_cast<const float4*>(&sm.edges[20 * t]);
     const float4 f0 = ef[0], f1 = ef[1], f2 = ef[2], f3 = ef[3], f4 = ef[4];
     const EdgeLin E0{f0.x, f0.y, f0.z, f0.w, f1.x, f1.y};
     const EdgeLin E1{f1.z, f1.w, f2.x, f2.y, f2.z, f2.w};
     const EdgeLin E2{f3.x, f3.y, f3.z, f3.w, f4.x, f4.y};
-    if (COUNT && lane < n) { ++n_cell; n_test += sm.run_k0[sub + 1] - k0; }
+    if (COUNT && lane < n) {
+        const int sub = (int)(sm.unit[j] >> 26);
+        ++n_cell;
+        n_test += sm.run_k0[sub + 1] - k0;
+    }
     const unsigned hit = cell_steps<CULL>(sm, E0, E1, E2, sm.xl[cell & (kTile - 1)],
                                           sm.yl[cell >> 5], k0, kmax, fr, bk);
     const unsigned long long m = (unsigned long long)hit << k0;
@@ -533,8 +537,8 @@ __device__ __forceinline__ int lane_prefix(int x) {
 
 // Rows rb .. rb + 31 of the batch's units: one lane per row finds its unit and its span; one
 // lane per covered cell checks whether the cell is already shadowed at every step its unit
-// could set (a stale read only skips less) and queues the others, (unit << 10) | cell, for
-// the step tests, 32 at a time whichever unit they come from.
+// could set (a stale read only skips less) and queues the others for the step tests, 32
+// at a time whichever unit they come from.
 template <bool COUNT, bool CULL>
 __device__ __forceinline__ void raster_rows(TileSmem& sm, int rb, int rows, int n_units, int kmax, float inv_dx,
                                             int& qn, unsigned long long& n_cell,
@@ -548,12 +552,14 @@ __device__ __forceinline__ void raster_rows(TileSmem& sm, int rb, int rows, int 
     const int jn = j0 + 1 + lane, at = jn < n_units ? (int)sm.start[jn] - rb : 32;
     const unsigned starts = __reduce_or_sync(0xffffffffu, at < 32 ? 1u << at : 0u);
     const int j = j0 + __popc(starts & upto), ridx = rb + lane;
-    int cs = 0, w = 0;
+    int cs = 0, w = 0, what = 0;
     unsigned long long can = 0ull;
     if (ridx < rows) {
         const unsigned un = sm.unit[j];
         const int row = (int)((un >> 10) & 31u) + (ridx - sm.start[j]), sub = (int)(un >> 26);
-        can = (unsigned long long)(CULL ? sm.fr[j] : (sm.fr[j] | sm.bk[j])) << sm.run_k0[sub];
+        const int k0 = sm.run_k0[sub];
+        can = (unsigned long long)(CULL ? sm.fr[j] : (sm.fr[j] | sm.bk[j])) << k0;
+        what = (j << 22) | (int)((un >> 4) & 0x3f0000u) | (k0 << 10);
         if ((sm.row_full[row] & can) != can)
             row_span(sm, (int)((un >> 20) & 63u), sub, (int)(un & 0xfffffu), row, inv_dx, &cs, &w);
         cs += row * kTile;                                      // the row's first cell
@@ -565,7 +571,7 @@ __device__ __forceinline__ void raster_rows(TileSmem& sm, int rb, int rows, int 
     const unsigned some = __ballot_sync(0xffffffffu, w > 0);
     // the rows with cells, in order
     if (w > 0)
-        sm.row[warp][__popc(some & (upto >> 1))] = make_int4(cs - cex, j, (int)(unsigned)can, (int)(unsigned)(can >> 32));
+        sm.row[warp][__popc(some & (upto >> 1))] = make_int4(cs - cex, what, (int)(unsigned)can, (int)(unsigned)(can >> 32));
     __syncwarp();
     int before = -1;                                            // rows that started before this window, less one
     for (int base = 0; base < total; base += 32) {
@@ -578,7 +584,7 @@ __device__ __forceinline__ void raster_rows(TileSmem& sm, int rb, int rows, int 
         const int cell = in ? (int)SA_CHK(info.x + idx, kTile * kTile, sa::CK_RASTER_CELL) : 0;
         const bool need = in && (((unsigned)info.z & ~sm.lo[cell]) | ((unsigned)info.w & ~sm.hi[cell])) != 0u;
         const unsigned bal = __ballot_sync(0xffffffffu, need);
-        if (need) q[qn + __popc(bal & (upto >> 1))] = ((unsigned)info.y << 10) | (unsigned)cell;
+        if (need) q[qn + __popc(bal & (upto >> 1))] = (unsigned)info.y | (unsigned)cell;
         qn += __popc(bal);
         if (qn >= 32) {
             __syncwarp();
