@@ -111,14 +111,15 @@ struct Grid {
 // gathered and ORed into memory once, when the line leaves it.  (Reading the word first to
 // skip bits that are set made every lane of the warp wait: 3.20 ms against 2.76 for 613 x 457
 // cells x 481 steps.)
+template <class Cell>
 struct Marker {
     unsigned long long* masks;
-    long long cell;
+    Cell cell;
     unsigned long long bits;
     __device__ __forceinline__ void flush() {
         if (bits) atomicOr(&masks[cell], bits);
     }
-    __device__ __forceinline__ void mark(long long c, unsigned long long bit) {
+    __device__ __forceinline__ void mark(Cell c, unsigned long long bit) {
         if (c != cell) {
             flush();
             cell = c;
@@ -129,8 +130,9 @@ struct Marker {
 };
 
 // Every closed grid cell touched by the segment P -> Q gets `bit`.
+template <class Cell>
 __device__ void draw_segment(const Grid& g, float px, float py, float qx, float qy,
-                             Marker& mk, unsigned long long bit) {
+                             Marker<Cell>& mk, unsigned long long bit) {
     const float inv = 1.f / g.dx;
     const float ymin = fminf(py, qy), ymax = fmaxf(py, qy);
     int iy0 = (int)ceilf((ymin - g.y0) * inv) - 1;
@@ -155,20 +157,30 @@ __device__ void draw_segment(const Grid& g, float px, float py, float qx, float 
         int ix1 = (int)floorf((xb - g.x0) * inv);
         ix0 = max(ix0, 0);
         ix1 = min(ix1, g.nx - 1);
-        for (int ix = ix0; ix <= ix1; ++ix) mk.mark((long long)iy * g.nx + ix, bit);
+        const Cell row = (Cell)iy * (Cell)g.nx;
+        for (int ix = ix0; ix <= ix1; ++ix) mk.mark(row + (Cell)ix, bit);
     }
 }
 
-__global__ void __launch_bounds__(32 * kWarps)
+// A CTA finds the sources of its 128 cells, 32 in a patch of 8 x 4 per warp, and lists them;
+// then its threads draw them, one line per thread whichever cell it comes from: most cells
+// are lit or have two sources where their neighbours have four, and a warp that drew its own
+// cells' sources waited for the longest list.  Bound by issue: the pieces of the lines, one
+// after the other (12 CTAs per SM: 2.17 ms the call, 2.21 at 10, 2.24 at 14).  613 x 457
+// cells x 481 steps: 2.76 ms with each thread's own sources, 2.17; 1024^2 9.84 -> 7.79; 400 x
+// 300 on 21 December, when most cells have all four, 3.23 -> 3.13.
+template <class Cell>
+__global__ void __launch_bounds__(32 * kWarps, 12)
 k_iam_draw(DevScene sc, Grid g, const StepConst* __restrict__ steps, const BlockConst* __restrict__ blocks,
            int L, unsigned long long* __restrict__ all_masks) {
-    const int lane = threadIdx.x & 31;
+    __shared__ float s_t[32 * kWarps * kMaxLevels * 2];               // the sources' distances,
+    __shared__ unsigned short s_from[32 * kWarps * kMaxLevels * 2];   // thread | direction << 15
+    __shared__ float2 s_o[32 * kWarps], s_u[kMaxBlock];
+    __shared__ int s_n;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int j0 = blocks[blockIdx.y].j0, K = blocks[blockIdx.y].K;
-    Marker mk{all_masks + (long long)blockIdx.y * g.nx * g.ny, -1, 0ull};
-    const long long warp_id = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    const long long warp_id = (long long)blockIdx.x * kWarps + (tid >> 5);
     const int tiles_x = (g.nx + 7) >> 3;
-    const long long n_warps = (long long)tiles_x * ((g.ny + 3) >> 2);
-    if (warp_id >= n_warps) return;
     const long long ty = warp_id / tiles_x;
     const int tx = (int)(warp_id - ty * tiles_x);
     const int ix = tx * 8 + (lane & 7);
@@ -178,6 +190,10 @@ k_iam_draw(DevScene sc, Grid g, const StepConst* __restrict__ steps, const Block
     o.x = __fadd_rn(g.x0, __fmul_rn(__fadd_rn((float)ix, 0.5f), g.dx));
     o.y = __fadd_rn(g.y0, __fmul_rn(__fadd_rn((float)iy, 0.5f), g.dx));
     o.z = 0.f;
+    s_o[tid] = make_float2(o.x, o.y);
+    if (tid < K) s_u[tid] = make_float2(steps[j0 + tid].ux, steps[j0 + tid].uy);
+    if (tid == 0) s_n = 0;
+    __syncthreads();
     for (int dir = 0; dir < 2; ++dir) {
         const StepConst s = steps[dir == 0 ? j0 : j0 + K - 1];
         float best[kMaxLevels];
@@ -185,30 +201,39 @@ k_iam_draw(DevScene sc, Grid g, const StepConst* __restrict__ steps, const Block
         if (s.kz == 2) n = nearest_sources<2>(sc, o, s, active, L, best);
         else if (s.kz == 0) n = nearest_sources<0>(sc, o, s, active, L, best);
         else n = nearest_sources<1>(sc, o, s, active, L, best);
-        for (int l = 0; l < n; ++l) {
-            const float sx = fmaf(best[l], s.dx, o.x), sy = fmaf(best[l], s.dy, o.y),
-                        sz = best[l] * s.dz;
-            // q_k for the block's steps; the pieces run forward (dir 0) or backward (dir 1)
-            if (dir == 0) {
-                float px = fmaf(-sz, steps[j0].ux, sx), py = fmaf(-sz, steps[j0].uy, sy);
-                for (int k = 0; k + 1 < K; ++k) {
-                    const float qx = fmaf(-sz, steps[j0 + k + 1].ux, sx);
-                    const float qy = fmaf(-sz, steps[j0 + k + 1].uy, sy);
-                    draw_segment(g, px, py, qx, qy, mk, 1ull << k);
-                    px = qx; py = qy;
-                }
-                draw_segment(g, px, py, px, py, mk, 1ull << (K - 1));
-            } else {
-                float px = fmaf(-sz, steps[j0 + K - 1].ux, sx), py = fmaf(-sz, steps[j0 + K - 1].uy, sy);
-                for (int k = K - 1; k >= 1; --k) {
-                    const float qx = fmaf(-sz, steps[j0 + k - 1].ux, sx);
-                    const float qy = fmaf(-sz, steps[j0 + k - 1].uy, sy);
-                    draw_segment(g, px, py, qx, qy, mk, 1ull << k);
-                    px = qx; py = qy;
-                }
-                draw_segment(g, px, py, px, py, mk, 1ull);
+        // level by level, so that neighbours' lines of one source surface stay together
+        for (int l = 0; l < L; ++l) {
+            const unsigned has = __ballot_sync(kFull, l < n);
+            if (!has) break;
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_n, __popc(has));
+            at = __shfl_sync(kFull, at, 0) + __popc(has & ((1u << lane) - 1u));
+            if (l < n) {
+                s_t[at] = best[l];
+                s_from[at] = (unsigned short)(tid | (dir << 15));
             }
         }
+    }
+    __syncthreads();
+    Marker<Cell> mk{all_masks + (long long)blockIdx.y * g.nx * g.ny, (Cell)-1, 0ull};
+    for (int e = tid; e < s_n; e += 32 * kWarps) {
+        const float t = s_t[e];
+        const int from = s_from[e], dir = from >> 15;
+        const float2 p0 = s_o[from & 0x7fff];
+        // q_k for the block's steps; the pieces run forward (dir 0) or backward (dir 1)
+        int k = dir == 0 ? 0 : K - 1;
+        const int dk = dir == 0 ? 1 : -1;
+        const StepConst& s = steps[j0 + k];
+        const float sx = fmaf(t, s.dx, p0.x), sy = fmaf(t, s.dy, p0.y), sz = t * s.dz;
+        float px = fmaf(-sz, s_u[k].x, sx), py = fmaf(-sz, s_u[k].y, sy);
+        for (int i = 0; i + 1 < K; ++i) {
+            const float2 u = s_u[k + dk];
+            const float qx = fmaf(-sz, u.x, sx), qy = fmaf(-sz, u.y, sy);
+            draw_segment(g, px, py, qx, qy, mk, 1ull << k);
+            px = qx; py = qy;
+            k += dk;
+        }
+        draw_segment(g, px, py, px, py, mk, 1ull << k);
     }
     mk.flush();
 }
@@ -257,7 +282,9 @@ cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
         if (e != cudaSuccess) break;
         {
             KernelTimer kt(KT_IAM, st);
-            k_iam_draw<<<dim3(ctas, (unsigned)nbc), 32 * kWarps, 0, st>>>(sc, g, sun.steps, sun.blocks + b0, L, masks);
+            const dim3 grid(ctas, (unsigned)nbc);
+            if (R < (1ll << 31)) k_iam_draw<unsigned><<<grid, 32 * kWarps, 0, st>>>(sc, g, sun.steps, sun.blocks + b0, L, masks);
+            else k_iam_draw<long long><<<grid, 32 * kWarps, 0, st>>>(sc, g, sun.steps, sun.blocks + b0, L, masks);
         }
         k_iam_fold<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(R, sun.blocks + b0, nbc, masks, out, b0 == 0,
                                                                b0 + nbc == sun.n_blocks);
