@@ -1,9 +1,10 @@
 // sa_iam.cu -- inverse accrual map (Sec. 5) of a ground receiver grid.
 //
 // Per block of K steps:
-//   k_iam_draw  every cell centre p traces toward the sun at the block's first step and
+//   k_iam_sources  every cell centre p traces toward the sun at the block's first step and
 //               keeps the L nearest intersections farther than 1 m (the paper's source
-//               levels and its 100 cm acne rule).  Each source s casts its shadow at step
+//               levels and its 100 cm acne rule).
+//   k_iam_draw  each source s casts its shadow at step
 //               k at q_k, the projection of s along d_k onto the ground; the shadow line
 //               q_0 -> q_{K-1} is cut into K - 1 pieces and piece [q_k, q_{k+1}] sets bit
 //               k of every grid cell it touches (closed cells), bit K-1 being set at
@@ -20,6 +21,7 @@
 #include <algorithm>
 
 #include "sa_internal.cuh"
+#include "sa_light.cuh"
 
 namespace sa {
 
@@ -56,50 +58,6 @@ __device__ __forceinline__ bool hit_tri_t(const float3& o, const float4& a, cons
     if (!(t > tmin)) return false;
     *t_out = t;
     return true;
-}
-
-// Slab test with an upper bound on the entry distance.
-__device__ __forceinline__ bool hit_box_before(const float3& o, const StepConst& s, const float4& lo,
-                                               const float4& hi, float tmax) {
-    float tx0 = (lo.x - o.x) * s.ix, tx1 = (hi.x - o.x) * s.ix;
-    float ty0 = (lo.y - o.y) * s.iy, ty1 = (hi.y - o.y) * s.iy;
-    float tz0 = (lo.z - o.z) * s.iz, tz1 = (hi.z - o.z) * s.iz;
-    float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.f));
-    float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1));
-    return tn <= tf * 1.0000005f && tn <= tmax;
-}
-
-// The L nearest hits (ascending) of the ray from o along step s; warp-coherent traversal.
-template <int KZ>
-__device__ int nearest_sources(const DevScene& sc, const float3& o, const StepConst& s,
-                               bool active, int L, float* best) {
-    int n = 0;
-    int i = 0;
-    while (i < sc.n_nodes && __any_sync(kFull, active)) {
-        const float4 lo = __ldg(&sc.nodes[2 * i]);
-        const float4 hi = __ldg(&sc.nodes[2 * i + 1]);
-        const int esc = SA_ESC(__float_as_int(lo.w), i, sc.n_nodes, sa::CK_IAM_ESCAPE);
-        const int tri = SA_LEAF(__float_as_int(hi.w), sc.T, sa::CK_IAM_LEAF);
-        const float bound = n < L ? 3.4e38f : best[L - 1];
-        const bool in = active && hit_box_before(o, s, lo, hi, bound);
-        if (tri >= 0) {
-            if (in) {
-                const float4 a = __ldg(&sc.tris[3 * tri]);
-                const float4 b = __ldg(&sc.tris[3 * tri + 1]);
-                const float4 c = __ldg(&sc.tris[3 * tri + 2]);
-                float t;
-                if (hit_tri_t<KZ>(o, a, b, c, s.Sx, s.Sy, s.Sz, kSourceTmin, &t) && t < bound) {
-                    int k = n < L ? n++ : L - 1;
-                    while (k > 0 && best[k - 1] > t) { best[k] = best[k - 1]; --k; }
-                    best[k] = t;
-                }
-            }
-            i = esc;
-        } else {
-            i = __any_sync(kFull, in) ? i + 1 : esc;
-        }
-    }
-    return n;
 }
 
 struct Grid {
@@ -162,23 +120,122 @@ __device__ void draw_segment(const Grid& g, float px, float py, float qx, float 
     }
 }
 
-// A CTA finds the sources of its 128 cells, 32 in a patch of 8 x 4 per warp, and lists them;
-// then its threads draw them, one line per thread whichever cell it comes from: most cells
-// are lit or have two sources where their neighbours have four, and a warp that drew its own
-// cells' sources waited for the longest list.  Bound by issue: the pieces of the lines, one
-// after the other (12 CTAs per SM: 2.17 ms the call, 2.21 at 10, 2.24 at 14).  613 x 457
-// cells x 481 steps: 2.76 ms with each thread's own sources, 2.17; 1024^2 9.84 -> 7.79; 400 x
-// 300 on 21 December, when most cells have all four, 3.23 -> 3.13.
+// A walk of the BVH for the sources of one or two ends of blocks (end 2 b: block b's first
+// step, 2 b + 1: its last): a block's last step and the next one's first are neighbours
+// within a day, and their rays share a walk.
+struct IamWalk {
+    int step, n;          // the walk's steps: step, and step + 1 where n is 2; none where n is 0
+    int end;              // the first step's end; a second step's is the next
+};
+
+// The walk of every end of the n blocks (none for an end that shares the one before).
+__global__ void k_iam_walks(const StepConst* __restrict__ steps, const BlockConst* __restrict__ blocks, int n,
+                            IamWalk* __restrict__ walks, RunLight* __restrict__ runs) {
+    const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x), b = i >> 1;
+    if (b >= n) return;
+    auto joins = [&](int q) {       // block q's first step shares the walk of the one before
+        return q > 0 && q < n && !blocks[q].new_day && blocks[q - 1].j0 + blocks[q - 1].K == blocks[q].j0;
+    };
+    const int j = i & 1 ? blocks[b].j0 + blocks[b].K - 1 : blocks[b].j0;
+    const int m = i & 1 ? (joins(b + 1) ? 2 : 1) : (joins(b) ? 0 : 1);
+    walks[i] = IamWalk{j, m, i};
+    if (m == 0) return;
+    const int k = j + m - 1;
+    const LightBasis L = light_basis(steps[k], steps[j], steps[k]);
+    LightStep ls = light_drift(L, steps[j]);         // (the bounds on d . n are not used)
+    light_merge(ls, light_drift(L, steps[k]));
+    light_finish(L, ls, &runs[i]);
+    runs[i].k0 = 0;
+    runs[i].kn = m;
+    runs[i].j0 = j;
+    runs[i].blk = b;
+}
+
+// Tests n <= 32 queued pairs of a warp, one per lane, and puts the hits into their cells'
+// lists: the distance's bits order as the distance does, and what a slot's minimum pushes
+// out goes on to the next slot, so the L slots end with the L least in order, whichever
+// order the hits came in.
+template <int KZ, class Smem>
+__device__ __forceinline__ void drain_sources(Smem& sm, unsigned (*near)[kTileThreads], const unsigned short* q, int n,
+                                              const StepConst& s, int L) {
+    const int lane = threadIdx.x & 31;
+    if (lane >= n) return;
+    const unsigned e = q[lane];
+    const int who = (int)(e >> 8), i = (int)(e & 0xffu);
+    const float4 p = sm.o[who];
+    float t;
+    if (!hit_tri_t<KZ>(make_float3(p.x, p.y, p.z), sm.tri[3 * i], sm.tri[3 * i + 1], sm.tri[3 * i + 2], s.Sx, s.Sy, s.Sz,
+                       kSourceTmin, &t)) return;
+    unsigned v = __float_as_uint(t);
+    for (int l = 0; l < L && v != 0xffffffffu; ++l) v = max(v, atomicMin(&near[l][who], v));
+}
+
+constexpr int kIamChunk = 64;
+constexpr int kPatchX = 16, kPatchY = 8;       // a group's cells: 8 x 4 per warp
+
+// The sources of a group of 128 cells at the ends of blocks of one walk: the CTA walks the BVH
+// once for all of its rays (walk_group) and tests the pairs that their common direction lets
+// through.  src [2 blocks][L][R]: distances, ascending, 0 past the last.  Bound by the latency
+// of the walk's steps.  613 x 457 cells, 18 ends: 403 us, 630 with a walk per end, some 800
+// with a node-list walk per 32 cells and end, whose lanes tested a ray each.
+__global__ void __launch_bounds__(kTileThreads, 8)
+k_iam_sources(DevScene sc, Grid g, const StepConst* __restrict__ steps, const IamWalk* __restrict__ walks,
+              const RunLight* __restrict__ runs, int L, float* __restrict__ src) {
+    __shared__ LightSmem<kIamChunk> sm;
+    __shared__ GroupSmem<kIamChunk, 512> gs;
+    __shared__ unsigned near[2][kMaxLevels][kTileThreads];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int groups_x = (g.nx + kPatchX - 1) / kPatchX;
+    const int gy = (int)(blockIdx.x / (unsigned)groups_x), gx = (int)(blockIdx.x - (unsigned)gy * (unsigned)groups_x);
+    const int ix = gx * kPatchX + (warp & 1) * 8 + (lane & 7), iy = gy * kPatchY + (warp >> 1) * 4 + (lane >> 3);
+    const bool active = ix < g.nx && iy < g.ny;
+    const RunLight& rl = runs[blockIdx.y];
+    const IamWalk walk = walks[blockIdx.y];
+    if (walk.n == 0) return;
+    const float4 p = make_float4(__fadd_rn(g.x0, __fmul_rn(__fadd_rn((float)ix, 0.5f), g.dx)),
+                                 __fadd_rn(g.y0, __fmul_rn(__fadd_rn((float)iy, 0.5f), g.dx)), 0.f, 0.f);
+    sm.o[tid] = p;
+    sm.m[tid] = 0u;
+    for (int h = 0; h < walk.n; ++h)
+        for (int l = 0; l < L; ++l) near[h][l][tid] = 0xffffffffu;
+    unsigned long long n_box = 0;
+    walk_group<false>(sm, gs, sc, rl, active, p, [](int) { return 1u; }, n_box, [&](int nt, float la, float lb) {
+        light_pass<false>(sm, rl, nt, active, p, la, lb, 1u, [&](const unsigned short* q, int n) {
+            for (int h = 0; h < walk.n; ++h) {
+                const StepConst& s = steps[walk.step + h];
+                if (s.kz == 2) drain_sources<2>(sm, near[h], q, n, s, L);
+                else if (s.kz == 0) drain_sources<0>(sm, near[h], q, n, s, L);
+                else drain_sources<1>(sm, near[h], q, n, s, L);
+            }
+        });
+        return false;
+    });
+    if (!active) return;
+    const long long R = (long long)g.nx * g.ny;
+    for (int h = 0; h < walk.n; ++h) {
+        float* out = src + (long long)(walk.end + h) * L * R + (long long)iy * g.nx + ix;
+        for (int l = 0; l < L; ++l) {
+            const unsigned v = near[h][l][tid];
+            out[(long long)l * R] = v == 0xffffffffu ? 0.f : __uint_as_float(v);
+        }
+    }
+}
+
+// A CTA lists the sources of its 128 cells, 32 in a patch of 8 x 4 per warp; then its threads
+// draw them, one line per thread whichever cell it comes from: most cells are lit or have two
+// sources where their neighbours have four, and a warp that drew its own cells' sources
+// waited for the longest list.  Bound by issue: the pieces of the lines, one after the other.
 template <class Cell>
 __global__ void __launch_bounds__(32 * kWarps, 12)
-k_iam_draw(DevScene sc, Grid g, const StepConst* __restrict__ steps, const BlockConst* __restrict__ blocks,
-           int L, unsigned long long* __restrict__ all_masks) {
+k_iam_draw(Grid g, const StepConst* __restrict__ steps, const BlockConst* __restrict__ blocks,
+           int L, const float* __restrict__ src, unsigned long long* __restrict__ all_masks) {
     __shared__ float s_t[32 * kWarps * kMaxLevels * 2];               // the sources' distances,
     __shared__ unsigned short s_from[32 * kWarps * kMaxLevels * 2];   // thread | direction << 15
     __shared__ float2 s_o[32 * kWarps], s_u[kMaxBlock];
     __shared__ int s_n;
     const int tid = threadIdx.x, lane = tid & 31;
     const int j0 = blocks[blockIdx.y].j0, K = blocks[blockIdx.y].K;
+    const long long R = (long long)g.nx * g.ny;
     const long long warp_id = (long long)blockIdx.x * kWarps + (tid >> 5);
     const int tiles_x = (g.nx + 7) >> 3;
     const long long ty = warp_id / tiles_x;
@@ -186,30 +243,23 @@ k_iam_draw(DevScene sc, Grid g, const StepConst* __restrict__ steps, const Block
     const int ix = tx * 8 + (lane & 7);
     const long long iy = ty * 4 + (lane >> 3);
     const bool active = ix < g.nx && iy < g.ny;
-    float3 o;
-    o.x = __fadd_rn(g.x0, __fmul_rn(__fadd_rn((float)ix, 0.5f), g.dx));
-    o.y = __fadd_rn(g.y0, __fmul_rn(__fadd_rn((float)iy, 0.5f), g.dx));
-    o.z = 0.f;
-    s_o[tid] = make_float2(o.x, o.y);
+    s_o[tid] = make_float2(__fadd_rn(g.x0, __fmul_rn(__fadd_rn((float)ix, 0.5f), g.dx)),
+                           __fadd_rn(g.y0, __fmul_rn(__fadd_rn((float)iy, 0.5f), g.dx)));
     if (tid < K) s_u[tid] = make_float2(steps[j0 + tid].ux, steps[j0 + tid].uy);
     if (tid == 0) s_n = 0;
     __syncthreads();
     for (int dir = 0; dir < 2; ++dir) {
-        const StepConst s = steps[dir == 0 ? j0 : j0 + K - 1];
-        float best[kMaxLevels];
-        int n;
-        if (s.kz == 2) n = nearest_sources<2>(sc, o, s, active, L, best);
-        else if (s.kz == 0) n = nearest_sources<0>(sc, o, s, active, L, best);
-        else n = nearest_sources<1>(sc, o, s, active, L, best);
         // level by level, so that neighbours' lines of one source surface stay together
+        const float* in = src + ((long long)blockIdx.y * 2 + dir) * L * R + iy * g.nx + ix;
         for (int l = 0; l < L; ++l) {
-            const unsigned has = __ballot_sync(kFull, l < n);
+            const float t = active ? __ldcs(&in[(long long)l * R]) : 0.f;
+            const unsigned has = __ballot_sync(kFull, t > 0.f);
             if (!has) break;
             int at = 0;
             if (lane == 0) at = atomicAdd(&s_n, __popc(has));
             at = __shfl_sync(kFull, at, 0) + __popc(has & ((1u << lane) - 1u));
-            if (l < n) {
-                s_t[at] = best[l];
+            if (t > 0.f) {
+                s_t[at] = t;
                 s_from[at] = (unsigned short)(tid | (dir << 15));
             }
         }
@@ -267,12 +317,16 @@ cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     const long long R = (long long)rc.nx * rc.ny;
     if (R == 0) return cudaSuccess;
     if (L < 1 || L > kMaxLevels) return cudaErrorInvalidValue;
-    // the blocks go in one launch, as many as 1 GiB of masks holds
-    const int chunk = (int)std::max(1ll, std::min({(long long)sun.n_blocks, 65535ll, (1ll << 30) / (8ll * R)}));
-    const size_t words = (size_t)R * chunk;
+    // the blocks go in one launch, as many as 1 GiB of masks and sources holds
+    const int chunk = (int)std::max(1ll, std::min({(long long)sun.n_blocks, 32767ll, (1ll << 30) / ((8ll + 8ll * L) * R)}));
     unsigned long long* masks = nullptr;
-    cudaError_t e = sa::scratch_alloc(&masks, sizeof(unsigned long long) * words, st);
-    if (e != cudaSuccess) return e;
+    float* src = nullptr;
+    RunLight* runs = nullptr;
+    IamWalk* d_walks = nullptr;
+    cudaError_t e = sa::scratch_alloc(&masks, sizeof(unsigned long long) * (size_t)R * chunk, st);
+    if (e == cudaSuccess) e = sa::scratch_alloc(&src, sizeof(float) * 2 * (size_t)L * (size_t)R * chunk, st);
+    if (e == cudaSuccess) e = sa::scratch_alloc(&runs, sizeof(RunLight) * 2 * (size_t)chunk, st);
+    if (e == cudaSuccess) e = sa::scratch_alloc(&d_walks, sizeof(IamWalk) * 2 * (size_t)chunk, st);
     Grid g{rc.x0, rc.y0, rc.dx, rc.nx, rc.ny};
     const long long warps = (long long)((rc.nx + 7) / 8) * ((rc.ny + 3) / 4);
     const unsigned ctas = (unsigned)((warps + kWarps - 1) / kWarps);
@@ -282,16 +336,21 @@ cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
         if (e != cudaSuccess) break;
         {
             KernelTimer kt(KT_IAM, st);
+            const dim3 groups((unsigned)((rc.nx + kPatchX - 1) / kPatchX) * (unsigned)((rc.ny + kPatchY - 1) / kPatchY),
+                              2u * (unsigned)nbc);
+            k_iam_walks<<<(2 * nbc + 63) / 64, 64, 0, st>>>(sun.steps, sun.blocks + b0, nbc, d_walks, runs);
+            k_iam_sources<<<groups, kTileThreads, 0, st>>>(sc, g, sun.steps, d_walks, runs, L, src);
             const dim3 grid(ctas, (unsigned)nbc);
-            if (R < (1ll << 31)) k_iam_draw<unsigned><<<grid, 32 * kWarps, 0, st>>>(sc, g, sun.steps, sun.blocks + b0, L, masks);
-            else k_iam_draw<long long><<<grid, 32 * kWarps, 0, st>>>(sc, g, sun.steps, sun.blocks + b0, L, masks);
+            if (R < (1ll << 31)) k_iam_draw<unsigned><<<grid, 32 * kWarps, 0, st>>>(g, sun.steps, sun.blocks + b0, L, src, masks);
+            else k_iam_draw<long long><<<grid, 32 * kWarps, 0, st>>>(g, sun.steps, sun.blocks + b0, L, src, masks);
         }
         k_iam_fold<<<(unsigned)((R + 255) / 256), 256, 0, st>>>(R, sun.blocks + b0, nbc, masks, out, b0 == 0,
                                                                b0 + nbc == sun.n_blocks);
         e = cudaGetLastError();
     }
-    cudaError_t e2 = cudaFreeAsync(masks, st);
-    return e != cudaSuccess ? e : e2;
+    for (void* p : {(void*)masks, (void*)src, (void*)runs, (void*)d_walks})
+        if (p) cudaFreeAsync(p, st);
+    return e;
 }
 
 }  // namespace sa

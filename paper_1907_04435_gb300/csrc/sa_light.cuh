@@ -98,18 +98,24 @@ __host__ __device__ inline LightBasis light_basis(const StepConst& mid, const St
 }
 
 // One step's share of a run's bounds: its drift per metre of height in light space, and the
-// |coefficients| of d - d_m in the FP32 basis (Cramer's rule).
+// |coefficients| of d - d_m in the FP32 basis (Cramer's rule); light_drift: the drift alone.
 struct LightStep {
     double da_lo, da_hi, db_lo, db_hi, mx[3];
 };
 
-__host__ __device__ inline LightStep light_step(const LightBasis& L, const StepConst& s) {
+__host__ __device__ inline LightStep light_drift(const LightBasis& L, const StepConst& s) {
     LightStep r;
     const double dz = s.dz > 1e-12f ? (double)s.dz : 1e-12;
     const double da = (L.e1[0] * s.dx + L.e1[1] * s.dy + L.e1[2] * s.dz) / dz;
     const double db = (L.e2[0] * s.dx + L.e2[1] * s.dy + L.e2[2] * s.dz) / dz;
     r.da_lo = fmin(0.0, da); r.da_hi = fmax(0.0, da);
     r.db_lo = fmin(0.0, db); r.db_hi = fmax(0.0, db);
+    r.mx[0] = r.mx[1] = r.mx[2] = 0.0;
+    return r;
+}
+
+__host__ __device__ inline LightStep light_step(const LightBasis& L, const StepConst& s) {
+    LightStep r = light_drift(L, s);
     const double M[3][3] = {{L.t[0], L.b[0], L.n[0]}, {L.t[1], L.b[1], L.n[1]}, {L.t[2], L.b[2], L.n[2]}};
     const double D = light_det(M);
     const double dl[3] = {(double)s.dx - L.dm[0], (double)s.dy - L.dm[1], (double)s.dz - L.dm[2]};
@@ -326,7 +332,9 @@ __device__ __forceinline__ void drain_pairs(Smem& sm, const unsigned short* q, i
 // at once, the other pairs are culled per lane, queued, and tested 32 at a time.
 // drain(queue, n) tests n <= 32 pairs, receiver slot << 8 | triangle each, one per lane.  A
 // receiver whose sm.m has come to `full` needs no more, and the pass ends when none does.
-template <class Smem, class Drain>
+// SIDE: also drops the pairs whose receiver lies on the side of the triangle's plane that no ray
+// leaves toward it, by the Pluecker test's own distance check (p.w: t_min).
+template <bool SIDE = true, class Smem, class Drain>
 __device__ __forceinline__ void light_pass(Smem& sm, const RunLight& rl, int nt, bool live, const float4& p,
                                            float la, float lb, unsigned full, Drain drain) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -380,16 +388,18 @@ __device__ __forceinline__ void light_pass(Smem& sm, const RunLight& rl, int nt,
                 const float4 e = sm.edge[q3][t];
                 pass &= fmaf(h, e.w, fmaf(e.x, la, fmaf(e.y, lb, e.z))) >= 0.f;
             }
-            // the receiver on the side of the triangle's plane that no ray of the run
-            // leaves toward it: the step test's own distance check (a . n against
-            // t_min d . n, same roundings) fails at every step
-            const float4 v0 = sm.tri[3 * t];
-            const float4 nv = sm.n[t];
-            const float aon = fmaf(nv.z, __fsub_rn(v0.z, p.z),
-                                   fmaf(nv.y, __fsub_rn(v0.y, p.y), __fmul_rn(nv.x, __fsub_rn(v0.x, p.x))));
-            const float2 nd = make_float2(sm.tri[3 * t + 1].w, sm.tri[3 * t + 2].w);
-            if (nd.x > 0.f) pass &= aon > __fmul_rn(p.w, nd.x);
-            else if (nd.y < 0.f) pass &= aon < __fmul_rn(p.w, nd.y);
+            if (SIDE) {
+                // the receiver on the side of the triangle's plane that no ray of the run
+                // leaves toward it: the step test's own distance check (a . n against
+                // t_min d . n, same roundings) fails at every step
+                const float4 v0 = sm.tri[3 * t];
+                const float4 nv = sm.n[t];
+                const float aon = fmaf(nv.z, __fsub_rn(v0.z, p.z),
+                                       fmaf(nv.y, __fsub_rn(v0.y, p.y), __fmul_rn(nv.x, __fsub_rn(v0.x, p.x))));
+                const float2 nd = make_float2(sm.tri[3 * t + 1].w, sm.tri[3 * t + 2].w);
+                if (nd.x > 0.f) pass &= aon > __fmul_rn(p.w, nd.x);
+                else if (nd.y < 0.f) pass &= aon < __fmul_rn(p.w, nd.y);
+            }
         }
         const unsigned bal = __ballot_sync(0xffffffffu, pass);
         if (pass) q[n + __popc(bal & ((1u << lane) - 1u))] =
