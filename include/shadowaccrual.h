@@ -124,7 +124,7 @@ int32_t sa_get_option(int32_t key);
 #define SA_KERNEL_IAM 4          /* inverse accrual map line drawing (Sec. 5) */
 #define SA_KERNEL_GRAPH 5        /* direction graph: edge run summaries and day-path reduce (Sec. 6) */
 #define SA_KERNEL_RASTER_BIN 6   /* triangle binning of the ground raster (count and fill passes) */
-#define SA_KERNEL_CONTRIB 7      /* building contribution: fan traversal of the shadowed steps (Sec. 7.2) */
+#define SA_KERNEL_CONTRIB 7      /* building contribution: grouped walks of the shadowed steps (Sec. 7.2) */
 #define SA_KERNEL_CLASSES 8
 
 /* Collect the timed launches recorded since the last collection: waits for their events,
@@ -315,7 +315,10 @@ typedef struct sa_batch sa_batch;
  * and the base counts of the whole grid are computed per interval.  A work item (interval,
  * variant, tile) is rastered only if the shadow of a removed building or of a tower, swept
  * over the interval's sun directions, can reach the tile; the others take the base counts
- * (their impact is zero).  with_impact is kept for compatibility and may be 0 or 1.
+ * (their impact is zero).  The base city's step masks, 8 bytes per cell and block of the
+ * intervals, stay on the device with the batch while they take at most a quarter of its
+ * free memory at creation; an item is then a single block of a tile, and only what its
+ * variant changes there is rastered.  with_impact is kept for compatibility and may be 0 or 1.
  * The scene, grid and suns must outlive the batch.  Synchronises `stream`.
  * Errors: SA_ERR_INVALID_ARG (offsets, regions outside the grid, bad towers),
  * SA_ERR_UNSUPPORTED (point receivers, geometry below z = 0), SA_ERR_OOM, SA_ERR_CUDA. */
@@ -345,7 +348,8 @@ sa_status sa_batch_work_counters(sa_batch* b, uint64_t* counters, void* stream);
 /* Work counters of one accumulation (diagnostics for roofline accounting): runs `method`
  * with counting enabled and writes counters uint64 [4] dev.
  *   trace methods: [0] ray/fan-versus-box tests, [1] ray-versus-triangle tests per
- *   receiver lane.
+ *   receiver lane (SA_ACCRUAL_TRACE by groups: [0] node tests of a group's query, [1] step
+ *   tests of its receiver-triangle pairs).
  *   raster methods (ground grids): [0] work units (triangle, run of steps) that reached
  *   the tile's cells, [1] cells their row spans enumerated, [2] cell set-ups (cells not
  *   already shadowed at every step of the unit), [3] cell-step coverage tests.
@@ -412,8 +416,9 @@ sa_status sa_direction_graph(const float* dirs, int32_t S, const int32_t* day_st
  * sa_accumulate (SA_ACCUMULATE_INTO is not offered); *n_edges (host, nullable) receives
  * the number of maps computed, against sa_sun_info's n_blocks for the exact result.  With
  * a bin_deg small enough that no two blocks share an edge the result is sa_accumulate's.
- * Scratch: 4 bytes per receiver and edge, plus the step masks of at most 4 GiB of edges
- * at a time.  Synchronises `stream` once per chunk of edges.  Errors: as sa_accumulate,
+ * Scratch: 4 bytes per receiver and edge, plus, but for the accrual raster of a ground grid
+ * (which leaves the edges' runs itself), the step masks of at most 4 GiB of edges at a
+ * time.  Synchronises `stream` once per chunk of edges.  Errors: as sa_accumulate,
  * SA_ERR_INVALID_ARG (bin_deg outside (0, 90]). */
 sa_status sa_accumulate_graph(const sa_scene* scene, const sa_receivers* recv, const sa_sun* sun,
                               sa_method method, int32_t iam_levels, float bin_deg, float step_minutes,
@@ -477,9 +482,9 @@ sa_status sa_shadow_score(const sa_receivers* grid, const int32_t* steps, int32_
  * The shadowed steps come from the ground accrual raster (as SA_ACCRUAL_SAM computes
  * them); the call keeps its per-step masks, 8 bytes per cell and block of steps, and
  * rejects with SA_ERR_INVALID_ARG a grid and sun table whose masks exceed 4 GiB (split the
- * interval).  The buildings are found by one traversal per cell and run of <= 32 steps,
- * whose query is the fan of the run's rays (as SA_ACCRUAL_TRACE), testing every triangle
- * in the fan against the cell's shadowed steps with the exact ray test.  Synchronises
+ * interval).  The buildings are found by one traversal per group of 128 cells and run of
+ * <= 16 steps, whose query is the fan of the run's rays (as SA_ACCRUAL_TRACE), testing every
+ * triangle in it against the cells' shadowed steps with the exact ray test.  Synchronises
  * `stream`.  Errors: SA_ERR_INVALID_ARG (NULL, not a grid, n < 3), SA_ERR_DEGENERATE
  * (non-finite vertex), SA_ERR_UNSUPPORTED (geometry below z = 0, as for the raster
  * methods; a ray meeting more than 64 buildings, above), SA_ERR_OOM, SA_ERR_CUDA. */

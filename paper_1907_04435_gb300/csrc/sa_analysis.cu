@@ -359,10 +359,11 @@ k_building_contribution(ContribArgs a) {
         }
         if (mine && !ovf) {
             for (int e = 0; e < kCastList && s.cb[e][tid] >= 0; ++e) {
-                const unsigned met = s.cm[e][tid];
-                atomicAdd(&a.cast_cnt[s.cb[e][tid]], (unsigned long long)__popc(met));
-                if (level > 0)
-                    for (unsigned w = met; w; w &= w - 1u) ++s.key[__ffs(w) - 1][tid];
+                unsigned met = s.cm[e][tid];
+                if (level > 0)                    // a ray's first kRayMost buildings are credited
+                    for (unsigned w = met; w; w &= w - 1u)
+                        if (s.key[__ffs(w) - 1][tid]++ >= kRayMost) met &= ~(w & (0u - w));
+                if (met) atomicAdd(&a.cast_cnt[s.cb[e][tid]], (unsigned long long)__popc(met));
             }
         }
         if (__syncthreads_or(ovf)) {          // split the pass

@@ -6,8 +6,11 @@
 // creation it bins the base city's triangles once per block of every interval (the bins
 // do not depend on the variant), computes the base counts over the whole grid, and lists
 // the work items (interval, variant, tile of the region).  sa_batch_run then executes a
-// CUDA graph holding one persistent launch that drains the work queue: each item rasters
-// its tile with the base bins minus the removed buildings plus the variant's towers.
+// CUDA graph holding one persistent launch that drains the work queue.  With the base city's
+// step masks (kept while they take at most a quarter of the free memory) an item is a block
+// of a tile that a changed building's shadow reaches, and only the bits it can change are
+// decided again; without them an item rasters its tile over all blocks with the base bins
+// minus the removed buildings plus the variant's towers.
 #include <string.h>
 
 #include <algorithm>

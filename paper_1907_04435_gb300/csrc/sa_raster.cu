@@ -10,6 +10,8 @@
 // receivers themselves, as one bit per step: no texel resampling, no aliasing, no bias.
 //
 // Per block of <= 64 steps:
+//   k_reach           with many (triangle, block) pairs, lists the triangles that can reach
+//                     the grid at some step
 //   k_bin             one pass over the triangles bins each into the 32 x 32-cell tiles its
 //                     projection can reach during the block (the triangle swept along the
 //                     block's slope box)
@@ -21,6 +23,8 @@
 //   k_raster          one CTA per tile, its blocks in series, the reduction fused (the raster
 //                     in fixed scratch, and the per-step raster of a large grid)
 // With one step per block the same kernels form the per-step shadow raster baseline.
+// Batched scenarios: k_batch_base and k_batch_delta change the base city's masks where a
+// variant does; k_batch rasters every block of an affected tile (no room for the masks).
 //
 // Coverage is decided with edge functions evaluated from canonically ordered endpoints,
 // so an edge shared by two projected triangles yields exactly negated values in the two

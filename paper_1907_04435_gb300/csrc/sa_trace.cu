@@ -249,7 +249,7 @@ __device__ __forceinline__ Receiver load_group_receiver(const DevRecv& rc, long 
 // a group shadowed at every step stops.  Bound by issue in the pair culls and tests.  The
 // traversal by one warp's 32 fans (k_accrual_fan, 80 instructions a node for every warp of
 // receivers and block in series) took 3.43 ms on 517 x 389 cells x 481 steps, 2.35 ms as
-// items; the grouped one 0.83 ms.  1024^2 cells: 13.8 -> 4.03 ms; 1M facade points: 16.5 ->
+// items; the grouped one 0.76 ms.  1024^2 cells: 13.8 -> 4.03 ms; 1M facade points: 16.5 ->
 // 6.7 ms.
 template <bool COUNT>
 __global__ void __launch_bounds__(kTileThreads, 8)
