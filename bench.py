@@ -463,11 +463,11 @@ OPS_BOX, OPS_TRI = 12, 25
 # profile summary gives the command).  A figure is reported only while the kernel's
 # sources hash to the value they had when it was captured; otherwise traffic is null.
 TRAFFIC = {
-    "k_raster": {"bytes": 7002880 + 14976768, "workload": "district",
-                 "sources": ("sa_raster.cu", "sa_internal.cuh"), "sha256_16": "fbe5e1cde17ff661"},
-    "k_sam_tile": {"bytes": 155689216 + 26193152, "workload": "district",
-                   "sources": ("sa_sam_points.cu", "sa_internal.cuh", "sa_handles.cuh"),
-                   "sha256_16": "e9ff7eeb4764c3a4"},
+    "k_raster": {"bytes": 8668160 + 94879744, "workload": "district",
+                 "sources": ("sa_raster.cu", "sa_internal.cuh"), "sha256_16": "6d6679ad3b5c3124"},
+    "k_sam_tile": {"bytes": 156936448 + 27335168, "workload": "district",
+                   "sources": ("sa_sam_points.cu", "sa_light.cuh", "sa_internal.cuh", "sa_handles.cuh"),
+                   "sha256_16": "c1f1c7fda39c47c2"},
 }
 
 
@@ -507,7 +507,7 @@ def roofline(B, scene, grid, fac, sun, ktimes, steps, workload):
                      "ops_per_launch": ops_launch, "work": work}
 
     c = B.sa_work_counters(scene, grid, sun, "accrual_sam")
-    entry("k_raster", "k_raster (ground accrual raster)", c[2] * OPS_CELL + c[3] * OPS_TEST,
+    entry("k_raster", "k_raster_items (ground accrual raster)", c[2] * OPS_CELL + c[3] * OPS_TEST,
           "raster", {"cell_setups": c[2], "cell_step_tests": c[3],
                      "ops_per_setup": OPS_CELL, "ops_per_test": OPS_TEST,
                      "work_units": c[0], "cells_enumerated": c[1]})
