@@ -474,7 +474,9 @@ __device__ __noinline__ bool solve_fp64(const FootprintSet& fs, const float* hei
 // slack at the root and at the shadowed end.  The root itself, and its derivative with respect to h, are FP64 from the two
 // constraints' exact coefficients.  FP64 runs at 1/64 of the FP32 rate here, and the search
 // in it kept that pipe 83 % busy (park of 600k cells, 200 buildings: 12.2 ms for all flips,
-// now 1.06, and 0.67 for the 6 % that are left to it).
+// now 1.06, and 0.46 for the 5 % that are left to it; 0.67
+// and 9 % with the pair's middle alone as the point inside at the shadowed end, and a park
+// on 16 December 1.29 -> 0.41).
 // Returns 1 with the root, 0 when undecided.  *dbe_dh: derivative of a roof-edge flip.
 __device__ __forceinline__ int solve_fast(const FootprintSet& fs, int fa, int v, float h, float px, float py,
                                           const ArcConst& arc, bool c0, double* be_star, double* dbe_dh) {
@@ -586,16 +588,25 @@ __device__ __forceinline__ int solve_fast(const FootprintSet& fs, int fa, int v,
     }
     // at be: the pair's denominators above a hundredth of their edge (z then errs by 2e-5 of
     // reach + z at the most), its mean height within the prism, every other constraint slack
-    // there.  At the root the two bounds meet, so the others hold around it; at the shadowed
-    // end the pair is open (the root lies between it and the lit end), so some height between
-    // its bounds is inside.
+    // there.  The two bounds meet at the root and the others hold around it, so the arc
+    // leaves the prism there toward the lit end.  At the shadowed end any height inside will
+    // do: the pair's middle (the pair is open there, since the root lies between it and the
+    // lit end), or, where another edge is nearer there, the middle of all constraints' bounds
+    // with every constraint slack.
     auto holds = [&](float at) {
         const float dz = fmaf(at, ez, az), denl = fmaf(at, E1l, E0l), denu = fmaf(at, E1u, E0u);
         const float zl = __fdividef(-Al * dz, denl);
         const float z = 0.5f * (zl + (pu < 0 ? h : __fdividef(-Au * dz, denu)));
         return denl > 100.f * Tl && denu < -100.f * Tu && z > zm && (pu < 0 || z < h - zm) && slack(at, z, pl, pu);
     };
-    const bool ok = fmaf(lit, E1l, E0l) > 100.f * Tl && fmaf(lit, E1u, E0u) < -100.f * Tu && holds(rf) && holds(sh);
+    auto inside = [&](float at) {
+        float l, u;
+        int i, j;
+        bounds(at, l, u, i, j);
+        const float z = 0.5f * (l + u);
+        return z > zm && z < h - zm && slack(at, z, -1, -1);
+    };
+    const bool ok = fmaf(lit, E1l, E0l) > 100.f * Tl && fmaf(lit, E1u, E0u) < -100.f * Tu && holds(rf) && (holds(sh) || inside(sh));
     if (!ok) return 0;
     *be_star = r;
     return 1;
