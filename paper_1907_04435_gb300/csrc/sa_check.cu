@@ -45,7 +45,8 @@ const char* check_site_name(int site) {
         "light-space map: binned triangle", "light-space map: binned receiver",
         "light-space map: receiver permutation", "light-space map: receiver mask",
         "building contribution: building id", "building contribution: listed cell",
-        "height adjoint: leaf triangle", "height adjoint: escape link"};
+        "height adjoint: leaf triangle", "height adjoint: escape link",
+        "grouped walk: leaf triangle", "grouped walk: child nodes", "grouped walk: stack"};
     return site >= 0 && site < CK_SITES ? names[site] : "unknown";
 }
 

@@ -19,14 +19,15 @@ namespace sa {
 // BVH leaf's triangle, an escape link, a binned triangle or receiver, a permutation
 // entry, a tile cell) before using it.  The first index out of range is recorded in a
 // device word of its translation unit -- the site, the index and its bound -- and replaced
-// by an index in range (an escape link by the end of the list), so that no access leaves
-// its buffer and no loop runs on; the public calls then return SA_ERR_INTERNAL.  Without
-// the flag the checks compile to nothing.
+// by an index in range (an escape link by the end of the list; a grouped walk drops children
+// that are out of place or find no room on its stack), so that no access leaves its buffer
+// and no loop runs on; the public calls then return SA_ERR_INTERNAL.  Without the flag the
+// checks compile to nothing.
 enum CheckSite {
     CK_NONE = 0, CK_TRACE_LEAF, CK_TRACE_ESCAPE, CK_RASTER_BIN, CK_RASTER_CELL, CK_BIN_SLOT,
     CK_POINTS_TRI, CK_POINTS_RECV, CK_POINTS_PERM, CK_POINTS_MASK,
     CK_CONTRIB_BUILDING, CK_CONTRIB_CELL, CK_ADJ_LEAF,
-    CK_ADJ_ESCAPE, CK_SITES
+    CK_ADJ_ESCAPE, CK_WALK_LEAF, CK_WALK_CHILD, CK_WALK_STACK, CK_SITES
 };
 const char* check_site_name(int site);
 // Reader of one translation unit's word: copies [site, index, bound] into w and, if a
@@ -41,21 +42,33 @@ cudaError_t read_check_words(unsigned long long* w);
 #ifdef SA_CHECKED
 namespace {
 __device__ unsigned long long g_sa_check[3];
-__device__ __forceinline__ long long sa_checked_index(long long i, long long n, int site) {
-    if (i >= 0 && i < n) return i;
+// true if lo < i < n; the first i that is not is recorded
+__device__ __forceinline__ bool sa_check_between(long long lo, long long i, long long n, int site) {
+    if (i > lo && i < n) return true;
     if (atomicCAS(&g_sa_check[0], 0ull, (unsigned long long)site) == 0ull) {
         g_sa_check[1] = (unsigned long long)i;
         g_sa_check[2] = (unsigned long long)n;
     }
-    return 0;
+    return false;
+}
+__device__ __forceinline__ long long sa_checked_index(long long i, long long n, int site) {
+    return sa_check_between(-1, i, n, site) ? i : 0;
 }
 __device__ __forceinline__ int sa_checked_escape(int esc, int i, int n, int site) {
     if (esc > i && esc <= n) return esc;
-    if (atomicCAS(&g_sa_check[0], 0ull, (unsigned long long)site) == 0ull) {
-        g_sa_check[1] = (unsigned long long)(long long)esc;
-        g_sa_check[2] = (unsigned long long)(long long)n;
-    }
+    sa_check_between(i, esc, n, site);
     return n;
+}
+// Inner node i of a depth-first list of n nodes has the subtree [i, end), end its escape link;
+// its left child follows it, and the right one, at the left one's escape link, lies in the
+// subtree too, as does its own.  Where that holds at every node, the subtrees of two
+// children never overlap: a walk reaches no node twice, whatever the links are.
+__device__ __forceinline__ bool sa_checked_children(const float4* nodes, int i, int n, int site) {
+    const int end = __float_as_int(nodes[2 * i].w);
+    if (!sa_check_between(i, end, n + 1ll, site) || !sa_check_between(i, i + 1, end, site)) return false;
+    const int right = __float_as_int(nodes[2 * (i + 1)].w);
+    if (!sa_check_between(i + 1, right, end, site)) return false;
+    return sa_check_between(right, __float_as_int(nodes[2 * right].w), end + 1ll, site);
 }
 cudaError_t sa_read_check_tu(unsigned long long* w, int reset) {
     cudaError_t e = cudaMemcpyFromSymbol(w, g_sa_check, sizeof(unsigned long long) * 3);
@@ -70,9 +83,16 @@ const int g_sa_check_registered = sa::register_check_reader(&sa_read_check_tu);
 // index i checked against [0, n); an escape link checked against (i, n]
 #define SA_CHK(i, n, site) sa_checked_index((long long)(i), (long long)(n), (int)(site))
 #define SA_ESC(esc, i, n, site) sa_checked_escape((esc), (i), (n), (int)(site))
+// node i's children are in place; entry i of a stack of n exists; a stack's count is at most n
+#define SA_CHILDREN(nodes, i, n, site) sa_checked_children((nodes), (i), (n), (int)(site))
+#define SA_ROOM(i, n, site) sa_check_between(-1, (i), (n), (int)(site))
+#define SA_AT_MOST(i, n) min((i), (n))
 #else
 #define SA_CHK(i, n, site) (i)
 #define SA_ESC(esc, i, n, site) (esc)
+#define SA_CHILDREN(nodes, i, n, site) true
+#define SA_ROOM(i, n, site) true
+#define SA_AT_MOST(i, n) (i)
 #endif
 // a node's triangle: -1 for an inner node, else checked against [0, T)
 #define SA_LEAF(tri, T, site) ((tri) < 0 ? (tri) : (int)SA_CHK((tri), (T), (site)))

@@ -475,10 +475,11 @@ __device__ __forceinline__ void walk_group(LightSmem<CHUNK>& sm, GroupSmem<CHUNK
     light_ab(rl, ref, p.x, p.y, p.z, &la, &lb);
     while (true) {
         __syncthreads();
-        int nst = gs.nst, nleaf = gs.nleaf;
+        int nst = SA_AT_MOST(gs.nst, STACK), nleaf = gs.nleaf;
         while (nst > 0 && nleaf < CHUNK) {
-            // a wave pops up to kTileThreads nodes and pushes at most twice as many; near the
-            // stack's end it goes node by node, and the tree's depth (<= 62) fits what is left
+            // A wave of w nodes leaves at most w more, so waves end at STACK - 96; from there it
+            // goes node by node, depth first, which adds one per level of the tree.  The tree
+            // is at most 62 deep (30 bits of Morton code, then the index's), so 96 are enough.
             const int take = min(kTileThreads, min(nst, max(1, STACK - 96 - nst)));
             const int i = tid < take ? gs.stack[nst - 1 - tid] : -1;
             __syncthreads();
@@ -489,7 +490,7 @@ __device__ __forceinline__ void walk_group(LightSmem<CHUNK>& sm, GroupSmem<CHUNK
             if (i >= 0) {
                 const float4 nlo = __ldg(&sc.nodes[2 * i]);
                 const float4 nhi = __ldg(&sc.nodes[2 * i + 1]);
-                tri = SA_LEAF(__float_as_int(nhi.w), sc.T, sa::CK_TRACE_LEAF);
+                tri = SA_LEAF(__float_as_int(nhi.w), sc.T, sa::CK_WALK_LEAF);
                 if (COUNT) ++n_box;
                 const float hx = 0.5f * (nhi.x - nlo.x), hy = 0.5f * (nhi.y - nlo.y), hz = 0.5f * (nhi.z - nlo.z);
                 float a, b;
@@ -500,7 +501,7 @@ __device__ __forceinline__ void walk_group(LightSmem<CHUNK>& sm, GroupSmem<CHUNK
                 in = (rise >= 0.f) & (fmaf(rise, rl.da_hi, ga) >= a - ra) & (fmaf(-rise, rl.da_lo, -ga) <= a + ra) &
                      (fmaf(rise, rl.db_hi, gb) >= b - rb) & (fmaf(-rise, rl.db_lo, -gb) <= b + rb);
             }
-            const bool leaf = in && tri >= 0, node = in && tri < 0;
+            const bool leaf = in && tri >= 0, node = in && tri < 0 && SA_CHILDREN(sc.nodes, i, sc.n_nodes, sa::CK_WALK_CHILD);
             const unsigned bn = __ballot_sync(kAll, node), bl = __ballot_sync(kAll, leaf);
             int pn = 0, pl = 0;
             if (lane == 0) {
@@ -512,14 +513,14 @@ __device__ __forceinline__ void walk_group(LightSmem<CHUNK>& sm, GroupSmem<CHUNK
             const unsigned below = (1u << lane) - 1u;
             if (node) {
                 // in depth-first order the left child follows, and the right one follows it
-                const int left = i + 1;
-                const int right = SA_ESC(__float_as_int(__ldg(&sc.nodes[2 * left]).w), left, sc.n_nodes, sa::CK_TRACE_ESCAPE);
-                gs.stack[pn + 2 * __popc(bn & below)] = right;
-                gs.stack[pn + 2 * __popc(bn & below) + 1] = left;
+                const int left = i + 1, right = __float_as_int(__ldg(&sc.nodes[2 * left]).w);
+                const int at = pn + 2 * __popc(bn & below);
+                if (SA_ROOM(at, STACK, sa::CK_WALK_STACK)) gs.stack[at] = right;
+                if (SA_ROOM(at + 1, STACK, sa::CK_WALK_STACK)) gs.stack[at + 1] = left;
             }
             if (leaf) gs.leaf[pl + __popc(bl & below)] = tri;
             __syncthreads();
-            nst = gs.nst;
+            nst = SA_AT_MOST(gs.nst, STACK);
             nleaf = gs.nleaf;
         }
         const int nt = min(nleaf, CHUNK), left = nleaf - nt;
