@@ -317,8 +317,8 @@ typedef struct sa_batch sa_batch;
  * over the interval's sun directions, can reach the tile; the others take the base counts
  * (their impact is zero).  The base city's step masks, 8 bytes per cell and block of the
  * intervals, stay on the device with the batch while they take at most a quarter of its
- * free memory at creation; an item is then a single block of a tile, and only what its
- * variant changes there is rastered.  with_impact is kept for compatibility and may be 0 or 1.
+ * free memory at creation and the rest of the batch fits beside them; an item is then a
+ * single block of a tile, and only what its variant changes there is rastered.  with_impact is kept for compatibility and may be 0 or 1.
  * The scene, grid and suns must outlive the batch.  Synchronises `stream`.
  * Errors: SA_ERR_INVALID_ARG (offsets, regions outside the grid, bad towers),
  * SA_ERR_UNSUPPORTED (point receivers, geometry below z = 0), SA_ERR_OOM, SA_ERR_CUDA. */
@@ -373,6 +373,11 @@ sa_status sa_work_counters(const sa_scene* scene, const sa_receivers* recv, cons
  *   clearing the record), SA_OK otherwise (always SA_OK in the plain build); SA_ERR_CUDA
  *   if the device reports an error. */
 int32_t sa_checked_build(void);
+/* In the checked build, makes the n-th device allocation from now fail once as if the memory
+ * were exhausted (0: none), for tests of what the calls do then.  Returns what was left of
+ * the count set before: 0 if that allocation has failed or none was set; -1 in the plain
+ * build, which fails none. */
+int32_t sa_check_fail_alloc(int32_t n);
 sa_status sa_check_status(int32_t* site, int64_t* index, int64_t* bound);
 
 /* Statistics of the library's device memory pool (diagnostics): stats uint64 [4] host gets

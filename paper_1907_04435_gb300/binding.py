@@ -100,6 +100,8 @@ def lib():
             L.sa_block_partition.argtypes = [P, i32, i32, P, P, P]
             L.sa_scratch_stats.argtypes = [P]
             L.sa_checked_build.restype = i32
+            L.sa_check_fail_alloc.argtypes = [i32]
+            L.sa_check_fail_alloc.restype = i32
             L.sa_check_status.argtypes = [P, P, P]
             L.sa_building_contribution.argtypes = [P, P, P, P, i32, P, P, P, P]
             L.sa_sun_interpolate.argtypes = [P, i32, P, i32, i32, P]
@@ -363,6 +365,12 @@ def sa_work_counters(scene: Scene, recv: Receivers, sun: Sun, method, stream=Non
 def sa_checked_build() -> bool:
     """True when the loaded library is the bounds-checked build."""
     return bool(lib().sa_checked_build())
+
+
+def sa_check_fail_alloc(n: int) -> int:
+    """The checked build's n-th device allocation from now fails once (0: none); returns what
+    was left of the count set before, -1 in the plain build."""
+    return int(lib().sa_check_fail_alloc(int(n)))
 
 
 def sa_check_status():

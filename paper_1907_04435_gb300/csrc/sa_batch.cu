@@ -110,7 +110,7 @@ void drop_graph(sa_batch* b) {
 template <class T>
 cudaError_t dev_copy(sa_batch* b, const T* src, size_t n, T** dst) {
     *dst = nullptr;
-    cudaError_t e = cudaMalloc(dst, sizeof(T) * std::max<size_t>(n, 1));
+    cudaError_t e = sa::device_alloc(dst, sizeof(T) * std::max<size_t>(n, 1));
     if (e != cudaSuccess) return e;
     b->owned.push_back(*dst);
     if (n == 0) return cudaSuccess;
@@ -130,51 +130,16 @@ void sa_batch_destroy(sa_batch* b) {
     delete b;
 }
 
-sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const sa_variants* v,
-                          const sa_sun* const* intervals, int32_t n_intervals,
-                          int32_t with_impact, void* stream, sa_batch** out) {
-    if (!out) return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: out is NULL");
-    *out = nullptr;
-    if (!base || !grid || !v || (n_intervals > 0 && !intervals) || n_intervals < 0)
-        return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: NULL argument or bad count");
-    if (!grid->is_grid) return sa::report_error(SA_ERR_UNSUPPORTED, "sa_batch_create: receivers must be a ground grid");
-    if (base->min_z < 0.f) return sa::report_error(SA_ERR_UNSUPPORTED, "sa_batch_create: base geometry below z = 0");
-    const int V = v->n_variants;
-    if (V < 0 || (V > 0 && (!v->tower_off || !v->removed_off || !v->regions)))
-        return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: bad variant description");
-    for (int i = 0; i < n_intervals; ++i)
-        if (!intervals[i]) return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: NULL interval");
-    const int n_tow = V > 0 ? v->tower_off[V] : 0, n_rem = V > 0 ? v->removed_off[V] : 0;
-    if (V > 0 && (v->tower_off[0] != 0 || v->removed_off[0] != 0 || n_tow < 0 || n_rem < 0 ||
-                  (n_tow > 0 && !v->tower_tris) || (n_rem > 0 && !v->removed_ids)))
-        return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: bad offsets");
-    std::vector<sa::BatchVariant> hv(V);
+// Builds the batch of a checked description (hv: its variants, cells: of all regions).  On
+// failure *kept_masks says whether the base masks had been taken.
+static cudaError_t create(const sa_scene* base, const sa_receivers* grid, const sa_variants* v,
+                          const sa_sun* const* intervals, int n_intervals, std::vector<sa::BatchVariant> hv,
+                          long long cells, const std::vector<float4>& towers, bool keep_masks, cudaStream_t st,
+                          sa_batch** out, bool* kept_masks) {
+    const int V = v->n_variants, n_rem = V > 0 ? v->removed_off[V] : 0;
     const int tiles_x = (grid->nx + 31) / 32, tiles_y = (grid->ny + 31) / 32;
-    long long cells = 0;
-    for (int k = 0; k < V; ++k) {
-        const int* r = v->regions + 4 * k;
-        if (v->tower_off[k + 1] < v->tower_off[k] || v->removed_off[k + 1] < v->removed_off[k])
-            return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: offsets decrease");
-        if (r[0] < 0 || r[1] < 0 || r[2] < 0 || r[3] < 0 || r[0] + r[2] > grid->nx || r[1] + r[3] > grid->ny)
-            return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: region outside the grid");
-        hv[k].tower_off = v->tower_off[k];
-        hv[k].n_tower = v->tower_off[k + 1] - v->tower_off[k];
-        hv[k].rem_off = v->removed_off[k];
-        hv[k].n_rem = v->removed_off[k + 1] - v->removed_off[k];
-        hv[k].ix0 = r[0]; hv[k].iy0 = r[1]; hv[k].nx = r[2]; hv[k].ny = r[3];
-        hv[k].out_off = cells;
-        cells += (long long)r[2] * r[3];
-    }
-    std::vector<float4> towers((size_t)n_tow * 3);
-    for (int t = 0; t < n_tow; ++t)
-        for (int q = 0; q < 3; ++q) {
-            const float* f = v->tower_tris + 9 * (size_t)t + 3 * q;
-            if (!isfinite(f[0]) || !isfinite(f[1]) || !isfinite(f[2]) || f[2] < 0.f)
-                return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: tower vertex non-finite or below z = 0");
-            towers[3 * (size_t)t + q] = make_float4(f[0], f[1], f[2], 0.f);
-        }
     sa_batch* b = new (std::nothrow) sa_batch();
-    if (!b) return sa::report_error(SA_ERR_OOM, "sa_batch_create: host allocation");
+    if (!b) return cudaErrorMemoryAllocation;
     b->base = base;
     b->grid.is_grid = 1;
     b->grid.x0 = grid->x0; b->grid.y0 = grid->y0; b->grid.dx = grid->dx;
@@ -185,7 +150,6 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
     b->I = n_intervals;
     b->cells_per_interval = cells;
     for (int k = 0; k < V; ++k) b->var_off.push_back(hv[k].out_off);
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSuccess;
     int dev = 0;
     e = cudaGetDevice(&dev);
@@ -194,7 +158,7 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
     b->run = sa::get_raster_run();
     if (e == cudaSuccess) e = dev_copy(b, towers.data(), towers.size(), &b->d_towers);
     if (e == cudaSuccess) e = dev_copy(b, v->removed_ids, (size_t)n_rem, &b->d_removed);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counter, sizeof(unsigned));
+    if (e == cudaSuccess) e = sa::device_alloc(&b->d_counter, sizeof(unsigned));
     if (e == cudaSuccess) b->owned.push_back(b->d_counter);
     // The base masks of every interval, where they take at most a quarter of the device's free
     // memory (8 bytes per cell and block: 453 MB for 1024^2 cells, two intervals of 3 days);
@@ -202,7 +166,7 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
     size_t mask_words = 0;
     for (int i = 0; i < n_intervals; ++i) mask_words += intervals[i]->h_blocks.size() * (size_t)grid->R;
     unsigned long long* masks = nullptr;
-    if (e == cudaSuccess && mask_words > 0 && V > 0 && sa::get_batch_tile_skip()) {
+    if (e == cudaSuccess && keep_masks && mask_words > 0 && V > 0 && sa::get_batch_tile_skip()) {
         size_t free_b = 0, total_b = 0;
         e = cudaMemGetInfo(&free_b, &total_b);
         if (e == cudaSuccess && mask_words * 8 <= free_b / 4) {
@@ -210,9 +174,6 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
                 b->owned.push_back(masks);
                 e = cudaMemsetAsync(masks, 0, mask_words * 8, st);
                 b->by_delta = true;
-            } else {
-                cudaGetLastError();
-                masks = nullptr;
             }
         }
     }
@@ -243,7 +204,7 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
         bi.base_counts = nullptr;
         if (e == cudaSuccess && grid->R > 0) {
             int *bc = nullptr, *run = nullptr;
-            e = cudaMalloc(&bc, sizeof(int) * (size_t)grid->R);
+            e = sa::device_alloc(&bc, sizeof(int) * (size_t)grid->R);
             if (e == cudaSuccess) b->owned.push_back(bc);
             if (e == cudaSuccess) e = cudaMemsetAsync(bc, 0, sizeof(int) * (size_t)grid->R, st);
             if (e == cudaSuccess) e = sa::scratch_alloc(&run, sizeof(int) * (size_t)grid->R, st);
@@ -377,7 +338,7 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
     b->n_items = (int)items.size();
     if (e == cudaSuccess && b->by_delta) {
         // the blocks of the affected tiles that a change reaches, one item each; a batch with
-        // more than 64M of them rasters its tiles whole
+        // more than 64M of them rasters its tiles whole, and needs no masks
         int4* d_tiles = nullptr;
         int max_blocks = 0;
         for (const sa::BatchInterval& iv : b->h_iv) max_blocks = std::max(max_blocks, iv.n_blocks);
@@ -391,7 +352,7 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
         if (order) b->owned.push_back(order);
         b->delta.order = order;
         b->n_work = (int)std::min(n_work, 1u << 26);
-        if (n_work > (1u << 26)) b->by_delta = false;
+        if (e == cudaSuccess && n_work > (1u << 26)) e = cudaErrorMemoryAllocation;
     }
     if (!b->by_delta && e == cudaSuccess) {
         e = dev_copy(b, items.data(), items.size(), &b->d_items);
@@ -399,10 +360,66 @@ sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const 
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
+        *kept_masks = masks != nullptr;
         sa_batch_destroy(b);
-        return sa::report_error(e == cudaErrorMemoryAllocation ? SA_ERR_OOM : SA_ERR_CUDA, cudaGetErrorString(e));
+        return e;
     }
     *out = b;
+    return cudaSuccess;
+}
+
+sa_status sa_batch_create(const sa_scene* base, const sa_receivers* grid, const sa_variants* v,
+                          const sa_sun* const* intervals, int32_t n_intervals,
+                          int32_t with_impact, void* stream, sa_batch** out) {
+    if (!out) return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: out is NULL");
+    *out = nullptr;
+    if (!base || !grid || !v || (n_intervals > 0 && !intervals) || n_intervals < 0)
+        return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: NULL argument or bad count");
+    if (!grid->is_grid) return sa::report_error(SA_ERR_UNSUPPORTED, "sa_batch_create: receivers must be a ground grid");
+    if (base->min_z < 0.f) return sa::report_error(SA_ERR_UNSUPPORTED, "sa_batch_create: base geometry below z = 0");
+    const int V = v->n_variants;
+    if (V < 0 || (V > 0 && (!v->tower_off || !v->removed_off || !v->regions)))
+        return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: bad variant description");
+    for (int i = 0; i < n_intervals; ++i)
+        if (!intervals[i]) return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: NULL interval");
+    const int n_tow = V > 0 ? v->tower_off[V] : 0, n_rem = V > 0 ? v->removed_off[V] : 0;
+    if (V > 0 && (v->tower_off[0] != 0 || v->removed_off[0] != 0 || n_tow < 0 || n_rem < 0 ||
+                  (n_tow > 0 && !v->tower_tris) || (n_rem > 0 && !v->removed_ids)))
+        return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: bad offsets");
+    std::vector<sa::BatchVariant> hv(V);
+    long long cells = 0;
+    for (int k = 0; k < V; ++k) {
+        const int* r = v->regions + 4 * k;
+        if (v->tower_off[k + 1] < v->tower_off[k] || v->removed_off[k + 1] < v->removed_off[k])
+            return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: offsets decrease");
+        if (r[0] < 0 || r[1] < 0 || r[2] < 0 || r[3] < 0 || r[0] + r[2] > grid->nx || r[1] + r[3] > grid->ny)
+            return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: region outside the grid");
+        hv[k].tower_off = v->tower_off[k];
+        hv[k].n_tower = v->tower_off[k + 1] - v->tower_off[k];
+        hv[k].rem_off = v->removed_off[k];
+        hv[k].n_rem = v->removed_off[k + 1] - v->removed_off[k];
+        hv[k].ix0 = r[0]; hv[k].iy0 = r[1]; hv[k].nx = r[2]; hv[k].ny = r[3];
+        hv[k].out_off = cells;
+        cells += (long long)r[2] * r[3];
+    }
+    std::vector<float4> towers((size_t)n_tow * 3);
+    for (int t = 0; t < n_tow; ++t)
+        for (int q = 0; q < 3; ++q) {
+            const float* f = v->tower_tris + 9 * (size_t)t + 3 * q;
+            if (!isfinite(f[0]) || !isfinite(f[1]) || !isfinite(f[2]) || f[2] < 0.f)
+                return sa::report_error(SA_ERR_INVALID_ARG, "sa_batch_create: tower vertex non-finite or below z = 0");
+            towers[3 * (size_t)t + q] = make_float4(f[0], f[1], f[2], 0.f);
+        }
+    // A batch that the masks leave no memory for, or that has too many items, does without them.
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    bool kept_masks = false;
+    cudaError_t e = create(base, grid, v, intervals, n_intervals, hv, cells, towers, true, st, out, &kept_masks);
+    if (e == cudaErrorMemoryAllocation && kept_masks) {
+        sa::trim_scratch();
+        e = create(base, grid, v, intervals, n_intervals, hv, cells, towers, false, st, out, &kept_masks);
+    }
+    if (e != cudaSuccess)
+        return sa::report_error(e == cudaErrorMemoryAllocation ? SA_ERR_OOM : SA_ERR_CUDA, cudaGetErrorString(e));
     return SA_OK;
 }
 

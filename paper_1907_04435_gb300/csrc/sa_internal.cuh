@@ -107,6 +107,14 @@ template <class T>
 inline cudaError_t scratch_alloc(T** p, size_t bytes, cudaStream_t st) {
     return scratch_alloc_bytes(reinterpret_cast<void**>(p), bytes, st);
 }
+// Gives back what the pool holds and nobody uses (after a synchronisation of its users).
+void trim_scratch();
+// cudaMalloc for what a handle keeps outside the pool.
+cudaError_t device_alloc_bytes(void** p, size_t bytes);
+template <class T>
+inline cudaError_t device_alloc(T** p, size_t bytes) {
+    return device_alloc_bytes(reinterpret_cast<void**>(p), bytes);
+}
 
 // Two FP32 values in one 64-bit register.  The packed multiply-add and multiply of sm_100
 // and later (fma.rn.f32x2, mul.rn.f32x2) round each half exactly as the scalar instruction

@@ -6,6 +6,10 @@
 // the device at every synchronisation, so a repeated call would map it again each time;
 // this pool keeps up to kKeep bytes reserved instead, and a handle built again (a scene
 // rebuilt every step) takes memory already mapped instead of paying cudaMalloc's latency.
+//
+// A caller that can do with less memory goes on after a failed allocation, so one leaves no
+// error behind for a later cudaGetLastError.  The bounds-checked build can be told to fail
+// an allocation (sa_check_fail_alloc): how the callers are tested without exhausting a device.
 #include <atomic>
 #include <mutex>
 #include <vector>
@@ -19,6 +23,18 @@ constexpr unsigned long long kKeep = 4ull << 30;
 std::mutex g_pool_mu;
 std::vector<cudaMemPool_t> g_pools;   // by device ordinal; null until first use
 std::atomic<unsigned long long> g_n_allocs{0}, g_alloc_bytes{0};
+std::atomic<int> g_fail_in{0};        // checked build: the allocation that fails, 1 the next; 0 none
+
+// counts one allocation; true if it is the one to fail
+bool planned_failure() {
+#ifdef SA_CHECKED
+    int n = g_fail_in.load();
+    while (n > 0 && !g_fail_in.compare_exchange_weak(n, n - 1)) {}
+    return n == 1;
+#else
+    return false;
+#endif
+}
 
 cudaError_t pool_of_current_device(cudaMemPool_t* out) {
     int dev = 0;
@@ -55,10 +71,35 @@ cudaError_t scratch_alloc_bytes(void** p, size_t bytes, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     g_n_allocs.fetch_add(1, std::memory_order_relaxed);
     g_alloc_bytes.fetch_add(bytes, std::memory_order_relaxed);
-    return cudaMallocFromPoolAsync(p, bytes, pool, st);
+    if (planned_failure()) return cudaErrorMemoryAllocation;
+    e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
+void trim_scratch() {
+    cudaMemPool_t pool = nullptr;
+    if (pool_of_current_device(&pool) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+}
+
+cudaError_t device_alloc_bytes(void** p, size_t bytes) {
+    *p = nullptr;
+    if (planned_failure()) return cudaErrorMemoryAllocation;
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 }  // namespace sa
+
+extern "C" int32_t sa_check_fail_alloc(int32_t n) {
+#ifdef SA_CHECKED
+    return sa::g_fail_in.exchange(n > 0 ? n : 0);
+#else
+    (void)n;
+    return -1;
+#endif
+}
 
 extern "C" sa_status sa_scratch_stats(uint64_t* stats) {
     if (!stats) return sa::report_error(SA_ERR_INVALID_ARG, "sa_scratch_stats: stats is NULL");

@@ -1687,8 +1687,8 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     g.tiles_y = (rc.ny + kTile - 1) / kTile;
     const size_t nc = (size_t)sun.n_blocks * g.tiles_x * g.tiles_y;
     if (nc == 0) return cudaSuccess;
-    cudaError_t e = cudaMalloc(counts, sizeof(unsigned) * nc);
-    if (e == cudaSuccess) e = cudaMalloc(offsets, sizeof(unsigned) * nc);
+    cudaError_t e = device_alloc(counts, sizeof(unsigned) * nc);
+    if (e == cudaSuccess) e = device_alloc(offsets, sizeof(unsigned) * nc);
     unsigned* cursor = nullptr;
     unsigned* d_total = nullptr;
     if (e == cudaSuccess) e = sa::scratch_alloc(&cursor, sizeof(unsigned) * nc, st);
@@ -1708,7 +1708,7 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     } else if (e == cudaSuccess) {
         e = cudaMemsetAsync(*offsets, 0, sizeof(unsigned) * nc, st);
     }
-    if (e == cudaSuccess) e = cudaMalloc(bins, sizeof(int) * ((size_t)total + 1));
+    if (e == cudaSuccess) e = device_alloc(bins, sizeof(int) * ((size_t)total + 1));
     if (e == cudaSuccess && total > 0)
         k_bin<true><<<grid, kBinThreads, 0, st>>>(sc, nullptr, sc.T, sun.steps, sun.blocks, 0, sun.n_blocks, per, g, *offsets, 0u,
                                                   cursor, *bins);
@@ -1747,8 +1747,8 @@ cudaError_t pick_batch_items(const BatchLaunch& bl, const int4* d_tiles, long lo
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess && total > 0 && total <= max_items) {
-        e = cudaMalloc(items, sizeof(int4) * (size_t)total);
-        if (e == cudaSuccess) e = cudaMalloc(order, sizeof(int) * (size_t)total);
+        e = device_alloc(items, sizeof(int4) * (size_t)total);
+        if (e == cudaSuccess) e = device_alloc(order, sizeof(int) * (size_t)total);
         if (e == cudaSuccess) e = sa::scratch_alloc(&weights, sizeof(unsigned) * (size_t)total, st);
         if (e == cudaSuccess) {
             k_batch_pick<<<ctas, 128, 0, st>>>(g, bl.intervals, bl.variants, bl.delta->boxes, d_tiles, n, max_blocks,
