@@ -342,7 +342,7 @@ static cudaError_t create(const sa_scene* base, const sa_receivers* grid, const 
         int4* d_tiles = nullptr;
         int max_blocks = 0;
         for (const sa::BatchInterval& iv : b->h_iv) max_blocks = std::max(max_blocks, iv.n_blocks);
-        unsigned n_work = 0;
+        unsigned long long n_work = 0;
         int* order = nullptr;
         e = dev_copy(b, items.data(), (size_t)b->n_affected, &d_tiles);
         if (e == cudaSuccess)
@@ -351,8 +351,8 @@ static cudaError_t create(const sa_scene* base, const sa_receivers* grid, const 
         if (b->d_work) b->owned.push_back(b->d_work);
         if (order) b->owned.push_back(order);
         b->delta.order = order;
-        b->n_work = (int)std::min(n_work, 1u << 26);
-        if (e == cudaSuccess && n_work > (1u << 26)) e = cudaErrorMemoryAllocation;
+        b->n_work = (int)std::min(n_work, 1ull << 26);
+        if (e == cudaSuccess && n_work > (1ull << 26)) e = cudaErrorMemoryAllocation;
     }
     if (!b->by_delta && e == cudaSuccess) {
         e = dev_copy(b, items.data(), items.size(), &b->d_items);

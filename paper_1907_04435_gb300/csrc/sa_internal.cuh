@@ -716,7 +716,8 @@ cudaError_t launch_batch(const BatchLaunch& bl, cudaStream_t st);
 // launch order (device, freed by the caller with cudaFree); *n_items above max_items: none
 // are made.  Synchronises st.
 cudaError_t pick_batch_items(const BatchLaunch& bl, const int4* d_tiles, long long n, int max_blocks,
-                             unsigned max_items, unsigned* n_items, int4** items, int** order, cudaStream_t st);
+                             unsigned max_items, unsigned long long* n_items, int4** items, int** order,
+                             cudaStream_t st);
 
 // shadow accrual map of point receivers in light space (scene_box, recv_box: lo.xyz hi.xyz)
 cudaError_t launch_sam_points(const DevScene& sc, const float* scene_box, const DevRecv& rc,

@@ -1273,12 +1273,14 @@ k_batch_delta(BatchArgs ba, BatchDelta bd) {
 
 // The work items of k_batch_delta: for every affected (interval, variant, tile) and block,
 // whether a changed box's shadow, swept over the block, can reach the tile.  Counts them
-// (items null), or appends them with their weights: the base triangles to raster again, and
-// the boxes.
+// (items null; a count, unlike the items that are then made of it, may pass 32 bits), or
+// appends them with their weights: the base triangles to raster again, and the boxes.
 __global__ void k_batch_pick(TileGeom g, const BatchInterval* __restrict__ intervals,
                              const BatchVariant* __restrict__ variants, const float4* __restrict__ boxes,
                              const int4* __restrict__ tiles, long long n, int max_blocks,
-                             unsigned* __restrict__ total, int4* __restrict__ items, unsigned* __restrict__ weights) {
+                             unsigned long long* __restrict__ total, int4* __restrict__ items,
+                             unsigned* __restrict__ weights) {
+    unsigned long long found = 0;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n * max_blocks;
          i += (long long)gridDim.x * blockDim.x) {
         const int4 t = tiles[i / max_blocks];
@@ -1296,11 +1298,15 @@ __global__ void k_batch_pick(TileGeom g, const BatchInterval* __restrict__ inter
             else ++n_tow;
         }
         if (!n_rem && !n_tow) continue;
-        const unsigned at = atomicAdd(total, 1u);
-        if (!items) continue;
+        if (!items) {
+            ++found;
+            continue;
+        }
+        const unsigned long long at = atomicAdd(total, 1ull);
         items[at] = make_int4(t.x, t.y, t.z, bl * 4 + (remv ? 2 : 0) + (n_tow ? 1 : 0));
         weights[at] = 1u + 4u * n_tow + (remv ? 16u * n_rem + iv.counts[(size_t)bl * g.tiles_x * g.tiles_y + t.z] : 0u);
     }
+    if (found) atomicAdd(total, found);
 }
 
 // The base counts, and no impact, for every cell of every region.
@@ -1729,21 +1735,22 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
 int raster_ctas_per_sm() { return SA_RASTER_CTAS; }
 
 cudaError_t pick_batch_items(const BatchLaunch& bl, const int4* d_tiles, long long n, int max_blocks,
-                             unsigned max_items, unsigned* n_items, int4** items, int** order, cudaStream_t st) {
+                             unsigned max_items, unsigned long long* n_items, int4** items, int** order, cudaStream_t st) {
     *n_items = 0;
     *items = nullptr;
     *order = nullptr;
     if (n == 0 || max_blocks == 0) return cudaSuccess;
     const TileGeom g = tile_geom(bl.grid);
-    unsigned *words = nullptr, *weights = nullptr;
-    cudaError_t e = sa::scratch_alloc(&words, sizeof(unsigned) * (2 + kOrderBuckets), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(words, 0, sizeof(unsigned) * 2, st);
+    unsigned long long* totals = nullptr;        // of the two passes; the buckets of the order
+    unsigned* weights = nullptr;
+    cudaError_t e = sa::scratch_alloc(&totals, sizeof(unsigned long long) * 2 + sizeof(unsigned) * kOrderBuckets, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(totals, 0, sizeof(unsigned long long) * 2, st);
     const unsigned ctas = (unsigned)std::min(152ll * 32, (n * max_blocks + 127) / 128);
-    unsigned total = 0;
+    unsigned long long total = 0;
     if (e == cudaSuccess) {
         k_batch_pick<<<ctas, 128, 0, st>>>(g, bl.intervals, bl.variants, bl.delta->boxes, d_tiles, n, max_blocks,
-                                           words, nullptr, nullptr);
-        e = cudaMemcpyAsync(&total, words, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+                                           totals, nullptr, nullptr);
+        e = cudaMemcpyAsync(&total, totals, sizeof(total), cudaMemcpyDeviceToHost, st);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess && total > 0 && total <= max_items) {
@@ -1752,11 +1759,12 @@ cudaError_t pick_batch_items(const BatchLaunch& bl, const int4* d_tiles, long lo
         if (e == cudaSuccess) e = sa::scratch_alloc(&weights, sizeof(unsigned) * (size_t)total, st);
         if (e == cudaSuccess) {
             k_batch_pick<<<ctas, 128, 0, st>>>(g, bl.intervals, bl.variants, bl.delta->boxes, d_tiles, n, max_blocks,
-                                               words + 1, *items, weights);
-            e = launch_work_order(weights, nullptr, total, words + 2, *order, nullptr, st);
+                                               totals + 1, *items, weights);
+            e = launch_work_order(weights, nullptr, (long long)total, reinterpret_cast<unsigned*>(totals + 2), *order,
+                                  nullptr, st);
         }
     }
-    if (words) cudaFreeAsync(words, st);
+    if (totals) cudaFreeAsync(totals, st);
     if (weights) cudaFreeAsync(weights, st);
     *n_items = total;
     return e;
