@@ -59,7 +59,7 @@ int g_tile_skip = 1;
 }  // namespace
 void set_batch_tile_skip(int on) { g_tile_skip = on; }
 int get_batch_tile_skip() { return g_tile_skip; }
-int raster_ctas_per_sm();   // sa_raster.cu: the CTAs per SM its kernels are compiled for
+int batch_ctas_per_sm(bool by_delta);   // sa_raster.cu: the CTAs per SM its kernels are compiled for
 }  // namespace sa
 
 namespace {
@@ -154,7 +154,6 @@ static cudaError_t create(const sa_scene* base, const sa_receivers* grid, const 
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
-    b->ctas = sa::raster_ctas_per_sm() * b->sms;     // 16 variants: 6.2 ms at 4 CTAs per SM, 4.9 at 6
     b->run = sa::get_raster_run();
     if (e == cudaSuccess) e = dev_copy(b, towers.data(), towers.size(), &b->d_towers);
     if (e == cudaSuccess) e = dev_copy(b, v->removed_ids, (size_t)n_rem, &b->d_removed);
@@ -357,6 +356,7 @@ static cudaError_t create(const sa_scene* base, const sa_receivers* grid, const 
     if (!b->by_delta && e == cudaSuccess) {
         e = dev_copy(b, items.data(), items.size(), &b->d_items);
     }
+    b->ctas = sa::batch_ctas_per_sm(b->by_delta) * b->sms;
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
@@ -475,7 +475,7 @@ sa_status sa_batch_tune(sa_batch* b, int32_t* best_ctas, int32_t* best_run, void
     float best = 3.4e38f;
     int bc = b->ctas, br = b->run;
     const int runs[3] = {8, 16, 24};
-    for (int c = 2; c <= sa::raster_ctas_per_sm() && e == cudaSuccess; ++c)
+    for (int c = 2; c <= sa::batch_ctas_per_sm(b->by_delta) && e == cudaSuccess; ++c)
         for (int r : runs) {
             const sa::BatchLaunch bl = launch_of(b, scratch, nullptr, 8, c * b->sms, r, nullptr);
             e = sa::launch_batch(bl, st);                                   // warm-up

@@ -47,11 +47,14 @@ constexpr int kTriBatch = SA_RASTER_BATCH;
 static_assert(kTriBatch <= 64, "a unit packs its triangle in 6 bits");
 // work units (triangle, run of steps) of a batch: one per thread
 constexpr int kMaxUnits = kRasterThreads;
+constexpr int kChangeList = 256;        // k_batch_delta: changed triangles picked per round
 // resident CTAs per SM the raster kernels are compiled for (registers: 65536 / (256 x this));
-// 6 is also what the item kernels' 32 KB of shared memory allow
+// 6 is also what the item kernels' 32 KB of shared memory allow, and 5 what it leaves the
+// kernels that hold a tile's running counts beside it (k_raster, k_batch: 44 KB)
 #ifndef SA_RASTER_CTAS
 #define SA_RASTER_CTAS 6
 #endif
+constexpr int kStateCtas = 5;
 
 struct TileGeom {
     float x0, y0, dx;
@@ -343,6 +346,11 @@ struct TileSmem {
         hi[cell] = (unsigned)(m >> 32);
     }
 };
+
+// an SM's 228 KB hold the CTAs that the kernels are compiled for, with 1 KB each of the system's
+constexpr int kSmShared = 228 * 1024, kCtaShared = 1024;
+static_assert(SA_RASTER_CTAS * (sizeof(TileSmem) + sizeof(int) * (kChangeList + 2) + kCtaShared) <= kSmShared, "items");
+static_assert(kStateCtas * (sizeof(TileSmem) + sizeof(RunState) * kTile * kTile + kCtaShared) <= kSmShared, "by tile");
 
 // Tile origin and cell centres in tile-local coordinates; the centres are rounded exactly
 // as the receivers' world coordinates, then shifted.
@@ -997,7 +1005,7 @@ k_items_fold(const unsigned* __restrict__ summary, long long R, const BlockConst
 // It writes the counts of the tile's cells inside the region and, where the base counts
 // are given, the impact (variant minus base).
 template <bool COUNT, bool CULL>
-__global__ void __launch_bounds__(kRasterThreads, SA_RASTER_CTAS)
+__global__ void __launch_bounds__(kRasterThreads, kStateCtas)
 k_batch(BatchArgs ba) {
     __shared__ TileSmem sm;
     __shared__ RunState s_st[kTile * kTile];       // gross / run / best of the tile's cells
@@ -1100,7 +1108,6 @@ k_batch(BatchArgs ba) {
 // counts.  Against k_batch (every block of an affected tile rastered whole): 16 variants x 2
 // intervals x 3 days over 1024^2 cells 18.2 -> 3.05 ms (bound by issue, in the towers' rasters
 // and in the units that set up the few triangles of an item).
-constexpr int kChangeList = 256;          // changed triangles picked per round
 
 // Triangles of k_batch_delta's rasters: item i is tris[map[list[i]]] (either index may be
 // absent); one of the removed buildings' triangles is skipped.
@@ -1333,7 +1340,7 @@ __global__ void k_tile_sums(const unsigned* __restrict__ counts, int nbc, int n_
     sums[t] = c;
 }
 
-// A launch of more tiles than 4 CTAs per SM hold takes the build for SA_RASTER_CTAS
+// A launch of more tiles than 4 CTAs per SM hold takes the build for kStateCtas
 // resident CTAs per SM (fewer registers, more warps to hide latency); a smaller one, all of
 // whose tiles are resident at once anyway, takes the build for 4 (more registers, no
 // spills).
@@ -1341,9 +1348,9 @@ void launch_k_raster(const RasterArgs& ra, int n_tiles, cudaStream_t st) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 0;
-    if (SA_RASTER_CTAS > 4 && n_tiles > 4 * sms) {
-        if (ra.cull) k_raster<true, SA_RASTER_CTAS><<<n_tiles, kRasterThreads, 0, st>>>(ra);
-        else k_raster<false, SA_RASTER_CTAS><<<n_tiles, kRasterThreads, 0, st>>>(ra);
+    if (n_tiles > 4 * sms) {
+        if (ra.cull) k_raster<true, kStateCtas><<<n_tiles, kRasterThreads, 0, st>>>(ra);
+        else k_raster<false, kStateCtas><<<n_tiles, kRasterThreads, 0, st>>>(ra);
     } else {
         if (ra.cull) k_raster<true, 4><<<n_tiles, kRasterThreads, 0, st>>>(ra);
         else k_raster<false, 4><<<n_tiles, kRasterThreads, 0, st>>>(ra);
@@ -1732,7 +1739,7 @@ cudaError_t build_bins(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     return e;
 }
 
-int raster_ctas_per_sm() { return SA_RASTER_CTAS; }
+int batch_ctas_per_sm(bool by_delta) { return by_delta ? SA_RASTER_CTAS : kStateCtas; }
 
 cudaError_t pick_batch_items(const BatchLaunch& bl, const int4* d_tiles, long long n, int max_blocks,
                              unsigned max_items, unsigned long long* n_items, int4** items, int** order, cudaStream_t st) {
