@@ -814,8 +814,14 @@ cudaError_t launch_height_grad(const DevScene& sc, const FootprintSet& fs, const
         go.nx = rc.nx; go.ny = rc.ny; go.tiles_x = (rc.nx + 7) / 8;
         go.n = 32ll * go.tiles_x * ((rc.ny + 3) / 4);
         go.per = (sun.n_blocks + kGroups - 1) / kGroups;
-        const long long slots = go.n * ((sun.n_blocks + go.per - 1) / go.per);
-        TRY(sa::scratch_alloc(&counts, sizeof(unsigned) * (size_t)slots, st));
+        long long slots = go.n * ((sun.n_blocks + go.per - 1) / go.per);
+        e = sa::scratch_alloc(&counts, sizeof(unsigned) * (size_t)slots, st);
+        if (e == cudaErrorMemoryAllocation) {          // no room for the groups' counts: one group
+            go.per = sun.n_blocks;
+            slots = go.n;
+            e = sa::scratch_alloc(&counts, sizeof(unsigned) * (size_t)slots, st);
+        }
+        if (e != cudaSuccess) goto done;
         TRY(sa::scratch_alloc(&d_total, sizeof(unsigned), st));
         const double dt = step_minutes;
         const unsigned grid = (unsigned)((go.n + 255) / 256);
@@ -830,6 +836,11 @@ cudaError_t launch_height_grad(const DevScene& sc, const FootprintSet& fs, const
         if (total > 0) {
             TRY(sa::scratch_alloc(&flips, sizeof(int4) * (size_t)total, st));
             k_flip_fill<<<grid, 256, 0, st>>>(masks, R, go, sun.blocks, sun.n_blocks, counts, flips);
+            // the list replaces the masks and counts, whose memory serves what follows
+            cudaFreeAsync(masks, st);
+            cudaFreeAsync(counts, st);
+            masks = nullptr;
+            counts = nullptr;
             TRY(sa::scratch_alloc(&arcs, sizeof(ArcConst) * (size_t)sun.S, st));
             k_arcs<<<(sun.S + 127) / 128, 128, 0, st>>>(sun.steps, sun.S - 1, arcs);
             SolveArgs sa;

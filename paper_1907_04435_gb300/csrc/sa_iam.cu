@@ -317,14 +317,15 @@ cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
     const long long R = (long long)rc.nx * rc.ny;
     if (R == 0) return cudaSuccess;
     if (L < 1 || L > kMaxLevels) return cudaErrorInvalidValue;
-    // the blocks go in one launch, as many as 1 GiB of masks and sources holds
-    const int chunk = (int)std::max(1ll, std::min({(long long)sun.n_blocks, 32767ll, (1ll << 30) / ((8ll + 8ll * L) * R)}));
+    // the blocks go in one launch, as many as 1 GiB of masks and sources holds, or the memory
+    // there is
+    int chunk = (int)std::max(1ll, std::min({(long long)sun.n_blocks, 32767ll, (1ll << 30) / ((8ll + 8ll * L) * R)}));
     unsigned long long* masks = nullptr;
     float* src = nullptr;
     RunLight* runs = nullptr;
     IamWalk* d_walks = nullptr;
-    cudaError_t e = sa::scratch_alloc(&masks, sizeof(unsigned long long) * (size_t)R * chunk, st);
-    if (e == cudaSuccess) e = sa::scratch_alloc(&src, sizeof(float) * 2 * (size_t)L * (size_t)R * chunk, st);
+    cudaError_t e = sa::scratch_alloc_blocks(&src, sizeof(float) * 2 * (size_t)L * (size_t)R, &chunk, st);
+    if (e == cudaSuccess) e = sa::scratch_alloc_blocks(&masks, sizeof(unsigned long long) * (size_t)R, &chunk, st);
     if (e == cudaSuccess) e = sa::scratch_alloc(&runs, sizeof(RunLight) * 2 * (size_t)chunk, st);
     if (e == cudaSuccess) e = sa::scratch_alloc(&d_walks, sizeof(IamWalk) * 2 * (size_t)chunk, st);
     Grid g{rc.x0, rc.y0, rc.dx, rc.nx, rc.ny};

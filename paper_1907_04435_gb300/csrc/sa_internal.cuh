@@ -107,6 +107,17 @@ template <class T>
 inline cudaError_t scratch_alloc(T** p, size_t bytes, cudaStream_t st) {
     return scratch_alloc_bytes(reinterpret_cast<void**>(p), bytes, st);
 }
+// Scratch for *blocks blocks of `bytes` each, or for as many as there is memory for, halving
+// *blocks down to 1.
+template <class T>
+inline cudaError_t scratch_alloc_blocks(T** p, size_t bytes, int* blocks, cudaStream_t st) {
+    cudaError_t e = scratch_alloc(p, bytes * (size_t)*blocks, st);
+    while (e == cudaErrorMemoryAllocation && *blocks > 1) {
+        *blocks = (*blocks + 1) / 2;
+        e = scratch_alloc(p, bytes * (size_t)*blocks, st);
+    }
+    return e;
+}
 // Gives back what the pool holds and nobody uses (after a synchronisation of its users).
 void trim_scratch();
 // cudaMalloc for what a handle keeps outside the pool.

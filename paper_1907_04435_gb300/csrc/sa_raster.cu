@@ -1417,10 +1417,10 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
     // One-step blocks (the per-step raster) of a grid whose tiles fill the chip go by tile: a
     // summary per step is as much memory as the raster's own work (2048^2 cells, 481 steps:
     // 30.9 ms by tile, 32.3 by item; 300 x 200 cells, 70 tiles, 241 steps: 4.07 and 0.50 ms).
-    const bool by_tile = !summaries && out.gross && !out.stats && n_tiles >= 4 * 152 &&
-                         sun.S < 8ll * sun.n_blocks;
-    const int parts = summaries || by_tile ? 1 : raster_parts(n_tiles, sun.n_blocks);
-    const bool fold = !summaries && out.gross && !by_tile;
+    bool by_tile = !summaries && out.gross && !out.stats && n_tiles >= 4 * 152 &&
+                   sun.S < 8ll * sun.n_blocks;
+    int parts = summaries || by_tile ? 1 : raster_parts(n_tiles, sun.n_blocks);
+    bool fold = !summaries && out.gross && !by_tile;
     cudaError_t e = cudaSuccess;
     // blocks per chunk: 64, and more where a small grid's counters, bins (every triangle in
     // every tile at the most: the sums stay below 2^31) and run summaries (1 GiB) allow it
@@ -1461,6 +1461,18 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
             list = nullptr;
         }
     }
+    unsigned* summary = summaries;
+    if (e == cudaSuccess && fold) {
+        // without memory for the summaries of one block, by tile, which needs none
+        e = sa::scratch_alloc_blocks(&summary, sizeof(unsigned) * (size_t)parts * (size_t)R, &chunk, st);
+        if (e == cudaErrorMemoryAllocation && !out.stats) {
+            e = cudaSuccess;
+            by_tile = true;
+            fold = false;
+            parts = 1;
+            chunk = chunk_blocks(T);
+        }
+    }
     const size_t nc = (size_t)chunk * n_tiles;
     const bool direct = is_direct(chunk, T);
     // one block of words: counts | cursor (zeroed together) | offsets | order | total | buckets
@@ -1468,7 +1480,6 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
     int* bins = nullptr;
     int* best = out.continuous;
     int* best_scratch = nullptr;
-    unsigned* summary = summaries;
     size_t bins_cap = 0;
     if (e == cudaSuccess) e = sa::scratch_alloc(&words, sizeof(unsigned) * (4 * nc + 1 + kOrderBuckets), st);
     unsigned *counts = words, *cursor = words + nc, *offsets = words + 2 * nc, *d_total = words + 4 * nc,
@@ -1478,8 +1489,6 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
         e = sa::scratch_alloc(&best_scratch, sizeof(int) * (size_t)R, st);
         best = best_scratch;
     }
-    if (e == cudaSuccess && fold)
-        e = sa::scratch_alloc(&summary, sizeof(unsigned) * (size_t)chunk * parts * (size_t)R, st);
     if (e == cudaSuccess && direct) {
         bins_cap = nc * (size_t)T;
         e = sa::scratch_alloc(&bins, sizeof(int) * bins_cap, st);
@@ -1489,8 +1498,8 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
         e = cudaMemsetAsync(out.run, 0, sizeof(int) * (size_t)R, st);
         if (e == cudaSuccess && !out.continuous) e = cudaMemsetAsync(best, 0, sizeof(int) * (size_t)R, st);
     }
-    for (int b0 = 0; b0 < sun.n_blocks && e == cudaSuccess; b0 += chunk) {
-        const int nbc = std::min(sun.n_blocks - b0, chunk);
+    for (int b0 = 0, nbc = 0; b0 < sun.n_blocks && e == cudaSuccess; b0 += nbc) {
+        nbc = std::min(sun.n_blocks - b0, chunk);
         const size_t ncc = (size_t)nbc * n_tiles;
         int per = 1;
         const dim3 grid = bin_grid(std::max(T, 1), nbc, &per);
@@ -1526,7 +1535,14 @@ static cudaError_t raster_ground(const DevScene& sc, const DevRecv& rc, const De
                 if (bins) cudaFreeAsync(bins, st);
                 bins_cap = (size_t)total + total / 4 + 1024;
                 e = sa::scratch_alloc(&bins, sizeof(int) * bins_cap, st);
-                if (e != cudaSuccess) { bins = nullptr; break; }
+                if (e == cudaErrorMemoryAllocation && nbc > 1) {      // again, with half the blocks
+                    e = cudaSuccess;
+                    bins_cap = 0;
+                    chunk = (nbc + 1) / 2;
+                    nbc = 0;
+                    continue;
+                }
+                if (e != cudaSuccess) break;
             }
             if (total > 0) {
                 KernelTimer kt(KT_RASTER_BIN, st);

@@ -494,22 +494,24 @@ static bool use_lane(int which, const DevRecv& rc) {
     return mode == 2 || (mode == 0 && which == 0);
 }
 
-// Runs launch(items, grid.y) over every block in chunks whose summaries fit 1 GiB, folding
-// each chunk into the receivers' state.
+// Runs launch(items, grid.y) over every block in chunks whose summaries fit 1 GiB (and the
+// memory there is), folding each chunk into the receivers' state.  Without memory for one
+// block's summaries nothing has been launched.
 template <class Launch>
 static cudaError_t by_items(const DevRecv& rc, const DevSun& sun, const DevOut& out, int parts, cudaStream_t st,
                             Launch launch) {
     const long long R = rc.R;
-    const int chunk = (int)std::max(1ll, std::min({(long long)sun.n_blocks, 65535ll / parts, (1ll << 30) / (4ll * parts * R)}));
+    int chunk = (int)std::max(1ll, std::min({(long long)sun.n_blocks, 65535ll / parts, (1ll << 30) / (4ll * parts * R)}));
     unsigned* summary = nullptr;
     int *run = nullptr, *best = out.continuous, *best_scratch = nullptr;
-    cudaError_t e = sa::scratch_alloc(&summary, sizeof(unsigned) * (size_t)chunk * parts * (size_t)R, st);
-    if (e == cudaSuccess) e = sa::scratch_alloc(&run, sizeof(int) * (size_t)R, st);
+    cudaError_t e = sa::scratch_alloc(&run, sizeof(int) * (size_t)R, st);
     if (e == cudaSuccess && !best) {
         e = sa::scratch_alloc(&best_scratch, sizeof(int) * (size_t)R, st);
         best = best_scratch;
         if (e == cudaSuccess && out.accumulate_into) e = cudaMemsetAsync(best, 0, sizeof(int) * (size_t)R, st);
     }
+    if (e == cudaSuccess)
+        e = sa::scratch_alloc_blocks(&summary, sizeof(unsigned) * (size_t)parts * (size_t)R, &chunk, st);
     if (e == cudaSuccess && out.accumulate_into) e = cudaMemsetAsync(run, 0, sizeof(int) * (size_t)R, st);
     DevOut o = out;
     o.run = run;
@@ -545,15 +547,15 @@ cudaError_t launch_sweep_trace(const DevScene& sc, const DevRecv& rc, const DevS
     KernelTimer kt(KT_SWEEP, st);
     if (use_lane(0, rc)) {
         const int parts = trace_parts(warps, sun);
-        return by_items(rc, sun, out, parts, st, [&](const TraceItems& it, unsigned ny) {
+        const cudaError_t e = by_items(rc, sun, out, parts, st, [&](const TraceItems& it, unsigned ny) {
             if (out.stats) k_sweep_lane<true><<<dim3(ctas, ny), T, 0, st>>>(sc, rc, sun, out, it);
             else k_sweep_lane<false><<<dim3(ctas, ny), T, 0, st>>>(sc, rc, sun, out, it);
             return cudaGetLastError();
         });
-    } else {
-        if (out.stats) k_sweep<true><<<ctas, T, 0, st>>>(sc, rc, sun, out);
-        else k_sweep<false><<<ctas, T, 0, st>>>(sc, rc, sun, out);
+        if (e != cudaErrorMemoryAllocation) return e;      // else the walk that needs no memory
     }
+    if (out.stats) k_sweep<true><<<ctas, T, 0, st>>>(sc, rc, sun, out);
+    else k_sweep<false><<<ctas, T, 0, st>>>(sc, rc, sun, out);
     return cudaGetLastError();
 }
 
@@ -586,7 +588,8 @@ cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const fl
                 k_regroup_keys<<<(unsigned)((rc.R + 255) / 256), 256, 0, st>>>(
                     rc.orig, rc.R, recv_box[0], recv_box[1], recv_box[2], ext > 0.f ? 1.f / ext : 0.f, keys, order);
             if (e == cudaSuccess) e = radix_sort_pairs(keys, order, rc.R, st, 16);
-            rg.order = order;
+            if (e == cudaSuccess) rg.order = order;
+            if (e == cudaErrorMemoryAllocation) e = cudaSuccess;      // the points in their own order
         }
         // Points scattered thinly over a large scene make a group's box hold far more than its
         // rays: below a quarter as many points as triangles each receiver's own fan prunes

@@ -27,3 +27,14 @@ def test_a_batch_does_without_the_base_masks(cuda_lib):
     first = ends.index("same")
     assert set(ends[:first]) <= {"oom"} and first <= 4         # towers, removed buildings, counter, masks
     assert len(ends) > 12 and set(ends[first:]) == {"same"}
+
+
+def test_calls_go_on_with_less_memory(cuda_lib):
+    """The summaries, masks, sources and bins of many blocks are taken for fewer at a time when they
+    do not fit, down to paths that need none; any other failure is reported, and no
+    result is wrong."""
+    fewer = {"raster": 2, "raster, one block": 1, "steps by tile": 1, "sweep": 1, "sweep, one block": 1, "traced": 1,
+             "inverse": 2, "points": 3, "gradient": 1}      # allocations that a call does without
+    ends = _run(*fewer)
+    for name, n in fewer.items():
+        assert set(ends[name]) <= {"same", "oom"} and ends[name].count("same") >= n, (name, ends[name])
