@@ -90,9 +90,9 @@ int32_t sa_version(void);
 /* Process-wide tuning options (set between calls; not thread-safe against running calls).
  *   SA_OPT_SWEEP_TRAVERSAL, SA_OPT_ACCRUAL_TRAVERSAL: BVH traversal of the ray-traced
  *   methods -- 1 warp-coherent (the 32 lanes of a warp walk the node list together), 2 one
- *   traversal per lane, 0 the default (per lane for the sweep, warp-coherent for the
- *   accrual, the faster of the two on the district workload).  Results do not depend on
- *   the option.
+ *   traversal per lane, 0 the default (per lane for the sweep; for the accrual one per
+ *   group of 128 receivers, or warp-coherent for thin point sets, the faster of the two
+ *   there).  Results do not depend on the option.
  *   SA_OPT_RASTER_RUN: at most this many steps the ground accrual raster tests per cell
  *   set-up (1..32, default 24), and SA_OPT_POINT_RUN: at most this many steps per
  *   light-space map of point receivers (1..32, default 27); each block is split into
@@ -349,7 +349,8 @@ sa_status sa_batch_work_counters(sa_batch* b, uint64_t* counters, void* stream);
  * with counting enabled and writes counters uint64 [4] dev.
  *   trace methods: [0] ray/fan-versus-box tests, [1] ray-versus-triangle tests per
  *   receiver lane (SA_ACCRUAL_TRACE by groups: [0] node tests of a group's query, [1] step
- *   tests of its receiver-triangle pairs).
+ *   tests of its receiver-triangle pairs); of the walk that the option and the receivers
+ *   choose.
  *   raster methods (ground grids): [0] work units (triangle, run of steps) that reached
  *   the tile's cells, [1] cells their row spans enumerated, [2] cell set-ups (cells not
  *   already shadowed at every step of the unit), [3] cell-step coverage tests.

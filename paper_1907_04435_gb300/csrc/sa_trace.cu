@@ -304,12 +304,13 @@ __device__ __forceinline__ bool hit_tri_rt(const float3& o, const float4& a, con
     return det > 0.f ? (T > tmin * det) : (T < tmin * det);
 }
 
-
+template <bool COUNT>
 __global__ void __launch_bounds__(32 * kWarpsPerCta)
 k_accrual_fan(DevScene sc, DevRecv rc, DevSun sun, DevOut out, TraceItems it) {
     // block and step constants are copied per warp, so warps never wait for one another
     __shared__ BlockConst s_bc[kWarpsPerCta];
     __shared__ StepConst s_st[kWarpsPerCta][kMaxBlock];
+    unsigned long long n_box = 0, n_tri = 0;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const long long warp_id = (long long)blockIdx.x * kWarpsPerCta + wib;
     if (warp_id >= warp_count(rc)) return;
@@ -342,6 +343,7 @@ k_accrual_fan(DevScene sc, DevRecv rc, DevSun sun, DevOut out, TraceItems it) {
             const int tri = SA_LEAF(__float_as_int(hi.w), sc.T, sa::CK_TRACE_LEAF);
             const bool want = r.active && m != full;
             const bool in = want && (wedge ? fan_box(r.o, bc, lo, hi, front, r.n) : slope_box(r.o, bc, lo, hi));
+            if (COUNT && want) ++n_box;
             if (tri >= 0) {
                 int ka = K, kb = -1;
                 float4 ta, tb, tc;
@@ -360,6 +362,7 @@ k_accrual_fan(DevScene sc, DevRecv rc, DevSun sun, DevOut out, TraceItems it) {
                     for (int k = wa; k <= wb; ++k) {
                         const bool test = k >= ka && k <= kb && !((m >> k) & 1ull);
                         if (test) {
+                            if (COUNT) ++n_tri;
                             if (plucker_hit(pt, ss[k].dx, ss[k].dy, ss[k].dz, r.tmin)) {
                                 m |= 1ull << k;
                             }
@@ -374,6 +377,7 @@ k_accrual_fan(DevScene sc, DevRecv rc, DevSun sun, DevOut out, TraceItems it) {
         }
         store_item(out, rc, r, it, m, K, bc.mask_block, bc.mask_bit);
     }
+    if (COUNT) flush_counts(out, n_box, n_tri);
 }
 
 // Ray-traced accrual with one independent traversal per lane ("while-while": each lane
@@ -483,9 +487,9 @@ long long host_warps(const DevRecv& rc) {
 
 }  // namespace
 
-// Traversal mode: 1 = warp-coherent (packet), 2 = per lane, 0 = the measured default:
-// per lane for the per-step sweep (single rays: lanes rarely wait on each other), packet
-// for the accrual (its leaf work is a loop over steps that lanes share best in lockstep).
+// Traversal mode: 1 = warp-coherent (packet), 2 = per lane, 0 = the measured default: per lane
+// for the per-step sweep (single rays: lanes rarely wait on each other); for the accrual a
+// walk per group of 128 receivers, or the packet's for thin point sets (launch_accrual_trace).
 int g_trace_mode[2] = {0, 0};   // [0] sweep, [1] accrual
 
 static bool use_lane(int which, const DevRecv& rc) {
@@ -596,10 +600,11 @@ cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const fl
         // better (13,182 points over 120k triangles: 2.3 ms by fan, 8.8 by group; 3,001 over
         // 6k: 1.2 and 0.5), unless a low sun (slope above 4) stretches the fans (5,000 points
         // over 61k triangles in January: 34 and 7.5 ms).
-        const bool fan = !rc.is_grid && 4 * rc.R < sc.T && sun.max_slope < 4.f;
-        if (e == cudaSuccess && fan && !out.stats) {
+        const bool fan = g_trace_mode[1] == 1 || (!rc.is_grid && 4 * rc.R < sc.T && sun.max_slope < 4.f);
+        if (e == cudaSuccess && fan) {
             e = by_items(rg, sun, out, 1, st, [&](const TraceItems& it, unsigned ny) {
-                k_accrual_fan<<<dim3(ctas, ny), T, 0, st>>>(sc, rg, sun, out, it);
+                if (out.stats) k_accrual_fan<true><<<dim3(ctas, ny), T, 0, st>>>(sc, rg, sun, out, it);
+                else k_accrual_fan<false><<<dim3(ctas, ny), T, 0, st>>>(sc, rg, sun, out, it);
                 return cudaGetLastError();
             });
         } else if (e == cudaSuccess) {
