@@ -799,7 +799,10 @@ static sa_status run_method(const sa_scene* scene, const sa_receivers* recv, con
         dsun.blocks = sun->d_blocks;
         dsun.n_blocks = (int)sun->h_blocks.size();
         dsun.max_K = 1;
+        dsun.thin = true;
         for (const sa::BlockConst& b : sun->h_blocks) {
+            dsun.thin &= b.K == 1 || b.wedge_ok != 0.f;
+            if (b.wedge_ok != 0.f) dsun.max_angle = std::max(dsun.max_angle, fabsf(b.psi[b.K - 1] - b.psi[0]));
             dsun.max_K = std::max(dsun.max_K, b.K);
             dsun.max_slope = std::max({dsun.max_slope, fabsf(b.uxlo), fabsf(b.uxhi), fabsf(b.uylo), fabsf(b.uyhi)});
         }
@@ -833,7 +836,7 @@ static sa_status run_method(const sa_scene* scene, const sa_receivers* recv, con
         e = sa::launch_sam_points(dsc, scene->box, drc, recv->box, dsun, sun->h_blocks, sun->h_steps,
                                   out, st);
     } else {
-        e = sa::launch_accrual_trace(dsc, drc, recv->box, dsun, out, st);
+        e = sa::launch_accrual_trace(dsc, scene->box, drc, recv->box, dsun, out, st);
     }
     if (run) cudaFreeAsync(run, st);
     if (e != cudaSuccess) return cuda_fail(e, who);

@@ -584,6 +584,8 @@ struct DevSun {
     int S, n_blocks;
     int max_K = kMaxBlock;      // steps of the longest block, or a bound
     float max_slope = 0.f;      // largest |d_xy| / d_z of a block's slope box, if known
+    bool thin = false;          // every block's rays lie in a thin wedge, if known
+    float max_angle = 0.f;      // largest angle between a block's first and last rays, of thin ones
 };
 
 // outputs / state (state buffers hold gross, run, best per receiver in output order)
@@ -601,9 +603,9 @@ struct DevOut {
 
 cudaError_t launch_sweep_trace(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
                                const DevOut& out, cudaStream_t st);
-// (recv_box: bounds of point receivers, lo.xyz hi.xyz)
-cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const float* recv_box, const DevSun& sun,
-                                 const DevOut& out, cudaStream_t st);
+// (scene_box, and recv_box of point receivers: lo.xyz hi.xyz)
+cudaError_t launch_accrual_trace(const DevScene& sc, const float* scene_box, const DevRecv& rc, const float* recv_box,
+                                 const DevSun& sun, const DevOut& out, cudaStream_t st);
 // traversal mode of the sweep (which = 0) and accrual (which = 1) kernels
 void set_trace_mode(int which, int mode);
 int get_trace_mode(int which);

@@ -570,8 +570,35 @@ cudaError_t launch_run_lights(const StepConst* steps, const BlockConst* blocks, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const float* recv_box, const DevSun& sun,
-                                 const DevOut& out, cudaStream_t st) {
+// Whether point receivers walk by warps, each with its own fan, rather than by groups.  A
+// group's box must not hold far more than its rays do, and where 128 consecutive points
+// straddle a bisection of the plan it holds a good part of the scene: that group's CTA
+// takes time in proportion to the scene, 80 to 120 us per 1,000 triangles whatever the
+// points, while the walks by warps take about as much per point and block.  So points that
+// are few for the triangles go by warps, unless the sun is low (long fans: their cost grows
+// with the slope), the scene small, the blocks many (a group's cost grows less with them,
+// and less still where each spans hours) or a block's rays too far apart for a wedge.
+// Points spread over the scene, ms by warps / by groups, 481 steps in June if not said:
+// 122k triangles, 32k points 5.0 / 14, 147k 14 / 17, 294k 24 / 19; 365k, 95k 13 / 46; 2,340,
+// 600 1.4 / 0.4; 122k and 73k points: 29 steps 3.7 / 12, 7 days of 2 minutes 32 / 34, 30
+// days of 10 minutes 92 / 42, March to a slope of 4.9 11 / 16, February to 23 26 / 18,
+// December 57 / 28.  Where the two are close the line errs to the warps.
+static bool accrual_by_warps(const DevScene& sc, const float* box, const DevRecv& rc, const float* recv_box,
+                             const DevSun& sun) {
+    if (g_trace_mode[1] == 1) return true;
+    if (rc.is_grid || !sun.thin) return false;
+    // the scene's triangles under the points' plan
+    auto area = [](const float* b) { return ((double)b[3] - b[0]) * ((double)b[4] - b[1]); };
+    const double share = area(box) > 0.0 ? std::min(1.0, area(recv_box) / area(box)) : 1.0;
+    const double slope = std::max(2.0, (double)sun.max_slope);
+    double f = 9.0 / sun.n_blocks;
+    if (f < 1.0) f *= std::min(1.0, 0.5 / std::max(1e-3, (double)sun.max_angle));
+    if (slope > 5.0) f = std::min(1.0, f) * 5.0 / slope;
+    return (double)rc.R < 2.2 * f * (share * sc.T - 6000.0 * slope);
+}
+
+cudaError_t launch_accrual_trace(const DevScene& sc, const float* scene_box, const DevRecv& rc, const float* recv_box,
+                                 const DevSun& sun, const DevOut& out, cudaStream_t st) {
     const long long warps = host_warps(rc);
     if (warps == 0) return cudaSuccess;
     const unsigned ctas = (unsigned)((warps + kWarpsPerCta - 1) / kWarpsPerCta);
@@ -595,13 +622,7 @@ cudaError_t launch_accrual_trace(const DevScene& sc, const DevRecv& rc, const fl
             if (e == cudaSuccess) rg.order = order;
             if (e == cudaErrorMemoryAllocation) e = cudaSuccess;      // the points in their own order
         }
-        // Points scattered thinly over a large scene make a group's box hold far more than its
-        // rays: below a quarter as many points as triangles each receiver's own fan prunes
-        // better (13,182 points over 120k triangles: 2.3 ms by fan, 8.8 by group; 3,001 over
-        // 6k: 1.2 and 0.5), unless a low sun (slope above 4) stretches the fans (5,000 points
-        // over 61k triangles in January: 34 and 7.5 ms).
-        const bool fan = g_trace_mode[1] == 1 || (!rc.is_grid && 4 * rc.R < sc.T && sun.max_slope < 4.f);
-        if (e == cudaSuccess && fan) {
+        if (e == cudaSuccess && accrual_by_warps(sc, scene_box, rc, recv_box, sun)) {
             e = by_items(rg, sun, out, 1, st, [&](const TraceItems& it, unsigned ny) {
                 if (out.stats) k_accrual_fan<true><<<dim3(ctas, ny), T, 0, st>>>(sc, rg, sun, out, it);
                 else k_accrual_fan<false><<<dim3(ctas, ny), T, 0, st>>>(sc, rg, sun, out, it);

@@ -1,6 +1,6 @@
-"""The ray-traced accrual's walks by option: mode 1 is the warp-coherent walk for any receivers,
-which is also the default's choice for a thin point set; the work counters are those of the
-walk that runs, and no result depends on it."""
+"""The ray-traced accrual's walks: mode 1 is the warp-coherent walk for any receivers, which the
+default takes where points are few for the scene's triangles; the work counters are those
+of the walk that runs, and no result depends on it."""
 import numpy as np
 import pytest
 import torch
@@ -11,29 +11,66 @@ from synth.sun import sun_table
 pytestmark = pytest.mark.gpu
 
 
+def _by_mode(B, scene, recv, sun, mode):
+    B.sa_set_option(B.SA_OPT_ACCRUAL_TRAVERSAL, mode)
+    try:
+        return (B.sa_accumulate(scene, recv, sun, 4.0, "accrual_trace"),
+                B.sa_work_counters(scene, recv, sun, "accrual_trace"))
+    finally:
+        B.sa_set_option(B.SA_OPT_ACCRUAL_TRAVERSAL, 0)
+
+
+def _scene(B, n, extent):
+    city = C.city_district(C.SEED_BASE + 91, extent=extent, n_buildings=n)
+    m = C.extrude(city)
+    return city, B.Scene(m.verts, m.tris, m.tri_building, city.B)
+
+
 def test_packet_mode_and_its_counters(cuda_lib):
     B = cuda_lib
-    city = C.city_district(C.SEED_BASE + 91, extent=600.0, n_buildings=100)
-    m = C.extrude(city)
-    scene = B.Scene(m.verts, m.tris, m.tri_building, city.B)
+    _, scene = _scene(B, 100, 600.0)
     st = sun_table(40.7, [172, 200], 9.0, 16.5, 4.0)
     sun = B.Sun(st.dirs, st.day_start)
-    assert np.abs(st.dirs[:, :2] / st.dirs[:, 2:]).max() < 4.0
-    pos, nrm = C.facade_samples(city, 300, 5)
-    thin = B.Receivers.points(pos, nrm)                   # a quarter as many points as triangles are more
-    assert 4 * 300 < scene.info()["n_tris"]
     grid = B.Receivers.ground_grid(101.0, 83.0, 3.0, 75, 50)
-    counts, results = {}, {}
-    for name, recv in (("thin", thin), ("grid", grid)):
-        for mode in (0, 1):
-            B.sa_set_option(B.SA_OPT_ACCRUAL_TRAVERSAL, mode)
-            try:
-                results[name, mode] = B.sa_accumulate(scene, recv, sun, 4.0, "accrual_trace")
-                counts[name, mode] = B.sa_work_counters(scene, recv, sun, "accrual_trace")
-            finally:
-                B.sa_set_option(B.SA_OPT_ACCRUAL_TRAVERSAL, 0)
-        assert all(torch.equal(a, b) for a, b in zip(results[name, 0], results[name, 1])), name
-        assert int(results[name, 0][0].sum()) > 0
-    assert counts["thin", 0] == counts["thin", 1] != [0, 0, 0, 0]
+    (a, ca), (b, cb) = (_by_mode(B, scene, grid, sun, mode) for mode in (0, 1))
+    assert all(torch.equal(x, y) for x, y in zip(a, b)) and int(a[0].sum()) > 0
     # the grid's groups test a node once for 128 receivers, its warps once a receiver
-    assert counts["grid", 1][0] > 8 * counts["grid", 0][0] > 0
+    assert cb[0] > 8 * ca[0] > 0
+
+
+# about 29,000 triangles in a plan of 1,500 m; 8 blocks of 8 steps, slopes to 1.7
+@pytest.mark.parametrize("n,normals,corner,by_warps", [(700, True, 1.0, True), (20_000, True, 1.0, True),
+                                                       (20_000, False, 1.0, True), (80_000, True, 1.0, False),
+                                                       (20_000, False, 0.2, False)])
+def test_few_points_for_the_triangles_go_by_warps(cuda_lib, n, normals, corner, by_warps):
+    B = cuda_lib
+    city, scene = _scene(B, 900, 1500.0)
+    assert 25_000 < scene.info()["n_tris"] < 33_000
+    st = sun_table(40.7, [172], 9.0, 16.5, 8.0)
+    sun = B.Sun(st.dirs, st.day_start, 8)
+    assert sun.n_blocks == 8 and np.abs(st.dirs[:, :2] / st.dirs[:, 2:]).max() < 2.0
+    pos, nrm = C.facade_samples(city, n, 5)
+    if not normals:
+        pos = np.random.default_rng(4).uniform(0.0, 1500.0 * corner, (n, 3)).astype(np.float32)
+        pos[:, 2] *= 0.01
+    recv = B.Receivers.points(pos, nrm if normals else None)
+    (a, ca), (b, cb) = (_by_mode(B, scene, recv, sun, mode) for mode in (0, 1))
+    assert all(torch.equal(x, y) for x, y in zip(a, b)) and int(a[0].sum()) > 0
+    assert (ca == cb) == by_warps
+    c = B.sa_accumulate(scene, recv, sun, 4.0, "accrual_sam")
+    assert all(torch.equal(x, y) for x, y in zip(b, c))
+
+
+@pytest.mark.parametrize("n", [1, 31, 129, 700])
+@pytest.mark.parametrize("doys,step,block_len", [((172,), 4.0, 0), ((355, 20), 3.0, 64), ((80,), 8.0, 1)])
+def test_walks_by_warps_equal_the_light_space_map(cuda_lib, n, doys, step, block_len):
+    B = cuda_lib
+    city, scene = _scene(B, 100, 600.0)
+    pos, nrm = C.facade_samples(city, n, 5)
+    st = sun_table(40.7, list(doys), 9.0, 16.5, step)
+    sun = B.Sun(st.dirs, st.day_start, block_len)
+    for normals in (nrm, None):
+        recv = B.Receivers.points(pos, normals)
+        a, _ = _by_mode(B, scene, recv, sun, 1)
+        b = B.sa_accumulate(scene, recv, sun, 4.0, "accrual_sam")
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
