@@ -1078,8 +1078,8 @@ sa_status sa_building_contribution(const sa_scene* scene, const sa_receivers* gr
         }
     }
     unsigned long long h[2] = {0ull, 0ull};
-    cudaError_t e = sa::launch_building_contribution(dev_scene(scene), dev_recv(grid), dsun, runs,
-                                                     scene->n_buildings, poly_xy, n, casting, nearest, h,
+    cudaError_t e = sa::launch_building_contribution(dev_scene(scene), scene->box, dev_recv(grid), dsun, runs,
+                                                     sun->h_steps, scene->n_buildings, poly_xy, n, casting, nearest, h,
                                                      as_stream(stream));
     if (e != cudaSuccess) return cuda_fail(e, who);
     const sa_status chk = sa::check_after_call(as_stream(stream), who);

@@ -644,8 +644,9 @@ cudaError_t launch_height_grad(const DevScene& sc, const FootprintSet& fs, const
 // nearest_out are host arrays of n_buildings, stats_out two host counters (cell-steps past
 // 64 buildings, shadowed cell-steps whose ray met no building)
 constexpr int kContribRun = 16;   // steps of a run, at the most
-cudaError_t launch_building_contribution(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
-                                         const std::vector<BlockConst>& runs, int n_buildings,
+cudaError_t launch_building_contribution(const DevScene& sc, const float* scene_box, const DevRecv& rc, const DevSun& sun,
+                                         const std::vector<BlockConst>& runs,
+                                         const std::vector<StepConst>& h_steps, int n_buildings,
                                          const float* poly_xy, int n, double* casting_out,
                                          double* nearest_out, unsigned long long* stats_out,
                                          cudaStream_t st);
