@@ -528,14 +528,10 @@ k_contribution_fan(ContribArgs a) {
         int n = 0;
         bool more = false;
         for (int i = 0; i < a.sc.n_nodes;) {
-            float4 lo = __ldg(&a.sc.nodes[2 * i]), hi = __ldg(&a.sc.nodes[2 * i + 1]);
+            const float4 lo = __ldg(&a.sc.nodes[2 * i]), hi = __ldg(&a.sc.nodes[2 * i + 1]);
             const int esc = SA_ESC(__float_as_int(lo.w), i, a.sc.n_nodes, sa::CK_TRACE_ESCAPE);
             const int tri = SA_LEAF(__float_as_int(hi.w), a.sc.T, sa::CK_TRACE_LEAF);
-            // the fan's slack, so that a box's rounding loses no hit that the walk above found
-            const float pad = fmaf(1e-5f, fabsf(lo.x - o.x) + fabsf(lo.y - o.y) + hi.z + (hi.x - lo.x) + (hi.y - lo.y), 1e-4f);
-            lo.x -= pad; lo.y -= pad; lo.z -= pad;
-            hi.x += pad; hi.y += pad; hi.z += pad;
-            if (!hit_box(o, r.x, r.y, r.z, lo, hi)) {
+            if (!hit_box_before(o, r.x, r.y, r.z, lo, hi, 3.4e38f)) {
                 i = esc;
                 continue;
             }

@@ -824,7 +824,7 @@ static sa_status run_method(const sa_scene* scene, const sa_receivers* recv, con
         e = sa::scratch_alloc(&run, sizeof(int) * (size_t)R, st);
         if (e != cudaSuccess) return cuda_fail(e, who);
         out.run = run;
-        e = sa::launch_iam(dsc, drc, dsun, iam_levels ? iam_levels : 3, out, st);
+        e = sa::launch_iam(dsc, scene->box, drc, dsun, iam_levels ? iam_levels : 3, out, st);
     } else if (raster) {
         e = sa::scratch_alloc(&run, sizeof(int) * (size_t)R, st);
         if (e != cudaSuccess) return cuda_fail(e, who);

@@ -221,6 +221,76 @@ k_iam_sources(DevScene sc, Grid g, const StepConst* __restrict__ steps, const Ia
     }
 }
 
+// The L nearest hits of the warp's rays toward step s, in order (bits of the distances, past the
+// last 0xffffffff), by one walk of the node list: a node is entered when any ray meets it
+// before its L-th hit so far.
+template <int KZ>
+__device__ __forceinline__ void nearest_by_warp(const DevScene& sc, const float3& o, const StepConst& s, bool active, int L,
+                                                unsigned* best) {
+#pragma unroll
+    for (int l = 0; l < kMaxLevels; ++l) best[l] = 0xffffffffu;
+    float last = 3.4e38f;
+    for (int i = __any_sync(kFull, active) ? 0 : sc.n_nodes; i < sc.n_nodes;) {
+        const float4 lo = __ldg(&sc.nodes[2 * i]);
+        const float4 hi = __ldg(&sc.nodes[2 * i + 1]);
+        const int esc = SA_ESC(__float_as_int(lo.w), i, sc.n_nodes, sa::CK_TRACE_ESCAPE);
+        const int tri = SA_LEAF(__float_as_int(hi.w), sc.T, sa::CK_TRACE_LEAF);
+        const bool in = active && hit_box_before(o, s.ix, s.iy, s.iz, lo, hi, last);
+        if (tri < 0) {
+            i = __any_sync(kFull, in) ? i + 1 : esc;
+            continue;
+        }
+        i = esc;
+        float t;
+        if (!in || !hit_tri_t<KZ>(o, __ldg(&sc.tris[3 * tri]), __ldg(&sc.tris[3 * tri + 1]), __ldg(&sc.tris[3 * tri + 2]), s.Sx,
+                                  s.Sy, s.Sz, kSourceTmin, &t)) continue;
+        unsigned v = __float_as_uint(t);
+#pragma unroll
+        for (int l = 0; l < kMaxLevels; ++l) {
+            if (l >= L) break;
+            const unsigned b = best[l];
+            best[l] = min(b, v);
+            v = max(b, v);
+            if (l == L - 1 && best[l] != 0xffffffffu) last = __uint_as_float(best[l]);
+        }
+    }
+}
+
+// The scene's triangles over the ground of a group's 128 cells from which its box holds too many
+// of them against what its rays meet, and the sources are found by warps.  Whole call, ms
+// by groups / by warps, 122k triangles, 481 steps in June: 268 triangles 0.77 / 1.05, 1,677
+// 0.94 / 0.68, 6,708 4.1 / 0.79, 47,702 34 / 1.1; in December 745 2.2 / 3.0, 3,773 3.3 / 3.9,
+// 11,925 8.8 / 5.6; hour steps 745 0.73 / 0.85, 3,773 2.5 / 1.3.
+constexpr double kGroupHeld = 1600.0;
+
+// The same sources by warps of 8 x 4 cells and end, for cells far apart (kGroupHeld).
+__global__ void __launch_bounds__(32 * kWarps)
+k_iam_sources_warp(DevScene sc, Grid g, const StepConst* __restrict__ steps, const BlockConst* __restrict__ blocks, int L,
+                   float* __restrict__ src) {
+    const int lane = threadIdx.x & 31;
+    const long long warp_id = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5);
+    const int tiles_x = (g.nx + 7) >> 3, end = blockIdx.y;
+    const long long ty = warp_id / tiles_x;
+    const int tx = (int)(warp_id - ty * tiles_x);
+    const int ix = tx * 8 + (lane & 7);
+    const long long iy = ty * 4 + (lane >> 3);
+    const bool active = ix < g.nx && iy < g.ny;
+    const BlockConst& bc = blocks[end >> 1];
+    const StepConst s = steps[end & 1 ? bc.j0 + bc.K - 1 : bc.j0];
+    const float3 o = make_float3(__fadd_rn(g.x0, __fmul_rn(__fadd_rn((float)ix, 0.5f), g.dx)),
+                                 __fadd_rn(g.y0, __fmul_rn(__fadd_rn((float)iy, 0.5f), g.dx)), 0.f);
+    unsigned best[kMaxLevels];
+    if (s.kz == 2) nearest_by_warp<2>(sc, o, s, active, L, best);
+    else if (s.kz == 0) nearest_by_warp<0>(sc, o, s, active, L, best);
+    else nearest_by_warp<1>(sc, o, s, active, L, best);
+    if (!active) return;
+    const long long R = (long long)g.nx * g.ny;
+    float* out = src + (long long)end * L * R + iy * g.nx + ix;
+#pragma unroll
+    for (int l = 0; l < kMaxLevels; ++l)
+        if (l < L) out[(long long)l * R] = best[l] == 0xffffffffu ? 0.f : __uint_as_float(best[l]);
+}
+
 // A CTA lists the sources of its 128 cells, 32 in a patch of 8 x 4 per warp; then its threads
 // draw them, one line per thread whichever cell it comes from: most cells are lit or have two
 // sources where their neighbours have four, and a warp that drew its own cells' sources
@@ -312,11 +382,14 @@ __global__ void k_iam_fold(long long R, const BlockConst* __restrict__ blocks, i
 
 }  // namespace
 
-cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
+cudaError_t launch_iam(const DevScene& sc, const float* scene_box, const DevRecv& rc, const DevSun& sun,
                        int L, const DevOut& out, cudaStream_t st) {
     const long long R = (long long)rc.nx * rc.ny;
     if (R == 0) return cudaSuccess;
     if (L < 1 || L > kMaxLevels) return cudaErrorInvalidValue;
+    const double area = ((double)scene_box[3] - scene_box[0]) * ((double)scene_box[4] - scene_box[1]);
+    const double held = area > 0.0 ? (double)sc.T * kTileThreads * (double)rc.dx * rc.dx / area : 0.0;
+    const bool by_warps = held > kGroupHeld;
     // the blocks go in one launch, as many as 1 GiB of masks and sources holds, or the memory
     // there is
     int chunk = (int)std::max(1ll, std::min({(long long)sun.n_blocks, 32767ll, (1ll << 30) / ((8ll + 8ll * L) * R)}));
@@ -339,8 +412,12 @@ cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
             KernelTimer kt(KT_IAM, st);
             const dim3 groups((unsigned)((rc.nx + kPatchX - 1) / kPatchX) * (unsigned)((rc.ny + kPatchY - 1) / kPatchY),
                               2u * (unsigned)nbc);
-            k_iam_walks<<<(2 * nbc + 63) / 64, 64, 0, st>>>(sun.steps, sun.blocks + b0, nbc, d_walks, runs);
-            k_iam_sources<<<groups, kTileThreads, 0, st>>>(sc, g, sun.steps, d_walks, runs, L, src);
+            if (by_warps) {
+                k_iam_sources_warp<<<dim3(ctas, 2u * (unsigned)nbc), 32 * kWarps, 0, st>>>(sc, g, sun.steps, sun.blocks + b0, L, src);
+            } else {
+                k_iam_walks<<<(2 * nbc + 63) / 64, 64, 0, st>>>(sun.steps, sun.blocks + b0, nbc, d_walks, runs);
+                k_iam_sources<<<groups, kTileThreads, 0, st>>>(sc, g, sun.steps, d_walks, runs, L, src);
+            }
             const dim3 grid(ctas, (unsigned)nbc);
             if (R < (1ll << 31)) k_iam_draw<unsigned><<<grid, 32 * kWarps, 0, st>>>(g, sun.steps, sun.blocks + b0, L, src, masks);
             else k_iam_draw<long long><<<grid, 32 * kWarps, 0, st>>>(g, sun.steps, sun.blocks + b0, L, src, masks);

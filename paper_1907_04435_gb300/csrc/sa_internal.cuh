@@ -484,6 +484,21 @@ __device__ __forceinline__ bool hit_box(const float3& o, float ix, float iy, flo
     return tn <= tf * 1.0000005f;
 }
 
+// The same before distance tmax, for a box widened by more than the roundings of the exact tests
+// within it, so that no hit there is lost.
+__device__ __forceinline__ bool hit_box_before(const float3& o, float ix, float iy, float iz, float4 lo, float4 hi,
+                                               float tmax) {
+    const float pad = fmaf(1e-5f, fabsf(lo.x - o.x) + fabsf(lo.y - o.y) + fabsf(hi.z) + (hi.x - lo.x) + (hi.y - lo.y), 1e-4f);
+    lo.x -= pad; lo.y -= pad; lo.z -= pad;
+    hi.x += pad; hi.y += pad; hi.z += pad;
+    const float tx0 = (lo.x - o.x) * ix, tx1 = (hi.x - o.x) * ix;
+    const float ty0 = (lo.y - o.y) * iy, ty1 = (hi.y - o.y) * iy;
+    const float tz0 = (lo.z - o.z) * iz, tz1 = (hi.z - o.z) * iz;
+    const float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.f));
+    const float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1));
+    return tn <= tf * 1.0000005f && tn <= tmax;
+}
+
 // Plücker form of the exact ray/triangle test for one origin and many steps.  For the
 // line through o along d, the side of edge v -> v' is  d . ((v - o) x (v' - o)):  the
 // moment m_e = (v - o) x (v' - o) depends only on the origin and the edge, so a triangle
@@ -741,7 +756,7 @@ cudaError_t launch_sam_points(const DevScene& sc, const float* scene_box, const 
                               cudaStream_t st);
 
 // inverse accrual map of a ground grid
-cudaError_t launch_iam(const DevScene& sc, const DevRecv& rc, const DevSun& sun,
+cudaError_t launch_iam(const DevScene& sc, const float* scene_box, const DevRecv& rc, const DevSun& sun,
                        int L, const DevOut& out, cudaStream_t st);
 
 // LBVH build (device), returns node / triangle arrays owned by the caller
