@@ -836,7 +836,7 @@ static sa_status run_method(const sa_scene* scene, const sa_receivers* recv, con
         e = sa::launch_sam_points(dsc, scene->box, drc, recv->box, dsun, sun->h_blocks, sun->h_steps,
                                   out, st);
     } else {
-        e = sa::launch_accrual_trace(dsc, scene->box, drc, recv->box, dsun, out, st);
+        e = sa::launch_accrual_trace(dsc, scene->box, drc, recv->box, dsun, sun->h_blocks, sun->h_steps, out, st);
     }
     if (run) cudaFreeAsync(run, st);
     if (e != cudaSuccess) return cuda_fail(e, who);

@@ -620,7 +620,11 @@ cudaError_t launch_sweep_trace(const DevScene& sc, const DevRecv& rc, const DevS
                                const DevOut& out, cudaStream_t st);
 // (scene_box, and recv_box of point receivers: lo.xyz hi.xyz)
 cudaError_t launch_accrual_trace(const DevScene& sc, const float* scene_box, const DevRecv& rc, const float* recv_box,
-                                 const DevSun& sun, const DevOut& out, cudaStream_t st);
+                                 const DevSun& sun, const std::vector<BlockConst>& h_blocks,
+                                 const std::vector<StepConst>& h_steps, const DevOut& out, cudaStream_t st);
+// Pieces of a block for the grouped walk, `parts` or a multiple of it up to `most`: as many as
+// bring the drift box of every piece's rays (its area, per square metre of rise) to `limit`.
+int drift_parts(const BlockConst& b, const std::vector<StepConst>& steps, int parts, int most, double limit);
 // traversal mode of the sweep (which = 0) and accrual (which = 1) kernels
 void set_trace_mode(int which, int mode);
 int get_trace_mode(int which);

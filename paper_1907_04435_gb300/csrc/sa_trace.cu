@@ -597,8 +597,41 @@ static bool accrual_by_warps(const DevScene& sc, const float* box, const DevRecv
     return (double)rc.R < 2.2 * f * (share * sc.T - 6000.0 * slope);
 }
 
+int drift_parts(const BlockConst& b, const std::vector<StepConst>& steps, int parts, int most, double limit) {
+    // the drift is the ground slopes' spread, foreshortened: no side passes their box's diagonal
+    const double ux = (double)b.uxhi - b.uxlo, uy = (double)b.uyhi - b.uylo;
+    if (ux * ux + uy * uy <= limit) return parts;
+    const int base = parts;
+    while (parts < most) {
+        bool wide = false;
+        for (int q = 0; q < parts && !wide; ++q) {
+            const int k0 = q * b.K / parts, kn = (q + 1) * b.K / parts - k0, j = b.j0 + k0;
+            if (kn < 2) continue;
+            const LightBasis L = light_basis(steps[(size_t)(j + kn / 2)], steps[(size_t)j], steps[(size_t)(j + kn - 1)]);
+            LightStep s = light_drift(L, steps[(size_t)j]);
+            for (int k = 1; k < kn; ++k) light_merge(s, light_drift(L, steps[(size_t)(j + k)]));
+            wide = (s.da_hi - s.da_lo) * (s.db_hi - s.db_lo) > limit;
+        }
+        if (!wide) break;
+        parts += base;
+    }
+    return std::min(parts, most);
+}
+
+// A run's box is widened by its rays' drift, so a run whose rays spread far -- a low sun, or
+// hours between its first step and last -- reaches most of a city, and its groups work for
+// all of it: shorter runs then, by the largest drift box of any (area per square metre of
+// rise; 0.02 of a June day's 27-minute runs, 9 of a December day's, 225 where a 2-hour run
+// takes in sunrise).  400^2 cells at 0.5 m over 61,676 triangles, ms for a largest box of
+// 225 / 50 / 9 / 1.8: 26 / 6.7 / 1.4 / 0.93; 15 minutes a step until sunset 19 / 6.6 / 2 / 0.5: 7.8 /
+// 3.1 / 1.4 / 0.67; December 9 / 2.4 / 0.7 / 0.2: 4.1 / 2.3 / 2.9 / 4.9.  The groups of points are
+// wide themselves (60,000 facade points: December 7.5 / 10 / 15 / 25, sunrise 18 / 8.7 / 6.1 /
+// 6.3).
+constexpr double kDriftGrid = 4.0, kDriftPoints = 12.0;
+
 cudaError_t launch_accrual_trace(const DevScene& sc, const float* scene_box, const DevRecv& rc, const float* recv_box,
-                                 const DevSun& sun, const DevOut& out, cudaStream_t st) {
+                                 const DevSun& sun, const std::vector<BlockConst>& h_blocks,
+                                 const std::vector<StepConst>& h_steps, const DevOut& out, cudaStream_t st) {
     const long long warps = host_warps(rc);
     if (warps == 0) return cudaSuccess;
     const unsigned ctas = (unsigned)((warps + kWarpsPerCta - 1) / kWarpsPerCta);
@@ -629,8 +662,12 @@ cudaError_t launch_accrual_trace(const DevScene& sc, const float* scene_box, con
                 return cudaGetLastError();
             });
         } else if (e == cudaSuccess) {
-            // runs of balanced lengths: every block in as many pieces as the longest needs
-            const int parts = (sun.max_K + kAccrualRun - 1) / kAccrualRun;
+            // runs of balanced lengths: every block in as many pieces as any needs
+            const int base = (sun.max_K + kAccrualRun - 1) / kAccrualRun;
+            int parts = base;
+            for (const BlockConst& b : h_blocks)
+                parts = std::max(parts, drift_parts(b, h_steps, base, std::min(16 * base, sun.max_K),
+                                                    rc.is_grid ? kDriftGrid : kDriftPoints));
             const unsigned groups = (unsigned)(rc.is_grid ? (long long)((rc.nx + 15) / 16) * ((rc.ny + 7) / 8)
                                                           : (rc.R + kTileThreads - 1) / kTileThreads);
             RunLight* runs = nullptr;

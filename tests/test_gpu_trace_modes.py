@@ -74,3 +74,29 @@ def test_walks_by_warps_equal_the_light_space_map(cuda_lib, n, doys, step, block
         a, _ = _by_mode(B, scene, recv, sun, 1)
         b = B.sa_accumulate(scene, recv, sun, 4.0, "accrual_sam")
         assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("doy,t0,t1,step,block_len", [(233, 5.0, 13.0, 5.0, 0), (282, 11.0, 17.0, 15.0, 64),
+                                                      (80, 6.0, 18.0, 10.0, 0), (172, 4.6, 19.4, 15.0, 1),
+                                                      (355, 8.0, 16.0, 1.0, 33), (172, 8.0, 18.0, 60.0, 7)])
+def test_runs_whose_rays_spread_far(cuda_lib, doy, t0, t1, step, block_len):
+    """Sunrise, sunset and hours between the steps: runs are cut by their drift, into pieces of
+    down to one step, without a change of the results."""
+    B = cuda_lib
+    city, scene = _scene(B, 100, 600.0)
+    st = sun_table(40.7, [doy], t0, t1, step)
+    sun = B.Sun(st.dirs, st.day_start, block_len)
+    pos, nrm = C.facade_samples(city, 3000, 5)
+    for recv in (B.Receivers.points(pos, nrm), B.Receivers.points(pos)):
+        a, b = (B.sa_accumulate(scene, recv, sun, step, m) for m in ("accrual_trace", "accrual_sam"))
+        assert all(torch.equal(x, y) for x, y in zip(a, b)) and int(a[0].sum()) > 0
+    nx, ny, dx = 71, 45, 4.0
+    grid = B.Receivers.ground_grid(101.0, 83.0, dx, nx, ny)
+    a, c = B.sa_accumulate(scene, grid, sun, step, "accrual_trace"), _by_mode(B, scene, grid, sun, 1)[0]
+    xs = np.float32(101.0) + (np.arange(nx, dtype=np.float32) + np.float32(0.5)) * np.float32(dx)
+    ys = np.float32(83.0) + (np.arange(ny, dtype=np.float32) + np.float32(0.5)) * np.float32(dx)
+    X, Y = np.meshgrid(xs, ys)
+    pts = B.Receivers.points(np.stack([X.ravel(), Y.ravel(), np.zeros(nx * ny)], 1).astype(np.float32))
+    b = B.sa_accumulate(scene, pts, sun, step, "accrual_sam")
+    assert torch.equal(a[0], b[0]) and torch.equal(a[2], b[2])
+    assert torch.equal(a[0], c[0]) and torch.equal(a[2], c[2])
