@@ -41,6 +41,9 @@ __global__ void k_regroup_keys(const float4* __restrict__ orig, long long R, flo
     vals[s] = (unsigned)s;
 }
 
+// 192 triangles, 60,000 points by 29 to 481 steps: 0.21 to 0.30 ms sorted, 0.15 to 0.23 as they come.
+constexpr int kRegroupTris = 1000;
+
 struct Receiver {
     float3 o;
     float tmin;
@@ -644,7 +647,8 @@ cudaError_t launch_accrual_trace(const DevScene& sc, const float* scene_box, con
         DevRecv rg = rc;
         unsigned *keys = nullptr, *order = nullptr;
         cudaError_t e = cudaSuccess;
-        if (!rc.is_grid && rc.nrm) {
+        // (a small scene's few triangles are all staged by any group)
+        if (!rc.is_grid && rc.nrm && sc.T >= kRegroupTris) {
             e = sa::scratch_alloc(&keys, sizeof(unsigned) * (size_t)rc.R, st);
             if (e == cudaSuccess) e = sa::scratch_alloc(&order, sizeof(unsigned) * (size_t)rc.R, st);
             const float ext = std::max({recv_box[3] - recv_box[0], recv_box[4] - recv_box[1], recv_box[5] - recv_box[2]});

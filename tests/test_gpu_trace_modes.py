@@ -100,3 +100,19 @@ def test_runs_whose_rays_spread_far(cuda_lib, doy, t0, t1, step, block_len):
     b = B.sa_accumulate(scene, pts, sun, step, "accrual_sam")
     assert torch.equal(a[0], b[0]) and torch.equal(a[2], b[2])
     assert torch.equal(a[0], c[0]) and torch.equal(a[2], c[2])
+
+
+@pytest.mark.parametrize("n", [1, 129, 5000])
+def test_points_of_a_small_scene(cuda_lib, n):
+    """Under 1,000 triangles facade points are taken in their own order."""
+    B = cuda_lib
+    city = C.city_boxes(C.SEED_BASE + 1)
+    m = C.extrude(city)
+    assert len(m.tris) < 1000
+    scene = B.Scene(m.verts, m.tris, m.tri_building, city.B)
+    st = sun_table(40.7, [172, 355], 9.0, 16.0, 7.0)
+    sun = B.Sun(st.dirs, st.day_start)
+    pos, nrm = C.facade_samples(city, n, 5)
+    recv = B.Receivers.points(pos, nrm)
+    a, b = (B.sa_accumulate(scene, recv, sun, 7.0, m) for m in ("accrual_trace", "accrual_sam"))
+    assert all(torch.equal(x, y) for x, y in zip(a, b)) and (n == 1 or int(a[0].sum()) > 0)
