@@ -1059,7 +1059,8 @@ sa_status sa_building_contribution(const sa_scene* scene, const sa_receivers* gr
     dsun.blocks = sun->d_blocks;
     dsun.S = sun->S;
     dsun.n_blocks = (int)sun->h_blocks.size();
-    // runs of <= kContribRun steps of each block, pointing into the block's mask
+    // runs of <= kContribRun steps of each block, cut by their rays' drift, pointing into the
+    // block's mask
     std::vector<float> dirs(3 * (size_t)sun->S);
     for (int j = 0; j < sun->S; ++j) {
         dirs[3 * (size_t)j] = sun->h_steps[j].dx;
@@ -1068,7 +1069,8 @@ sa_status sa_building_contribution(const sa_scene* scene, const sa_receivers* gr
     }
     std::vector<sa::BlockConst> runs;
     for (const sa::BlockConst& b : sun->h_blocks) {
-        const int nsub = (b.K + sa::kContribRun - 1) / sa::kContribRun;
+        const int nsub = sa::drift_parts(b, sun->h_steps, (b.K + sa::kContribRun - 1) / sa::kContribRun, b.K,
+                                         sa::kContribDrift);
         for (int q = 0; q < nsub; ++q) {
             const int k0 = q * b.K / nsub, k1 = (q + 1) * b.K / nsub;
             sa::BlockConst r = make_block(dirs.data(), sun->h_steps, b.j0 + k0, k1 - k0, 0, true);

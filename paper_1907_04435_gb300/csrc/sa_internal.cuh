@@ -662,7 +662,8 @@ cudaError_t launch_height_grad(const DevScene& sc, const FootprintSet& fs, const
 // building contribution over a polygonal region (sa_analysis.cu); casting_out and
 // nearest_out are host arrays of n_buildings, stats_out two host counters (cell-steps past
 // 64 buildings, shadowed cell-steps whose ray met no building)
-constexpr int kContribRun = 16;   // steps of a run, at the most
+constexpr int kContribRun = 16;   // steps of a run, at the most,
+constexpr double kContribDrift = 4.0;   // and its drift box's area (drift_parts)
 cudaError_t launch_building_contribution(const DevScene& sc, const float* scene_box, const DevRecv& rc, const DevSun& sun,
                                          const std::vector<BlockConst>& runs,
                                          const std::vector<StepConst>& h_steps, int n_buildings,
