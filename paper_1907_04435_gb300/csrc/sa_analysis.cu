@@ -228,8 +228,13 @@ struct ContribCell {
 
 __device__ __forceinline__ ContribCell contrib_cell(const ContribArgs& a) {
     ContribCell c;
+    // the first run whose CTAs end past this one (runs without cells have none)
     c.r = 0;
-    while (a.cta_base[c.r + 1] <= (int)blockIdx.x) ++c.r;
+    for (int end = a.n_runs - 1; c.r < end;) {
+        const int mid = (c.r + end) >> 1;
+        if (a.cta_base[mid + 1] <= (int)blockIdx.x) c.r = mid + 1;
+        else end = mid;
+    }
     const unsigned slot = (unsigned)((int)blockIdx.x - a.cta_base[c.r]) * (unsigned)kTileThreads + threadIdx.x;
     c.live = slot < a.n_items[c.r];
     const long long cell = c.live ? (long long)SA_CHK(a.items[(long long)a.item0[c.r] + slot], a.R, sa::CK_CONTRIB_CELL) : 0;
