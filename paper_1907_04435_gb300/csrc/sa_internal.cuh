@@ -446,31 +446,12 @@ __device__ __forceinline__ bool hit_tri(const float3& o, const float4& a, const 
     return det > 0.f ? (T > tmin * det) : (T < tmin * det);
 }
 
-// the same decision, returning the hit distance T / det (in units of |d|), or -1
-template <int KZ>
-__device__ __forceinline__ float hit_tri_dist(const float3& o, const float4& a, const float4& b,
-                                              const float4& c, float Sx, float Sy, float Sz,
-                                              float tmin) {
-    float T, det;
-    if (!woop_td<KZ>(o, a, b, c, Sx, Sy, Sz, T, det)) return -1.f;
-    const bool ahead = det > 0.f ? (T > tmin * det) : (T < tmin * det);
-    return ahead ? T / det : -1.f;
-}
-
 __device__ __forceinline__ bool hit_tri_any(int kz, const float3& o, const float4& a,
                                             const float4& b, const float4& c,
                                             const StepConst& s, float tmin) {
     if (kz == 2) return hit_tri<2>(o, a, b, c, s.Sx, s.Sy, s.Sz, tmin);
     if (kz == 0) return hit_tri<0>(o, a, b, c, s.Sx, s.Sy, s.Sz, tmin);
     return hit_tri<1>(o, a, b, c, s.Sx, s.Sy, s.Sz, tmin);
-}
-
-__device__ __forceinline__ float hit_dist_any(int kz, const float3& o, const float4& a,
-                                              const float4& b, const float4& c,
-                                              const StepConst& s, float tmin) {
-    if (kz == 2) return hit_tri_dist<2>(o, a, b, c, s.Sx, s.Sy, s.Sz, tmin);
-    if (kz == 0) return hit_tri_dist<0>(o, a, b, c, s.Sx, s.Sy, s.Sz, tmin);
-    return hit_tri_dist<1>(o, a, b, c, s.Sx, s.Sy, s.Sz, tmin);
 }
 
 // Slab test of the ray o + t d, t in [0, inf), against a (padded) box.
@@ -562,20 +543,6 @@ __device__ __forceinline__ bool plucker_hit(const PluckerTri& p, float dx, float
     if (nd == 0.f) return false;
     const float lim = __fmul_rn(tmin, nd);
     return nd > 0.f ? (p.aon > lim) : (p.aon < lim);
-}
-
-// the same decision as plucker_hit, evaluated without early exits, so the steps of a run
-// form independent chains
-__device__ __forceinline__ bool plucker_hit_all(const PluckerTri& p, float dx, float dy, float dz,
-                                                float tmin) {
-    const float s0 = fmaf(dz, p.m[0][2], fmaf(dy, p.m[0][1], __fmul_rn(dx, p.m[0][0])));
-    const float s1 = fmaf(dz, p.m[1][2], fmaf(dy, p.m[1][1], __fmul_rn(dx, p.m[1][0])));
-    const float s2 = fmaf(dz, p.m[2][2], fmaf(dy, p.m[2][1], __fmul_rn(dx, p.m[2][0])));
-    const float nd = fmaf(dz, p.nz, fmaf(dy, p.ny, __fmul_rn(dx, p.nx)));
-    const bool inside = fminf(s0, fminf(s1, s2)) >= 0.f || fmaxf(s0, fmaxf(s1, s2)) <= 0.f;
-    const float lim = __fmul_rn(tmin, nd);
-    const bool ahead = (nd > 0.f && p.aon > lim) || (nd < 0.f && p.aon < lim);
-    return inside && ahead;
 }
 
 // --------------------------------------------------------------- host-side launchers

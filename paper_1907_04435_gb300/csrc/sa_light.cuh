@@ -276,7 +276,7 @@ __device__ __forceinline__ void drain_pairs(Smem& sm, const unsigned short* q, i
     const float4 nv = sm.n[t];
     const PluckerTri pt = plucker_setup_n(o, a, b, c, make_float3(nv.x, nv.y, nv.z));
     // every step of the run is tested without branches, two steps per packed instruction
-    // (the same roundings as plucker_hit_all); steps the triangle turns away from, and the
+    // (the same roundings as plucker_hit); steps the triangle turns away from, and the
     // repeated step of an odd run's last pair, are masked off afterwards
     unsigned long long M[3][3];
 #pragma unroll
