@@ -58,9 +58,10 @@ typedef enum {
  *                     the triangles onto the ground separately (the per-minute
  *                     shadow-map baseline, Sec. 8.1).  Ground grids only.
  *   SA_ACCRUAL_TRACE  ray-traced accrual: one BVH traversal per group of 128 neighbouring
- *                     receivers and run of <= 27 steps (per warp and block for thin point
- *                     sets), whose query is the whole fan of the run's rays (the
- *                     moving-shadow observation of Sec. 3.2 applied to rays).
+ *                     receivers and run of <= 27 steps, fewer where its rays spread far
+ *                     (per warp and block for points that are few for the triangles),
+ *                     whose query is the whole fan of the run's rays (the moving-shadow
+ *                     observation of Sec. 3.2 applied to rays).
  *   SA_ACCRUAL_SAM    shadow accrual map (Sec. 4): one pass over the geometry serves all
  *                     the steps of a block (ground grids: the receiver-space accrual
  *                     raster) or of a run of <= 32 steps (points: a light-space map
@@ -91,8 +92,8 @@ int32_t sa_version(void);
  *   SA_OPT_SWEEP_TRAVERSAL, SA_OPT_ACCRUAL_TRAVERSAL: BVH traversal of the ray-traced
  *   methods -- 1 warp-coherent (the 32 lanes of a warp walk the node list together), 2 one
  *   traversal per lane, 0 the default (per lane for the sweep; for the accrual one per
- *   group of 128 receivers, or warp-coherent for thin point sets, the faster of the two
- *   there).  Results do not depend on the option.
+ *   group of 128 receivers, or warp-coherent for points that are few for the triangles, the
+ *   faster of the two there).  Results do not depend on the option.
  *   SA_OPT_RASTER_RUN: at most this many steps the ground accrual raster tests per cell
  *   set-up (1..32, default 24), and SA_OPT_POINT_RUN: at most this many steps per
  *   light-space map of point receivers (1..32, default 27); each block is split into
@@ -104,8 +105,9 @@ int32_t sa_version(void);
  *   stream capture, and those of sa_accumulate_grid_noalloc, are never timed.
  *   SA_OPT_BATCH_TILE_SKIP: read by sa_batch_create.  1 (default): a work item whose tile
  *   no removed building and no tower can shadow during the interval keeps the base counts
- *   without rastering; 0: every tile of every region is rastered.  Results do not depend
- *   on the option; 0 exists to measure what the skipping saves.
+ *   without rastering, and the others are put together from the base city's masks, block by
+ *   block, where those fit; 0: every tile of every region is rastered whole, without the
+ *   masks.  Results do not depend on the option; 0 exists to measure what both save.
  * sa_get_option returns the current value, or -1 for an unknown key. */
 #define SA_OPT_SWEEP_TRAVERSAL 1
 #define SA_OPT_ACCRUAL_TRAVERSAL 2
@@ -340,7 +342,7 @@ int32_t sa_batch_affected_items(const sa_batch* b);
 sa_status sa_batch_run(sa_batch* b, int32_t* counts, int32_t* impact, void* stream);
 /* Autotuner: times 2 to 6 persistent CTAs per SM (as many as the raster kernels are built
  * to hold) x raster runs of 8, 16 or 24 steps on an eighth of the work items and keeps the
- * fastest; reports the choice. */
+ * fastest; reports the choice.  (5 at the most where tiles are rastered whole.) */
 sa_status sa_batch_tune(sa_batch* b, int32_t* best_ctas, int32_t* best_run, void* stream);
 /* Work counters of one batch run (counters [2] cell set-ups, [3] cell-step tests). */
 sa_status sa_batch_work_counters(sa_batch* b, uint64_t* counters, void* stream);
@@ -363,8 +365,8 @@ sa_status sa_work_counters(const sa_scene* scene, const sa_receivers* recv, cons
  * every index its kernels take from data -- a BVH leaf's triangle, an escape link, a
  * binned triangle or receiver, a permutation entry, a tile cell, a building id -- before
  * using it.  The first index out of range is recorded (site, index, bound) and replaced by
- * one in range (an escape link by the end of the node list), so that no access leaves its
- * buffer and no loop runs on; the computing calls (sa_accumulate, sa_shadow_masks,
+ * one in range (an escape link by the end of the node list; a grouped walk drops children out
+ * of place), so that no access leaves its buffer and no loop runs on; the computing calls (sa_accumulate, sa_shadow_masks,
  * sa_accumulate_graph, sa_height_grad, sa_building_contribution, sa_batch_run,
  * sa_accumulate_grid_noalloc) then synchronise their stream and return SA_ERR_INTERNAL
  * naming the site.  In the plain build the checks compile to nothing.
@@ -488,9 +490,9 @@ sa_status sa_shadow_score(const sa_receivers* grid, const int32_t* steps, int32_
  * The shadowed steps come from the ground accrual raster (as SA_ACCRUAL_SAM computes
  * them); the call keeps its per-step masks, 8 bytes per cell and block of steps, and
  * rejects with SA_ERR_INVALID_ARG a grid and sun table whose masks exceed 4 GiB (split the
- * interval).  The buildings are found by one traversal per group of 128 cells and run of
- * <= 16 steps, whose query is the fan of the run's rays (as SA_ACCRUAL_TRACE), testing every
- * triangle in it against the cells' shadowed steps with the exact ray test.  Synchronises
+ * interval).  The buildings are found by one traversal per group of 128 cells (per warp of 32
+ * where they lie far apart) and run of <= 16 steps, whose query is the fan of the run's rays
+ * (as SA_ACCRUAL_TRACE), testing every triangle in it against the cells' shadowed steps with the exact ray test.  Synchronises
  * `stream`.  Errors: SA_ERR_INVALID_ARG (NULL, not a grid, n < 3), SA_ERR_DEGENERATE
  * (non-finite vertex), SA_ERR_UNSUPPORTED (geometry below z = 0, as for the raster
  * methods; a ray meeting more than 64 buildings, above), SA_ERR_OOM, SA_ERR_CUDA. */

@@ -402,8 +402,8 @@ __device__ __forceinline__ double slerp_param(const ArcConst& c, double be) {
     if (c.inv_theta == 0.0) return be;
     double ang;
     if (c.theta < 0.1) {
-        // steps up to about 20 minutes: the arctangent's power series (the next term is below
-        // 1e-18 of the first at t = 0.1)
+        // steps up to about 20 minutes: the arctangent's power series (the next term, t^16 / 17
+        // of the first, is 6e-18 of it at t = 0.1)
         const double t = be * c.sin_theta / (1.0 - be * c.omc), q = t * t;
         double p = -1.0 / 15.0;
         p = fma(p, q, 1.0 / 13.0);

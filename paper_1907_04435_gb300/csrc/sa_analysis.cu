@@ -109,10 +109,10 @@ __global__ void k_shadow_score(const int* __restrict__ steps, long long R, int n
 //
 // A first pass lists, per run of <= 16 consecutive steps of a block, the region's cells
 // with a shadowed step in it.  A CTA then takes 128 listed cells of one run (each warp alone
-// where the cells are far apart: contrib_by_fan) and walks the
-// BVH once for all of them (walk_group, as the ray-traced accrual does): the pairs of a
-// cell and a triangle that the run's rays may reach are tested exactly at each of the
-// cell's shadowed steps (Plucker form, with the distance).  Per cell and step the nearest
+// where the cells are far apart: contrib_by_fan) and walks the BVH once for all of them
+// (walk_group, as the ray-traced accrual does): the pairs of a cell and a triangle that the
+// run's rays may reach are tested exactly at each of the cell's shadowed steps (Plucker
+// form, with the distance).  Per cell and step the nearest
 // hit is kept in shared memory -- distance and triangle in one 64-bit key, so the minimum
 // does not depend on the order; equal distances go to the lower triangle index, as a walk
 // of the node list in its order gives -- and per cell and run a short list of kCastList

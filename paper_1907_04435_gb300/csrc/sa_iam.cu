@@ -3,7 +3,7 @@
 // Per block of K steps:
 //   k_iam_sources  every cell centre p traces toward the sun at the block's first step and
 //               keeps the L nearest intersections farther than 1 m (the paper's source
-//               levels and its 100 cm acne rule).
+//               levels and its 100 cm acne rule); k_iam_sources_warp for very coarse grids.
 //   k_iam_draw  each source s casts its shadow at step
 //               k at q_k, the projection of s along d_k onto the ground; the shadow line
 //               q_0 -> q_{K-1} is cut into K - 1 pieces and piece [q_k, q_{k+1}] sets bit

@@ -115,7 +115,8 @@ __device__ __forceinline__ bool faces_sun(const float3& n, const StepConst* step
 // tile range swept over the union of the blocks' slope boxes, with swept_tiles's own margin
 // (so a triangle it drops has no tile in any block).  A grid in the middle of a city is
 // reached by few: 1024^2 cells among 1.3M triangles, 132 blocks, 3 chunks of k_bin 1.25 ms
-// -> 0.27 in 2 and 16 us here; 231 x 187 cells, 92 days 3.38 -> 3.06 ms.
+// -> 0.27 in 2 and 16 us here, the whole call 8.43 -> 7.47; 231 x 187 cells among 60k, 92 days
+// 4.13 -> 3.79 ms.
 constexpr int kReachThreads = 256;
 __global__ void __launch_bounds__(kReachThreads)
 k_reach(DevScene sc, const BlockConst* __restrict__ blocks, int n_blocks, TileGeom g, unsigned* __restrict__ n,

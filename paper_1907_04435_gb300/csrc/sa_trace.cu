@@ -9,8 +9,8 @@
 //              geometry inside that wedge can shadow it in the run.  Each candidate
 //              triangle is tested exactly, per step (Plucker form).
 //   k_accrual_fan  the same with a warp's 32 receivers and whole blocks, a node entered when
-//              any receiver's own wedge overlaps it: for point sets so thin that a
-//              group's box holds far more than its rays.
+//              any receiver's own wedge overlaps it: for points so few for the triangles
+//              that a group's box holds far more than its rays (accrual_by_warps).
 //
 // The work is cut into items (TraceItems) that leave run summaries for launch_fold.
 // k_sweep (an option) and k_accrual_fan are warp-coherent: the 32 lanes of a warp hold
